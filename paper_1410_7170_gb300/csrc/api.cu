@@ -206,38 +206,60 @@ ovl_status Ctx::norm2_f(const float *x, double *out) {
     return fetch(d_scal, 1, out);
 }
 
-// Copy a boundary vector (host or device, lexicographic) into an internal FP64 eo vector.
-ovl_status Ctx::import_vec(const double *src, double2 *dst) {
+// Internal storage words per spinor.
+template <typename ST> static long spinor_words(const Geom &g);
+template <> long spinor_words<double2>(const Geom &g) { return 12L * g.V; }
+template <> long spinor_words<ffw>(const Geom &g) { return 12L * g.V; }
+template <> long spinor_words<float4>(const Geom &g) { return 6L * g.V; }
+
+// Waits for the stream; OVL_EINVAL (with the flags cleared) if an imported vector was not finite.
+ovl_status Ctx::check_finite() {
     Ctx *c = this;
-    const double *lex = src;
-    if (!is_device_ptr(src)) {
-        CK(cudaMemcpyAsync(io_lex, src, n64 * sizeof(double), cudaMemcpyHostToDevice, stream));
-        lex = io_lex;
-    }
-    CK(pack_spinor_f64(g, dst, lex, stream));
-    CK(cudaMemsetAsync(d_flag, 0, sizeof(int), stream));
-    CK(dev_nonfinite((const double *)dst, n64, d_flag, stream));
-    int h = 0;
-    CK(cudaMemcpyAsync(h_flag, d_flag, sizeof(int), cudaMemcpyDeviceToHost, stream));
     ST(sync());
-    h = *h_flag;
-    if (h) {
-        err = "input vector holds NaN or Inf";
-        return OVL_EINVAL;
-    }
-    return OVL_OK;
+    if (!*(volatile int *)h_flag) return OVL_OK;
+    *h_flag = 0;
+    CK(cudaMemsetAsync(d_flag, 0, sizeof(int), stream));
+    err = "input vector holds NaN or Inf";
+    return OVL_EINVAL;
 }
 
-ovl_status Ctx::export_vec(const double2 *src, double *dst) {
+// Boundary vectors (host or device, lexicographic, back to back) into internal even-odd spinors.
+template <typename ST>
+ovl_status Ctx::import_vec(const double *src, ST *dst, int n, bool check) {
     Ctx *c = this;
-    if (is_device_ptr(dst)) {
-        CK(unpack_spinor_f64(g, dst, src, stream));
-        return sync();
+    const long w = spinor_words<ST>(g);
+    const InputFlags bad{d_flag, h_flag};
+    if (is_device_ptr(src)) {
+        CK(spinor_in(g, dst, w, src, n, bad, stream));
+    } else {
+        for (int y = 0; y < n; y++) {
+            CK(cudaMemcpyAsync(io_lex, src + (size_t)y * n64, n64 * sizeof(double), cudaMemcpyHostToDevice, stream));
+            CK(spinor_in(g, dst + (size_t)y * w, w, io_lex, 1, bad, stream));
+        }
     }
-    CK(unpack_spinor_f64(g, io_lex, src, stream));
-    CK(cudaMemcpyAsync(dst, io_lex, n64 * sizeof(double), cudaMemcpyDeviceToHost, stream));
+    return check ? check_finite() : OVL_OK;
+}
+
+template <typename ST>
+ovl_status Ctx::export_vec(const ST *src, double *dst, int n, bool gate) {
+    Ctx *c = this;
+    const long w = spinor_words<ST>(g);
+    if (is_device_ptr(dst)) {
+        CK(spinor_out(g, dst, src, w, n, gate ? d_flag : nullptr, stream));
+        return gate ? check_finite() : sync();
+    }
+    if (gate) ST(check_finite());
+    for (int y = 0; y < n; y++) {
+        CK(spinor_out(g, io_lex, src + (size_t)y * w, w, 1, nullptr, stream));
+        CK(cudaMemcpyAsync(dst + (size_t)y * n64, io_lex, n64 * sizeof(double), cudaMemcpyDeviceToHost, stream));
+    }
     return sync();
 }
+// the forms other translation units use
+template ovl_status Ctx::import_vec<double2>(const double *, double2 *, int, bool);
+template ovl_status Ctx::import_vec<float4>(const double *, float4 *, int, bool);
+template ovl_status Ctx::export_vec<double2>(const double2 *, double *, int, bool);
+template ovl_status Ctx::export_vec<float4>(const float4 *, double *, int, bool);
 
 // ------------------------------------------------------------------ multishift sign
 // Zolotarev degree for a sign application of relative accuracy tol: the smallest n <=
@@ -1336,6 +1358,10 @@ static ovl_status check_ctx_ptrs(Ctx *c, const void *a, const void *b) {
     return OVL_OK;
 }
 
+// Whether the finite check of a call's input can be left to its end (import_vec): host buffers
+// are checked before anything is copied back into them.
+static bool on_device(const double *in, const double *out) { return is_device_ptr(in) && is_device_ptr(out); }
+
 extern "C" ovl_status wilson_apply(ovl_ctx *ctx, double *out, const double *in, double m0) {
     Ctx *c = reinterpret_cast<Ctx *>(ctx);
     ST(check_ctx_ptrs(c, out, in));
@@ -1343,9 +1369,10 @@ extern "C" ovl_status wilson_apply(ovl_ctx *ctx, double *out, const double *in, 
         c->err = "m0 must be finite";
         return OVL_EINVAL;
     }
-    ST(c->import_vec(in, c->io_a));
+    const bool late = on_device(in, out);
+    ST(c->import_vec(in, c->io_a, 1, !late));
     CK(wilson_f64(c->g, c->U64, c->io_a, c->io_b, m0, 0, 1.0, nullptr, 0.0, c->stream));
-    return c->export_vec(c->io_b, out);
+    return c->export_vec(c->io_b, out, 1, late);
 }
 
 static ovl_status check_tol(Ctx *c, double tol) {
@@ -1534,11 +1561,18 @@ extern "C" ovl_status wilson_solve(ovl_ctx *ctx, double *x, const double *b, dou
         ST(c->autotune_sap());
         c->sap_tuned = true;
     }
-    ST(c->import_vec(b, c->io_a));
     int it = 0;
-    ST(wilson_solve_eo(c, c->io_a, c->io_b, m0, tol, &it));
+    if (c->p.precision == OVL_FP64) {
+        ST(c->import_vec(b, c->io_a));
+        ST(wilson_solve_eo(c, c->io_a, c->io_b, m0, tol, &it));
+        if (iters) *iters = it;
+        return c->export_vec(c->io_b, x);
+    }
+    ST(ensure_f32_buffers(c));
+    ST(c->import_vec(b, (float4 *)c->f_a));
+    ST(wilson_solve_eo(c, (const float4 *)c->f_a, (float4 *)c->f_b, m0, tol, &it));
     if (iters) *iters = it;
-    return c->export_vec(c->io_b, x);
+    return c->export_vec((const float4 *)c->f_b, x);
 }
 
 extern "C" ovl_status wilson_sap_apply(ovl_ctx *ctx, double *out, const double *in, double m0) {
@@ -1563,9 +1597,16 @@ extern "C" ovl_status wilson_sap_apply(ovl_ctx *ctx, double *out, const double *
         ST(c->autotune_sap());
         c->sap_tuned = true;
     }
-    ST(c->import_vec(in, c->io_a));
-    ST(sap_apply_eo(c, c->io_a, c->io_b, m0));
-    return c->export_vec(c->io_b, out);
+    const bool late = on_device(in, out);
+    if (c->p.precision == OVL_FP64) {
+        ST(c->import_vec(in, c->io_a, 1, !late));
+        ST(sap_apply_eo(c, c->io_a, c->io_b, m0));
+        return c->export_vec(c->io_b, out, 1, late);
+    }
+    ST(ensure_f32_buffers(c));
+    ST(c->import_vec(in, (float4 *)c->f_a, 1, !late));
+    ST(sap_apply_eo(c, (const float4 *)c->f_a, (float4 *)c->f_b, m0));
+    return c->export_vec((const float4 *)c->f_b, out, 1, late);
 }
 
 // ------------------------------------------------------------------ operators in a chosen arithmetic
@@ -1581,33 +1622,31 @@ extern "C" ovl_status wilson_apply_arith(ovl_ctx *ctx, double *out, const double
         c->err = "wilson_apply_arith: need finite m0 and an ovl_arith value";
         return OVL_EINVAL;
     }
-    ST(c->import_vec(in, c->io_a));
-    const long w = (long)c->g.V * 12;
-    if (arith == OVL_ARITH_FP64) {
-        CK(wilson_f64(c->g, c->U64, c->io_a, c->io_b, m0, 0, 1.0, nullptr, 0.0, c->stream));
-    } else if (arith == OVL_ARITH_FF) {
+    if (arith == OVL_ARITH_FP64) return wilson_apply(ctx, out, in, m0);
+    const bool late = on_device(in, out);
+    if (arith == OVL_ARITH_FF) {
         ST(c->ensure_msff());
-        CK(dev_d2ff(c->io_a, c->msff.t, w, c->stream));
+        ST(c->import_vec(in, c->msff.t, 1, !late));
         CK(wilson_ff(c->g, c->Uff, c->msff.t, c->msff.y, m0, 0, 1.0, nullptr, 0.0, c->stream));
-        CK(dev_ff2d(c->msff.y, c->io_b, w, c->stream));
-    } else if (arith == OVL_ARITH_FP16 || arith == OVL_ARITH_BF16) {
-        // 16-bit links and spinors, FP32 arithmetic: FP64 -> FP32 -> 16 bits, stencil, and back
-        const bool bf = arith == OVL_ARITH_BF16;
-        ST(ensure_f32_buffers(c));
-        ST(c->ensure_16(bf));
-        CK(spinor_d2f(c->g, c->io_a, (float4 *)c->f_a, c->stream));
-        CK(spinor_f2h(c->g, (const float4 *)c->f_a, c->h16a, c->h16na, bf, c->stream));
-        CK(wilson_16(c->g, c->U16[bf ? 1 : 0], c->h16a, c->h16na, c->h16b, c->h16nb, (float)m0, bf, c->stream));
-        CK(spinor_h2f(c->g, c->h16b, c->h16nb, (float4 *)c->f_b, bf, c->stream));
-        CK(spinor_f2d(c->g, (const float4 *)c->f_b, c->io_b, c->stream));
-    } else {
-        ST(ensure_f32_buffers(c));
-        CK(spinor_d2f(c->g, c->io_a, (float4 *)c->f_a, c->stream));
-        CK(wilson_f32(c->g, c->U32, (const float4 *)c->f_a, (float4 *)c->f_b, (float)m0, 0, 1.f, nullptr, 0.f,
-                      c->stream));
-        CK(spinor_f2d(c->g, (const float4 *)c->f_b, c->io_b, c->stream));
+        return c->export_vec(c->msff.y, out, 1, late);
     }
-    return c->export_vec(c->io_b, out);
+    float4 *fa, *fb;
+    ST(ensure_f32_buffers(c));
+    fa = (float4 *)c->f_a;
+    fb = (float4 *)c->f_b;
+    if (arith == OVL_ARITH_FP32) {
+        ST(c->import_vec(in, fa, 1, !late));
+        CK(wilson_f32(c->g, c->U32, fa, fb, (float)m0, 0, 1.f, nullptr, 0.f, c->stream));
+    } else {
+        // 16-bit links and spinors, FP32 arithmetic: FP32 -> 16 bits, stencil, and back
+        const bool bf = arith == OVL_ARITH_BF16;
+        ST(c->ensure_16(bf));
+        ST(c->import_vec(in, fa, 1, !late));
+        CK(spinor_f2h(c->g, fa, c->h16a, c->h16na, bf, c->stream));
+        CK(wilson_16(c->g, c->U16[bf ? 1 : 0], c->h16a, c->h16na, c->h16b, c->h16nb, (float)m0, bf, c->stream));
+        CK(spinor_h2f(c->g, c->h16b, c->h16nb, fb, bf, c->stream));
+    }
+    return c->export_vec(fb, out, 1, late);
 }
 
 extern "C" ovl_status wilson_apply_n_arith(ovl_ctx *ctx, double *out, const double *in, int n_rhs, double m0,
@@ -1620,28 +1659,20 @@ extern "C" ovl_status wilson_apply_n_arith(ovl_ctx *ctx, double *out, const doub
         return OVL_EINVAL;
     }
     const int blk = std::min(kMaxBatch, n_rhs);
-    if (!c->xbat || c->xbat_cap < blk) {
-        void *buf;
-        ST(c->alloc(&buf, (size_t)c->n64 * sizeof(double) * 2 * blk));
-        c->xbat = (double2 *)buf;
-        c->bbat = c->xbat + (size_t)blk * c->g.V * 12;
-        c->xbat_cap = blk;
-    }
     if (!c->fbat || c->fbat_cap < blk) {
         void *buf;
         ST(c->alloc(&buf, (size_t)c->n64 * sizeof(float) * 2 * blk));
         c->fbat = (float *)buf;
         c->fbat_cap = blk;
     }
-    const long w = (long)c->g.V * 12, wf = (long)c->g.V * 6;
+    const long wf = (long)c->g.V * 6;
+    const bool late = on_device(in, out);
     float4 *fa = (float4 *)c->fbat, *fb = fa + (size_t)blk * wf;
     for (int r0 = 0; r0 < n_rhs; r0 += blk) {
         const int nb = std::min(blk, n_rhs - r0);
-        for (int y = 0; y < nb; y++) ST(c->import_vec(in + (size_t)(r0 + y) * c->n64, c->bbat + y * w));
-        CK(spinor_d2f_n(c, c->bbat, fa, nb));
+        ST(c->import_vec(in + (size_t)r0 * c->n64, fa, nb, !late));
         CK(wilson_batch_f32(c->g, c->U32, fa, fb, wf, nb, (float)m0, 0, 1.f, nullptr, 0.f, c->stream));
-        CK(spinor_f2d_n(c, fb, c->xbat, nb));
-        for (int y = 0; y < nb; y++) ST(c->export_vec(c->xbat + y * w, out + (size_t)(r0 + y) * c->n64));
+        ST(c->export_vec(fb, out + (size_t)r0 * c->n64, nb, late));
     }
     return OVL_OK;
 }
@@ -1654,21 +1685,18 @@ extern "C" ovl_status sign_apply_arith(ovl_ctx *ctx, double *out, const double *
         c->err = "sign_apply_arith: arith must be an ovl_arith value";
         return OVL_EINVAL;
     }
-    ST(c->import_vec(in, c->io_a));
     ovl_status st;
-    if (arith == OVL_ARITH_FP64) {
-        st = c->sign64(c->io_a, c->io_b, tol, 0);
-    } else if (arith == OVL_ARITH_FF) {
-        st = c->sign_ff(c->io_a, c->io_b, tol, 0);
+    if (arith == OVL_ARITH_FP64 || arith == OVL_ARITH_FF) {
+        ST(c->import_vec(in, c->io_a));
+        st = arith == OVL_ARITH_FP64 ? c->sign64(c->io_a, c->io_b, tol, 0) : c->sign_ff(c->io_a, c->io_b, tol, 0);
+        if (st == OVL_OK || st == OVL_ENOCONV) ST(c->export_vec(c->io_b, out));
     } else {
         ST(ensure_f32_buffers(c));
-        CK(spinor_d2f(c->g, c->io_a, (float4 *)c->f_a, c->stream));
+        ST(c->import_vec(in, (float4 *)c->f_a));
         st = c->sign32((const float4 *)c->f_a, (float4 *)c->f_b, tol, 0,
                        arith == OVL_ARITH_FP16 ? 1 : arith == OVL_ARITH_BF16 ? 2 : 0);
-        if (st == OVL_OK || st == OVL_ENOCONV) CK(spinor_f2d(c->g, (const float4 *)c->f_b, c->io_b, c->stream));
+        if (st == OVL_OK || st == OVL_ENOCONV) ST(c->export_vec((const float4 *)c->f_b, out));
     }
-    if (st != OVL_OK && st != OVL_ENOCONV) return st;
-    ST(c->export_vec(c->io_b, out));
     return st;
 }
 
@@ -1772,11 +1800,12 @@ extern "C" ovl_status wilson_apply_n(ovl_ctx *ctx, double *out, const double *in
     }
     const int blk = c->xbat_cap;
     const long w = (long)c->g.V * 12;
+    const bool late = on_device(in, out);
     for (int r0 = 0; r0 < n_rhs; r0 += blk) {
         const int nb = std::min(blk, n_rhs - r0);
-        for (int y = 0; y < nb; y++) ST(c->import_vec(in + (size_t)(r0 + y) * c->n64, c->bbat + y * w));
+        ST(c->import_vec(in + (size_t)r0 * c->n64, c->bbat, nb, !late));
         CK(wilson_batch_f64(c->g, c->U64, c->bbat, c->xbat, w, nb, m0, 0, 1.0, nullptr, 0.0, c->stream));
-        for (int y = 0; y < nb; y++) ST(c->export_vec(c->xbat + y * w, out + (size_t)(r0 + y) * c->n64));
+        ST(c->export_vec(c->xbat, out + (size_t)r0 * c->n64, nb, late));
     }
     return OVL_OK;
 }
@@ -1804,9 +1833,9 @@ extern "C" ovl_status ovl_apply_n(ovl_ctx *ctx, double *out, const double *in, i
     for (int y = 0; y < kMaxBatch; y++) t[y] = tol;
     for (int r0 = 0; r0 < n_rhs; r0 += blk) {
         const int nb = std::min(blk, n_rhs - r0);
-        for (int y = 0; y < nb; y++) ST(c->import_vec(in + (size_t)(r0 + y) * c->n64, c->bbat + y * w));
+        ST(c->import_vec(in + (size_t)r0 * c->n64, c->bbat, nb));
         ST(c->sign64_batch(c->bbat, c->xbat, nb, t, 1));
-        for (int y = 0; y < nb; y++) ST(c->export_vec(c->xbat + y * w, out + (size_t)(r0 + y) * c->n64));
+        ST(c->export_vec(c->xbat, out + (size_t)r0 * c->n64, nb));
     }
     return OVL_OK;
 }

@@ -142,10 +142,6 @@ __global__ void k_f2d(const float *__restrict__ x, double *__restrict__ y, long 
     for (long k = (long)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (long)gridDim.x * blockDim.x)
         y[k] = (double)x[k];
 }
-__global__ void k_nonfinite(const double *__restrict__ x, long n, int *flag) {
-    for (long k = (long)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (long)gridDim.x * blockDim.x)
-        if (!isfinite(x[k])) atomicExch(flag, 1);
-}
 
 inline int stream_grid(long n) {
     long b = (n + kBlock - 1) / kBlock;
@@ -253,11 +249,6 @@ cudaError_t dev_d2f(const double *x, float *y, long n, cudaStream_t st) {
 }
 cudaError_t dev_f2d(const float *x, double *y, long n, cudaStream_t st) {
     k_f2d<<<stream_grid(n), kBlock, 0, st>>>(x, y, n);
-    count_launches(1);
-    return cudaGetLastError();
-}
-cudaError_t dev_nonfinite(const double *x, long n, int *flag, cudaStream_t st) {
-    k_nonfinite<<<stream_grid(n), kBlock, 0, st>>>(x, n, flag);
     count_launches(1);
     return cudaGetLastError();
 }

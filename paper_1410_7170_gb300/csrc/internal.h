@@ -75,13 +75,20 @@ inline int plain_grid(long n_threads) {
 // sets *bad to 1 if some link misses unitarity or det = 1 by more than tol.
 cudaError_t pack_gauge(const Geom &g, const double *lex, double2 *u64, float4 *u32, int *bad, double tol,
                        cudaStream_t st);
-// lex spinor [s][12] complex doubles <-> internal even-odd layouts
-cudaError_t pack_spinor_f64(const Geom &g, double2 *dst, const double *lex, cudaStream_t st);
-cudaError_t unpack_spinor_f64(const Geom &g, double *lex, const double2 *src, cudaStream_t st);
+// n boundary vectors [V][12] complex doubles, back to back <-> even-odd spinors `stride` storage
+// words apart, ST = double2, float4 or ffw. Reading sets both flags of `bad` (if given) when a
+// component is NaN or Inf; writing does nothing if *skip (device memory, nullable) is set.
+struct InputFlags {
+    int *device, *host;   // host: pinned memory, written from the device
+};
+template <typename ST>
+cudaError_t spinor_in(const Geom &g, ST *dst, long stride, const double *lex, int n, InputFlags bad, cudaStream_t st);
+template <typename ST>
+cudaError_t spinor_out(const Geom &g, double *lex, const ST *src, long stride, int n, const int *skip, cudaStream_t st);
 
-// even-odd FP64 <-> FP32 spinor conversion
-cudaError_t spinor_d2f(const Geom &g, const double2 *a, float4 *b, cudaStream_t st);
-cudaError_t spinor_f2d(const Geom &g, const float4 *a, double2 *b, cudaStream_t st);
+// even-odd FP64 <-> FP32 conversion of n spinors back to back
+cudaError_t spinor_d2f(const Geom &g, const double2 *a, float4 *b, cudaStream_t st, int n = 1);
+cudaError_t spinor_f2d(const Geom &g, const float4 *a, double2 *b, cudaStream_t st, int n = 1);
 
 // ---------------------------------------------------------------- stencils
 // out = a * [gamma5] D_W(m0) in + b * z   (z may be NULL; then b is ignored)
@@ -139,8 +146,6 @@ cudaError_t dev_multiaxpy_f(const float *base, long stride, int m, const double 
                             cudaStream_t st);
 // x[k] = seeded pseudo-random values in [-1, 1) (a counter hash of k and the seed)
 cudaError_t fill_random_f32(float *x, long n, unsigned seed, cudaStream_t st);
-// Finite check of a flat array: *flag = 1 if some entry is NaN/Inf.
-cudaError_t dev_nonfinite(const double *x, long n, int *flag, cudaStream_t st);
 
 // ---------------------------------------------------------------- multishift CG
 // Device-side state of one multishift solve (Q^2 + sigma_l) x_l = b, l < n, with the

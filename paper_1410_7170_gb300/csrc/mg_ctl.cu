@@ -164,8 +164,7 @@ ovl_status mg_setup(Ctx *c, double m0, const double *start, int n_start) {
     for (int k = 0; k < nv; k++) {
         float4 *v = mg.P + k * vw;
         if (start) {
-            ST(c->import_vec(start + (size_t)k * c->n64, c->io_a));
-            CK(spinor_d2f(g, c->io_a, v, st));
+            ST(c->import_vec(start + (size_t)k * c->n64, v));
         } else {
             CK(fill_random_f32((float *)v, vw * 4, 0x51ed270bu + 7919u * (unsigned)k, st));
         }
@@ -321,12 +320,10 @@ extern "C" ovl_status wilson_mg_apply(ovl_ctx *ctx, double *out, const double *i
         ST(c->autotune_sap());
         c->sap_tuned = true;
     }
-    ST(c->import_vec(in, c->io_a));
     ST(ensure_f32_buffers(c));
-    CK(spinor_d2f(c->g, c->io_a, (float4 *)c->f_a, c->stream));
+    ST(c->import_vec(in, (float4 *)c->f_a));
     ST(mg_apply_f32(c, (const float4 *)c->f_a, (float4 *)c->f_b, m0));
-    CK(spinor_f2d(c->g, (const float4 *)c->f_b, c->io_b, c->stream));
-    return c->export_vec(c->io_b, out);
+    return c->export_vec((const float4 *)c->f_b, out);
 }
 
 extern "C" ovl_status ovl_mg_info(const ovl_ctx *ctx, int *nv, int *coarse_sites, int *last_coarse_steps,

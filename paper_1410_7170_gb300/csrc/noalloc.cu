@@ -137,9 +137,9 @@ extern "C" ovl_status wilson_apply_noalloc(double *out, const double *in, const 
     k_noalloc_pack_links<<<plain_grid(V * 4), kBlock, 0, st>>>(g, (const double2 *)gauge);
     count_launches(1);
     if ((e = cudaGetLastError()) != cudaSuccess ||
-        (e = pack_spinor_f64(g, pin, in, st)) != cudaSuccess ||
+        (e = spinor_in(g, pin, 0, in, 1, InputFlags{nullptr, nullptr}, st)) != cudaSuccess ||
         (e = wilson_f64(g, links, pin, pout, m0, 0, 1.0, nullptr, 0.0, st)) != cudaSuccess ||
-        (e = unpack_spinor_f64(g, out, pout, st)) != cudaSuccess) {
+        (e = spinor_out(g, out, pout, 0, 1, nullptr, st)) != cudaSuccess) {
         cudaGetLastError();
         return fail(OVL_ECUDA, std::string("wilson_apply_noalloc: ") + cudaGetErrorString(e));
     }

@@ -412,41 +412,33 @@ static ovl_status outer_precond(Ctx *c, const double *v, double *z) {
     return OVL_OK;
 }
 
-ovl_status wilson_solve_eo(Ctx *c, const double2 *b, double2 *x, double m0, double tol, int *iters) {
-    if (c->p.precision == OVL_FP64) return wilson_solve<double>(c, c->kry_wil64, (const double *)b, (double *)x, m0, tol, iters);
-    ST(ensure_f32_buffers(c));
-    CK(spinor_d2f(c->g, b, (float4 *)c->f_a, c->stream));
-    ST(wilson_solve<float>(c, c->kry_wil32, c->f_a, c->f_b, m0, tol, iters));
-    CK(spinor_f2d(c->g, (const float4 *)c->f_b, x, c->stream));
-    return OVL_OK;
+template <>
+ovl_status wilson_solve_eo<double2>(Ctx *c, const double2 *b, double2 *x, double m0, double tol, int *iters) {
+    return wilson_solve<double>(c, c->kry_wil64, (const double *)b, (double *)x, m0, tol, iters);
+}
+template <>
+ovl_status wilson_solve_eo<float4>(Ctx *c, const float4 *b, float4 *x, double m0, double tol, int *iters) {
+    return wilson_solve<float>(c, c->kry_wil32, (const float *)b, (float *)x, m0, tol, iters);
 }
 
 // One application of the Schwarz preconditioner, x = M_SAP b: params.sap_cycles red-black
 // cycles from x = 0 over params.sap_block blocks, params.sap_mr_iters MR steps per block
-// solve, on D_W(m0); FP64 even-odd spinors in and out, FP32 inside unless precision ==
-// OVL_FP64. The same call the Wilson FGMRES makes for its preconditioner.
-ovl_status sap_apply_eo(Ctx *c, const double2 *b, double2 *x, double m0) {
+// solve, on D_W(m0). The same call the Wilson FGMRES makes for its preconditioner.
+template <typename T>
+static ovl_status sap_apply_t(Ctx *c, const T *b, T *x, void *&scratch, double m0) {
     SapGeom sg = make_sap_geom(c->g, c->p.sap_block);
     sg.tps = c->sap_tps;
-    if (c->p.precision == OVL_FP64) {
-        if (!c->sap_r64) {
-            void *buf;
-            ST(c->alloc(&buf, (size_t)c->n64 * sizeof(double)));
-            c->sap_r64 = buf;
-        }
-        CK(Ops<double>::sap(c, sg, (const double *)b, (double *)x, (double *)c->sap_r64, m0));
-        return OVL_OK;
-    }
-    ST(ensure_f32_buffers(c));
-    if (!c->sap_r32) {
-        void *buf;
-        ST(c->alloc(&buf, (size_t)c->n64 * sizeof(float)));
-        c->sap_r32 = buf;
-    }
-    CK(spinor_d2f(c->g, b, (float4 *)c->f_a, c->stream));
-    CK(Ops<float>::sap(c, sg, c->f_a, c->f_b, (float *)c->sap_r32, m0));
-    CK(spinor_f2d(c->g, (const float4 *)c->f_b, x, c->stream));
+    if (!scratch) ST(c->alloc(&scratch, (size_t)c->n64 * sizeof(T)));
+    CK(Ops<T>::sap(c, sg, b, x, (T *)scratch, m0));
     return OVL_OK;
+}
+template <>
+ovl_status sap_apply_eo<double2>(Ctx *c, const double2 *b, double2 *x, double m0) {
+    return sap_apply_t<double>(c, (const double *)b, (double *)x, c->sap_r64, m0);
+}
+template <>
+ovl_status sap_apply_eo<float4>(Ctx *c, const float4 *b, float4 *x, double m0) {
+    return sap_apply_t<float>(c, (const float *)b, (float *)x, c->sap_r32, m0);
 }
 
 int batch_size_for(Ctx *c, int want);
@@ -493,10 +485,8 @@ ovl_status solve_all(Ctx *c, double *x, const double *b, int n_rhs, double tol, 
         }
         for (int r0 = 0; r0 < n_rhs; r0 += nbmax) {
             const int nb = std::min(nbmax, n_rhs - r0);
-            for (int y = 0; y < nb; y++) {
-                ST(c->import_vec(b + (size_t)(r0 + y) * c->n64, c->bbat + (size_t)y * c->g.V * 12));
-                ST(c->import_vec(x + (size_t)(r0 + y) * c->n64, c->xbat + (size_t)y * c->g.V * 12));
-            }
+            ST(c->import_vec(b + (size_t)r0 * c->n64, c->bbat, nb, false));
+            ST(c->import_vec(x + (size_t)r0 * c->n64, c->xbat, nb));   // checks both
             int its;
             double wr;
             bool cv;
@@ -504,7 +494,7 @@ ovl_status solve_all(Ctx *c, double *x, const double *b, int n_rhs, double tol, 
             outer_total += its;
             worst = std::max(worst, wr);
             all_conv = all_conv && cv;
-            for (int y = 0; y < nb; y++) ST(c->export_vec(c->xbat + (size_t)y * c->g.V * 12, x + (size_t)(r0 + y) * c->n64));
+            ST(c->export_vec(c->xbat, x + (size_t)r0 * c->n64, nb));
         }
         n_rhs = 0;   // done; fall through to the statistics
     }
@@ -520,8 +510,8 @@ ovl_status solve_all(Ctx *c, double *x, const double *b, int n_rhs, double tol, 
     for (int r = 0; r < n_rhs; r++) {
         const double *br = b + (size_t)r * c->n64;
         double *xr = x + (size_t)r * c->n64;
-        ST(c->import_vec(br, c->d_b));
-        ST(c->import_vec(xr, c->d_x));
+        ST(c->import_vec(br, c->d_b, 1, false));
+        ST(c->import_vec(xr, c->d_x));   // checks both
         double xx;
         ST(c->norm2_d((const double *)c->d_x, &xx));
         // D_N in FP64; in the mixed modes, a relaxed product whose requested accuracy is
@@ -586,22 +576,6 @@ ovl_status solve_all(Ctx *c, double *x, const double *b, int n_rhs, double tol, 
 // A system that has converged is dropped from the Gram-Schmidt work and its operator
 // applications are skipped inside the batched calls (tolerance <= 0).
 // ====================================================================================
-// nb FP64 <-> FP32 internal spinors back to back
-cudaError_t spinor_d2f_n(Ctx *c, const double2 *a, float4 *b, int nb) {
-    for (int y = 0; y < nb; y++) {
-        cudaError_t e = spinor_d2f(c->g, a + (long)y * c->g.V * 12, b + (long)y * c->g.V * 6, c->stream);
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
-}
-cudaError_t spinor_f2d_n(Ctx *c, const float4 *a, double2 *b, int nb) {
-    for (int y = 0; y < nb; y++) {
-        cudaError_t e = spinor_f2d(c->g, a + (long)y * c->g.V * 6, b + (long)y * c->g.V * 12, c->stream);
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
-}
-
 namespace {
 
 // Zero the input rows of systems that are not iterating, so a nested batched solve
@@ -954,9 +928,9 @@ ovl_status solve_batch(Ctx *c, double2 *x, const double2 *b, int nb, double tol,
             if (t[y] > 0 && (relv[y] < 0 || t[y] < low_ok)) low = false;
         }
         if (low) {
-            CK(spinor_d2f_n(c, (const double2 *)a, (float4 *)fa, nb));
+            CK(spinor_d2f(c->g, (const double2 *)a, (float4 *)fa, c->stream, nb));
             ST(c->sign32_batch((const float4 *)fa, (float4 *)fb, nb, t, 1));
-            CK(spinor_f2d_n(c, (const float4 *)fb, (double2 *)o, nb));
+            CK(spinor_f2d(c->g, (const float4 *)fb, (double2 *)o, c->stream, nb));
             return OVL_OK;
         }
         return c->sign_outer_batch((const double2 *)a, (double2 *)o, nb, t, 1);
@@ -970,11 +944,11 @@ ovl_status solve_batch(Ctx *c, double2 *x, const double2 *b, int nb, double tol,
             CK(cudaMemcpyAsync(o, a, (size_t)nb * n * sizeof(double), cudaMemcpyDeviceToDevice, c->stream));
             return OVL_OK;
         }
-        CK(spinor_d2f_n(c, (const double2 *)a, (float4 *)fa, nb));
+        CK(spinor_d2f(c->g, (const double2 *)a, (float4 *)fa, c->stream, nb));
         CK(zero_inactive<float>(c, fa, nb, act));
         if (c->p.precond == OVL_PREC_WILSON) ST(wilson_solve_batch<float>(c, nb, fa, fb, c->m0_prec, c->p.eps_prec, act));
         else ST(inner(fa, fb, act));
-        CK(spinor_f2d_n(c, (const float4 *)fb, (double2 *)o, nb));
+        CK(spinor_f2d(c->g, (const float4 *)fb, (double2 *)o, c->stream, nb));
         return OVL_OK;
     };
     // x holds the initial guesses; start from zero when all of them are zero

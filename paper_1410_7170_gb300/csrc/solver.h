@@ -198,8 +198,16 @@ struct Ctx {
     ovl_status fetch(const double *d, int n, double *h);
     ovl_status norm2_d(const double *x, double *out);
     ovl_status norm2_f(const float *x, double *out);
-    ovl_status import_vec(const double *src, double2 *dst);
-    ovl_status export_vec(const double2 *src, double *dst);
+    // n boundary vectors into internal spinors and back, ST = double2, float4 or ffw. import_vec
+    // with check = true waits and returns OVL_EINVAL for NaN or Inf. With check = false (device
+    // memory on both sides) the answer is left to the export_vec of the same call: with gate =
+    // true that writes nothing and returns OVL_EINVAL if an input since the last check was not
+    // finite, so that the call waits for the GPU once, at its end.
+    template <typename ST>
+    ovl_status import_vec(const double *src, ST *dst, int n = 1, bool check = true);
+    template <typename ST>
+    ovl_status export_vec(const ST *src, double *dst, int n = 1, bool gate = false);
+    ovl_status check_finite();
     int pick_poles(double tol) const;
     void fill_poles(MsState &s, int n, double tol) const;
     ovl_status ms_setup(MsState *d_state, double tol, int *n_out);
@@ -264,16 +272,15 @@ ovl_status upload_coef(Ctx *c, const std::vector<std::complex<double>> &v);
 ovl_status solve_all(Ctx *c, double *x, const double *b, int n_rhs, double tol, ovl_stats *stats);
 // FP32 conversion buffers f_a, f_b (one spinor each), allocated on first use
 ovl_status ensure_f32_buffers(Ctx *c);
-// FP64 <-> FP32 even-odd conversion of nb spinors back to back
-cudaError_t spinor_d2f_n(Ctx *c, const double2 *a, float4 *b, int nb);
-cudaError_t spinor_f2d_n(Ctx *c, const float4 *a, double2 *b, int nb);
 // Lock-step batched solve of nrhs <= kMaxBatch systems on internal FP64 vectors.
 ovl_status solve_batch(Ctx *c, double2 *x, const double2 *b, int nrhs, double tol, int *outer_iters,
                        double *worst_res, bool *all_conv);
-// Inexact Wilson solve on FP64 even-odd spinors (FP32 inside unless precision == FP64).
-ovl_status wilson_solve_eo(Ctx *c, const double2 *b, double2 *x, double m0, double tol, int *iters);
-// One Schwarz preconditioner application x = M_SAP b on FP64 even-odd spinors.
-ovl_status sap_apply_eo(Ctx *c, const double2 *b, double2 *x, double m0);
+// Inexact Wilson solve on even-odd spinors, in their precision (ST = double2 or float4).
+template <typename ST>
+ovl_status wilson_solve_eo(Ctx *c, const ST *b, ST *x, double m0, double tol, int *iters);
+// One Schwarz preconditioner application x = M_SAP b on even-odd spinors, in their precision.
+template <typename ST>
+ovl_status sap_apply_eo(Ctx *c, const ST *b, ST *x, double m0);
 // Two-level multigrid for D_W(m0) (mg_ctl.cu): setup from n_start start vectors (boundary
 // layout; NULL = seeded pseudo-random ones), and one preconditioner application on FP32
 // even-odd spinors (the setup is made, or remade for a new m0, first).
