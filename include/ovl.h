@@ -119,7 +119,7 @@ typedef struct {
                                fastest measured at 16^4 with 12 right-hand sides; 1 = one after another) */
     int use_graphs;         /* 1: capture multishift iterations in CUDA graphs */
     int check_every;        /* multishift iterations between host convergence checks */
-    int stencil_tps;        /* threads per lattice site of the stencils: 0 = autotune, 1 or 4 = forced */
+    int stencil_tps;        /* threads per lattice site of the FP32 stencils: 0 = autotune, 1 or 4 = forced */
     int sap_tps;            /* threads per block site of the FP32 Schwarz block solves: 0 = autotune, 1, 2 or 4 */
     int adaptive_poles;     /* 1 (default): each sign application uses the smallest Zolotarev degree
                                n <= n_poles whose uniform error delta(k, n) is <= 1/10 of its requested
@@ -232,9 +232,10 @@ ovl_status wilson_solve(ovl_ctx *ctx, double *x, const double *b, double m0, dou
  * sap_cycles or sap_mr_iters < 1. */
 ovl_status wilson_sap_apply(ovl_ctx *ctx, double *out, const double *in, double m0);
 
-/* Stencil variant chosen by the autotuner (threads per site, 1 or 4, for FP64 and FP32)
- * and the measured ms per full-lattice stencil application of each variant
- * (ms[0..3] = FP64 x1, FP64 x4, FP32 x1, FP32 x4; zeros when forced). Nullable outputs. */
+/* FP32 stencil variant chosen by the autotuner (threads per site, 1 or 4) and the measured ms
+ * per full-lattice stencil application of each variant (ms[2], ms[3] = FP32 x1, x4). The FP64
+ * stencil is one kernel (a warp per hop) at every size: *tps64 is 1, ms[0] = ms[1] its time. All
+ * ms are zero when the variant is forced. Nullable outputs. */
 ovl_status ovl_tuning(const ovl_ctx *ctx, int *tps64, int *tps32, float *ms);
 
 /* FP32 multi-RHS stencil kernels chosen for this lattice shape (params.mrhs_kernel numbering,
@@ -374,7 +375,7 @@ ovl_status ovl_prof_get(ovl_ctx *ctx, ovl_prof *out, int reset);
  * --------------------------------------------------------------------------------- */
 
 /* out = D_W(m0) in (Eq. Wilson-Dirac) in any ovl_arith, with the context's stencil variant
- * (params.stencil_tps for FP64 and FP32; float-float and 16-bit always 1 thread per site). The
+ * (params.stencil_tps for FP32; FP64 and float-float one warp per hop, 16-bit 1 thread per site). The
  * 16-bit stencil reads 200 B per site in FP16 (192 B in BF16) against 384 B in FP32. */
 ovl_status wilson_apply_arith(ovl_ctx *ctx, double *out, const double *in, double m0, int arith);
 

@@ -355,7 +355,8 @@ def wilson_solve(ctx, x, b, m0, tol):
 
 
 def ovl_tuning(ctx):
-    """Stencil threads per site chosen by the autotuner (FP64, FP32) and the timed variants (ms)."""
+    """Threads per site of the FP32 stencil chosen by the autotuner (tps64 is 1: one FP64 kernel)
+    and the timed variants (ms: FP64 twice, FP32 with 1 and 4)."""
     import numpy as np
     a, b = ctypes.c_int(), ctypes.c_int()
     ms = np.zeros(4, dtype=np.float32)

@@ -303,6 +303,9 @@ void Ctx::fill_poles(MsState &s, int n, double tol) const {
         s.zeta_prev[l] = 1.0;
         s.active[l] = 1;
     }
+    const ff s0(s.sigma[0]);
+    s.sigma0_f[0] = s0.hi;
+    s.sigma0_f[1] = s0.lo;
 }
 
 // Fills the multishift state for tolerance tol and uploads it; *n_out = the degree used.
@@ -462,11 +465,10 @@ ovl_status Ctx::sign_ff(const double2 *b, double2 *out, double tol, int mode) {
         ST(defl_project64(b, defl_tmp64, dc));
         bm = defl_tmp64;
     }
-    const long words = (long)g.V * 12;
     int n;
     ST(ms_setup(msff_state, tol, &n));
     // b in float-float into t (t is overwritten by the first iteration's Q p)
-    CK(dev_d2ff(bm, msff.t, words, stream));
+    CK(spinor_d2ff(g, bm, msff.t, stream));
     CK(ms_init_ff(g, n, msff_state, msff, msff.t, rs, stream));
     int iters = 0;
     auto fn = [&](cudaEvent_t *e, unsigned f) { return ms_iter_ff(g, Uff, m0_ker, msff_state, msff, rs, stream, e, f); };
@@ -476,8 +478,8 @@ ovl_status Ctx::sign_ff(const double2 *b, double2 *out, double tol, int mode) {
     const double sc = zs_d0[n - 1] / lam_min;
     // s = (d0/lmin) [gamma5] D_W y in float-float, then FP64; D_N b = rho b + s without gamma5
     CK(wilson_ff(g, Uff, msff.y, msff.t, m0_ker, mode == 0, sc, nullptr, 0.0, stream));
-    CK(dev_ff2d(msff.t, out, words, stream));
-    if (mode == 1) CK(dev_axpby(rho, (const double *)b, 1.0, (double *)out, 2 * words, stream));
+    CK(spinor_ff2d(g, msff.t, out, stream));
+    if (mode == 1) CK(dev_axpby(rho, (const double *)b, 1.0, (double *)out, n64, stream));
     if (ndefl) ST(defl_add64(dc, out, mode));
     return ms;
 }
@@ -486,8 +488,8 @@ ovl_status Ctx::ensure_ff_links() {
     Ctx *c = this;
     if (Uff) return OVL_OK;
     const long words = (long)g.V * 4 * kLink64Words;
-    ST(alloc((void **)&Uff, (size_t)words * sizeof(ffw)));
-    CK(dev_d2ff(U64, Uff, words, stream));
+    ST(alloc((void **)&Uff, (size_t)words * sizeof(ffl)));
+    CK(links_d2ff(U64, Uff, words, stream));
     return OVL_OK;
 }
 
@@ -725,7 +727,7 @@ ovl_status Ctx::sign64_batch(const double2 *b, double2 *out, int nrhs, const dou
         msb64_cap = nrhs;
     }
     long iters = 0;
-    auto init = [&]() { return msb_init_f64(g, nrhs, npole, msb_state, msb64, b, rsb, stream); };
+    auto init = [&]() { return msb_init_f64(g, nrhs, npole, msb_state, msb64, b, rsb, bcounters, stream); };
     auto it = [&]() { return msb_iter_f64(g, U64, m0_ker, nrhs, npole, msb_state, msb64, rsb, bcounters, stream); };
     const int n = pick_poles(min_positive(tol, nrhs));
     ST((msb_run<double2>(nrhs, tol, n, 3, init, it, &iters)));
@@ -924,12 +926,12 @@ ovl_status Ctx::sigma_min_estimate(double *smin) {
 }
 
 // ------------------------------------------------------------------ autotuner
-// Threads per site of the stencils (1 or 4) for this lattice shape: both variants of
-// each precision are timed with CUDA events on the context's stream and the faster is
-// kept. Results are cached per process and shape.
+// Threads per site of the FP32 stencil (1 or 4) for this lattice shape: both variants are timed
+// with CUDA events on the context's stream and the faster is kept; the FP64 stencil (one kernel
+// for all sizes) is timed beside them. Results are cached per process and shape.
 static std::mutex g_tune_mu;
 struct TuneEntry {
-    int tps64, tps32;
+    int tps32;
     float ms[4];
 };
 static std::map<std::tuple<int, int, int, int>, TuneEntry> g_tune_cache;
@@ -941,7 +943,6 @@ ovl_status Ctx::autotune() {
         std::lock_guard<std::mutex> lk(g_tune_mu);
         auto it = g_tune_cache.find(key);
         if (it != g_tune_cache.end()) {
-            g.tps64 = it->second.tps64;
             g.tps32 = it->second.tps32;
             for (int k = 0; k < 4; k++) tune_ms[k] = it->second.ms[k];
             return OVL_OK;
@@ -956,30 +957,25 @@ ovl_status Ctx::autotune() {
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
     const int reps = g.V >= (1 << 20) ? 5 : 20;
-    float best[2][2];
-    for (int prec = 0; prec < 2; prec++) {
-        for (int v = 0; v < 2; v++) {
-            const int tps = v == 0 ? 1 : 4;
-            Geom gg = g;
-            gg.tps64 = gg.tps32 = tps;
-            for (int k = 0; k < 3 + reps; k++) {
-                if (k == 3) CK(cudaEventRecord(e0, stream));
-                if (prec == 0) CK(wilson_f64(gg, U64, io_a, io_b, m0_ker, 0, 1.0, nullptr, 0.0, stream));
-                else CK(wilson_f32(gg, U32, fa, fb, (float)m0_ker, 0, 1.f, nullptr, 0.f, stream));
-            }
-            CK(cudaEventRecord(e1, stream));
-            CK(cudaEventSynchronize(e1));
-            CK(cudaEventElapsedTime(&best[prec][v], e0, e1));
+    float best[3];   // FP64, FP32 with 1 and with 4 threads per site
+    for (int v = 0; v < 3; v++) {
+        Geom gg = g;
+        gg.tps32 = v == 2 ? 4 : 1;
+        for (int k = 0; k < 3 + reps; k++) {
+            if (k == 3) CK(cudaEventRecord(e0, stream));
+            if (v == 0) CK(wilson_f64(gg, U64, io_a, io_b, m0_ker, 0, 1.0, nullptr, 0.0, stream));
+            else CK(wilson_f32(gg, U32, fa, fb, (float)m0_ker, 0, 1.f, nullptr, 0.f, stream));
         }
+        CK(cudaEventRecord(e1, stream));
+        CK(cudaEventSynchronize(e1));
+        CK(cudaEventElapsedTime(&best[v], e0, e1));
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    g.tps64 = best[0][1] < best[0][0] ? 4 : 1;
-    g.tps32 = best[1][1] < best[1][0] ? 4 : 1;
-    tune_ms[0] = best[0][0] / reps;
-    tune_ms[1] = best[0][1] / reps;
-    tune_ms[2] = best[1][0] / reps;
-    tune_ms[3] = best[1][1] / reps;
+    g.tps32 = best[2] < best[1] ? 4 : 1;
+    tune_ms[0] = tune_ms[1] = best[0] / reps;
+    tune_ms[2] = best[1] / reps;
+    tune_ms[3] = best[2] / reps;
     {
         // first writer wins: a context of the same shape that finished tuning first (for
         // instance concurrently in the serving loop) has fixed the variant for the whole
@@ -988,11 +984,10 @@ ovl_status Ctx::autotune() {
         std::lock_guard<std::mutex> lk(g_tune_mu);
         auto it = g_tune_cache.find(key);
         if (it != g_tune_cache.end()) {
-            g.tps64 = it->second.tps64;
             g.tps32 = it->second.tps32;
             for (int k = 0; k < 4; k++) tune_ms[k] = it->second.ms[k];
         } else {
-            g_tune_cache[key] = TuneEntry{g.tps64, g.tps32, {tune_ms[0], tune_ms[1], tune_ms[2], tune_ms[3]}};
+            g_tune_cache[key] = TuneEntry{g.tps32, {tune_ms[0], tune_ms[1], tune_ms[2], tune_ms[3]}};
         }
     }
     cudaFree(buf);
@@ -1186,10 +1181,7 @@ static ovl_status create_impl(Ctx *c, const double *gauge, const int dims[4], do
         c->err = "lattice too large";
         return OVL_EINVAL;
     }
-    for (int m = 0; m < 4; m++) c->g.L[m] = dims[m];
-    c->g.V = (int)V;
-    c->g.Vh = (int)(V / 2);
-    c->g.Lh3 = dims[3] / 2;
+    c->g.set_dims(dims);
     c->g.antiperiodic = c->p.antiperiodic;
     {
         int dev = 0, nsm = 0;
@@ -1266,8 +1258,8 @@ static ovl_status create_impl(Ctx *c, const double *gauge, const int dims[4], do
         c->err = "gauge field: some link is not SU(3) to 1e-10 (or holds NaN)";
         return OVL_EINVAL;
     }
-    c->g.tps64 = c->g.tps32 = 1;
-    if (c->p.stencil_tps) c->g.tps64 = c->g.tps32 = c->p.stencil_tps;
+    c->g.tps32 = 1;
+    if (c->p.stencil_tps) c->g.tps32 = c->p.stencil_tps;
     else ST(c->autotune());
     if (c->p.mrhs_kernel) c->g.mrhs32 = c->g.mrhs32l = c->p.mrhs_kernel;
     else ST(c->autotune_mrhs());
@@ -1461,7 +1453,7 @@ extern "C" ovl_status ovl_prof_get(ovl_ctx *ctx, ovl_prof *out, int reset) {
 extern "C" ovl_status ovl_tuning(const ovl_ctx *ctx, int *tps64, int *tps32, float *ms) {
     const Ctx *c = reinterpret_cast<const Ctx *>(ctx);
     if (!c) return OVL_EINVAL;
-    if (tps64) *tps64 = c->g.tps64;
+    if (tps64) *tps64 = 1;
     if (tps32) *tps32 = c->g.tps32;
     if (ms)
         for (int k = 0; k < 4; k++) ms[k] = c->tune_ms[k];

@@ -63,12 +63,36 @@ struct Geom {
     int Vh;     // V / 2
     int V;
     int antiperiodic;
-    int tps64, tps32;   // threads per site of the FP64 / FP32 stencils (1 or 4), chosen by the autotuner
+    int tps32;          // threads per site of the FP32 stencils (1 or 4), chosen by the autotuner
     int mrhs32;         // FP32 multi-RHS stencil kernel for <= 6 right-hand sides (1 RHS pairs, 2 tiles of 32
                         // sites, 3 staged links); mrhs32l for 7..12
     int mrhs32l;
     int nsm;            // streaming multiprocessors of the device (grid sizing)
+    unsigned inv[3];    // floor((2^32 - 1) / d) for d = L1, L2, L3 / 2 (div_mod)
+
+    void set_dims(const int dims[4]) {
+        for (int m = 0; m < 4; m++) L[m] = dims[m];
+        V = dims[0] * dims[1] * dims[2] * dims[3];
+        Vh = V / 2;
+        Lh3 = dims[3] / 2;
+        inv[0] = 0xffffffffu / (unsigned)L[1];
+        inv[1] = 0xffffffffu / (unsigned)L[2];
+        inv[2] = 0xffffffffu / (unsigned)Lh3;
+    }
 };
+
+// n / d and n % d for 0 <= n < 2^31 with inv = floor((2^32 - 1) / d): the product's high word is
+// the quotient or one less. A run-time integer division costs about 25 instructions, and a
+// stencil's site coordinates take three of them (10% of the instructions of the float-float one).
+__device__ __forceinline__ int div_mod(int n, int d, unsigned inv, int &rem) {
+    int q = (int)__umulhi((unsigned)n, inv);
+    rem = n - q * d;
+    if (rem >= d) {
+        rem -= d;
+        q++;
+    }
+    return q;
+}
 
 // Site visited by thread t of a full-lattice kernel: parities interleave (t even: even
 // site, t odd: odd site, same checkerboard index), so the two sites that read a link
@@ -81,12 +105,10 @@ __device__ __forceinline__ void site_of_thread(int t, int &p, int &i) {
 
 // Coordinates of checkerboard site (p, i).
 __device__ __forceinline__ void eo_coords(const Geom &g, int p, int i, int x[4]) {
-    int x3h = i % g.Lh3;
-    int r = i / g.Lh3;
-    x[2] = r % g.L[2];
-    r /= g.L[2];
-    x[1] = r % g.L[1];
-    x[0] = r / g.L[1];
+    int x3h;
+    int r = div_mod(i, g.Lh3, g.inv[2], x3h);
+    r = div_mod(r, g.L[2], g.inv[1], x[2]);
+    x[0] = div_mod(r, g.L[1], g.inv[0], x[1]);
     int b = (p + x[0] + x[1] + x[2]) & 1;
     x[3] = 2 * x3h + b;
 }

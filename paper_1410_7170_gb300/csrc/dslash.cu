@@ -1,4 +1,5 @@
 // Layout conversion and the Wilson-Dirac stencil kernels (Eq. Wilson-Dirac).
+#include "hops.cuh"
 #include "internal.h"
 #include "reduce.cuh"
 #include "wilson_quad.cuh"
@@ -131,12 +132,17 @@ template <> struct IoWord<float4> {
 };
 template <> struct IoWord<ffw> {
     static constexpr int N = 12;
+    // word j: real (j even) or imaginary part of one colour of two spins; its two complex numbers
+    __device__ static int first(int j) { return j < 6 ? j >> 1 : 3 + (j >> 1); }
     __device__ static ffw get(const double2 *v, int j) {
-        const ff re(v[j].x), im(v[j].y);
-        return ffw{re.hi, re.lo, im.hi, im.lo};
+        const double2 x = v[first(j)], y = v[first(j) + 3];
+        const ff a(j & 1 ? x.y : x.x), b(j & 1 ? y.y : y.x);
+        return ffw{a.hi, b.hi, a.lo, b.lo};
     }
     __device__ static void put(double2 *v, int j, ffw w) {
-        v[j] = make_double2(ff(w.rh, w.rl).to_double(), ff(w.ih, w.il).to_double());
+        double *x = reinterpret_cast<double *>(v + first(j)) + (j & 1);
+        x[0] = ff(w.h0, w.l0).to_double();
+        x[6] = ff(w.h1, w.l1).to_double();
     }
 };
 
@@ -144,10 +150,9 @@ __device__ __forceinline__ int io_row(int s) { return ((s >> 1) + (kIoTile / 2) 
 // parity of x0 + x1 + x2 at checkerboard index i: site (p, i) is lexicographic site
 // 2 i + ((p + this) & 1)
 __device__ __forceinline__ int io_row_parity(const Geom &g, int i) {
-    int r = i / g.Lh3;
-    const int x2 = r % g.L[2];
-    r /= g.L[2];
-    return (x2 + r % g.L[1] + r / g.L[1]) & 1;
+    int x3h, x2, x1;
+    const int r = div_mod(i, g.Lh3, g.inv[2], x3h), q = div_mod(r, g.L[2], g.inv[1], x2);
+    return (div_mod(q, g.L[1], g.inv[0], x1) + x1 + x2) & 1;
 }
 
 // bad: flags set when a component is NaN or Inf (device memory, and the host's copy), or NULL
@@ -336,18 +341,44 @@ __global__ void __launch_bounds__(kBlock, MinBlocks<R>::value) k_wilson4(Geom g,
     }
 }
 
-cudaError_t wilson_f64(const Geom &g, const double2 *U, const double2 *in, double2 *out, double m0, int g5,
-                       double a, const double2 *z, double b, cudaStream_t st) {
-    if (g.tps64 == 4)
-        k_wilson4<double, double2, double2><<<plain_grid(4L * g.V), kBlock, 0, st>>>(g, U, in, out, m0 + 4.0, g5,
-                                                                                     a, z, b);
-    else {
-        const LaunchShape ls = balanced_shape(g.V, g.nsm, MinBlocks<double>::value, 1 << 30);
-        k_wilson<double, double2, double2><<<ls.grid, ls.block, 0, st>>>(g, U, in, out, m0 + 4.0, g5, a, z, b,
-                                                                         ls.spb);
-    }
+// out = a [g5] D_W(m0) in + b z in FP64 or float-float, one warp per hop (hops.cuh); blockIdx.y =
+// right-hand side, vectors `stride` words apart.
+template <typename R>
+__global__ void __launch_bounds__(kHopBlock, HopBlocks<R>::value)
+    k_wilson_hops(Geom g, const typename HopTiles<R>::Link *__restrict__ U,
+                  const typename HopTiles<R>::Store *__restrict__ in, typename HopTiles<R>::Store *__restrict__ out,
+                  long stride, R m4, int g5, R a, const typename HopTiles<R>::Store *z, R b) {
+    using H = HopTiles<R>;
+    in += blockIdx.y * stride;
+    out += blockIdx.y * stride;
+    if (z) z += blockIdx.y * stride;
+    const auto fm = H::factor(m4), fa = H::factor(a), fb = H::factor(b);
+    hop_tiles<R>(g, blockIdx.x, gridDim.x, U, in, [&](int p, int i, int it, int e, typename H::Elem hop) {
+        typename H::Elem r = H::fma(fm, H::load(in, g.Vh, p, i, it, e), hop);
+        r = H::mul(fa, H::neg_if(r, g5 && H::upper(it)));
+        if (z) r = H::fma(fb, H::load(z, g.Vh, p, i, it, e), r);
+        H::store(out, g.Vh, p, i, it, e, r);
+    });
+}
+template <typename R, typename LT, typename ST>
+static cudaError_t wilson_hops(const Geom &g, const LT *U, const ST *in, ST *out, long stride, int n, double m0, int g5,
+                               double a, const ST *z, double b, cudaStream_t st) {
+    k_wilson_hops<R><<<dim3(hop_grid<R>(g, n, false), n), kHopBlock, 0, st>>>(g, U, in, out, stride, R(m0 + 4.0), g5,
+                                                                               R(a), z, R(b));
     count_launches(1);
     return cudaGetLastError();
+}
+cudaError_t wilson_f64(const Geom &g, const double2 *U, const double2 *in, double2 *out, double m0, int g5,
+                       double a, const double2 *z, double b, cudaStream_t st) {
+    return wilson_hops<double>(g, U, in, out, 0, 1, m0, g5, a, z, b, st);
+}
+cudaError_t wilson_batch_f64(const Geom &g, const double2 *U, const double2 *in, double2 *out, long stride, int nrhs,
+                             double m0, int g5, double a, const double2 *z, double b, cudaStream_t st) {
+    return wilson_hops<double>(g, U, in, out, stride, nrhs, m0, g5, a, z, b, st);
+}
+cudaError_t wilson_ff(const Geom &g, const ffl *U, const ffw *in, ffw *out, double m0, int g5, double a,
+                      const ffw *z, double b, cudaStream_t st) {
+    return wilson_hops<ff>(g, U, in, out, 0, 1, m0, g5, a, z, b, st);
 }
 cudaError_t wilson_f32(const Geom &g, const float4 *U, const float4 *in, float4 *out, float m0, int g5,
                        float a, const float4 *z, float b, cudaStream_t st) {
@@ -359,14 +390,6 @@ cudaError_t wilson_f32(const Geom &g, const float4 *U, const float4 *in, float4 
         k_wilson<float, float4, float4><<<ls.grid, ls.block, 0, st>>>(g, U, in, out, m0 + 4.0f, g5, a, z, b,
                                                                       ls.spb);
     }
-    count_launches(1);
-    return cudaGetLastError();
-}
-
-cudaError_t wilson_ff(const Geom &g, const ffw *U, const ffw *in, ffw *out, double m0, int g5, double a,
-                      const ffw *z, double b, cudaStream_t st) {
-    const LaunchShape ls = balanced_shape(g.V, g.nsm, MinBlocks<ff>::value, 1 << 30);
-    k_wilson<ff, ffw, ffw><<<ls.grid, ls.block, 0, st>>>(g, U, in, out, ff(m0 + 4.0), g5, ff(a), z, ff(b), ls.spb);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -453,18 +476,33 @@ cudaError_t wilson_16(const Geom &g, const void *u16, const uint4 *in, const flo
 }
 
 // ------------------------------------------------------------------ float-float conversion
-// double2 word k <-> ffw word k: hi = fl32(x), lo = fl32(x - hi) per real; back, hi + lo in FP64.
-__global__ void k_d2ff(const double2 *__restrict__ x, ffw *__restrict__ y, long n) {
+// hi = fl32(x), lo = fl32(x - hi) per real; back, hi + lo in FP64.
+__global__ void k_links_d2ff(const double2 *__restrict__ x, ffl *__restrict__ y, long n) {
     for (long k = (long)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (long)gridDim.x * blockDim.x) {
         const double2 v = x[k];
         const ff re(v.x), im(v.y);
-        reinterpret_cast<float4 *>(y)[k] = make_float4(re.hi, re.lo, im.hi, im.lo);
+        y[k] = ffl{re.hi, re.lo, im.hi, im.lo};
     }
 }
-__global__ void k_ff2d(const ffw *__restrict__ x, double2 *__restrict__ y, long n) {
+// Thread k: checkerboard index, colour and spin pair of one parity of one spinor (6 Vh of them
+// per parity): two complex numbers of two spins <-> the words of their real and imaginary parts.
+__global__ void k_spinor_d2ff(const double2 *__restrict__ x, ffw *__restrict__ y, int Vh, long n) {
     for (long k = (long)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (long)gridDim.x * blockDim.x) {
-        const float4 v = reinterpret_cast<const float4 *>(x)[k];
-        y[k] = make_double2(ff(v.x, v.y).to_double(), ff(v.z, v.w).to_double());
+        const long i = k % Vh, r = k / Vh;         // r = 6 * (parity and spinor) + 3 * pair + colour
+        const long m = r / 6, w = r % 6, c = w % 3 + 6 * (w / 3);
+        const double2 a = x[(12 * m + c) * Vh + i], b = x[(12 * m + c + 3) * Vh + i];
+        const ff ar(a.x), ai(a.y), br(b.x), bi(b.y);
+        y[(12 * m + 2 * w) * Vh + i] = ffw{ar.hi, br.hi, ar.lo, br.lo};
+        y[(12 * m + 2 * w + 1) * Vh + i] = ffw{ai.hi, bi.hi, ai.lo, bi.lo};
+    }
+}
+__global__ void k_spinor_ff2d(const ffw *__restrict__ x, double2 *__restrict__ y, int Vh, long n) {
+    for (long k = (long)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (long)gridDim.x * blockDim.x) {
+        const long i = k % Vh, r = k / Vh;
+        const long m = r / 6, w = r % 6, c = w % 3 + 6 * (w / 3);
+        const ffw a = x[(12 * m + 2 * w) * Vh + i], b = x[(12 * m + 2 * w + 1) * Vh + i];
+        y[(12 * m + c) * Vh + i] = make_double2(ff(a.h0, a.l0).to_double(), ff(b.h0, b.l0).to_double());
+        y[(12 * m + c + 3) * Vh + i] = make_double2(ff(a.h1, a.l1).to_double(), ff(b.h1, b.l1).to_double());
     }
 }
 static int conv_grid(long n) {
@@ -472,13 +510,20 @@ static int conv_grid(long n) {
     const long cap = 16L * device_sm_count();
     return (int)(b < 1 ? 1 : (b > cap ? cap : b));
 }
-cudaError_t dev_d2ff(const double2 *x, ffw *y, long n, cudaStream_t st) {
-    k_d2ff<<<conv_grid(n), kBlock, 0, st>>>(x, y, n);
+cudaError_t links_d2ff(const double2 *x, ffl *y, long n, cudaStream_t st) {
+    k_links_d2ff<<<conv_grid(n), kBlock, 0, st>>>(x, y, n);
     count_launches(1);
     return cudaGetLastError();
 }
-cudaError_t dev_ff2d(const ffw *x, double2 *y, long n, cudaStream_t st) {
-    k_ff2d<<<conv_grid(n), kBlock, 0, st>>>(x, y, n);
+cudaError_t spinor_d2ff(const Geom &g, const double2 *x, ffw *y, cudaStream_t st, int n) {
+    const long k = 6L * g.V * n;
+    k_spinor_d2ff<<<conv_grid(k), kBlock, 0, st>>>(x, y, g.Vh, k);
+    count_launches(1);
+    return cudaGetLastError();
+}
+cudaError_t spinor_ff2d(const Geom &g, const ffw *x, double2 *y, cudaStream_t st, int n) {
+    const long k = 6L * g.V * n;
+    k_spinor_ff2d<<<conv_grid(k), kBlock, 0, st>>>(x, y, g.Vh, k);
     count_launches(1);
     return cudaGetLastError();
 }

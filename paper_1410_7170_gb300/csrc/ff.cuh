@@ -71,36 +71,16 @@ __device__ __forceinline__ ff ff_fma(ff a, ff b, ff c) {
     return ff_fast_two_sum(s.hi, __fadd_rn(s.lo, __fadd_rn(e, c.lo)));
 }
 
-// Storage word of one complex number in float-float: (re.hi, re.lo, im.hi, im.lo), 16 bytes,
-// the same size and word layout as an FP64 complex (double2), so the FP64 even-odd layouts
-// carry over word for word:
-//   float-float spinor: ffw [p][12 spin-colour][Vh]        (192 B per site)
-//   float-float link:   ffw [p][mu][9][Vh]   all 18 reals of -1/2 U_mu(x)
+// Storage words of float-float fields, 16 bytes each (as many as an FP64 complex number):
+//   spinor: ffw [p][12][Vh], word ((s / 2) * 3 + colour) * 2 + (0 real, 1 imaginary) holds that
+//           real of spins s and s + 1 (s = 0 or 2) as (hi, hi, lo, lo): two numbers side by side,
+//           ready for the packed FP32 instructions (hops.cuh);
+//   link:   ffl [p][mu][9][Vh], all nine entries of -1/2 U_mu(x) as (re.hi, re.lo, im.hi, im.lo).
 struct __align__(16) ffw {
+    float h0, h1, l0, l1;
+};
+struct __align__(16) ffl {
     float rh, rl, ih, il;
 };
-
-__device__ __forceinline__ cpx<ff> ffw_get(const float4 v) { return cpx<ff>{ff(v.x, v.y), ff(v.z, v.w)}; }
-__device__ __forceinline__ float4 ffw_put(const cpx<ff> &c) { return make_float4(c.re.hi, c.re.lo, c.im.hi, c.im.lo); }
-
-template <typename R>
-__device__ __forceinline__ void load_spinor(const ffw *__restrict__ f, int Vh, int p, int i, cpx<R> s[12]) {
-    static_assert(sizeof(R) == sizeof(ff), "float-float storage is read as float-float");
-    const float4 *b = reinterpret_cast<const float4 *>(f) + (size_t)p * 12 * Vh + i;
-#pragma unroll
-    for (int c = 0; c < 12; c++) s[c] = ffw_get(__ldg(b + (size_t)c * Vh));
-}
-template <typename R>
-__device__ __forceinline__ void store_spinor(ffw *__restrict__ f, int Vh, int p, int i, const cpx<R> s[12]) {
-    float4 *b = reinterpret_cast<float4 *>(f) + (size_t)p * 12 * Vh + i;
-#pragma unroll
-    for (int c = 0; c < 12; c++) b[(size_t)c * Vh] = ffw_put(s[c]);
-}
-template <typename R>
-__device__ __forceinline__ void load_link(const ffw *__restrict__ g, int Vh, int p, int mu, int i, cpx<R> u[3][3]) {
-    const float4 *b = reinterpret_cast<const float4 *>(g) + ((size_t)(p * 4 + mu) * kLink64Words) * Vh + i;
-#pragma unroll
-    for (int c = 0; c < 9; c++) u[c / 3][c % 3] = ffw_get(__ldg(b + (size_t)c * Vh));
-}
 
 }  // namespace ovl

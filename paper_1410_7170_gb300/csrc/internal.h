@@ -21,15 +21,14 @@ constexpr int kMaxRedValues = 4;        // doubles reduced by one kernel
 struct RedScratch {
     double *partials;      // [kMaxRedValues][kMaxRedBlocks]
     unsigned *counter;     // one word, zero between launches
+    // of grid row y, where each has one reduced value and a counter of its own
+    __device__ RedScratch row(int y) const { return RedScratch{partials + (size_t)y * kMaxRedBlocks, counter + y}; }
 };
 
-// Minimum resident blocks per SM requested from the compiler: the FP64 stencils are
-// held to 128 registers so two 256-thread blocks fit on an SM (one wave of 256 blocks
-// at 16^4 on 152 SMs).
+// Minimum resident blocks per SM requested from the compiler for the one-thread-per-site stencils:
+// at 128 registers two 256-thread blocks fit on an SM (one wave of 256 blocks at 16^4 on 152 SMs).
 template <typename R> struct MinBlocks { static constexpr int value = 1; };
-template <> struct MinBlocks<double> { static constexpr int value = 2; };
 template <> struct MinBlocks<float> { static constexpr int value = 2; };
-template <> struct MinBlocks<ff> { static constexpr int value = 2; };
 
 // SMs of the current device (queried once per device and cached).
 int device_sm_count();
@@ -96,8 +95,8 @@ cudaError_t wilson_f64(const Geom &g, const double2 *U, const double2 *in, doubl
                        double a, const double2 *z, double b, cudaStream_t st);
 cudaError_t wilson_f32(const Geom &g, const float4 *U, const float4 *in, float4 *out, float m0, int g5,
                        float a, const float4 *z, float b, cudaStream_t st);
-// float-float stencil (one thread per site); links in the float-float layout of ff.cuh
-cudaError_t wilson_ff(const Geom &g, const ffw *U, const ffw *in, ffw *out, double m0, int g5, double a,
+// float-float stencil; fields in the layouts of ff.cuh
+cudaError_t wilson_ff(const Geom &g, const ffl *U, const ffw *in, ffw *out, double m0, int g5, double a,
                       const ffw *z, double b, cudaStream_t st);
 // 16-bit stencil: out = D_W(m0) in with 16-bit links (from links_to16) and 16-bit spinors,
 // FP16 with a per-site scale (norm arrays of V floats) or BF16 (norms unused), FP32 arithmetic
@@ -106,10 +105,11 @@ cudaError_t spinor_f2h(const Geom &g, const float4 *a, uint4 *v, float *norm, bo
 cudaError_t spinor_h2f(const Geom &g, const uint4 *v, const float *norm, float4 *b, bool bf16, cudaStream_t st);
 cudaError_t wilson_16(const Geom &g, const void *u16, const uint4 *in, const float *in_norm, uint4 *out, float *out_norm,
                       float m0, bool bf16, cudaStream_t st);
-// FP64 <-> float-float conversion of n complex words (double2 <-> ffw, same word order; used
-// for even-odd spinors and for the FP64 link array)
-cudaError_t dev_d2ff(const double2 *x, ffw *y, long n, cudaStream_t st);
-cudaError_t dev_ff2d(const ffw *x, double2 *y, long n, cudaStream_t st);
+// FP64 -> float-float links (n complex words), and FP64 <-> float-float conversion of n even-odd
+// spinors back to back
+cudaError_t links_d2ff(const double2 *x, ffl *y, long n, cudaStream_t st);
+cudaError_t spinor_d2ff(const Geom &g, const double2 *x, ffw *y, cudaStream_t st, int n = 1);
+cudaError_t spinor_ff2d(const Geom &g, const ffw *x, double2 *y, cudaStream_t st, int n = 1);
 
 // ---------------------------------------------------------------- BLAS-1 (flat arrays of n doubles)
 // Reductions return through device memory `res` (written by the last block).
@@ -159,6 +159,7 @@ struct MsState {
     double rr;                 // ||r_k||^2 (base residual)
     double pp;                 // ||p_0||^2 by the recurrence ||p_k||^2 = ||r_k||^2 + b_{k-1}^2 ||p_{k-1}||^2
     double alpha, alpha_prev, beta_prev;
+    float alpha_f[2], sigma0_f[2];   // alpha and sigma[0] as float-float (hi, lo)
     double tol;                // target relative accuracy of the rational function
     double sigma[kMaxPoles];   // shifts
     double w[kMaxPoles];       // weights of x_l in y
@@ -166,6 +167,8 @@ struct MsState {
     double zeta[kMaxPoles], zeta_prev[kMaxPoles];
     double alpha_l[kMaxPoles], beta_l[kMaxPoles];   // this iteration's coefficients of the rescaled directions
                                                     // (y += w_l alpha_l p~_l, p~_l = r + beta_l p~_l)
+    double ratio[kMaxPoles], critz2[kMaxPoles];     // zeta_{k+1} / zeta_k, (crit zeta_{k+1})^2
+    double scale, inv_rr, inv_bb;                   // scale, 1 / (scale ||r||^2), 1 / (scale ||b||^2)
     int active[kMaxPoles];
     int *hist;                 // optional: hist[k] = shifts updated in iteration k (instrumentation)
     int hist_cap;
@@ -209,7 +212,7 @@ cudaError_t ms_init_half(const Geom &g, int n, MsState *s, MsVectorsH v, const f
 // float-float multishift (the FP64-accuracy sign on the FP32 pipes)
 cudaError_t ms_init_ff(const Geom &g, int n, MsState *s, MsVectors<ffw> v, const ffw *b, RedScratch rs,
                        cudaStream_t st);
-cudaError_t ms_iter_ff(const Geom &g, const ffw *U, double m0, MsState *s, MsVectors<ffw> v, RedScratch rs,
+cudaError_t ms_iter_ff(const Geom &g, const ffl *U, double m0, MsState *s, MsVectors<ffw> v, RedScratch rs,
                        cudaStream_t st, cudaEvent_t *ev = nullptr, unsigned ev_flags = 0);
 cudaError_t ms_iter_half(const Geom &g, const float4 *U, float m0, MsState *s, MsVectorsH v, RedScratch rs, bool bf16,
                          cudaStream_t st, cudaEvent_t *ev = nullptr, unsigned ev_flags = 0);
@@ -232,8 +235,12 @@ struct MsBatch {
 };
 // One state per right-hand side (st[y]); partial sums need nrhs * 2 * kMaxRedBlocks doubles;
 // counters: nrhs words, zero between launches.
+cudaError_t msb_init_ff(const Geom &g, int nrhs, int npole, MsState *st, MsBatch<ffw> v, const ffw *b, RedScratch rs,
+                        unsigned *counters, cudaStream_t s);
+cudaError_t msb_iter_ff(const Geom &g, const ffl *U, double m0, int nrhs, int npole, MsState *st, MsBatch<ffw> v,
+                        RedScratch rs, unsigned *counters, cudaStream_t s);
 cudaError_t msb_init_f64(const Geom &g, int nrhs, int npole, MsState *st, MsBatch<double2> v, const double2 *b,
-                         RedScratch rs, cudaStream_t s);
+                         RedScratch rs, unsigned *counters, cudaStream_t s);
 cudaError_t msb_init_f32(const Geom &g, int nrhs, int npole, MsState *st, MsBatch<float4> v, const float4 *b,
                          RedScratch rs, cudaStream_t s);
 cudaError_t msb_iter_f64(const Geom &g, const double2 *U, double m0, int nrhs, int npole, MsState *st,

@@ -382,12 +382,6 @@ __global__ void __launch_bounds__(384) k_msb_r(Geom g, const LT *__restrict__ U,
 }
 
 template <typename ST> struct WordB;
-template <> struct WordB<double2> {
-    static constexpr int N = 2;
-    using A = double;
-    __device__ static void get(const double2 &w, A *o) { o[0] = w.x; o[1] = w.y; }
-    __device__ static double2 put(const A *o) { return make_double2(o[0], o[1]); }
-};
 template <> struct WordB<float4> {
     static constexpr int N = 4;
     using A = float;
@@ -515,13 +509,6 @@ inline int stream_grid_b(long n) {
 }  // namespace
 
 // out_y = a [gamma5] D_W(m0) in_y + b z_y, y < nrhs (nrhs <= 12), vectors `stride` words apart
-cudaError_t wilson_batch_f64(const Geom &g, const double2 *U, const double2 *in, double2 *out, long stride, int nrhs,
-                             double m0, int g5, double a, const double2 *z, double b, cudaStream_t st) {
-    k_wilson_mrhs<double, double2, double2><<<dim3((g.V + kTile - 1) / kTile, 1), dim3(kTile, nrhs), 0, st>>>(
-        g, U, in, out, stride, nrhs, m0 + 4.0, g5, a, z, b);
-    count_launches(1);
-    return cudaGetLastError();
-}
 cudaError_t wilson_batch_f32(const Geom &g, const float4 *U, const float4 *in, float4 *out, long stride, int nrhs,
                              float m0, int g5, float a, const float4 *z, float b, cudaStream_t st) {
     const int kern = nrhs > 6 ? g.mrhs32l : g.mrhs32;
@@ -573,17 +560,9 @@ static cudaError_t msb_iter_t(const Geom &g, const LT *U, R m0, int nrhs, int np
     return cudaGetLastError();
 }
 
-cudaError_t msb_init_f64(const Geom &g, int nrhs, int npole, MsState *st, MsBatch<double2> v, const double2 *b,
-                         RedScratch rs, cudaStream_t s) {
-    return msb_init_t<double2>(g, nrhs, npole, st, v, b, rs, s);
-}
 cudaError_t msb_init_f32(const Geom &g, int nrhs, int npole, MsState *st, MsBatch<float4> v, const float4 *b,
                          RedScratch rs, cudaStream_t s) {
     return msb_init_t<float4>(g, nrhs, npole, st, v, b, rs, s);
-}
-cudaError_t msb_iter_f64(const Geom &g, const double2 *U, double m0, int nrhs, int npole, MsState *st,
-                         MsBatch<double2> v, RedScratch rs, unsigned *counters, cudaStream_t s) {
-    return msb_iter_t<double, double2, double2>(g, U, m0, nrhs, npole, st, v, rs, counters, s);
 }
 cudaError_t msb_iter_f32(const Geom &g, const float4 *U, float m0, int nrhs, int npole, MsState *st,
                          MsBatch<float4> v, RedScratch rs, unsigned *counters, cudaStream_t s) {

@@ -46,6 +46,9 @@
 // of iterations can be queued or captured in a CUDA graph without host round trips.
 #include <math.h>
 
+#include <algorithm>
+
+#include "hops.cuh"
 #include "internal.h"
 #include "reduce.cuh"
 #include "wilson_quad.cuh"
@@ -69,6 +72,9 @@ struct AlphaFin {
             return;
         }
         s->alpha = a;
+        const ff af(a);
+        s->alpha_f[0] = af.hi;
+        s->alpha_f[1] = af.lo;
     }
 };
 
@@ -128,6 +134,79 @@ struct ShiftFin {
             s->rr = rr_new;
             s->iter += 1;
             if (!any) s->done = 2;   // finish this iteration's shift updates, then stop
+        }
+    }
+};
+
+// The same in two parts. A dependent FP64 instruction takes 64 clocks or more on GB300 (half a lane
+// per clock and scheduler), so the divisions and roots of ShiftFin cost about 3 us at the end of
+// every residual kernel. ShiftScalars does what does not need ||r_{k+1}||^2, in a block of its own
+// during the kernel: zeta_{k+1}, alpha^l_k, zeta_{k+1} / zeta_k, the squared drop criterion and
+// the reciprocals of ||r_k||^2 and ||b||^2 (scaled, so that they exist for any ||b||^2 > 0).
+struct ShiftScalars {
+    MsState *s;
+    __device__ void operator()(int lane) const {
+        const double a = s->alpha, ap = s->alpha_prev, bp = s->beta_prev;
+        for (int l = lane; l < s->n; l += 32) {
+            if (!s->active[l]) {
+                s->alpha_l[l] = 0.0;
+                continue;
+            }
+            const double z = s->zeta[l], zp = s->zeta_prev[l];
+            double zn = 1.0;
+            if (l > 0) {
+                const double den = a * bp * (zp - z) + zp * ap * (1.0 + (s->sigma[l] - s->sigma[0]) * a);
+                zn = (den != 0.0) ? z * zp * ap / den : 0.0;
+            }
+            s->alpha_l[l] = a * zn;
+            s->ratio[l] = (z != 0.0) ? zn / z : 0.0;
+            const double c = s->crit[l] * zn;
+            s->critz2[l] = c * c;
+            s->zeta_prev[l] = z;
+            s->zeta[l] = zn;
+        }
+        if (lane == 0) {
+            const double scale = s->bb < 1e-150 ? 0x1p500 : 1.0;
+            s->scale = scale;
+            s->inv_rr = 1.0 / (s->rr * scale);
+            s->inv_bb = 1.0 / (s->bb * scale);
+        }
+    }
+};
+struct ShiftFinS {
+    MsState *s;
+    __device__ void operator()(const double *v, int lane) const {
+        const double rr_new = v[0], rs = rr_new * s->scale;
+        const double beta = rs * s->inv_rr;
+        if (!isfinite(beta)) {
+            if (lane == 0) {
+                s->status = 1;
+                s->done = 1;
+            }
+            return;
+        }
+        const double rel = rs * s->inv_bb, tol2 = s->tol * s->tol;
+        int any = 0, nupd = 0;
+        for (int l = lane; l < s->n; l += 32) {
+            if (!s->active[l]) continue;
+            nupd++;
+            s->beta_l[l] = beta * s->ratio[l];
+            if (s->critz2[l] * rel <= tol2) s->active[l] = 2;   // last update
+            else any = 1;
+        }
+        any = __any_sync(0xffffffffu, any);
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) nupd += __shfl_down_sync(0xffffffffu, nupd, off);
+        __syncwarp();
+        if (lane == 0) {
+            if (any && s->active[0] == 2) s->active[0] = 1;
+            if (s->hist && s->iter < s->hist_cap) s->hist[s->iter] = nupd;
+            s->alpha_prev = s->alpha;
+            s->beta_prev = beta;
+            s->pp = rr_new + beta * beta * s->pp;
+            s->rr = rr_new;
+            s->iter += 1;
+            if (!any) s->done = 2;
         }
     }
 };
@@ -346,61 +425,97 @@ __global__ void __launch_bounds__(kBlock, MinBlocks<R>::value) k_ms_r4(Geom g, c
     grid_reduce_warp<1>(v, rs, ShiftFin{s});
 }
 
-// Elementwise access to a storage word as NR reals.
+// Elementwise arithmetic on storage words: V is a word in registers, C a real coefficient in the
+// word's arithmetic; N reals of A per word where a word is a plain array of reals.
 template <typename ST> struct Word;
-// A = arithmetic type of the elementwise updates (the storage precision).
 template <> struct Word<double2> {
-    static constexpr int N = 2;
-    using A = double;
-    __device__ static void get(const double2 &w, A *o) { o[0] = w.x; o[1] = w.y; }
-    __device__ static double2 put(const A *o) { return make_double2(o[0], o[1]); }
+    using V = double2;
+    using C = double;
+    using Sum = double;
+    __device__ static V get(const double2 &w) { return w; }
+    __device__ static double2 put(const V &v) { return v; }
+    __device__ static C coef(double a) { return a; }
+    __device__ static V fma(C a, const V &b, const V &c) {
+        return make_double2(fma_r(a, b.x, c.x), fma_r(a, b.y, c.y));
+    }
+    __device__ static Sum norm2(const V &v) { return v.x * v.x + v.y * v.y; }
 };
 template <> struct Word<float4> {
     static constexpr int N = 4;
     using A = float;
+    using V = float4;
+    using C = float;
+    using Sum = float;
     __device__ static void get(const float4 &w, A *o) { o[0] = w.x; o[1] = w.y; o[2] = w.z; o[3] = w.w; }
     __device__ static float4 put(const A *o) { return make_float4(o[0], o[1], o[2], o[3]); }
+    __device__ static V get(const float4 &w) { return w; }
+    __device__ static float4 put(const V &v) { return v; }
+    __device__ static C coef(double a) { return (float)a; }
+    __device__ static V fma(C a, const V &b, const V &c) {
+        return make_float4(fma_r(a, b.x, c.x), fma_r(a, b.y, c.y), fma_r(a, b.z, c.z), fma_r(a, b.w, c.w));
+    }
+    __device__ static Sum norm2(const V &v) { return v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w; }
 };
-// float-float: one complex number per 16-byte word, (re.hi, re.lo, im.hi, im.lo)
 template <> struct Word<ffw> {
-    static constexpr int N = 2;
-    using A = ff;
-    __device__ static void get(const ffw &w, A *o) { o[0] = ff(w.rh, w.rl); o[1] = ff(w.ih, w.il); }
-    __device__ static ffw put(const A *o) { return ffw{o[0].hi, o[0].lo, o[1].hi, o[1].lo}; }
+    using V = ff2;
+    using C = ff2_factor;
+    using Sum = ff;
+    __device__ static V get(const ffw &w) { return ff2_load(reinterpret_cast<const float4 &>(w)); }
+    __device__ static ffw put(const V &v) {
+        const float4 w = ff2_word(v);
+        return ffw{w.x, w.y, w.z, w.w};
+    }
+    __device__ static C coef(double a) { return ff2_scale(ff(a)); }
+    __device__ static V fma(const C &a, const V &b, const V &c) { return ff2_fma(a, b, c); }
+    __device__ static Sum norm2(const V &v) {
+        return HopTiles<ff>::total(ff2_square_add(v, HopTiles<ff>::zero()));
+    }
 };
 
-// y += sum_l w_l a^l p_l ; p_l = zeta_l r + b^l p_l   (words of ST; nw words per vector).
+// y += sum_l w_l a^l p_l ; p_l = zeta_l r + b^l p_l for right-hand side blockIdx.y, whose vectors
+// start `stride` words and whose directions start `pstride` words after the previous one's.
 // The active shifts are compacted into a list in shared memory and processed four at
 // a time: the four loads of a batch are issued before any store, so each thread keeps
 // four independent memory requests in flight.
 template <typename ST>
-__global__ void __launch_bounds__(kBlock) k_ms_shifts(MsState *s, const ST *__restrict__ r, ST *__restrict__ y,
-                                                      ST *__restrict__ P, long stride, long nw, unsigned *counter) {
-    using A = typename Word<ST>::A;
-    __shared__ A sw[kMaxPoles], sb[kMaxPoles];
+__global__ void __launch_bounds__(kBlock) k_ms_shifts(MsState *st, const ST *__restrict__ r, ST *__restrict__ y,
+                                                      ST *__restrict__ P, long stride, long pstride,
+                                                      unsigned *counters) {
+    using W = Word<ST>;
+    __shared__ typename W::C sw[kMaxPoles], sb[kMaxPoles];
     __shared__ int sidx[kMaxPoles];
     __shared__ int sact, sdone;
-    if (threadIdx.x == 0) {
-        sdone = s->done;
+    MsState *s = st + blockIdx.y;
+    if (threadIdx.x < 32) {
+        const int lane = threadIdx.x;
+        const int done = s->done;
         int na = 0;
-        if (sdone != 1)
-            for (int l = 0; l < s->n; l++)
-                if (s->active[l]) {
-                    sidx[na] = l;
-                    sw[na] = (A)(s->w[l] * s->alpha_l[l]);
-                    sb[na] = (A)s->beta_l[l];
-                    na++;
-                }
-        sact = na;
+        for (int l0 = 0; l0 < s->n && done != 1; l0 += 32) {
+            const int l = l0 + lane;
+            const bool on = l < s->n && s->active[l];
+            const unsigned m = __ballot_sync(0xffffffffu, on);
+            if (on) {
+                const int k = na + __popc(m & ((1u << lane) - 1));
+                sidx[k] = l;
+                sw[k] = W::coef(s->w[l] * s->alpha_l[l]);
+                sb[k] = W::coef(s->beta_l[l]);
+            }
+            na += __popc(m);
+        }
+        if (lane == 0) {
+            sdone = done;
+            sact = na;
+        }
     }
     __syncthreads();
-    if (sdone == 1) return;
+    if (sdone == 1) return;   // uniform over the blocks of this right-hand side
     const int na = sact;
-    constexpr int N = Word<ST>::N;
-    for (long k = (long)blockIdx.x * blockDim.x + threadIdx.x; k < nw; k += (long)gridDim.x * blockDim.x) {
-        A rv[N], yv[N];
-        Word<ST>::get(r[k], rv);
-        Word<ST>::get(y[k], yv);
+    r += blockIdx.y * stride;
+    y += blockIdx.y * stride;
+    P += blockIdx.y * pstride;
+    for (long k = (long)blockIdx.x * blockDim.x + threadIdx.x; k < stride; k += (long)gridDim.x * blockDim.x) {
+        const typename W::V rv = W::get(r[k]);
+        typename W::V yv = W::get(y[k]);
         for (int a0 = 0; a0 < na; a0 += 4) {
             ST w[4];
 #pragma unroll
@@ -409,26 +524,72 @@ __global__ void __launch_bounds__(kBlock) k_ms_shifts(MsState *s, const ST *__re
 #pragma unroll
             for (int u = 0; u < 4; u++) {
                 if (a0 + u >= na) break;
-                A pv[N];
-                Word<ST>::get(w[u], pv);
-                const A wl = sw[a0 + u], bl = sb[a0 + u];
-#pragma unroll
-                for (int e = 0; e < N; e++) {
-                    yv[e] = fma_r(wl, pv[e], yv[e]);
-                    pv[e] = fma_r(bl, pv[e], rv[e]);
-                }
-                P[(long)sidx[a0 + u] * stride + k] = Word<ST>::put(pv);
+                const typename W::V pv = W::get(w[u]);
+                yv = W::fma(sw[a0 + u], pv, yv);
+                P[(long)sidx[a0 + u] * stride + k] = W::put(W::fma(sb[a0 + u], pv, rv));
             }
         }
-        y[k] = Word<ST>::put(yv);
+        y[k] = W::put(yv);
     }
     // the last block retires the shifts that made their final update and ends a finished solve
-    if (grid_last_block(counter)) {
+    if (grid_last_block(counters + blockIdx.y)) {
         for (int l = threadIdx.x; l < s->n; l += blockDim.x)
             if (s->active[l] == 2) s->active[l] = 0;
         __syncthreads();
         if (threadIdx.x == 0 && s->done == 2) s->done = 1;
     }
+}
+
+// t = gamma5 D_W p0 ; ||t||^2 -> alpha of right-hand side blockIdx.y, one warp per hop (hops.cuh).
+// FP64 and float-float.
+template <typename R>
+__global__ void __launch_bounds__(kHopBlock, HopBlocks<R>::value)
+    k_ms_q_hops(Geom g, const typename HopTiles<R>::Link *__restrict__ U, R m4, MsState *st,
+                const typename HopTiles<R>::Store *__restrict__ p0, long pstride,
+                typename HopTiles<R>::Store *__restrict__ t, long stride, RedScratch rs) {
+    using H = HopTiles<R>;
+    MsState *s = st + blockIdx.y;
+    if (s->done) return;
+    p0 += blockIdx.y * pstride;
+    t += blockIdx.y * stride;
+    typename H::Sum sum = H::zero();
+    const auto fm = H::factor(m4);
+    hop_tiles<R>(g, blockIdx.x, gridDim.x, U, p0, [&](int p, int i, int it, int e, typename H::Elem hop) {
+        typename H::Elem v = H::fma(fm, H::load(p0, g.Vh, p, i, it, e), hop);
+        v = H::neg_if(v, H::upper(it));
+        H::store(t, g.Vh, p, i, it, e, v);
+        H::square_add(v, sum);
+    });
+    const R v[1] = {H::total(sum)};
+    grid_reduce<1>(v, rs.row(blockIdx.y), AlphaFin{s});
+}
+
+// r -= alpha (gamma5 D_W t + sigma0 p0) ; ||r||^2 -> shift scalars, as above. Block 0 takes no
+// tiles: it forms the shift scalars that need only alpha_k while the others compute (ShiftScalars).
+template <typename R>
+__global__ void __launch_bounds__(kHopBlock, HopBlocks<R>::value)
+    k_ms_r_hops(Geom g, const typename HopTiles<R>::Link *__restrict__ U, R m4, MsState *st,
+                const typename HopTiles<R>::Store *__restrict__ t, const typename HopTiles<R>::Store *__restrict__ p0,
+                long pstride, typename HopTiles<R>::Store *__restrict__ r, long stride, RedScratch rs) {
+    using H = HopTiles<R>;
+    MsState *s = st + blockIdx.y;
+    if (s->done) return;
+    p0 += blockIdx.y * pstride;
+    t += blockIdx.y * stride;
+    r += blockIdx.y * stride;
+    typename H::Sum sum = H::zero();
+    if (blockIdx.x == 0 && threadIdx.x < 32) ShiftScalars{s}(threadIdx.x);
+    const int first = blockIdx.x ? blockIdx.x - 1 : g.V;   // block 0: past the last tile
+    const auto fm = H::factor(m4), fa = H::minus_alpha(*s), fs = H::sigma0(*s);
+    hop_tiles<R>(g, first, gridDim.x - 1, U, t, [&](int p, int i, int it, int e, typename H::Elem hop) {
+        typename H::Elem v = H::fma(fm, H::load(t, g.Vh, p, i, it, e), hop);
+        v = H::fma(fs, H::load(p0, g.Vh, p, i, it, e), H::neg_if(v, H::upper(it)));
+        v = H::fma(fa, v, H::load_rw(r, g.Vh, p, i, it, e));
+        H::store(r, g.Vh, p, i, it, e, v);
+        H::square_add(v, sum);
+    });
+    const R v[1] = {H::total(sum)};
+    grid_reduce_warp<1>(v, rs.row(blockIdx.y), ShiftFinS{s});
 }
 
 // Lagged shift updates at site (p, i), word by word: y += wa0 p_0 ; for the active shifts
@@ -541,17 +702,10 @@ __global__ void __launch_bounds__(kBlock) k_ms_p0(const MsState *s, const ST *__
                                                   const ST *__restrict__ rb1, ST *__restrict__ P0, long nw) {
     if (s->done) return;
     const ST *__restrict__ r = (s->iter & 1) ? rb1 : rb0;
-    using A = typename Word<ST>::A;
-    constexpr int N = Word<ST>::N;
-    const A b = A(s->beta_prev);
-    for (long k = (long)blockIdx.x * blockDim.x + threadIdx.x; k < nw; k += (long)gridDim.x * blockDim.x) {
-        A rv[N], pv[N];
-        Word<ST>::get(r[k], rv);
-        Word<ST>::get(P0[k], pv);
-#pragma unroll
-        for (int e = 0; e < N; e++) pv[e] = fma_r(b, pv[e], rv[e]);
-        P0[k] = Word<ST>::put(pv);
-    }
+    using W = Word<ST>;
+    const typename W::C b = W::coef(s->beta_prev);
+    for (long k = (long)blockIdx.x * blockDim.x + threadIdx.x; k < nw; k += (long)gridDim.x * blockDim.x)
+        P0[k] = W::put(W::fma(b, W::get(P0[k]), W::get(r[k])));
 }
 
 struct InitFin {
@@ -568,25 +722,26 @@ struct InitFin {
     }
 };
 
-// r = y = p_l = b ; ||b||^2
+// r = y = p_l = b ; ||b||^2 of right-hand side blockIdx.y
 template <typename ST>
-__global__ void k_ms_init(MsState *s, const ST *__restrict__ b, ST *r, ST *y, ST *P, long stride, long nw,
-                          int n, RedScratch rs) {
-    constexpr int N = Word<ST>::N;
-    using A = typename Word<ST>::A;
-    A v[1] = {A(0)};
-    for (long k = (long)blockIdx.x * blockDim.x + threadIdx.x; k < nw; k += (long)gridDim.x * blockDim.x) {
+__global__ void k_ms_init(MsState *st, const ST *__restrict__ b, ST *r, ST *y, ST *P, long stride, long pstride,
+                          RedScratch rs) {
+    using W = Word<ST>;
+    MsState *s = st + blockIdx.y;
+    b += blockIdx.y * stride;
+    r += blockIdx.y * stride;
+    y += blockIdx.y * stride;
+    P += blockIdx.y * pstride;
+    const int n = s->n;
+    typename W::Sum v[1] = {typename W::Sum(0)};
+    for (long k = (long)blockIdx.x * blockDim.x + threadIdx.x; k < stride; k += (long)gridDim.x * blockDim.x) {
         const ST w = b[k];
         r[k] = w;
         y[k] = w;
         for (int l = 0; l < n; l++) P[l * stride + k] = w;
-        A e[N], a = A(0);
-        Word<ST>::get(w, e);
-#pragma unroll
-        for (int q = 0; q < N; q++) a += e[q] * e[q];
-        v[0] += a;
+        v[0] += W::norm2(W::get(w));
     }
-    grid_reduce<1>(v, rs, InitFin{s});
+    grid_reduce<1>(v, rs.row(blockIdx.y), InitFin{s});
 }
 
 inline int stream_grid(long n) {
@@ -682,82 +837,100 @@ __global__ void k_ms_init_half(Geom g, MsState *s, MsVectorsH v, const float4 *_
     grid_reduce<1>(acc, rs, InitFin{s});
 }
 
+// One iteration of nrhs right-hand sides in FP64 or float-float: Q p, residual, shifts.
 template <typename R, typename LT, typename ST>
-cudaError_t ms_iter_t(const Geom &g, const LT *U, R m0, MsState *s, MsVectors<ST> v, RedScratch rs,
-                      cudaStream_t st, cudaEvent_t *ev, unsigned ev_flags) {
-    const int tps = sizeof(R) == 8 ? g.tps64 : g.tps32;
-    const int gs = red_grid(4L * g.V);
-    const LaunchShape ls = balanced_shape(g.V, g.nsm, MinBlocks<R>::value, kMaxRedBlocks);
+cudaError_t ms_iter_hops(const Geom &g, const LT *U, double m0, int nrhs, MsState *s, MsBatch<ST> v, long pstride,
+                         RedScratch rs, unsigned *counters, cudaStream_t st, cudaEvent_t *ev, unsigned ev_flags) {
+    const dim3 grid(hop_grid<R>(g, nrhs, true), nrhs), grid1(grid.x + 1, nrhs);
+    const RedScratch rows{rs.partials, counters};
     cudaError_t e;
     if (ev && (e = cudaEventRecordWithFlags(ev[0], st, ev_flags)) != cudaSuccess) return e;
-    // the fused form pays where the stencil waits on memory (FP32); the FP64 and float-float
-    // stencils are bound by arithmetic that the shift updates would add to
-    if (tps == 4 || sizeof(R) != 4) {   // three-kernel form (4 or 1 threads per site)
-        if (tps == 4) k_ms_q4<R, LT, ST><<<gs, kBlock, 0, st>>>(g, U, m0 + (R)4, s, v.p, v.t, rs);
-        else k_ms_q<R, LT, ST, false><<<ls.grid, ls.block, 0, st>>>(g, U, m0 + (R)4, s, v.p, v.t, rs, ls.spb);
+    k_ms_q_hops<R><<<grid, kHopBlock, 0, st>>>(g, U, R(m0 + 4.0), s, v.p, pstride, v.t, v.stride, rows);
+    if (ev && (e = cudaEventRecordWithFlags(ev[1], st, ev_flags)) != cudaSuccess) return e;
+    k_ms_r_hops<R><<<grid1, kHopBlock, 0, st>>>(g, U, R(m0 + 4.0), s, v.t, v.p, pstride, v.r, v.stride, rows);
+    if (ev && (e = cudaEventRecordWithFlags(ev[2], st, ev_flags)) != cudaSuccess) return e;
+    const int gs = nrhs > 1 ? std::max(1, std::min(stream_grid(v.stride), 16 * g.nsm / nrhs)) : stream_grid(v.stride);
+    k_ms_shifts<ST><<<dim3(gs, nrhs), kBlock, 0, st>>>(s, v.r, v.y, v.p, v.stride, pstride, counters);
+    if (ev && (e = cudaEventRecordWithFlags(ev[3], st, ev_flags)) != cudaSuccess) return e;
+    count_launches(3);
+    return cudaGetLastError();
+}
+template <typename ST>
+cudaError_t ms_init_rows(int nrhs, MsState *s, MsBatch<ST> v, long pstride, const ST *b, RedScratch rs,
+                         unsigned *counters, cudaStream_t st) {
+    const int gx = std::max(1, red_grid(v.stride) / nrhs);
+    k_ms_init<ST><<<dim3(gx, nrhs), kBlock, 0, st>>>(s, b, v.r, v.y, v.p, v.stride, pstride,
+                                                    RedScratch{rs.partials, counters});
+    count_launches(1);
+    return cudaGetLastError();
+}
+template <typename ST> MsBatch<ST> one_row(const MsVectors<ST> &v) { return MsBatch<ST>{v.r, v.t, v.y, v.p, v.stride}; }
+
+}  // namespace
+
+cudaError_t ms_init_f64(const Geom &g, int n, MsState *s, MsVectors<double2> v, const double2 *b, RedScratch rs,
+                        cudaStream_t st) {
+    return ms_init_rows(1, s, one_row(v), 0, b, rs, rs.counter, st);
+}
+cudaError_t ms_init_f32(const Geom &g, int n, MsState *s, MsVectors<float4> v, const float4 *b, RedScratch rs,
+                        cudaStream_t st) {
+    return ms_init_rows(1, s, one_row(v), 0, b, rs, rs.counter, st);
+}
+cudaError_t ms_init_ff(const Geom &g, int n, MsState *s, MsVectors<ffw> v, const ffw *b, RedScratch rs,
+                       cudaStream_t st) {
+    return ms_init_rows(1, s, one_row(v), 0, b, rs, rs.counter, st);
+}
+cudaError_t ms_iter_f64(const Geom &g, const double2 *U, double m0, MsState *s, MsVectors<double2> v,
+                        RedScratch rs, cudaStream_t st, cudaEvent_t *ev, unsigned ev_flags) {
+    return ms_iter_hops<double>(g, U, m0, 1, s, one_row(v), 0, rs, rs.counter, st, ev, ev_flags);
+}
+// float-float multishift: the scalar recurrences stay FP64 on the device
+cudaError_t ms_iter_ff(const Geom &g, const ffl *U, double m0, MsState *s, MsVectors<ffw> v, RedScratch rs,
+                       cudaStream_t st, cudaEvent_t *ev, unsigned ev_flags) {
+    return ms_iter_hops<ff>(g, U, m0, 1, s, one_row(v), 0, rs, rs.counter, st, ev, ev_flags);
+}
+
+cudaError_t ms_iter_f32(const Geom &g, const float4 *U, float m0, MsState *s, MsVectors<float4> v,
+                        RedScratch rs, cudaStream_t st, cudaEvent_t *ev, unsigned ev_flags) {
+    const int gs = red_grid(4L * g.V);
+    const LaunchShape ls = balanced_shape(g.V, g.nsm, MinBlocks<float>::value, kMaxRedBlocks);
+    cudaError_t e;
+    if (ev && (e = cudaEventRecordWithFlags(ev[0], st, ev_flags)) != cudaSuccess) return e;
+    if (g.tps32 == 4) {   // three-kernel form (4 threads per site)
+        k_ms_q4<float, float4, float4><<<gs, kBlock, 0, st>>>(g, U, m0 + 4.f, s, v.p, v.t, rs);
         if (ev && (e = cudaEventRecordWithFlags(ev[1], st, ev_flags)) != cudaSuccess) return e;
-        if (tps == 4) k_ms_r4<R, LT, ST><<<gs, kBlock, 0, st>>>(g, U, m0 + (R)4, s, v.t, v.p, v.r, rs);
-        else k_ms_r<R, LT, ST><<<ls.grid, ls.block, 0, st>>>(g, U, m0 + (R)4, s, v.t, v.p, v.r, rs, ls.spb);
+        k_ms_r4<float, float4, float4><<<gs, kBlock, 0, st>>>(g, U, m0 + 4.f, s, v.t, v.p, v.r, rs);
         if (ev && (e = cudaEventRecordWithFlags(ev[2], st, ev_flags)) != cudaSuccess) return e;
-        k_ms_shifts<ST><<<stream_grid(v.stride), kBlock, 0, st>>>(s, v.r, v.y, v.p, v.stride, v.stride, rs.counter);
-    } else {          // fused form
-        k_ms_q<R, LT, ST, true><<<ls.grid, ls.block, 0, st>>>(g, U, m0 + (R)4, s, v.p, v.t, rs, ls.spb);
+        k_ms_shifts<float4><<<stream_grid(v.stride), kBlock, 0, st>>>(s, v.r, v.y, v.p, v.stride, 0, rs.counter);
+    } else {   // fused form: it pays where the stencil waits on memory
+        k_ms_q<float, float4, float4, true><<<ls.grid, ls.block, 0, st>>>(g, U, m0 + 4.f, s, v.p, v.t, rs, ls.spb);
         if (ev && (e = cudaEventRecordWithFlags(ev[1], st, ev_flags)) != cudaSuccess) return e;
-        k_ms_rf<R, LT, ST><<<ls.grid, ls.block, 0, st>>>(g, U, m0 + (R)4, s, v.t, v.p, v.stride, v.r, v.r2, v.y,
-                                                         rs, ls.spb);
+        k_ms_rf<float, float4, float4><<<ls.grid, ls.block, 0, st>>>(g, U, m0 + 4.f, s, v.t, v.p, v.stride, v.r, v.r2,
+                                                                     v.y, rs, ls.spb);
         if (ev && (e = cudaEventRecordWithFlags(ev[2], st, ev_flags)) != cudaSuccess) return e;
-        k_ms_p0<ST><<<stream_grid(v.stride), kBlock, 0, st>>>(s, v.r, v.r2, v.p, v.stride);
+        k_ms_p0<float4><<<stream_grid(v.stride), kBlock, 0, st>>>(s, v.r, v.r2, v.p, v.stride);
     }
     if (ev && (e = cudaEventRecordWithFlags(ev[3], st, ev_flags)) != cudaSuccess) return e;
     count_launches(3);
     return cudaGetLastError();
 }
 
-}  // namespace
-
-cudaError_t ms_init_f64(const Geom &g, int n, MsState *s, MsVectors<double2> v, const double2 *b, RedScratch rs,
-                        cudaStream_t st) {
-    k_ms_init<double2><<<red_grid(v.stride), kBlock, 0, st>>>(s, b, v.r, v.y, v.p, v.stride, v.stride, n, rs);
-    count_launches(1);
-    return cudaGetLastError();
+// several right-hand sides in lock-step: one grid row each
+cudaError_t msb_init_f64(const Geom &g, int nrhs, int npole, MsState *st, MsBatch<double2> v, const double2 *b,
+                         RedScratch rs, unsigned *counters, cudaStream_t s) {
+    return ms_init_rows(nrhs, st, v, npole * v.stride, b, rs, counters, s);
 }
-cudaError_t ms_init_f32(const Geom &g, int n, MsState *s, MsVectors<float4> v, const float4 *b, RedScratch rs,
-                        cudaStream_t st) {
-    k_ms_init<float4><<<red_grid(v.stride), kBlock, 0, st>>>(s, b, v.r, v.y, v.p, v.stride, v.stride, n, rs);
-    count_launches(1);
-    return cudaGetLastError();
+cudaError_t msb_init_ff(const Geom &g, int nrhs, int npole, MsState *st, MsBatch<ffw> v, const ffw *b, RedScratch rs,
+                        unsigned *counters, cudaStream_t s) {
+    return ms_init_rows(nrhs, st, v, npole * v.stride, b, rs, counters, s);
 }
-cudaError_t ms_iter_f64(const Geom &g, const double2 *U, double m0, MsState *s, MsVectors<double2> v,
-                        RedScratch rs, cudaStream_t st, cudaEvent_t *ev, unsigned ev_flags) {
-    return ms_iter_t<double, double2, double2>(g, U, m0, s, v, rs, st, ev, ev_flags);
+cudaError_t msb_iter_f64(const Geom &g, const double2 *U, double m0, int nrhs, int npole, MsState *st,
+                         MsBatch<double2> v, RedScratch rs, unsigned *counters, cudaStream_t s) {
+    return ms_iter_hops<double>(g, U, m0, nrhs, st, v, npole * v.stride, rs, counters, s, nullptr, 0);
 }
-cudaError_t ms_iter_f32(const Geom &g, const float4 *U, float m0, MsState *s, MsVectors<float4> v,
-                        RedScratch rs, cudaStream_t st, cudaEvent_t *ev, unsigned ev_flags) {
-    return ms_iter_t<float, float4, float4>(g, U, m0, s, v, rs, st, ev, ev_flags);
-}
-
-// float-float multishift: the same three kernels on float-float vectors and links (one
-// thread per site); the scalar recurrences stay FP64 on the device.
-cudaError_t ms_init_ff(const Geom &g, int n, MsState *s, MsVectors<ffw> v, const ffw *b, RedScratch rs,
-                       cudaStream_t st) {
-    k_ms_init<ffw><<<red_grid(v.stride), kBlock, 0, st>>>(s, b, v.r, v.y, v.p, v.stride, v.stride, n, rs);
-    count_launches(1);
-    return cudaGetLastError();
-}
-cudaError_t ms_iter_ff(const Geom &g, const ffw *U, double m0, MsState *s, MsVectors<ffw> v, RedScratch rs,
-                       cudaStream_t st, cudaEvent_t *ev, unsigned ev_flags) {
-    const LaunchShape ls = balanced_shape(g.V, g.nsm, MinBlocks<ff>::value, kMaxRedBlocks);
-    const ff m4(m0 + 4.0);
-    cudaError_t e;
-    if (ev && (e = cudaEventRecordWithFlags(ev[0], st, ev_flags)) != cudaSuccess) return e;
-    k_ms_q<ff, ffw, ffw, false><<<ls.grid, ls.block, 0, st>>>(g, U, m4, s, v.p, v.t, rs, ls.spb);
-    if (ev && (e = cudaEventRecordWithFlags(ev[1], st, ev_flags)) != cudaSuccess) return e;
-    k_ms_r<ff, ffw, ffw><<<ls.grid, ls.block, 0, st>>>(g, U, m4, s, v.t, v.p, v.r, rs, ls.spb);
-    if (ev && (e = cudaEventRecordWithFlags(ev[2], st, ev_flags)) != cudaSuccess) return e;
-    k_ms_shifts<ffw><<<stream_grid(v.stride), kBlock, 0, st>>>(s, v.r, v.y, v.p, v.stride, v.stride, rs.counter);
-    if (ev && (e = cudaEventRecordWithFlags(ev[3], st, ev_flags)) != cudaSuccess) return e;
-    count_launches(3);
-    return cudaGetLastError();
+cudaError_t msb_iter_ff(const Geom &g, const ffl *U, double m0, int nrhs, int npole, MsState *st, MsBatch<ffw> v,
+                        RedScratch rs, unsigned *counters, cudaStream_t s) {
+    return ms_iter_hops<ff>(g, U, m0, nrhs, st, v, npole * v.stride, rs, counters, s, nullptr, 0);
 }
 
 }  // namespace ovl

@@ -119,12 +119,9 @@ extern "C" ovl_status wilson_apply_noalloc(double *out, const double *in, const 
         scratch = (unsigned char *)g_noalloc_addr[dev];
     }
     Geom g{};
-    for (int m = 0; m < 4; m++) g.L[m] = dims[m];
-    g.V = (int)V;
-    g.Vh = (int)(V / 2);
-    g.Lh3 = dims[3] / 2;
+    g.set_dims(dims);
     g.antiperiodic = antiperiodic ? 1 : 0;
-    g.tps64 = g.tps32 = 1;
+    g.tps32 = 1;
     g.mrhs32 = g.mrhs32l = 1;
     if (cudaDeviceGetAttribute(&g.nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
         cudaGetLastError();

@@ -16,24 +16,28 @@ __device__ __forceinline__ void warp_sum(double v[NV]) {
         for (int off = 16; off > 0; off >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], off);
 }
 
-// Block-wide sum of v[NV]; the result is valid in thread 0. blockDim.x <= 1024.
+// Block-wide sum of per-thread FP64 values, blockDim.x <= kBlock, valid in thread 0: the first warp adds the warps'
+// values lane by lane and then its lanes, 13 FP64 instructions of one warp instead of 5 of every warp
+// and 5 more (each occupies the SM's FP64 unit for 16 clocks).
 template <int NV>
-__device__ __forceinline__ void block_sum(double v[NV]) {
-    __shared__ double sm[NV][32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+__device__ __forceinline__ void block_sum(const double vd[NV], double v[NV]) {
+    __shared__ double sm[NV][kBlock];
     const int nw = (blockDim.x + 31) >> 5;
-    warp_sum<NV>(v);
     __syncthreads();   // protect sm from a previous use in the same kernel
-    if (lane == 0)
 #pragma unroll
-        for (int k = 0; k < NV; k++) sm[k][warp] = v[k];
+    for (int k = 0; k < NV; k++) sm[k][threadIdx.x] = vd[k];
     __syncthreads();
-    if (warp == 0) {
+    if (threadIdx.x < 32) {
 #pragma unroll
-        for (int k = 0; k < NV; k++) v[k] = lane < nw ? sm[k][lane] : 0.0;
+        for (int k = 0; k < NV; k++) {
+            v[k] = sm[k][threadIdx.x];
+            for (int w = 1; w < nw; w++) v[k] += sm[k][32 * w + threadIdx.x];
+        }
         warp_sum<NV>(v);
     }
 }
+template <int NV>
+__device__ __forceinline__ void block_sum(double v[NV]) { block_sum<NV>(v, v); }
 
 // Block-wide sum of per-thread FP32 values: the warp stage in FP32 (shuffles), the sum
 // over warps in FP64 by the first warp; the FP64 result is valid in thread 0. GB300 runs
@@ -87,13 +91,6 @@ __device__ __forceinline__ void block_sum(const ff vf[NV], double v[NV]) {
         warp_sum<NV>(v);
     }
 }
-template <int NV>
-__device__ __forceinline__ void block_sum(const double vd[NV], double v[NV]) {
-#pragma unroll
-    for (int k = 0; k < NV; k++) v[k] = vd[k];
-    block_sum<NV>(v);
-}
-
 // Reduce v[NV] (per-thread FP64 or FP32 partial sums) over the grid; the last block calls
 // fin(total) on thread 0 and resets the counter. Must be reached by every thread of every
 // block.

@@ -83,7 +83,7 @@ struct Ctx {
     // gauge field (12-real links)
     double2 *U64 = nullptr;
     float4 *U32 = nullptr;
-    ffw *Uff = nullptr;           // float-float copy of U64 (made on first use)
+    ffl *Uff = nullptr;           // float-float copy of U64 (made on first use)
     void *U16[2] = {nullptr, nullptr};    // 16-bit links: FP16 [0], BF16 [1] (made on first use)
     uint4 *h16a = nullptr, *h16b = nullptr;   // two 16-bit spinors (48 B per site)
     float *h16na = nullptr, *h16nb = nullptr; // their per-site FP16 scales

@@ -138,18 +138,6 @@ __device__ __forceinline__ void quad_allreduce(cpx<R> acc[12]) {
 
 // Chunk access: a storage word holds CPC complex numbers; a site has 12 / CPC words.
 template <typename ST> struct Chunk;
-template <> struct Chunk<double2> {
-    static constexpr int CPC = 1, NC = 12;
-    template <typename R>
-    __device__ static void load(const double2 *f, int Vh, int p, int i, int j, cpx<R> v[1]) {
-        double2 w = __ldg(f + ((size_t)p * NC + j) * Vh + i);
-        v[0] = cpx<R>{(R)w.x, (R)w.y};
-    }
-    template <typename R>
-    __device__ static void store(double2 *f, int Vh, int p, int i, int j, const cpx<R> v[1]) {
-        f[((size_t)p * NC + j) * Vh + i] = make_double2((double)v[0].re, (double)v[0].im);
-    }
-};
 template <> struct Chunk<float4> {
     static constexpr int CPC = 2, NC = 6;
     template <typename R>
