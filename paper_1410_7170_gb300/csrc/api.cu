@@ -538,10 +538,7 @@ ovl_status Ctx::sign_outer(const double2 *b, double2 *out, double tol, int mode)
 
 ovl_status Ctx::sign_outer_batch(const double2 *b, double2 *out, int nrhs, const double *tol, int mode) {
     if (!(p.precision != OVL_FP64 && p.ff_outer)) return sign64_batch(b, out, nrhs, tol, mode);
-    const long w = (long)g.V * 12;   // float-float: one right-hand side at a time
-    for (int y = 0; y < nrhs; y++)
-        if (tol[y] > 0) ST(sign_ff(b + y * w, out + y * w, tol[y], mode));
-    return OVL_OK;
+    return sign_ff_batch(b, out, nrhs, tol, mode);
 }
 
 // FP32 version for the inner (low-accuracy) D_N: b, out FP32 eo spinors.
@@ -619,6 +616,33 @@ ovl_status Ctx::ensure_batch() {
     CK(cudaMallocHost(&h_pinned_b, sizeof(MsState) * kMaxBatch + 4096));
     h_msb = (MsState *)h_pinned_b;
     h_msb_small = (int *)((char *)h_pinned_b + sizeof(MsState) * kMaxBatch);
+    return OVL_OK;
+}
+
+// Batched multishift vectors for nrhs right-hand sides (grown when a larger batch comes).
+template <typename W>
+ovl_status Ctx::ensure_msb(MsBatch<W> &v, int &cap, int nrhs) {
+    if (v.p && cap >= nrhs) return OVL_OK;
+    if (v.p) {
+        cudaFree(v.r);
+        allocs.erase(std::find(allocs.begin(), allocs.end(), (void *)v.r));
+        v.p = nullptr;
+        for (int k : {3, 4, 7})   // the batches' graphs hold the old addresses
+            if (graphs[k].exec) {
+                cudaGraphExecDestroy(graphs[k].exec);
+                graphs[k].exec = nullptr;
+            }
+    }
+    const long words = spinor_words<W>(g);
+    void *buf;
+    ST(alloc(&buf, (size_t)words * sizeof(W) * nrhs * (npole + 3)));
+    W *d = (W *)buf;
+    v.r = d;
+    v.t = d + words * nrhs;
+    v.y = d + 2 * words * nrhs;
+    v.p = d + 3 * words * nrhs;
+    v.stride = words;
+    cap = nrhs;
     return OVL_OK;
 }
 
@@ -710,22 +734,7 @@ ovl_status Ctx::sign64_batch(const double2 *b, double2 *out, int nrhs, const dou
         return OVL_OK;
     }
     ST(ensure_batch());
-    if (!msb64.p || msb64_cap < nrhs) {   // sized to the batch (grown when a larger one comes)
-        if (msb64.p) {
-            cudaFree(msb64.r);
-            allocs.erase(std::find(allocs.begin(), allocs.end(), (void *)msb64.r));
-        }
-        const long words = (long)g.V * 12;
-        void *buf;
-        ST(alloc(&buf, (size_t)words * sizeof(double2) * nrhs * (npole + 3)));
-        double2 *d = (double2 *)buf;
-        msb64.r = d;
-        msb64.t = d + words * nrhs;
-        msb64.y = d + 2 * words * nrhs;
-        msb64.p = d + 3 * words * nrhs;
-        msb64.stride = words;
-        msb64_cap = nrhs;
-    }
+    ST(ensure_msb(msb64, msb64_cap, nrhs));
     long iters = 0;
     auto init = [&]() { return msb_init_f64(g, nrhs, npole, msb_state, msb64, b, rsb, bcounters, stream); };
     auto it = [&]() { return msb_iter_f64(g, U64, m0_ker, nrhs, npole, msb_state, msb64, rsb, bcounters, stream); };
@@ -738,6 +747,37 @@ ovl_status Ctx::sign64_batch(const double2 *b, double2 *out, int nrhs, const dou
     return OVL_OK;
 }
 
+// The same in float-float arithmetic (sign_ff).
+ovl_status Ctx::sign_ff_batch(const double2 *b, double2 *out, int nrhs, const double *tol, int mode) {
+    Ctx *c = this;
+    const long words = (long)g.V * 12;
+    // the FP64 batch's vectors serve both arithmetics (words of the same size, one call at a time);
+    // a batch that does not fit runs one vector at a time in the single vector's memory
+    static_assert(sizeof(ffw) == sizeof(double2), "");
+    if (nrhs == 1 || ndefl || p.sign_method == OVL_SIGN_KRYLOV || ensure_msb(msb64, msb64_cap, nrhs) != OVL_OK) {
+        for (int y = 0; y < nrhs; y++)
+            if (tol[y] > 0) ST(sign_ff(b + y * words, out + y * words, tol[y], mode));
+        return OVL_OK;
+    }
+    PhaseClock pclk(this, &t_sign64);
+    ST(ensure_batch());
+    ST(ensure_ff_links());
+    const MsBatch<ffw> vf{(ffw *)msb64.r, (ffw *)msb64.t, (ffw *)msb64.y, (ffw *)msb64.p, msb64.stride};
+    // b in float-float into t (t is overwritten by the first iteration's Q p)
+    CK(spinor_d2ff(g, b, vf.t, stream, nrhs));
+    long iters = 0;
+    auto init = [&]() { return msb_init_ff(g, nrhs, npole, msb_state, vf, vf.t, rsb, bcounters, stream); };
+    auto it = [&]() { return msb_iter_ff(g, Uff, m0_ker, nrhs, npole, msb_state, vf, rsb, bcounters, stream); };
+    const int n = pick_poles(min_positive(tol, nrhs));
+    ST((msb_run<ffw>(nrhs, tol, n, 7, init, it, &iters)));
+    stat_msff += iters * nrhs;
+    const double sc = zs_d0[n - 1] / lam_min;
+    CK(wilson_batch_ff(g, Uff, vf.y, vf.t, words, nrhs, m0_ker, mode == 0, sc, nullptr, 0.0, stream));
+    CK(spinor_ff2d(g, vf.t, out, stream, nrhs));
+    if (mode == 1) CK(dev_axpby(rho, (const double *)b, 1.0, (double *)out, n64 * nrhs, stream));
+    return OVL_OK;
+}
+
 ovl_status Ctx::sign32_batch(const float4 *b, float4 *out, int nrhs, const double *tol, int mode) {
     Ctx *c = this;
     if (ndefl) {
@@ -747,22 +787,7 @@ ovl_status Ctx::sign32_batch(const float4 *b, float4 *out, int nrhs, const doubl
         return OVL_OK;
     }
     ST(ensure_batch());
-    if (!msb32.p || msb32_cap < nrhs) {
-        if (msb32.p) {
-            cudaFree(msb32.r);
-            allocs.erase(std::find(allocs.begin(), allocs.end(), (void *)msb32.r));
-        }
-        const long words = (long)g.V * 6;
-        void *buf;
-        ST(alloc(&buf, (size_t)words * sizeof(float4) * nrhs * (npole + 3)));
-        float4 *d = (float4 *)buf;
-        msb32.r = d;
-        msb32.t = d + words * nrhs;
-        msb32.y = d + 2 * words * nrhs;
-        msb32.p = d + 3 * words * nrhs;
-        msb32.stride = words;
-        msb32_cap = nrhs;
-    }
+    ST(ensure_msb(msb32, msb32_cap, nrhs));
     long iters = 0;
     auto init = [&]() { return msb_init_f32(g, nrhs, npole, msb_state, msb32, b, rsb, stream); };
     auto it = [&]() {

@@ -376,6 +376,10 @@ cudaError_t wilson_batch_f64(const Geom &g, const double2 *U, const double2 *in,
                              double m0, int g5, double a, const double2 *z, double b, cudaStream_t st) {
     return wilson_hops<double>(g, U, in, out, stride, nrhs, m0, g5, a, z, b, st);
 }
+cudaError_t wilson_batch_ff(const Geom &g, const ffl *U, const ffw *in, ffw *out, long stride, int nrhs, double m0,
+                            int g5, double a, const ffw *z, double b, cudaStream_t st) {
+    return wilson_hops<ff>(g, U, in, out, stride, nrhs, m0, g5, a, z, b, st);
+}
 cudaError_t wilson_ff(const Geom &g, const ffl *U, const ffw *in, ffw *out, double m0, int g5, double a,
                       const ffw *z, double b, cudaStream_t st) {
     return wilson_hops<ff>(g, U, in, out, 0, 1, m0, g5, a, z, b, st);

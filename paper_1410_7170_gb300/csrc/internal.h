@@ -223,6 +223,8 @@ constexpr int kMaxBatch = 12;   // right-hand sides per batch (threads 32 x nrhs
 // out_y = a [gamma5] D_W(m0) in_y + b z_y for y < nrhs; vectors `stride` storage words apart.
 cudaError_t wilson_batch_f64(const Geom &g, const double2 *U, const double2 *in, double2 *out, long stride, int nrhs,
                              double m0, int g5, double a, const double2 *z, double b, cudaStream_t st);
+cudaError_t wilson_batch_ff(const Geom &g, const ffl *U, const ffw *in, ffw *out, long stride, int nrhs, double m0,
+                            int g5, double a, const ffw *z, double b, cudaStream_t st);
 cudaError_t wilson_batch_f32(const Geom &g, const float4 *U, const float4 *in, float4 *out, long stride, int nrhs,
                              float m0, int g5, float a, const float4 *z, float b, cudaStream_t st);
 

@@ -108,7 +108,7 @@ struct Ctx {
     MsState *msff_state = nullptr;
     GraphSlot graphs[8];
     // batched multishift (several right-hand sides in lock-step)
-    MsBatch<double2> msb64{};
+    MsBatch<double2> msb64{};          // FP64 and float-float batches (sign_ff_batch)
     MsBatch<float4> msb32{};
     int msb64_cap = 0, msb32_cap = 0;
     MsState *msb_state = nullptr;      // kMaxBatch states
@@ -234,7 +234,10 @@ struct Ctx {
     ovl_status ensure_msh();
     // several right-hand sides: b, out hold nrhs internal vectors back to back
     ovl_status ensure_batch();
+    template <typename W>
+    ovl_status ensure_msb(MsBatch<W> &v, int &cap, int nrhs);
     ovl_status sign64_batch(const double2 *b, double2 *out, int nrhs, const double *tol, int mode);
+    ovl_status sign_ff_batch(const double2 *b, double2 *out, int nrhs, const double *tol, int mode);
     ovl_status sign_outer_batch(const double2 *b, double2 *out, int nrhs, const double *tol, int mode);
     ovl_status sign32_batch(const float4 *b, float4 *out, int nrhs, const double *tol, int mode);
     template <typename ST, typename Init, typename Iter>

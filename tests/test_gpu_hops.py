@@ -71,3 +71,29 @@ def test_sign_scales_with_its_argument(power):
     op.sign_apply(out, b * 2.0 ** power, 1e-13)
     assert ((out * 2.0 ** -power - ref).norm() / ref.norm()).item() < 1e-11
     op.close()
+
+
+def test_batches_of_both_arithmetics_share_vectors():
+    """The mixed solve's float-float batches and D_N's FP64 batches use the same vectors, which
+    grow with the batch: results are the same before and after the other has moved them."""
+    dims = (4, 4, 4, 8)
+    U, op = _op(dims, precision=ovl.OVL_MIXED_FP32, precond=ovl.OVL_PREC_RECURSIVE, sap_block=(2, 2, 2, 2))
+    b = dev(synth.rhs_gaussian(dims, 34, n_rhs=9))
+
+    def solve(n):
+        x = torch.zeros_like(b[:n])
+        op.ovl_solve(x, b[:n], n, 1e-10)
+        return x
+
+    def apply(n):
+        y = torch.empty_like(b[:n])
+        op.ovl_apply_n(y, b[:n], n, 1e-12)
+        return y
+
+    x2, y2, x3, y9 = solve(2), apply(2), solve(3), apply(9)
+    assert torch.equal(solve(2), x2) and torch.equal(solve(3), x3)
+    assert torch.equal(apply(2), y2) and torch.equal(apply(9), y9)
+    r = torch.empty_like(x3)
+    op.ovl_apply_n(r, x3, 3, 1e-13)
+    assert ((r - b[:3]).norm() / b[:3].norm()).item() < 2e-10
+    op.close()
