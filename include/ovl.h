@@ -120,7 +120,7 @@ typedef struct {
     int use_graphs;         /* 1: capture multishift iterations in CUDA graphs */
     int check_every;        /* multishift iterations between host convergence checks */
     int stencil_tps;        /* threads per lattice site of the FP32 stencils: 0 = autotune, 1 or 4 = forced */
-    int sap_tps;            /* threads per block site of the FP32 Schwarz block solves: 0 = autotune, 1, 2 or 4 */
+    int sap_tps;            /* 0, 1, 2 or 4; accepted and reported by ovl_tuning_sap (one FP32 block kernel) */
     int adaptive_poles;     /* 1 (default): each sign application uses the smallest Zolotarev degree
                                n <= n_poles whose uniform error delta(k, n) is <= 1/10 of its requested
                                accuracy; 0: always n_poles */
@@ -267,10 +267,10 @@ ovl_status ovl_krylov_sign_info(const ovl_ctx *ctx, long *cycles, long *matvecs)
  * more than 60 n + 100 steps. */
 ovl_status ovl_hermitian_eig(int n, const double *A, double *w, double *Z);
 
-/* Threads per block site chosen for the FP32 Schwarz block solves of the Wilson
- * preconditioner (Sec. 5.1 smoother; an implementation choice, the paper has no
- * counterpart) and the measured time of one Schwarz cycle per variant (ms[3]: 1, 2, 4
- * threads per site; zeros when not tuned). tps, ms nullable. */
+/* FP32 Schwarz block solves of the Wilson preconditioner (Sec. 5.1 smoother; an implementation
+ * choice, the paper has no counterpart): they have one form, two threads per block site. *tps is
+ * params.sap_tps if that is set and 2 otherwise; ms[0..2] the measured time of one Schwarz cycle
+ * (zeros when sap_tps is set or precond is OVL_PREC_NONE). tps, ms nullable. */
 ovl_status ovl_tuning_sap(const ovl_ctx *ctx, int *tps, float *ms);
 
 /* out_k = D_W(m0) in_k for k < n_rhs (n_rhs vectors back to back), with the multi-RHS

@@ -1091,25 +1091,10 @@ ovl_status Ctx::autotune_mrhs() {
     return OVL_OK;
 }
 
-// Threads per site of the FP32 Schwarz block kernel (1, 2 or 4): one Schwarz cycle of
-// each variant is timed on a constant non-zero input and the fastest kept. Cached per
-// process, lattice shape and block shape.
-static std::map<std::tuple<int, int, int, int, int, int, int, int, int>, std::pair<int, std::array<float, 3>>>
-    g_sap_cache;
-
-ovl_status Ctx::autotune_sap() {
+// Time of one FP32 Schwarz cycle on a constant non-zero input, for ovl_tuning_sap (the block kernel
+// has one form, two threads per block site).
+ovl_status Ctx::time_sap() {
     Ctx *c = this;
-    const auto key = std::make_tuple(g.L[0], g.L[1], g.L[2], g.L[3], p.sap_block[0], p.sap_block[1], p.sap_block[2],
-                                     p.sap_block[3], p.sap_mr_iters);
-    {
-        std::lock_guard<std::mutex> lk(g_tune_mu);
-        auto it = g_sap_cache.find(key);
-        if (it != g_sap_cache.end()) {
-            sap_tps = it->second.first;
-            for (int k = 0; k < 3; k++) sap_ms[k] = it->second.second[k];
-            return OVL_OK;
-        }
-    }
     void *buf;
     const size_t bytes = (size_t)n64 * sizeof(float);
     ST(alloc(&buf, bytes * 3));
@@ -1119,39 +1104,18 @@ ovl_status Ctx::autotune_sap() {
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
     const int reps = g.V >= (1 << 20) ? 3 : 10;
-    const int tps_of[3] = {1, 2, 4};
-    float best = 0.f;
-    int best_tps = 1;
-    for (int v = 0; v < 3; v++) {
-        SapGeom sg = make_sap_geom(g, p.sap_block);
-        sg.tps = tps_of[v];
-        for (int k = 0; k < 2 + reps; k++) {
-            if (k == 2) CK(cudaEventRecord(e0, stream));
-            CK(sap_f32(g, sg, U32, fv, fx, fr, -0.5f, 1, p.sap_mr_iters, stream));
-        }
-        CK(cudaEventRecord(e1, stream));
-        CK(cudaEventSynchronize(e1));
-        float ms;
-        CK(cudaEventElapsedTime(&ms, e0, e1));
-        sap_ms[v] = ms / reps;
-        if (v == 0 || sap_ms[v] < best) {
-            best = sap_ms[v];
-            best_tps = tps_of[v];
-        }
+    const SapGeom sg = make_sap_geom(g, p.sap_block);
+    for (int k = 0; k < 2 + reps; k++) {
+        if (k == 2) CK(cudaEventRecord(e0, stream));
+        CK(sap_f32(g, sg, U32, fv, fx, fr, -0.5f, 1, p.sap_mr_iters, stream));
     }
+    CK(cudaEventRecord(e1, stream));
+    CK(cudaEventSynchronize(e1));
+    float ms;
+    CK(cudaEventElapsedTime(&ms, e0, e1));
+    sap_ms[0] = sap_ms[1] = sap_ms[2] = ms / reps;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    sap_tps = best_tps;
-    {
-        std::lock_guard<std::mutex> lk(g_tune_mu);   // first writer wins, as in autotune()
-        auto it = g_sap_cache.find(key);
-        if (it != g_sap_cache.end()) {
-            sap_tps = it->second.first;
-            for (int k = 0; k < 3; k++) sap_ms[k] = it->second.second[k];
-        } else {
-            g_sap_cache[key] = {sap_tps, {sap_ms[0], sap_ms[1], sap_ms[2]}};
-        }
-    }
     cudaFree(buf);
     allocs.erase(std::find(allocs.begin(), allocs.end(), buf));
     return OVL_OK;
@@ -1288,13 +1252,7 @@ static ovl_status create_impl(Ctx *c, const double *gauge, const int dims[4], do
     else ST(c->autotune());
     if (c->p.mrhs_kernel) c->g.mrhs32 = c->g.mrhs32l = c->p.mrhs_kernel;
     else ST(c->autotune_mrhs());
-    if (c->p.sap_tps) {
-        c->sap_tps = c->p.sap_tps;
-        c->sap_tuned = true;
-    } else if (c->p.precond != OVL_PREC_NONE) {
-        ST(c->autotune_sap());
-        c->sap_tuned = true;
-    }
+    if (!c->p.sap_tps && c->p.precond != OVL_PREC_NONE) ST(c->time_sap());
     // spectral interval of |Q|
     if (c->p.lambda_min > 0) {
         c->lam_min = c->p.lambda_min;
@@ -1550,7 +1508,7 @@ extern "C" ovl_status ovl_m0_adapt_info(const ovl_ctx *ctx, double *cand, double
 extern "C" ovl_status ovl_tuning_sap(const ovl_ctx *ctx, int *tps, float *ms) {
     const Ctx *c = reinterpret_cast<const Ctx *>(ctx);
     if (!c) return OVL_EINVAL;
-    if (tps) *tps = c->sap_tps;
+    if (tps) *tps = c->p.sap_tps ? c->p.sap_tps : 2;
     if (ms)
         for (int k = 0; k < 3; k++) ms[k] = c->sap_ms[k];
     return OVL_OK;
@@ -1573,10 +1531,6 @@ extern "C" ovl_status wilson_solve(ovl_ctx *ctx, double *x, const double *b, dou
             c->err = "sap_block must be even, divide the lattice extent and hold <= 256 sites";
             return OVL_EINVAL;
         }
-    }
-    if (!c->sap_tuned) {
-        ST(c->autotune_sap());
-        c->sap_tuned = true;
     }
     int it = 0;
     if (c->p.precision == OVL_FP64) {
@@ -1609,10 +1563,6 @@ extern "C" ovl_status wilson_sap_apply(ovl_ctx *ctx, double *out, const double *
     if (c->p.sap_cycles < 1 || c->p.sap_mr_iters < 1) {
         c->err = "sap_cycles and sap_mr_iters must be >= 1";
         return OVL_EINVAL;
-    }
-    if (!c->sap_tuned) {
-        ST(c->autotune_sap());
-        c->sap_tuned = true;
     }
     const bool late = on_device(in, out);
     if (c->p.precision == OVL_FP64) {

@@ -156,8 +156,7 @@ ovl_status mg_setup(Ctx *c, double m0, const double *start, int n_start) {
         mg.graph = nullptr;
     }
     const Geom &g = c->g;
-    SapGeom sg = make_sap_geom(g, c->p.sap_block);
-    sg.tps = c->sap_tps;
+    const SapGeom sg = make_sap_geom(g, c->p.sap_block);
     const long vw = (long)g.V * 6;   // float4 words per FP32 spinor
     cudaStream_t st = c->stream;
     // start vectors
@@ -241,8 +240,7 @@ ovl_status mg_setup(Ctx *c, double m0, const double *start, int n_start) {
 static cudaError_t mg_apply_kernels(Ctx *c, const float4 *r, float4 *x, double m0) {
     MgData &mg = c->mg;
     const Geom &g = c->g;
-    SapGeom sg = make_sap_geom(g, c->p.sap_block);
-    sg.tps = c->sap_tps;
+    const SapGeom sg = make_sap_geom(g, c->p.sap_block);
     cudaStream_t st = c->stream;
     cudaError_t e;
     if ((e = mg_restrict(g, sg, mg.P, mg.nv, r, mg.rc, mg.nc, 0, st)) != cudaSuccess) return e;
@@ -301,10 +299,6 @@ extern "C" ovl_status ovl_mg_setup(ovl_ctx *ctx, double m0, const double *start,
         c->err = "ovl_mg_setup: need finite m0 and n_start >= 1 with start vectors";
         return OVL_EINVAL;
     }
-    if (!c->sap_tuned) {
-        ST(c->autotune_sap());
-        c->sap_tuned = true;
-    }
     return mg_setup(c, m0, start, n_start);
 }
 
@@ -316,10 +310,6 @@ extern "C" ovl_status wilson_mg_apply(ovl_ctx *ctx, double *out, const double *i
         return OVL_EINVAL;
     }
     ST(mg_check(c, c->mg.ready ? c->mg.nv : c->p.mg_nv));
-    if (!c->sap_tuned) {
-        ST(c->autotune_sap());
-        c->sap_tuned = true;
-    }
     ST(ensure_f32_buffers(c));
     ST(c->import_vec(in, (float4 *)c->f_a));
     ST(mg_apply_f32(c, (const float4 *)c->f_a, (float4 *)c->f_b, m0));

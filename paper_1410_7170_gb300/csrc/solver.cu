@@ -294,8 +294,7 @@ static ovl_status wilson_solve(Ctx *c, Krylov<T> &k, const T *in, T *out, double
         ST(c->alloc(&buf, (size_t)c->n64 * sizeof(T)));
         scratch = (T *)buf;
     }
-    SapGeom sg = make_sap_geom(c->g, c->p.sap_block);
-    sg.tps = c->sap_tps;
+    const SapGeom sg = make_sap_geom(c->g, c->p.sap_block);
     auto mv = [&](const T *a, T *o, double) -> ovl_status {
         CK(Ops<T>::wilson(c, a, o, m0));
         return OVL_OK;
@@ -426,8 +425,7 @@ ovl_status wilson_solve_eo<float4>(Ctx *c, const float4 *b, float4 *x, double m0
 // solve, on D_W(m0). The same call the Wilson FGMRES makes for its preconditioner.
 template <typename T>
 static ovl_status sap_apply_t(Ctx *c, const T *b, T *x, void *&scratch, double m0) {
-    SapGeom sg = make_sap_geom(c->g, c->p.sap_block);
-    sg.tps = c->sap_tps;
+    const SapGeom sg = make_sap_geom(c->g, c->p.sap_block);
     if (!scratch) ST(c->alloc(&scratch, (size_t)c->n64 * sizeof(T)));
     CK(Ops<T>::sap(c, sg, b, x, (T *)scratch, m0));
     return OVL_OK;
@@ -817,8 +815,7 @@ ovl_status wilson_solve_batch(Ctx *c, int nb, const T *in, T *out, double m0, do
         ST(c->alloc(&buf, (size_t)c->n64 * sizeof(T)));
         scratch = (T *)buf;
     }
-    SapGeom sg = make_sap_geom(c->g, c->p.sap_block);
-    sg.tps = c->sap_tps;
+    const SapGeom sg = make_sap_geom(c->g, c->p.sap_block);
     const long n = c->n64;
     auto mv = [&](const T *a, T *o, const double *) -> ovl_status {
         if (sizeof(T) == 8)
@@ -830,6 +827,11 @@ ovl_status wilson_solve_batch(Ctx *c, int nb, const T *in, T *out, double m0, do
         return OVL_OK;
     };
     auto pc = [&](const T *a, T *o, const char *act) -> ovl_status {
+        if (sizeof(T) == 4 && !c->p.wilson_mg) {
+            CK(sap_f32_rows(c->g, sg, c->U32, (const float4 *)a, (float4 *)o, (float4 *)scratch, (long)c->g.V * 6, nb,
+                            act, (float)m0, c->p.sap_cycles, c->p.sap_mr_iters, c->stream));
+            return OVL_OK;
+        }
         for (int y = 0; y < nb; y++) {
             if (!act[y]) CK(cudaMemsetAsync(o + (long)y * n, 0, n * sizeof(T), c->stream));
             else if (sizeof(T) == 4 && c->p.wilson_mg)

@@ -145,10 +145,8 @@ struct Ctx {
     float tune_ms[4] = {0, 0, 0, 0};   // stencil ms: fp64 1/4 tps, fp32 1/4 tps
     float tune_mrhs_ms[6] = {0, 0, 0, 0, 0, 0};   // FP32 multi-RHS stencil ms per RHS of kernels 1, 2, 3
                                                     // at 4 right-hand sides, then at 12
-    int sap_tps = 1;                   // threads per site of the FP32 Schwarz block kernel
     double t_sign64 = 0, t_sign_low = 0, t_prec = 0;   // phase wall times of the current solve (s)
-    bool sap_tuned = false;
-    float sap_ms[3] = {0, 0, 0};       // one FP32 Schwarz cycle, ms: 1, 2, 4 threads per site
+    float sap_ms[3] = {0, 0, 0};       // one FP32 Schwarz cycle, ms (the same value three times)
     // low-mode deflation of the sign function (params.n_deflate > 0)
     int ndefl = 0;
     double2 *defl64 = nullptr, *defl64g5 = nullptr;   // eigenvectors xi_i of Q and gamma5 xi_i (FP64)
@@ -247,7 +245,7 @@ struct Ctx {
     ovl_status set_zolotarev();
     ovl_status autotune();
     ovl_status autotune_mrhs();
-    ovl_status autotune_sap();
+    ovl_status time_sap();
     ovl_status deflation_setup();
     ovl_status defl_project64(const double2 *b, double2 *bp, std::vector<double> &coef);
     ovl_status defl_add64(const std::vector<double> &coef, double2 *out, int mode);
