@@ -171,7 +171,7 @@ Ctx::~Ctx() {
     if (mg.graph) cudaGraphExecDestroy(mg.graph);
     for (int w = 0; w < 3; w++)
         if (ev_ready[w])
-            for (int k = 0; k < 4; k++) cudaEventDestroy(ev[w][k]);
+            for (int k = 0; k < 6; k++) cudaEventDestroy(ev[w][k]);
     for (void *p : allocs) cudaFree(p);
     if (h_pinned) cudaFreeHost(h_pinned);
     if (own_stream && stream) cudaStreamDestroy(stream);
@@ -320,37 +320,49 @@ ovl_status Ctx::ms_setup(MsState *d_state, double tol, int *n_out) {
     return OVL_OK;
 }
 
+// Iteration k of a chunk ends with the pending shift updates: every ring-th one and the last.
+static bool ms_flush(int k, int chunk, int ring) { return (k + 1) % ring == 0 || k == chunk - 1; }
+
 // Polls the device state every check_every iterations; graphs replay the chunk.
-// With instrumentation on, event records around the first three kernels of every
-// iteration are part of the queued work (event record nodes inside graphs) and the
-// device logs how many shifts each iteration updated, so per-kernel durations and
-// algorithmic bytes come from the same launches that do the work.
+// With instrumentation on, event records around the three kernels of one iteration (the first
+// that updates the shifts) and around the p_0 kernel of the one before are part of the queued
+// work (event record nodes inside graphs) and the device logs how many shifts each iteration
+// updated, so per-kernel durations and algorithmic bytes come from the same launches that do the
+// work.
 template <typename Iter>
-ovl_status Ctx::ms_run(MsState *d_state, int which, int slot, double shift_bytes, bool fused, Iter iter_fn,
+ovl_status Ctx::ms_run(MsState *d_state, int which, int slot, int ring, double shift_bytes, Iter iter_fn,
                        int *iters_out) {
     Ctx *c = this;
     const int chunk = std::min(p.check_every, kMaxChunk);
-    const int sample = chunk / 2;   // the iteration of every chunk whose kernels are timed
+    const int sample = std::min(ring, chunk) - 1;   // the iteration of every chunk whose kernels are timed
     const double rbytes = which == 1 ? 4.0 : 8.0;   // bytes per real: FP32 slot 4, FP64 and float-float 8
     int done_iters = 0, iter_before = 0;
     GraphSlot &gs = graphs[slot];
     if (prof && !ev_ready[which]) {
-        for (int k = 0; k < 4; k++) CK(cudaEventCreate(&ev[which][k]));
+        for (int k = 0; k < 6; k++) CK(cudaEventCreate(&ev[which][k]));
         ev_ready[which] = true;
     }
     if (gs.exec && (gs.chunk != chunk || gs.prof != prof)) {
         cudaGraphExecDestroy(gs.exec);
         gs.exec = nullptr;
     }
+    auto queue = [&](unsigned flags) {
+        cudaError_t ce = cudaSuccess;
+        for (int k = 0; k < chunk && ce == cudaSuccess; k++) {
+            MsEvents e;
+            if (prof && k == sample) e = MsEvents{ev[which], flags, 0};
+            if (prof && k == sample - 1) e = MsEvents{ev[which] + 2, flags, 2};   // records 4 and 5
+            ce = iter_fn(ms_flush(k, chunk, ring), e);
+        }
+        return ce;
+    };
     while (true) {
         if (p.use_graphs) {
             if (!gs.exec) {
                 cudaGraph_t graph;
                 set_launch_counting(false);
                 CK(cudaStreamBeginCapture(stream, cudaStreamCaptureModeThreadLocal));
-                cudaError_t ce = cudaSuccess;
-                for (int k = 0; k < chunk && ce == cudaSuccess; k++)
-                    ce = iter_fn(prof && k == sample ? ev[which] : nullptr, cudaEventRecordExternal);
+                const cudaError_t ce = queue(cudaEventRecordExternal);
                 cudaError_t ee = cudaStreamEndCapture(stream, &graph);
                 set_launch_counting(true);
                 CK(ce);
@@ -364,7 +376,7 @@ ovl_status Ctx::ms_run(MsState *d_state, int which, int slot, double shift_bytes
             CK(cudaGraphLaunch(gs.exec, stream));
             count_launches(3L * chunk);
         } else {
-            for (int k = 0; k < chunk; k++) CK(iter_fn(prof && k == sample ? ev[which] : nullptr, 0u));
+            CK(queue(0u));
         }
         done_iters += chunk;
         CK(cudaMemcpyAsync(h_ms_small, d_state, 4 * sizeof(int), cudaMemcpyDeviceToHost, stream));
@@ -377,26 +389,29 @@ ovl_status Ctx::ms_run(MsState *d_state, int which, int slot, double shift_bytes
             const double V = (double)g.V;
             ProfAcc &pa = pacc[which];
             // algorithmic reals per site: Q p: p, 4 links x 12, t; residual: t, links, p, r in/out;
-            // shifts: r, y in/out, each updated p_l in/out. Fused form: the residual kernel also
-            // moves y in/out and the p_l (l >= 1), the third kernel r, p_0 in/out.
-            const double qb = 96.0 * V * rbytes;
+            // p_0: r, p in/out; shift updates of np iterations: np residuals and base directions, p_0
+            // out, y in/out, each updated p_l (l >= 1) in/out; an iteration's share of its block
+            const double qb = 96.0 * V * rbytes, rb = 144.0 * V * rbytes;
             for (int k = 0; k < ran; k++) {
-                const double rb = fused ? (192.0 * rbytes + shift_bytes * (h_hist[k] - 1)) * V : 144.0 * V * rbytes;
-                const double sb = fused ? 72.0 * rbytes * V : (72.0 * rbytes + shift_bytes * h_hist[k]) * V;
+                const int first = k - k % ring, np = std::min({ring, ran - first, chunk - first});
+                const double sb = ring == 1 ? (72.0 * rbytes + shift_bytes * h_hist[k]) * V
+                                            : ((48.0 * np + 72.0 + 72.0 * (np - 1)) * rbytes +
+                                               shift_bytes * (h_hist[first] - 1)) * V / np;
                 pa.n++;
                 pa.q_bytes += qb;
                 pa.r_bytes += rb;
                 pa.s_bytes += sb;
                 if (k != sample) continue;
-                float a = 0, b = 0, d = 0;
+                float a = 0, b = 0, d = 0, d0 = 0;
                 if (cudaEventElapsedTime(&a, ev[which][0], ev[which][1]) != cudaSuccess ||
                     cudaEventElapsedTime(&b, ev[which][1], ev[which][2]) != cudaSuccess ||
-                    cudaEventElapsedTime(&d, ev[which][2], ev[which][3]) != cudaSuccess) {
+                    cudaEventElapsedTime(&d, ev[which][2], ev[which][3]) != cudaSuccess ||
+                    (sample > 0 && cudaEventElapsedTime(&d0, ev[which][4], ev[which][5]) != cudaSuccess)) {
                     cudaGetLastError();
                     pa.valid = false;
                     continue;
                 }
-                pa.q_ms += a; pa.r_ms += b; pa.s_ms += d;
+                pa.q_ms += a; pa.r_ms += b; pa.s_ms += (d + sample * d0) / (sample + 1);
                 pa.q_t++; pa.r_t++; pa.s_t++;
                 pa.q_tb += qb; pa.r_tb += rb; pa.s_tb += sb;
             }
@@ -436,11 +451,13 @@ ovl_status Ctx::sign64(const double2 *b, double2 *out, double tol, int mode) {
     }
     int n;
     ST(ms_setup(ms64_state, tol, &n));
-    CK(ms_init_f64(g, n, ms64_state, ms64, bm, rs, stream));
+    CK(ms_init(g, 1, ms64_state, ms64, bm, rs, rs.counter, stream));
     int iters = 0;
-    auto fn = [&](cudaEvent_t *e, unsigned f) { return ms_iter_f64(g, U64, m0_ker, ms64_state, ms64, rs, stream, e, f); };
+    auto fn = [&](bool flush, const MsEvents &e) {
+        return ms_iter(g, U64, m0_ker, 1, ms64_state, ms64, rs, rs.counter, flush, stream, e);
+    };
     // at the iteration cap the output is still formed from the last iterate (status ENOCONV)
-    const ovl_status ms = ms_run(ms64_state, 0, 0, 48.0 * 8.0, false, fn, &iters);
+    const ovl_status ms = ms_run(ms64_state, 0, 0, ms64.ring, 48.0 * 8.0, fn, &iters);
     if (ms != OVL_OK && ms != OVL_ENOCONV) return ms;
     stat_ms64 += iters;
     const double sc = zs_d0[n - 1] / lam_min;
@@ -469,10 +486,12 @@ ovl_status Ctx::sign_ff(const double2 *b, double2 *out, double tol, int mode) {
     ST(ms_setup(msff_state, tol, &n));
     // b in float-float into t (t is overwritten by the first iteration's Q p)
     CK(spinor_d2ff(g, bm, msff.t, stream));
-    CK(ms_init_ff(g, n, msff_state, msff, msff.t, rs, stream));
+    CK(ms_init(g, 1, msff_state, msff, msff.t, rs, rs.counter, stream));
     int iters = 0;
-    auto fn = [&](cudaEvent_t *e, unsigned f) { return ms_iter_ff(g, Uff, m0_ker, msff_state, msff, rs, stream, e, f); };
-    const ovl_status ms = ms_run(msff_state, 2, 5, 48.0 * 8.0, false, fn, &iters);
+    auto fn = [&](bool flush, const MsEvents &e) {
+        return ms_iter(g, Uff, m0_ker, 1, msff_state, msff, rs, rs.counter, flush, stream, e);
+    };
+    const ovl_status ms = ms_run(msff_state, 2, 5, msff.ring, 48.0 * 8.0, fn, &iters);
     if (ms != OVL_OK && ms != OVL_ENOCONV) return ms;
     stat_msff += iters;
     const double sc = zs_d0[n - 1] / lam_min;
@@ -514,21 +533,13 @@ ovl_status Ctx::ensure_16(bool bf16) {
 
 ovl_status Ctx::ensure_msff() {
     ST(ensure_ff_links());
-    if (msff.p) return OVL_OK;
+    if (msff.r) return OVL_OK;
     void *buf;
     if (!msff_state) {
         ST(alloc(&buf, sizeof(MsState)));
         msff_state = (MsState *)buf;
     }
-    const long words = (long)g.V * 12;   // ffw per vector
-    ST(alloc(&buf, (size_t)words * sizeof(ffw) * (npole + 3)));
-    ffw *f = (ffw *)buf;
-    msff.r = f;
-    msff.t = f + words;
-    msff.y = f + 2 * words;
-    msff.p = f + 3 * words;
-    msff.stride = words;
-    return OVL_OK;
+    return alloc_ms(msff, 1, kMaxRing);
 }
 
 ovl_status Ctx::sign_outer(const double2 *b, double2 *out, double tol, int mode) {
@@ -561,20 +572,20 @@ ovl_status Ctx::sign32(const float4 *b, float4 *out, double tol, int mode, int s
         ST(ensure_msh());
         ST(ms_setup(msh_state, tol, &n));
         CK(ms_init_half(g, n, msh_state, msh, b, rs, bf, stream));
-        auto fn = [&](cudaEvent_t *e, unsigned f) {
-            return ms_iter_half(g, U32, (float)m0_ker, msh_state, msh, rs, bf, stream, e, f);
+        auto fn = [&](bool, const MsEvents &e) {
+            return ms_iter_half(g, U32, m0_ker, msh_state, msh, rs, bf, stream, e);
         };
-        ms = ms_run(msh_state, 1, bf ? 6 : 2, bf ? 96.0 : 104.0, false, fn, &iters);
+        ms = ms_run(msh_state, 1, bf ? 6 : 2, 1, bf ? 96.0 : 104.0, fn, &iters);
         if (ms != OVL_OK && ms != OVL_ENOCONV) return ms;
         y = msh.y;
     } else {
         ST(ensure_ms32());
         ST(ms_setup(ms32_state, tol, &n));
-        CK(ms_init_f32(g, n, ms32_state, ms32, b, rs, stream));
-        auto fn = [&](cudaEvent_t *e, unsigned f) {
-            return ms_iter_f32(g, U32, (float)m0_ker, ms32_state, ms32, rs, stream, e, f);
+        CK(ms_init(g, 1, ms32_state, ms32, b, rs, rs.counter, stream));
+        auto fn = [&](bool flush, const MsEvents &e) {
+            return ms_iter(g, U32, m0_ker, 1, ms32_state, ms32, rs, rs.counter, flush, stream, e);
         };
-        ms = ms_run(ms32_state, 1, 1, 48.0 * 4.0, g.tps32 != 4, fn, &iters);
+        ms = ms_run(ms32_state, 1, 1, ms32.ring, 48.0 * 4.0, fn, &iters);
         if (ms != OVL_OK && ms != OVL_ENOCONV) return ms;
         y = ms32.y;
     }
@@ -586,19 +597,7 @@ ovl_status Ctx::sign32(const float4 *b, float4 *out, double tol, int mode, int s
     return ms;
 }
 
-ovl_status Ctx::ensure_ms64() {
-    if (ms64.p) return OVL_OK;
-    const long words = (long)g.V * 12;   // double2 per vector
-    void *buf;
-    ST(alloc(&buf, (size_t)words * sizeof(double2) * (npole + 3)));
-    double2 *b2 = (double2 *)buf;
-    ms64.r = b2;
-    ms64.t = b2 + words;
-    ms64.y = b2 + 2 * words;
-    ms64.p = b2 + 3 * words;
-    ms64.stride = words;
-    return OVL_OK;
-}
+ovl_status Ctx::ensure_ms64() { return ms64.r ? OVL_OK : alloc_ms(ms64, 1, kMaxRing); }
 // ---- several right-hand sides
 ovl_status Ctx::ensure_batch() {
     Ctx *c = this;
@@ -619,29 +618,35 @@ ovl_status Ctx::ensure_batch() {
     return OVL_OK;
 }
 
-// Batched multishift vectors for nrhs right-hand sides (grown when a larger batch comes).
+// Multishift vectors for nrhs right-hand sides, one allocation that starts at v.r.
+template <typename W>
+ovl_status Ctx::alloc_ms(MsBatch<W> &v, int nrhs, int ring) {
+    const long words = spinor_words<W>(g);
+    void *buf;
+    ST(alloc(&buf, (size_t)words * sizeof(W) * nrhs * ms_vectors(npole, ring)));
+    W *d = (W *)buf;
+    const long n = words * nrhs;
+    v = MsBatch<W>{d, d + n * ring, d + 2 * n * ring, d + (2 * ring + 1) * n, d + (2 * ring + 2) * n, words,
+                   words * (npole - 1), ring};
+    return OVL_OK;
+}
+
+// Batched multishift vectors (grown when a larger batch comes).
+constexpr int kBatchRing = 2;
 template <typename W>
 ovl_status Ctx::ensure_msb(MsBatch<W> &v, int &cap, int nrhs) {
-    if (v.p && cap >= nrhs) return OVL_OK;
-    if (v.p) {
+    if (v.r && cap >= nrhs) return OVL_OK;
+    if (v.r) {
         cudaFree(v.r);
         allocs.erase(std::find(allocs.begin(), allocs.end(), (void *)v.r));
-        v.p = nullptr;
+        v.r = nullptr;
         for (int k : {3, 4, 7})   // the batches' graphs hold the old addresses
             if (graphs[k].exec) {
                 cudaGraphExecDestroy(graphs[k].exec);
                 graphs[k].exec = nullptr;
             }
     }
-    const long words = spinor_words<W>(g);
-    void *buf;
-    ST(alloc(&buf, (size_t)words * sizeof(W) * nrhs * (npole + 3)));
-    W *d = (W *)buf;
-    v.r = d;
-    v.t = d + words * nrhs;
-    v.y = d + 2 * words * nrhs;
-    v.p = d + 3 * words * nrhs;
-    v.stride = words;
+    ST(alloc_ms(v, nrhs, kBatchRing));
     cap = nrhs;
     return OVL_OK;
 }
@@ -672,7 +677,7 @@ ovl_status Ctx::msb_run(int nrhs, const double *tol, int n, int slot, Init init_
                 set_launch_counting(false);
                 CK(cudaStreamBeginCapture(stream, cudaStreamCaptureModeThreadLocal));
                 cudaError_t ce = cudaSuccess;
-                for (int k = 0; k < chunk && ce == cudaSuccess; k++) ce = iter_fn();
+                for (int k = 0; k < chunk && ce == cudaSuccess; k++) ce = iter_fn(ms_flush(k, chunk, kBatchRing));
                 cudaError_t ee = cudaStreamEndCapture(stream, &graph);
                 set_launch_counting(true);
                 CK(ce);
@@ -686,7 +691,7 @@ ovl_status Ctx::msb_run(int nrhs, const double *tol, int n, int slot, Init init_
             CK(cudaGraphLaunch(gs.exec, stream));
             count_launches(3L * chunk);
         } else {
-            for (int k = 0; k < chunk; k++) CK(iter_fn());
+            for (int k = 0; k < chunk; k++) CK(iter_fn(ms_flush(k, chunk, kBatchRing)));
         }
         done_iters += chunk;
         CK(cudaMemcpy2DAsync(h_msb_small, 4 * sizeof(int), msb_state, sizeof(MsState), 4 * sizeof(int), nrhs,
@@ -736,8 +741,10 @@ ovl_status Ctx::sign64_batch(const double2 *b, double2 *out, int nrhs, const dou
     ST(ensure_batch());
     ST(ensure_msb(msb64, msb64_cap, nrhs));
     long iters = 0;
-    auto init = [&]() { return msb_init_f64(g, nrhs, npole, msb_state, msb64, b, rsb, bcounters, stream); };
-    auto it = [&]() { return msb_iter_f64(g, U64, m0_ker, nrhs, npole, msb_state, msb64, rsb, bcounters, stream); };
+    auto init = [&]() { return ms_init(g, nrhs, msb_state, msb64, b, rsb, bcounters, stream); };
+    auto it = [&](bool flush) {
+        return ms_iter(g, U64, m0_ker, nrhs, msb_state, msb64, rsb, bcounters, flush, stream, MsEvents{});
+    };
     const int n = pick_poles(min_positive(tol, nrhs));
     ST((msb_run<double2>(nrhs, tol, n, 3, init, it, &iters)));
     stat_ms64 += iters * nrhs;
@@ -762,12 +769,15 @@ ovl_status Ctx::sign_ff_batch(const double2 *b, double2 *out, int nrhs, const do
     PhaseClock pclk(this, &t_sign64);
     ST(ensure_batch());
     ST(ensure_ff_links());
-    const MsBatch<ffw> vf{(ffw *)msb64.r, (ffw *)msb64.t, (ffw *)msb64.y, (ffw *)msb64.p, msb64.stride};
+    const MsBatch<ffw> vf{(ffw *)msb64.r, (ffw *)msb64.p0, (ffw *)msb64.t, (ffw *)msb64.y, (ffw *)msb64.p, msb64.stride,
+                          msb64.prow, msb64.ring};
     // b in float-float into t (t is overwritten by the first iteration's Q p)
     CK(spinor_d2ff(g, b, vf.t, stream, nrhs));
     long iters = 0;
-    auto init = [&]() { return msb_init_ff(g, nrhs, npole, msb_state, vf, vf.t, rsb, bcounters, stream); };
-    auto it = [&]() { return msb_iter_ff(g, Uff, m0_ker, nrhs, npole, msb_state, vf, rsb, bcounters, stream); };
+    auto init = [&]() { return ms_init(g, nrhs, msb_state, vf, vf.t, rsb, bcounters, stream); };
+    auto it = [&](bool flush) {
+        return ms_iter(g, Uff, m0_ker, nrhs, msb_state, vf, rsb, bcounters, flush, stream, MsEvents{});
+    };
     const int n = pick_poles(min_positive(tol, nrhs));
     ST((msb_run<ffw>(nrhs, tol, n, 7, init, it, &iters)));
     stat_msff += iters * nrhs;
@@ -789,9 +799,9 @@ ovl_status Ctx::sign32_batch(const float4 *b, float4 *out, int nrhs, const doubl
     ST(ensure_batch());
     ST(ensure_msb(msb32, msb32_cap, nrhs));
     long iters = 0;
-    auto init = [&]() { return msb_init_f32(g, nrhs, npole, msb_state, msb32, b, rsb, stream); };
-    auto it = [&]() {
-        return msb_iter_f32(g, U32, (float)m0_ker, nrhs, npole, msb_state, msb32, rsb, bcounters, stream);
+    auto init = [&]() { return ms_init(g, nrhs, msb_state, msb32, b, rsb, bcounters, stream); };
+    auto it = [&](bool flush) {
+        return ms_iter(g, U32, m0_ker, nrhs, msb_state, msb32, rsb, bcounters, flush, stream, MsEvents{});
     };
     const int n = pick_poles(min_positive(tol, nrhs));
     ST((msb_run<float4>(nrhs, tol, n, 4, init, it, &iters)));
@@ -826,20 +836,7 @@ ovl_status Ctx::ensure_msh() {
     return OVL_OK;
 }
 
-ovl_status Ctx::ensure_ms32() {
-    if (ms32.p) return OVL_OK;
-    const long words = (long)g.V * 6;    // float4 per vector
-    void *buf;
-    ST(alloc(&buf, (size_t)words * sizeof(float4) * (npole + 4)));
-    float4 *b4 = (float4 *)buf;
-    ms32.r = b4;
-    ms32.t = b4 + words;
-    ms32.y = b4 + 2 * words;
-    ms32.p = b4 + 3 * words;
-    ms32.r2 = b4 + (3 + npole) * words;
-    ms32.stride = words;
-    return OVL_OK;
-}
+ovl_status Ctx::ensure_ms32() { return ms32.r ? OVL_OK : alloc_ms(ms32, 1, kMaxRing); }
 
 // ------------------------------------------------------------------ spectral estimates
 // Tridiagonal eigenvalue bounds by Sturm-sequence bisection.

@@ -2,7 +2,6 @@
 #include "hops.cuh"
 #include "internal.h"
 #include "reduce.cuh"
-#include "wilson_quad.cuh"
 #include "wilson_site.cuh"
 
 #include <algorithm>
@@ -304,43 +303,6 @@ __global__ void __launch_bounds__(kBlock, MinBlocks<R>::value) k_wilson(Geom g, 
     store_spinor<R>(out, g.Vh, p, i, res);
 }
 
-// Same with four threads per site (thread q of a quad owns direction mu = q and the
-// storage words j with j % 4 == q of the output).
-template <typename R, typename LT, typename ST>
-__global__ void __launch_bounds__(kBlock, MinBlocks<R>::value) k_wilson4(Geom g, const LT *__restrict__ U, const ST *__restrict__ in,
-                                                    ST *__restrict__ out, R m4, int g5, R a, const ST *z, R b) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    const int s0 = t >> 2, q = t & 3;
-    const int s = s0 < g.V ? s0 : g.V - 1;   // quads past the end compute a copy, store nothing
-    int p, i;
-    site_of_thread(s, p, i);
-    cpx<R> acc[12];
-    wilson_hop_dir<R>(g, U, in, p, i, q, acc);
-    quad_allreduce(acc);
-    if (s0 >= g.V) return;
-    using C = Chunk<ST>;
-#pragma unroll
-    for (int j = 0; j < C::NC; j++) {
-        if ((j & 3) != q) continue;
-        cpx<R> own[C::CPC], res[C::CPC];
-        C::template load<R>(in, g.Vh, p, i, j, own);
-#pragma unroll
-        for (int e = 0; e < C::CPC; e++) {
-            const int cix = j * C::CPC + e;
-            res[e] = m4 * own[e] + acc[cix];
-            if (g5 && cix < 6) res[e] = -res[e];
-            res[e] = a * res[e];
-        }
-        if (z) {
-            cpx<R> zz[C::CPC];
-            C::template load<R>(z, g.Vh, p, i, j, zz);
-#pragma unroll
-            for (int e = 0; e < C::CPC; e++) res[e] = res[e] + b * zz[e];
-        }
-        C::template store<R>(out, g.Vh, p, i, j, res);
-    }
-}
-
 // out = a [g5] D_W(m0) in + b z in FP64 or float-float, one warp per hop (hops.cuh); blockIdx.y =
 // right-hand side, vectors `stride` words apart.
 template <typename R>
@@ -386,14 +348,9 @@ cudaError_t wilson_ff(const Geom &g, const ffl *U, const ffw *in, ffw *out, doub
 }
 cudaError_t wilson_f32(const Geom &g, const float4 *U, const float4 *in, float4 *out, float m0, int g5,
                        float a, const float4 *z, float b, cudaStream_t st) {
-    if (g.tps32 == 4)
-        k_wilson4<float, float4, float4><<<plain_grid(4L * g.V), kBlock, 0, st>>>(g, U, in, out, m0 + 4.0f, g5, a,
-                                                                                  z, b);
-    else {
-        const LaunchShape ls = balanced_shape(g.V, g.nsm, MinBlocks<float>::value, 1 << 30);
-        k_wilson<float, float4, float4><<<ls.grid, ls.block, 0, st>>>(g, U, in, out, m0 + 4.0f, g5, a, z, b,
-                                                                      ls.spb);
-    }
+    if (g.tps32 == 4) return wilson_hops<float>(g, U, in, out, 0, 1, m0, g5, a, z, b, st);
+    const LaunchShape ls = balanced_shape(g.V, g.nsm, MinBlocks<float>::value, 1 << 30);
+    k_wilson<float, float4, float4><<<ls.grid, ls.block, 0, st>>>(g, U, in, out, m0 + 4.0f, g5, a, z, b, ls.spb);
     count_launches(1);
     return cudaGetLastError();
 }

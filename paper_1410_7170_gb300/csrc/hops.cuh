@@ -5,7 +5,9 @@
 // contributions in the order of the one-thread-per-site stencil (the same results bit for bit)
 // and run the caller's epilogue.
 //
-// Used for the arithmetics that are bound by their own instructions, FP64 (2 lanes per clock and
+// Used for small lattices in FP32 (the autotuner's choice: 8^4 5.8 -> 4.2 us a stencil, 16^4 8.3 -> 12.4,
+// where the shared memory traffic costs more than the extra warps give) and at all sizes for the
+// arithmetics that are bound by their own instructions, FP64 (2 lanes per clock and
 // SM on GB300, so a warp's FP64 instruction holds the SM's unit for 16 clocks) and float-float
 // (about 10k FP32 operations per site):
 //   * the work of a tile is spread evenly over the four schedulers. One thread per site fills
@@ -278,6 +280,105 @@ template <> struct HopTiles<double> {
     __device__ static double total(Sum s) { return s; }
 };
 
+// FP32. A tile is 32 sites; a hop leaves 12 reals per site, [h0, h1][colour][re, im]; item j is
+// storage word j, complex components 2 j and 2 j + 1 (six items: two of the eight warps idle in the
+// second part, which is a tenth of the work).
+template <> struct HopTiles<float> {
+    using Word = float;
+    using Elem = float4;
+    using Factor = float;
+    using Store = float4;
+    using Link = float4;
+    static constexpr int tile = 32, words = 12, items = 6;
+
+    template <int MU, bool FWD>
+    __device__ static void hop(const Geom &g, const float4 *__restrict__ U, const float4 *__restrict__ in, int p, int i,
+                               const int x[4], Word *out) {
+        bool flip;
+        const int j = hop_neighbour(g, x, MU, FWD, flip);
+        cpx<float> s[12], h0[3], h1[3], a0[3], a1[3], u[3][3];
+        load_spinor<float>(in, g.Vh, 1 - p, j, s);
+        if (FWD) load_link<float>(U, g.Vh, p, MU, i, u);
+        else load_link<float>(U, g.Vh, 1 - p, MU, j, u);
+        if (FWD) proj_fwd(MU, s, h0, h1);
+        else proj_bwd(MU, s, h0, h1);
+        if (MU == 0) flip_half(h0, h1, flip);
+        if (FWD) {
+            su3_mul(u, h0, a0);
+            su3_mul(u, h1, a1);
+        } else {
+            su3_dag_mul(u, h0, a0);
+            su3_dag_mul(u, h1, a1);
+        }
+#pragma unroll
+        for (int c = 0; c < 3; c++) {
+            out[(2 * c) * tile] = a0[c].re;
+            out[(2 * c + 1) * tile] = a0[c].im;
+            out[(6 + 2 * c) * tile] = a1[c].re;
+            out[(7 + 2 * c) * tile] = a1[c].im;
+        }
+    }
+    __device__ static void hop(const Geom &g, const Link *__restrict__ U, const Store *__restrict__ in, int p, int i,
+                               const int x[4], int w, int, Word *out) {
+        switch (w) {
+            case 0: hop<0, true>(g, U, in, p, i, x, out); break;
+            case 1: hop<0, false>(g, U, in, p, i, x, out); break;
+            case 2: hop<1, true>(g, U, in, p, i, x, out); break;
+            case 3: hop<1, false>(g, U, in, p, i, x, out); break;
+            case 4: hop<2, true>(g, U, in, p, i, x, out); break;
+            case 5: hop<2, false>(g, U, in, p, i, x, out); break;
+            case 6: hop<3, true>(g, U, in, p, i, x, out); break;
+            default: hop<3, false>(g, U, in, p, i, x, out); break;
+        }
+    }
+    __device__ static Elem sum(const Word *part, int it, int) {
+        float acc[4];
+#pragma unroll
+        for (int d = 0; d < 2; d++) {
+            const int cix = 2 * it + d, spin = cix / 3, c = cix - 3 * spin, k = spin & 1;
+            const bool low = spin >= 2;
+#pragma unroll
+            for (int h = 0; h < 8; h++) {
+                const int mu = h >> 1;
+                // lower spins are +-1 or +-i times h0 or h1 (acc_fwd, acc_bwd)
+                const bool cross = mu == 1 || mu == 2, turn = mu == 1 || mu == 3;
+                const int half = low && cross ? 1 - k : k;
+                const float *b = part + (h * words + 6 * half + 2 * c) * tile;
+                float re = b[0], im = b[tile];
+                if (low) {
+                    const bool sre = (mu == 0 || (mu == 2 && k == 0) || (mu == 3 && k == 1)) != ((h & 1) != 0);
+                    const bool sim = (mu == 0 || mu == 1 || (mu == 2 && k == 0) || (mu == 3 && k == 0)) != ((h & 1) != 0);
+                    const float a = turn ? im : re, e = turn ? re : im;
+                    re = flip_sign(a, sre);
+                    im = flip_sign(e, sim);
+                }
+                acc[2 * d] = h == 0 ? re : acc[2 * d] + re;
+                acc[2 * d + 1] = h == 0 ? im : acc[2 * d + 1] + im;
+            }
+        }
+        return make_float4(acc[0], acc[1], acc[2], acc[3]);
+    }
+    __device__ static bool upper(int it) { return it < 3; }
+    __device__ static size_t at(int Vh, int p, int i, int it) { return (size_t)(p * 6 + it) * Vh + i; }
+    __device__ static Elem load(const Store *f, int Vh, int p, int i, int it, int) { return __ldg(f + at(Vh, p, i, it)); }
+    __device__ static Elem load_rw(const Store *f, int Vh, int p, int i, int it, int) { return f[at(Vh, p, i, it)]; }
+    __device__ static void store(Store *f, int Vh, int p, int i, int it, int, Elem v) { f[at(Vh, p, i, it)] = v; }
+    __device__ static Factor factor(float a) { return a; }
+    __device__ static Factor minus_alpha(const MsState &s) { return -s.alpha_f[0]; }
+    __device__ static Factor sigma0(const MsState &s) { return s.sigma0_f[0]; }
+    __device__ static Elem fma(Factor a, Elem b, Elem c) {
+        return make_float4(__fmaf_rn(a, b.x, c.x), __fmaf_rn(a, b.y, c.y), __fmaf_rn(a, b.z, c.z), __fmaf_rn(a, b.w, c.w));
+    }
+    __device__ static Elem mul(Factor a, Elem b) { return make_float4(a * b.x, a * b.y, a * b.z, a * b.w); }
+    __device__ static Elem neg_if(Elem x, bool n) {
+        return make_float4(flip_sign(x.x, n), flip_sign(x.y, n), flip_sign(x.z, n), flip_sign(x.w, n));
+    }
+    using Sum = float;
+    __device__ static void square_add(Elem x, Sum &s) { s += x.x * x.x + x.y * x.y + x.z * x.z + x.w * x.w; }
+    __device__ static Sum zero() { return 0.f; }
+    __device__ static float total(Sum s) { return s; }
+};
+
 // Float-float. A word is a pair of float-float numbers, the same real of two spins, so that one
 // link entry multiplies both: a hop leaves six words per site, [colour][re, im] of (h0, h1), and a
 // spinor has twelve, [upper, lower spin pair][colour][re, im].
@@ -408,6 +509,7 @@ template <> struct HopTiles<ff> {
 template <typename R> struct HopBlocks;
 template <> struct HopBlocks<double> { static constexpr int value = 3; };
 template <> struct HopBlocks<ff> { static constexpr int value = 3; };
+template <> struct HopBlocks<float> { static constexpr int value = 4; };
 
 // Tiles first, first + step, ... : epi(p, i, item, sub, hop) is called for each of the warp's items in
 // every lane that holds a site, with the hopping sum (times -1/2, the stored links' factor).

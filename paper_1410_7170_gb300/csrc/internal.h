@@ -148,6 +148,8 @@ cudaError_t dev_multiaxpy_f(const float *base, long stride, int m, const double 
 cudaError_t fill_random_f32(float *x, long n, unsigned seed, cudaStream_t st);
 
 // ---------------------------------------------------------------- multishift CG
+constexpr int kMaxRing = 4;   // iterations whose shift updates are done together, at most
+
 // Device-side state of one multishift solve (Q^2 + sigma_l) x_l = b, l < n, with the
 // Zolotarev accumulation y = b + sum_l w_l x_l. sigma[0] is the base (smallest) shift.
 struct MsState {
@@ -165,24 +167,45 @@ struct MsState {
     double w[kMaxPoles];       // weights of x_l in y
     double crit[kMaxPoles];    // drop shift l when crit_l * |zeta_l| * ||r|| <= tol * ||b||
     double zeta[kMaxPoles], zeta_prev[kMaxPoles];
-    double alpha_l[kMaxPoles], beta_l[kMaxPoles];   // this iteration's coefficients of the rescaled directions
-                                                    // (y += w_l alpha_l p~_l, p~_l = r + beta_l p~_l)
     double ratio[kMaxPoles], critz2[kMaxPoles];     // zeta_{k+1} / zeta_k, (crit zeta_{k+1})^2
     double scale, inv_rr, inv_bb;                   // scale, 1 / (scale ||r||^2), 1 / (scale ||b||^2)
     int active[kMaxPoles];
+    // iterations whose shift updates are pending, oldest first: the coefficients of the rescaled
+    // directions (y += wa p~_l, p~_l = r + bl p~_l) and the shifts that take part (bit l)
+    int npend;
+    unsigned on[kMaxRing][kMaxPoles / 32];
+    double wa[kMaxRing][kMaxPoles], bl[kMaxRing][kMaxPoles];
+    float wa_f[kMaxRing][kMaxPoles][2], bl_f[kMaxRing][kMaxPoles][2], beta_f[2];   // the same and beta_prev as
+                                                                                   // float-float (hi, lo)
     int *hist;                 // optional: hist[k] = shifts updated in iteration k (instrumentation)
     int hist_cap;
 };
 
-// Workspace vectors of a multishift solve, in storage type ST.
+// Workspace vectors of nrhs multishift solves in storage type ST. Residuals and base directions are
+// rings of `ring` vectors per right-hand side (a power of two, at most kMaxRing): r_k and p_0(k) are
+// entry k % ring. t = Q p_0 and y (the accumulated argument of the rational function) are one vector
+// per right-hand side, the directions p_l, l >= 1, start at p + y * prow.
 template <typename ST>
-struct MsVectors {
-    ST *r;       // base residual
-    ST *t;       // Q p_0
-    ST *y;       // accumulated rational function argument
-    ST *p;       // n search directions, p[l] at p + l * stride
-    ST *r2;      // FP32 only: second residual buffer of the fused iteration (r_k in r for even k, r2 odd)
-    long stride; // elements of ST per vector
+struct MsBatch {
+    ST *r, *p0, *t, *y, *p;
+    long stride;   // words per vector
+    long prow;
+    int ring;
+    __host__ __device__ ST *r_at(int y_, int k) const { return r + ((long)y_ * ring + (k & (ring - 1))) * stride; }
+    __host__ __device__ ST *p0_at(int y_, int k) const { return p0 + ((long)y_ * ring + (k & (ring - 1))) * stride; }
+};
+// Vectors per right-hand side with npole directions.
+constexpr int ms_vectors(int npole, int ring) { return 2 * ring + 2 + npole - 1; }
+
+// Event records around the kernels of an iteration (instrumentation; ev = NULL: none). only >= 0:
+// just from record `only` on. flags: cudaEventRecordExternal inside graphs.
+struct MsEvents {
+    cudaEvent_t *ev = nullptr;
+    unsigned flags = 0;
+    int only = 0;
+    cudaError_t record(int k, cudaStream_t st) const {
+        return ev && k >= only ? cudaEventRecordWithFlags(ev[k], st, flags) : cudaSuccess;
+    }
 };
 
 // Half-precision variant of the FP32 multishift vectors: p_0 (the base direction, which
@@ -196,26 +219,27 @@ struct MsVectorsH {
     long words_h;       // uint4 words per FP16 vector (3 V)
 };
 
-// One multishift iteration = three launches (Q p, residual update, shift updates).
-// ev (optional, 4 events): recorded before/between/after the first three launches;
-// ev_flags is passed to cudaEventRecordWithFlags (cudaEventRecordExternal inside graphs).
-cudaError_t ms_init_f64(const Geom &g, int n, MsState *s, MsVectors<double2> v, const double2 *b, RedScratch rs,
-                        cudaStream_t st);
-cudaError_t ms_iter_f64(const Geom &g, const double2 *U, double m0, MsState *s, MsVectors<double2> v,
-                        RedScratch rs, cudaStream_t st, cudaEvent_t *ev = nullptr, unsigned ev_flags = 0);
-cudaError_t ms_init_f32(const Geom &g, int n, MsState *s, MsVectors<float4> v, const float4 *b, RedScratch rs,
-                        cudaStream_t st);
-cudaError_t ms_iter_f32(const Geom &g, const float4 *U, float m0, MsState *s, MsVectors<float4> v,
-                        RedScratch rs, cudaStream_t st, cudaEvent_t *ev = nullptr, unsigned ev_flags = 0);
+// One multishift iteration of nrhs right-hand sides (state st[y]; grid row y) = three launches: Q p,
+// residual update, and p_0 or, where flush is set, the pending shift updates with it. A caller sets
+// flush at least in every ring-th iteration, and in the last one before it reads y or the state.
+// rs.partials: nrhs * kMaxRedBlocks doubles; counters: nrhs words, zero between launches.
+cudaError_t ms_init(const Geom &g, int nrhs, MsState *s, MsBatch<double2> v, const double2 *b, RedScratch rs,
+                    unsigned *counters, cudaStream_t st);
+cudaError_t ms_init(const Geom &g, int nrhs, MsState *s, MsBatch<float4> v, const float4 *b, RedScratch rs,
+                    unsigned *counters, cudaStream_t st);
+cudaError_t ms_init(const Geom &g, int nrhs, MsState *s, MsBatch<ffw> v, const ffw *b, RedScratch rs,
+                    unsigned *counters, cudaStream_t st);
+cudaError_t ms_iter(const Geom &g, const double2 *U, double m0, int nrhs, MsState *s, MsBatch<double2> v, RedScratch rs,
+                    unsigned *counters, bool flush, cudaStream_t st, const MsEvents &ev);
+cudaError_t ms_iter(const Geom &g, const float4 *U, double m0, int nrhs, MsState *s, MsBatch<float4> v, RedScratch rs,
+                    unsigned *counters, bool flush, cudaStream_t st, const MsEvents &ev);
+cudaError_t ms_iter(const Geom &g, const ffl *U, double m0, int nrhs, MsState *s, MsBatch<ffw> v, RedScratch rs,
+                    unsigned *counters, bool flush, cudaStream_t st, const MsEvents &ev);
+// one right-hand side with 16-bit shifted directions, updated in every iteration
 cudaError_t ms_init_half(const Geom &g, int n, MsState *s, MsVectorsH v, const float4 *b, RedScratch rs, bool bf16,
                          cudaStream_t st);
-// float-float multishift (the FP64-accuracy sign on the FP32 pipes)
-cudaError_t ms_init_ff(const Geom &g, int n, MsState *s, MsVectors<ffw> v, const ffw *b, RedScratch rs,
-                       cudaStream_t st);
-cudaError_t ms_iter_ff(const Geom &g, const ffl *U, double m0, MsState *s, MsVectors<ffw> v, RedScratch rs,
-                       cudaStream_t st, cudaEvent_t *ev = nullptr, unsigned ev_flags = 0);
-cudaError_t ms_iter_half(const Geom &g, const float4 *U, float m0, MsState *s, MsVectorsH v, RedScratch rs, bool bf16,
-                         cudaStream_t st, cudaEvent_t *ev = nullptr, unsigned ev_flags = 0);
+cudaError_t ms_iter_half(const Geom &g, const float4 *U, double m0, MsState *s, MsVectorsH v, RedScratch rs, bool bf16,
+                         cudaStream_t st, const MsEvents &ev);
 
 // ---------------------------------------------------------------- several right-hand sides
 constexpr int kMaxBatch = 12;   // right-hand sides per batch (threads 32 x nrhs per block)
@@ -227,28 +251,6 @@ cudaError_t wilson_batch_ff(const Geom &g, const ffl *U, const ffw *in, ffw *out
                             int g5, double a, const ffw *z, double b, cudaStream_t st);
 cudaError_t wilson_batch_f32(const Geom &g, const float4 *U, const float4 *in, float4 *out, long stride, int nrhs,
                              float m0, int g5, float a, const float4 *z, float b, cudaStream_t st);
-
-// Batched multishift vectors: per right-hand side y, r/t/y at base + y * stride and its
-// npole directions at p + (y * npole + l) * stride.
-template <typename ST>
-struct MsBatch {
-    ST *r, *t, *y, *p;
-    long stride;
-};
-// One state per right-hand side (st[y]); partial sums need nrhs * 2 * kMaxRedBlocks doubles;
-// counters: nrhs words, zero between launches.
-cudaError_t msb_init_ff(const Geom &g, int nrhs, int npole, MsState *st, MsBatch<ffw> v, const ffw *b, RedScratch rs,
-                        unsigned *counters, cudaStream_t s);
-cudaError_t msb_iter_ff(const Geom &g, const ffl *U, double m0, int nrhs, int npole, MsState *st, MsBatch<ffw> v,
-                        RedScratch rs, unsigned *counters, cudaStream_t s);
-cudaError_t msb_init_f64(const Geom &g, int nrhs, int npole, MsState *st, MsBatch<double2> v, const double2 *b,
-                         RedScratch rs, unsigned *counters, cudaStream_t s);
-cudaError_t msb_init_f32(const Geom &g, int nrhs, int npole, MsState *st, MsBatch<float4> v, const float4 *b,
-                         RedScratch rs, cudaStream_t s);
-cudaError_t msb_iter_f64(const Geom &g, const double2 *U, double m0, int nrhs, int npole, MsState *st,
-                         MsBatch<double2> v, RedScratch rs, unsigned *counters, cudaStream_t s);
-cudaError_t msb_iter_f32(const Geom &g, const float4 *U, float m0, int nrhs, int npole, MsState *st,
-                         MsBatch<float4> v, RedScratch rs, unsigned *counters, cudaStream_t s);
 
 // Process-wide count of kernel launches issued by the library (instrumentation).
 void count_launches(long n);

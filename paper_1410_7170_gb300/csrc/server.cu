@@ -31,6 +31,7 @@
 #include <vector>
 
 #include "../../include/ovl.h"
+#include "internal.h"
 #include "solver.h"
 
 namespace {
@@ -96,9 +97,9 @@ size_t estimate_bytes(const ovl_request &r, const ovl_params &p) {
     double b = V * 4 * (9 * 16 + 3 * 16);                 // links: FP64 18 reals + FP32 12 reals
     b += 3 * v64 + 6 * v32;                               // staging, Lanczos / tuning vectors
     b += 24 * v32;                                        // multi-RHS stencil tuning (12 RHS in and out)
-    b += (p.n_poles + 3) * v64;                           // FP64 (or float-float) multishift
+    b += ovl::ms_vectors(p.n_poles, ovl::kMaxRing) * v64;   // FP64 (or float-float) multishift
     const bool mixed = p.precision != OVL_FP64 || p.precond == OVL_PREC_RECURSIVE;
-    if (mixed) b += (p.n_poles + 4) * v32;                 // FP32 multishift
+    if (mixed) b += ovl::ms_vectors(p.n_poles, ovl::kMaxRing) * v32;   // FP32 multishift
     if (mixed && p.ff_outer) b += V * 4 * 9 * 16;          // float-float links
     if (p.sign_method == OVL_SIGN_KRYLOV) b += (p.krylov_m + p.krylov_keep + 3) * v64;   // Krylov sign basis
     if (p.n_deflate > 0) {
@@ -112,8 +113,8 @@ size_t estimate_bytes(const ovl_request &r, const ovl_params &p) {
     if (nrhs > 1 && p.rhs_block > 1) {
         const int nb = std::min(std::min(p.rhs_block, nrhs), 12);
         const int mo = std::min(p.restart, 32), mi = std::min(p.restart_inner, 32), mw = std::min(p.prec_restart, 16);
-        b += nb * ((2 * mo + 5) * v64 + (p.n_poles + 3) * v64);
-        if (mixed) b += nb * ((2 * mi + 3) * v32 + (2 * mw + 3) * v32 + (p.n_poles + 3) * v32 + 2 * v32);
+        b += nb * ((2 * mo + 5) * v64 + ovl::ms_vectors(p.n_poles, 2) * v64);
+        if (mixed) b += nb * ((2 * mi + 3) * v32 + (2 * mw + 3) * v32 + ovl::ms_vectors(p.n_poles, 2) * v32 + 2 * v32);
     } else {
         b += (2 * p.restart + 5) * v64;                   // outer FGMRES basis (V and Z)
         if (p.precond == OVL_PREC_RECURSIVE) b += (2 * p.restart_inner + 3) * v32;

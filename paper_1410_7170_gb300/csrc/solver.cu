@@ -857,8 +857,9 @@ ovl_status wilson_solve_batch(Ctx *c, int nb, const T *in, T *out, double m0, do
 static size_t batch_bytes_per_rhs(const Ctx *c) {
     const double v64 = (double)c->n64 * 8.0, v32 = (double)c->n64 * 4.0;
     const int mo = std::min(c->p.restart, 32), mi = std::min(c->p.restart_inner, 32), mw = std::min(c->p.prec_restart, 16);
-    double b = (2 * mo + 3) * v64 + (c->npole + 3) * v64 + 2 * v64;                 // outer + FP64 multishift + x, b
-    b += (2 * mi + 3) * v32 + (2 * mw + 3) * v32 + (c->npole + 3) * v32 + 2 * v32;  // inner, Wilson, FP32 multishift
+    const int mv = ms_vectors(c->npole, 2);
+    double b = (2 * mo + 3) * v64 + mv * v64 + 2 * v64;                 // outer + FP64 multishift + x, b
+    b += (2 * mi + 3) * v32 + (2 * mw + 3) * v32 + mv * v32 + 2 * v32;  // inner, Wilson, FP32 multishift
     return (size_t)b;
 }
 

@@ -100,11 +100,11 @@ struct Ctx {
     std::vector<double> za, zc;
     // multishift
     MsState *ms64_state = nullptr, *ms32_state = nullptr;
-    MsVectors<double2> ms64{};
-    MsVectors<float4> ms32{};
+    MsBatch<double2> ms64{};
+    MsBatch<float4> ms32{};
     MsVectorsH msh{};
     MsState *msh_state = nullptr;
-    MsVectors<ffw> msff{};             // float-float multishift vectors
+    MsBatch<ffw> msff{};               // float-float multishift vectors
     MsState *msff_state = nullptr;
     GraphSlot graphs[8];
     // batched multishift (several right-hand sides in lock-step)
@@ -121,7 +121,7 @@ struct Ctx {
     bool prof = false;
     ProfAcc pacc[3];   // per arithmetic slot (0 FP64, 1 FP32 / 16-bit stored, 2 float-float)
     long launch_mark = 0;
-    cudaEvent_t ev[3][4] = {};   // profiling: events around the kernels of one sampled iteration
+    cudaEvent_t ev[3][6] = {};   // profiling: events around the kernels of one sampled iteration and a p_0 kernel
     bool ev_ready[3] = {false, false, false};
     int *d_hist = nullptr;
     int hist_cap = 0;
@@ -210,9 +210,10 @@ struct Ctx {
     void fill_poles(MsState &s, int n, double tol) const;
     ovl_status ms_setup(MsState *d_state, double tol, int *n_out);
     // which: instrumentation class (0 FP64, 1 FP32/FP16); slot: CUDA-graph slot;
-    // shift_bytes: algorithmic bytes per site of one shift update (read + write of p_l)
+    // ring: iterations whose shift updates go together; shift_bytes: algorithmic bytes per site of one
+    // shift update (read + write of p_l)
     template <typename Iter>
-    ovl_status ms_run(MsState *d_state, int which, int slot, double shift_bytes, bool fused, Iter iter_fn,
+    ovl_status ms_run(MsState *d_state, int which, int slot, int ring, double shift_bytes, Iter iter_fn,
                       int *iters_out);
     ovl_status sign64(const double2 *b, double2 *out, double tol, int mode);
     // store: -1 = from params.precision, 0 = FP32, 1 = FP16-stored, 2 = BF16-stored directions
@@ -232,6 +233,8 @@ struct Ctx {
     ovl_status ensure_msh();
     // several right-hand sides: b, out hold nrhs internal vectors back to back
     ovl_status ensure_batch();
+    template <typename W>
+    ovl_status alloc_ms(MsBatch<W> &v, int nrhs, int ring);
     template <typename W>
     ovl_status ensure_msb(MsBatch<W> &v, int &cap, int nrhs);
     ovl_status sign64_batch(const double2 *b, double2 *out, int nrhs, const double *tol, int mode);

@@ -97,3 +97,31 @@ def test_batches_of_both_arithmetics_share_vectors():
     op.ovl_apply_n(r, x3, 3, 1e-13)
     assert ((r - b[:3]).norm() / b[:3].norm()).item() < 2e-10
     op.close()
+
+
+@pytest.mark.parametrize("tps", [1, 4])
+@pytest.mark.parametrize("arith,tol,bar", [(ovl.OVL_ARITH_FP64, 1e-12, 1e-12), (ovl.OVL_ARITH_FF, 1e-11, 1e-11),
+                                           (ovl.OVL_ARITH_FP32, 1e-5, 2e-5)])
+def test_chunk_lengths_and_pending_updates(arith, tol, bar, tps):
+    """The shift updates are done four iterations at a time (two in a batch), and at the end of every
+    chunk of check_every iterations: any chunk length, captured or not, stops after the same iteration
+    and gives the same result up to the rounding of y (2e-5: 100 FP32 roundings, more in FP64 bars)."""
+    dims = (6, 4, 4, 10)
+    b = dev(synth.rhs_gaussian(dims, 35, n_rhs=3))
+    ref, its = None, None
+    for every, graphs in ((8, 1), (1, 1), (2, 0), (3, 1), (5, 0), (7, 1), (64, 1)):
+        U, op = _op(dims, check_every=every, use_graphs=graphs, stencil_tps=tps)
+        out = torch.empty_like(b)
+        op.prof_enable(True)
+        op.sign_apply_arith(out[0], b[0], tol, arith)
+        n = {k: v["launches"] for k, v in op.prof_get(reset=True).items() if k.startswith("ms_shifts")}
+        op.prof_enable(False)
+        if arith == ovl.OVL_ARITH_FP64:
+            op.ovl_apply_n(out, b, 3, tol)
+        op.close()
+        if ref is None:
+            ref, its = out.clone(), n
+            continue
+        assert n == its, (every, n, its)
+        m = 3 if arith == ovl.OVL_ARITH_FP64 else 1
+        assert ((out[:m] - ref[:m]).norm() / ref[:m].norm()).item() < bar, (every, graphs)
