@@ -1,4 +1,5 @@
 // Layout conversion and the Wilson-Dirac stencil kernels (Eq. Wilson-Dirac).
+#include "convert.h"
 #include "hops.cuh"
 #include "internal.h"
 #include "reduce.cuh"
@@ -105,10 +106,11 @@ cudaError_t pack_gauge(const Geom &g, const double *lex, double2 *u64, float4 *u
 // both sides are read and written in whole 512-byte rows. Sites 2i and 2i + 1 share the
 // checkerboard index i, so they are kept 32 rows apart in shared memory and a row is 13 words
 // long: the eight 16-byte reads of a quarter warp (consecutive i, one component) then fall on
-// different banks. The format conversion and the test for NaN and Inf ride along. Measured at
-// 64 x 32^3, FP32 format: 0.31 ms for pack + test + conversion and 0.40 ms for conversion +
-// unpack as separate kernels with one thread per site (pack 120, test 102, d2f 85; f2d 87,
-// unpack 310 us).
+// different banks. The format conversion (by integer instructions, convert.h) and the test for NaN
+// and Inf ride along. Measured at 64 x 32^3, FP32 format (603 MB each way): 308 us in and 397 us out
+// as separate kernels with one thread per site (pack 120, test 102, d2f 85; f2d 87, unpack 310),
+// 181 and 121 us in one pass with conversions on the FP64 unit, 104 and 114 us (5.8 and 5.3 TB/s)
+// with integer ones.
 constexpr int kIoTile = 64, kIoRow = 13;
 
 // Word j of a site's internal format from / to its 12 complex numbers.
@@ -122,11 +124,11 @@ template <> struct IoWord<float4> {
     static constexpr int N = 6;
     __device__ static float4 get(const double2 *v, int j) {
         const double2 a = v[2 * j], b = v[2 * j + 1];
-        return make_float4((float)a.x, (float)a.y, (float)b.x, (float)b.y);
+        return make_float4(d2f(a.x), d2f(a.y), d2f(b.x), d2f(b.y));
     }
     __device__ static void put(double2 *v, int j, float4 w) {
-        v[2 * j] = make_double2((double)w.x, (double)w.y);
-        v[2 * j + 1] = make_double2((double)w.z, (double)w.w);
+        v[2 * j] = make_double2(f2d(w.x), f2d(w.y));
+        v[2 * j + 1] = make_double2(f2d(w.z), f2d(w.w));
     }
 };
 template <> struct IoWord<ffw> {
@@ -134,14 +136,16 @@ template <> struct IoWord<ffw> {
     // word j: real (j even) or imaginary part of one colour of two spins; its two complex numbers
     __device__ static int first(int j) { return j < 6 ? j >> 1 : 3 + (j >> 1); }
     __device__ static ffw get(const double2 *v, int j) {
-        const double2 x = v[first(j)], y = v[first(j) + 3];
-        const ff a(j & 1 ? x.y : x.x), b(j & 1 ? y.y : y.x);
-        return ffw{a.hi, b.hi, a.lo, b.lo};
+        const double *x = reinterpret_cast<const double *>(v + first(j)) + (j & 1);
+        ffw w;
+        d2ff(x[0], w.h0, w.l0);
+        d2ff(x[6], w.h1, w.l1);
+        return w;
     }
     __device__ static void put(double2 *v, int j, ffw w) {
         double *x = reinterpret_cast<double *>(v + first(j)) + (j & 1);
-        x[0] = ff(w.h0, w.l0).to_double();
-        x[6] = ff(w.h1, w.l1).to_double();
+        x[0] = ff2d(w.h0, w.l0);
+        x[6] = ff2d(w.h1, w.l1);
     }
 };
 
@@ -169,7 +173,7 @@ __global__ void __launch_bounds__(kBlock) k_spinor_in(Geom g, ST *__restrict__ d
         const int e = threadIdx.x + q * kBlock;
         if (e < ns * 12) {
             const double2 v = __ldcs(lex + e);
-            fine = fine && isfinite(v.x) && isfinite(v.y);
+            fine = fine && finite_bits(v.x) && finite_bits(v.y);
             sm[io_row(e / 12) + e % 12] = v;
         }
     }
@@ -250,9 +254,13 @@ __global__ void k_spinor_d2f(Geom g, const double2 *__restrict__ a, float4 *__re
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= g.V) return;
     const int p = t >= g.Vh, i = t - p * g.Vh;
-    cpx<float> v[12];
-    load_spinor<float>(a, g.Vh, p, i, v);
-    store_spinor<float>(b, g.Vh, p, i, v);
+    const double2 *x = a + (size_t)p * 12 * g.Vh + i;
+    float4 *y = b + (size_t)p * 6 * g.Vh + i;
+#pragma unroll
+    for (int c = 0; c < 6; c++) {
+        const double2 u = x[(size_t)(2 * c) * g.Vh], v = x[(size_t)(2 * c + 1) * g.Vh];
+        y[(size_t)c * g.Vh] = make_float4(d2f(u.x), d2f(u.y), d2f(v.x), d2f(v.y));
+    }
 }
 __global__ void k_spinor_f2d(Geom g, const float4 *__restrict__ a, double2 *__restrict__ b) {
     a += (size_t)blockIdx.y * 6 * g.V;
@@ -260,9 +268,14 @@ __global__ void k_spinor_f2d(Geom g, const float4 *__restrict__ a, double2 *__re
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= g.V) return;
     const int p = t >= g.Vh, i = t - p * g.Vh;
-    cpx<double> v[12];
-    load_spinor<double>(a, g.Vh, p, i, v);
-    store_spinor<double>(b, g.Vh, p, i, v);
+    const float4 *x = a + (size_t)p * 6 * g.Vh + i;
+    double2 *y = b + (size_t)p * 12 * g.Vh + i;
+#pragma unroll
+    for (int c = 0; c < 6; c++) {
+        const float4 w = x[(size_t)c * g.Vh];
+        y[(size_t)(2 * c) * g.Vh] = make_double2(f2d(w.x), f2d(w.y));
+        y[(size_t)(2 * c + 1) * g.Vh] = make_double2(f2d(w.z), f2d(w.w));
+    }
 }
 cudaError_t spinor_d2f(const Geom &g, const double2 *a, float4 *b, cudaStream_t st, int n) {
     k_spinor_d2f<<<dim3(plain_grid(g.V), n), kBlock, 0, st>>>(g, a, b);
@@ -441,8 +454,10 @@ cudaError_t wilson_16(const Geom &g, const void *u16, const uint4 *in, const flo
 __global__ void k_links_d2ff(const double2 *__restrict__ x, ffl *__restrict__ y, long n) {
     for (long k = (long)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (long)gridDim.x * blockDim.x) {
         const double2 v = x[k];
-        const ff re(v.x), im(v.y);
-        y[k] = ffl{re.hi, re.lo, im.hi, im.lo};
+        ffl w;
+        d2ff(v.x, w.rh, w.rl);
+        d2ff(v.y, w.ih, w.il);
+        y[k] = w;
     }
 }
 // Thread k: checkerboard index, colour and spin pair of one parity of one spinor (6 Vh of them
@@ -452,9 +467,13 @@ __global__ void k_spinor_d2ff(const double2 *__restrict__ x, ffw *__restrict__ y
         const long i = k % Vh, r = k / Vh;         // r = 6 * (parity and spinor) + 3 * pair + colour
         const long m = r / 6, w = r % 6, c = w % 3 + 6 * (w / 3);
         const double2 a = x[(12 * m + c) * Vh + i], b = x[(12 * m + c + 3) * Vh + i];
-        const ff ar(a.x), ai(a.y), br(b.x), bi(b.y);
-        y[(12 * m + 2 * w) * Vh + i] = ffw{ar.hi, br.hi, ar.lo, br.lo};
-        y[(12 * m + 2 * w + 1) * Vh + i] = ffw{ai.hi, bi.hi, ai.lo, bi.lo};
+        ffw re, im;
+        d2ff(a.x, re.h0, re.l0);
+        d2ff(b.x, re.h1, re.l1);
+        d2ff(a.y, im.h0, im.l0);
+        d2ff(b.y, im.h1, im.l1);
+        y[(12 * m + 2 * w) * Vh + i] = re;
+        y[(12 * m + 2 * w + 1) * Vh + i] = im;
     }
 }
 __global__ void k_spinor_ff2d(const ffw *__restrict__ x, double2 *__restrict__ y, int Vh, long n) {
@@ -462,8 +481,8 @@ __global__ void k_spinor_ff2d(const ffw *__restrict__ x, double2 *__restrict__ y
         const long i = k % Vh, r = k / Vh;
         const long m = r / 6, w = r % 6, c = w % 3 + 6 * (w / 3);
         const ffw a = x[(12 * m + 2 * w) * Vh + i], b = x[(12 * m + 2 * w + 1) * Vh + i];
-        y[(12 * m + c) * Vh + i] = make_double2(ff(a.h0, a.l0).to_double(), ff(b.h0, b.l0).to_double());
-        y[(12 * m + c + 3) * Vh + i] = make_double2(ff(a.h1, a.l1).to_double(), ff(b.h1, b.l1).to_double());
+        y[(12 * m + c) * Vh + i] = make_double2(ff2d(a.h0, a.l0), ff2d(b.h0, b.l0));
+        y[(12 * m + c + 3) * Vh + i] = make_double2(ff2d(a.h1, a.l1), ff2d(b.h1, b.l1));
     }
 }
 static int conv_grid(long n) {
