@@ -1200,6 +1200,8 @@ static ovl_status create_impl(Ctx *c, const double *gauge, const int dims[4], do
     c->h_ms_small = (int *)(hp + 4096);
     c->h_ms = (MsState *)(hp + 8192);
     c->h_hist = (int *)(hp + 32768);
+    c->h_gs_coef = (double *)(hp + 40960);   // 12 x 256 doubles
+    static_assert(8192 + sizeof(MsState) <= 32768 && 40960 + 12 * 256 * sizeof(double) <= (1 << 16), "");
     c->launch_mark = launches_total();
     // device scratch
     void *buf;
@@ -1218,6 +1220,11 @@ static ovl_status create_impl(Ctx *c, const double *gauge, const int dims[4], do
     c->d_md_part = (double *)buf;
     ST(c->alloc(&buf, (size_t)2 * 128 * sizeof(double)));
     c->d_coef = (double *)buf;
+    ST(c->alloc(&buf, (size_t)(kScal + 12 * 256) * sizeof(double) + 256));
+    c->d_gs = (double *)buf;
+    c->d_gs_coef = c->d_gs + kScal;
+    c->gs_counters = (unsigned *)(c->d_gs_coef + 12 * 256);
+    CK(cudaMemsetAsync(c->gs_counters, 0, 256, c->stream));
     // gauge field
     ST(c->alloc((void **)&c->U64, (size_t)V * 4 * kLink64Words * sizeof(double2)));
     ST(c->alloc((void **)&c->U32, (size_t)V * 4 * 3 * sizeof(float4)));

@@ -1,6 +1,8 @@
 // BLAS-1 kernels on flat arrays: deterministic reductions (norms, complex dots,
 // multi-dots for Gram-Schmidt), axpy variants and precision conversion. All are
 // HBM-streaming; reductions accumulate in FP64 in a fixed order.
+#include <algorithm>
+
 #include "internal.h"
 #include "reduce.cuh"
 
@@ -59,12 +61,11 @@ __global__ void k_caxpy(double ar, double ai, const double *__restrict__ x, doub
     }
 }
 
-// Multi-dot: blockIdx.y = vector index; partials[k][blockIdx.x] (complex). Rows y >= m use
-// w itself, so an extra row gives (||w||^2, 0) in the same pass.
+// Multi-dot: blockIdx.y = vector index; partials[k][blockIdx.x] (complex).
 template <typename T>
 __global__ void k_multidot_part(const T *__restrict__ base, long stride, int m, const T *__restrict__ w, long nc,
                                 double *partials) {
-    const T *v = (int)blockIdx.y < m ? base + (long)blockIdx.y * stride : w;
+    const T *v = base + (long)blockIdx.y * stride;
     T a = 0, b = 0;
     for (long k = (long)blockIdx.x * blockDim.x + threadIdx.x; k < nc; k += (long)gridDim.x * blockDim.x) {
         const T vr = v[2 * k], vi = v[2 * k + 1];
@@ -93,28 +94,6 @@ __global__ void k_multidot_sum(const double *partials, int nb, double *out) {
     }
 }
 
-// out = scale (w - sum_j h_j v_j) with h the complex dot products of a multi-dot (device
-// memory, FP64): the Gram-Schmidt update and normalisation of an Arnoldi step in one pass.
-template <typename T>
-__global__ void k_orth_scale(const T *__restrict__ base, long stride, int m, const double *__restrict__ h,
-                             double scale, const T *__restrict__ w, T *__restrict__ out, long nc) {
-    __shared__ T cs[2 * 128];
-    for (int k = threadIdx.x; k < 2 * m; k += blockDim.x) cs[k] = (T)(-h[k]);
-    __syncthreads();
-    const T sc = (T)scale;
-    for (long k = (long)blockIdx.x * blockDim.x + threadIdx.x; k < nc; k += (long)gridDim.x * blockDim.x) {
-        T ar = w[2 * k], ai = w[2 * k + 1];
-        for (int j = 0; j < m; j++) {
-            const T *v = base + (long)j * stride;
-            const T vr = v[2 * k], vi = v[2 * k + 1];
-            ar += cs[2 * j] * vr - cs[2 * j + 1] * vi;
-            ai += cs[2 * j] * vi + cs[2 * j + 1] * vr;
-        }
-        out[2 * k] = sc * ar;
-        out[2 * k + 1] = sc * ai;
-    }
-}
-
 template <typename T>
 __global__ void k_multiaxpy(const T *__restrict__ base, long stride, int m, const double *__restrict__ c,
                             T *__restrict__ w, long nc) {
@@ -131,6 +110,164 @@ __global__ void k_multiaxpy(const T *__restrict__ base, long stride, int m, cons
         }
         w[2 * k] = ar;
         w[2 * k + 1] = ai;
+    }
+}
+
+// ---- Gram-Schmidt without the host (gs_dots, gs_subtract, gs_combine)
+// 16-byte words: one complex double or two complex floats.
+template <typename T> struct GsWord;
+template <> struct GsWord<double> {
+    using W = double2;
+    __device__ static void dot(W v, W w, double &a, double &b) {
+        a += v.x * w.x + v.y * w.y;
+        b += v.x * w.y - v.y * w.x;
+    }
+    __device__ static void axpy(double cr, double ci, W v, W &w) {
+        w.x += cr * v.x - ci * v.y;
+        w.y += cr * v.y + ci * v.x;
+    }
+    __device__ static W scaled(double s, W w) { return make_double2(s * w.x, s * w.y); }
+    __device__ static W zero() { return make_double2(0.0, 0.0); }
+};
+template <> struct GsWord<float> {
+    using W = float4;
+    __device__ static void dot(W v, W w, float &a, float &b) {
+        a += v.x * w.x + v.y * w.y + v.z * w.z + v.w * w.w;
+        b += v.x * w.y - v.y * w.x + v.z * w.w - v.w * w.z;
+    }
+    __device__ static void axpy(float cr, float ci, W v, W &w) {
+        w.x += cr * v.x - ci * v.y;
+        w.y += cr * v.y + ci * v.x;
+        w.z += cr * v.z - ci * v.w;
+        w.w += cr * v.w + ci * v.z;
+    }
+    __device__ static W scaled(float s, W w) { return make_float4(s * w.x, s * w.y, s * w.z, s * w.w); }
+    __device__ static W zero() { return make_float4(0.f, 0.f, 0.f, 0.f); }
+};
+constexpr int kGsMax = 128;   // basis vectors
+
+// Grid (blocks, m + 1, right-hand sides); vector m is w itself. The last block of a right-hand side
+// sums the partials in block order and writes its record.
+template <typename T>
+__global__ void __launch_bounds__(kBlock) k_gs_dots(const T *__restrict__ base, long stride, int m,
+                                                    const T *__restrict__ w, long n, RowList rows, double *out,
+                                                    long ostride, bool one_pass, const double *prev, double *partials,
+                                                    unsigned *counters) {
+    using G = GsWord<T>;
+    using W = typename G::W;
+    const int z = blockIdx.z, i = blockIdx.y;
+    if (prev && prev[z * ostride + 2 * m + 4] != 0.0) return;   // uniform over the right-hand side
+    const long off = (long)rows.row[z] * n, nw = n * (long)sizeof(T) / (long)sizeof(W);
+    const W *x = reinterpret_cast<const W *>(w + off);
+    const W *v = i < m ? reinterpret_cast<const W *>(base + (long)i * stride + off) : x;
+    // four words of each vector in flight per thread: the grid is small (gs_grid)
+    T a = 0, b = 0;
+    const long step = (long)gridDim.x * blockDim.x;
+    long k = (long)blockIdx.x * blockDim.x + threadIdx.x;
+    for (; k + 3 * step < nw; k += 4 * step) {
+        W p[4], q[4];
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            p[u] = v[k + u * step];
+            q[u] = x[k + u * step];
+        }
+#pragma unroll
+        for (int u = 0; u < 4; u++) G::dot(p[u], q[u], a, b);
+    }
+    for (; k < nw; k += step) G::dot(v[k], x[k], a, b);
+    const T t[2] = {a, b};
+    double s[2];
+    block_sum<2>(t, s);
+    __shared__ int is_last;
+    __shared__ double h[2 * kGsMax + 2];
+    const int gx = gridDim.x;
+    double *part = partials + (long)z * gridDim.y * gx * 2;
+    if (threadIdx.x == 0) {
+        part[((long)i * gx + blockIdx.x) * 2] = s[0];
+        part[((long)i * gx + blockIdx.x) * 2 + 1] = s[1];
+        __threadfence();
+        is_last = atomicAdd(counters + z, 1u) == (unsigned)(gridDim.y * gx - 1);
+    }
+    __syncthreads();
+    if (!is_last) return;
+    __threadfence();
+    double *o = out + z * ostride;
+    const int lane = threadIdx.x & 31;
+    for (int q = threadIdx.x >> 5; q <= m; q += kBlock / 32) {
+        double d[2] = {0.0, 0.0};
+        for (int k = lane; k < gx; k += 32) {
+            d[0] += __ldcg(part + ((long)q * gx + k) * 2);
+            d[1] += __ldcg(part + ((long)q * gx + k) * 2 + 1);
+        }
+        warp_sum<2>(d);
+        if (lane == 0) {
+            o[2 * q] = h[2 * q] = d[0];
+            o[2 * q + 1] = h[2 * q + 1] = q < m ? d[1] : 0.0;
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        double q[1] = {0.0};
+        for (int k = lane; k < 2 * m; k += 32) q[0] += h[k] * h[k];
+        warp_sum<1>(q);
+        if (lane == 0) {
+            const double ww = h[2 * m], left = ww - q[0];
+            const double hn = left <= 0.0 ? 0.0 : sqrt(left);   // NaN stays NaN
+            o[2 * m + 2] = hn;
+            o[2 * m + 3] = hn > 0.0 ? 1.0 / hn : 0.0;
+            o[2 * m + 4] = one_pass && left > 0.1 * ww ? 1.0 : 0.0;
+            counters[z] = 0u;
+        }
+    }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kBlock) k_gs_subtract(const T *__restrict__ base, long stride, int m,
+                                                        const double *__restrict__ h, long ostride,
+                                                        const double *__restrict__ prev, T *w, T *next, long n,
+                                                        RowList rows) {
+    using G = GsWord<T>;
+    using W = typename G::W;
+    __shared__ T cs[2 * kGsMax];
+    const int z = blockIdx.y;
+    const double *hz = h + z * ostride;
+    const bool one = hz[2 * m + 4] != 0.0;
+    if (prev && prev[z * ostride + 2 * m + 4] != 0.0) return;
+    for (int k = threadIdx.x; k < 2 * m; k += blockDim.x) cs[k] = (T)(-hz[k]);
+    __syncthreads();
+    const bool fin = prev || one;   // the last subtraction: normalise into next
+    const T sc = fin ? (T)hz[2 * m + 3] : T(1);
+    const long off = (long)rows.row[z] * n, nw = n * (long)sizeof(T) / (long)sizeof(W);
+    const W *v = reinterpret_cast<const W *>(base + off), *x = reinterpret_cast<const W *>(w + off);
+    W *o = reinterpret_cast<W *>((fin ? next : w) + off);
+    const long sw = stride * (long)sizeof(T) / (long)sizeof(W);
+    for (long k = (long)blockIdx.x * blockDim.x + threadIdx.x; k < nw; k += (long)gridDim.x * blockDim.x) {
+        W a = x[k];
+#pragma unroll 4
+        for (int j = 0; j < m; j++) G::axpy(cs[2 * j], cs[2 * j + 1], v[j * sw + k], a);
+        o[k] = fin ? G::scaled(sc, a) : a;
+    }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kBlock) k_gs_combine(const T *__restrict__ base, long stride, int m,
+                                                       const double *__restrict__ c, T *x, bool add, long n,
+                                                       RowList rows) {
+    using G = GsWord<T>;
+    using W = typename G::W;
+    __shared__ T cs[2 * kGsMax];
+    const int z = blockIdx.y;
+    for (int k = threadIdx.x; k < 2 * m; k += blockDim.x) cs[k] = (T)c[2 * m * z + k];
+    __syncthreads();
+    const long off = (long)rows.row[z] * n, nw = n * (long)sizeof(T) / (long)sizeof(W);
+    const W *v = reinterpret_cast<const W *>(base + off);
+    W *o = reinterpret_cast<W *>(x + off);
+    const long sw = stride * (long)sizeof(T) / (long)sizeof(W);
+    for (long k = (long)blockIdx.x * blockDim.x + threadIdx.x; k < nw; k += (long)gridDim.x * blockDim.x) {
+        W a = add ? o[k] : G::zero();
+#pragma unroll 4
+        for (int j = 0; j < m; j++) G::axpy(cs[2 * j], cs[2 * j + 1], v[j * sw + k], a);
+        o[k] = a;
     }
 }
 
@@ -212,22 +349,6 @@ cudaError_t dev_multidot_f(const float *base, long stride, int m, const float *w
     count_launches(2);
     return cudaGetLastError();
 }
-cudaError_t dev_multidot_norm_f(const float *base, long stride, int m, const float *w, long n, double *out,
-                                double *partials, cudaStream_t st) {
-    int gx = (int)((n / 2 + kBlock - 1) / kBlock);
-    if (gx > kMdBlocks) gx = kMdBlocks;
-    if (gx < 1) gx = 1;
-    k_multidot_part<float><<<dim3(gx, m + 1), kBlock, 0, st>>>(base, stride, m, w, n / 2, partials);
-    k_multidot_sum<<<m + 1, kBlock, 0, st>>>(partials, gx, out);
-    count_launches(2);
-    return cudaGetLastError();
-}
-cudaError_t dev_orth_scale_f(const float *base, long stride, int m, const double *h, double scale, const float *w,
-                             float *out, long n, cudaStream_t st) {
-    k_orth_scale<float><<<stream_grid(n / 2), kBlock, 0, st>>>(base, stride, m, h, scale, w, out, n / 2);
-    count_launches(1);
-    return cudaGetLastError();
-}
 cudaError_t dev_multiaxpy(const double *base, long stride, int m, const double *c, double *w, long n,
                           cudaStream_t st) {
     if (m <= 0) return cudaSuccess;
@@ -252,5 +373,50 @@ cudaError_t dev_f2d(const float *x, double *y, long n, cudaStream_t st) {
     count_launches(1);
     return cudaGetLastError();
 }
+
+// Blocks per vector: about per_sm per SM over all vectors and right-hand sides, none without words.
+// The dot products take few (each block ends with a fence and an atomic: at 16^4 17 us with 1216
+// blocks), and no more than the partial sums have room for.
+constexpr long kGsPartials = 128 * 256;   // complex partial sums
+static int gs_grid(long words, long vectors, int per_sm) {
+    const long b = (words + kBlock - 1) / kBlock, cap = std::max(4L, (long)per_sm * device_sm_count() / vectors);
+    return (int)std::max(1L, std::min({b, cap, kGsPartials / vectors}));
+}
+template <typename T>
+cudaError_t gs_dots(const T *base, long stride, int m, const T *w, long n, const RowList &rows, double *out,
+                    long ostride, bool one_pass, const double *prev, double *partials, unsigned *counters,
+                    cudaStream_t st) {
+    const int gx = gs_grid(n * (long)sizeof(T) / 16, (long)(m + 1) * rows.n, 2);
+    k_gs_dots<T><<<dim3(gx, m + 1, rows.n), kBlock, 0, st>>>(base, stride, m, w, n, rows, out, ostride, one_pass, prev,
+                                                             partials, counters);
+    count_launches(1);
+    return cudaGetLastError();
+}
+template <typename T>
+cudaError_t gs_subtract(const T *base, long stride, int m, const double *h, long ostride, const double *prev, T *w,
+                        T *next, long n, const RowList &rows, cudaStream_t st) {
+    k_gs_subtract<T><<<dim3(gs_grid(n * (long)sizeof(T) / 16, rows.n, 8), rows.n), kBlock, 0, st>>>(base, stride, m, h, ostride,
+                                                                                              prev, w, next, n, rows);
+    count_launches(1);
+    return cudaGetLastError();
+}
+template <typename T>
+cudaError_t gs_combine(const T *base, long stride, int m, const double *c, T *x, bool add, long n, const RowList &rows,
+                       cudaStream_t st) {
+    k_gs_combine<T><<<dim3(gs_grid(n * (long)sizeof(T) / 16, rows.n, 8), rows.n), kBlock, 0, st>>>(base, stride, m, c, x, add,
+                                                                                             n, rows);
+    count_launches(1);
+    return cudaGetLastError();
+}
+#define OVL_GS(T)                                                                                                     \
+    template cudaError_t gs_dots<T>(const T *, long, int, const T *, long, const RowList &, double *, long, bool,      \
+                                    const double *, double *, unsigned *, cudaStream_t);                              \
+    template cudaError_t gs_subtract<T>(const T *, long, int, const double *, long, const double *, T *, T *, long,    \
+                                        const RowList &, cudaStream_t);                                               \
+    template cudaError_t gs_combine<T>(const T *, long, int, const double *, T *, bool, long, const RowList &,         \
+                                       cudaStream_t);
+OVL_GS(float)
+OVL_GS(double)
+#undef OVL_GS
 
 }  // namespace ovl

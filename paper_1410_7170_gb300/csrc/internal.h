@@ -136,12 +136,31 @@ cudaError_t dev_cdot_f(const float *x, const float *y, long n, double *res, RedS
 // multi-dot / multi-axpy with float vectors (accumulation in double)
 cudaError_t dev_multidot_f(const float *base, long stride, int m, const float *w, long n, double *out,
                            double *partials, cudaStream_t st);
-// out[0 .. 2m-1] = <base_j, w> (complex), out[2m] = ||w||^2, out[2m+1] = 0, in one pass.
-cudaError_t dev_multidot_norm_f(const float *base, long stride, int m, const float *w, long n, double *out,
-                                double *partials, cudaStream_t st);
-// out = scale (w - sum_j h_j base_j), h = the complex dots of dev_multidot_norm_f (device).
-cudaError_t dev_orth_scale_f(const float *base, long stride, int m, const double *h, double scale, const float *w,
-                             float *out, long n, cudaStream_t st);
+
+// Gram-Schmidt steps of the FGMRES solvers, several right-hand sides at once, without the host.
+// Vector y of a basis entry is n reals after vector 0. T = float or double.
+struct RowList {
+    int n, row[12];   // the right-hand sides that take part (grid rows)
+};
+// Record of row k at out + k * ostride: [0, 2m) = <v_i, w> (complex), [2m] = ||w||^2, [2m+1] = 0,
+// then hn = sqrt(max(0, ||w||^2 - sum |<v_i, w>|^2)), 1 / hn (0 for hn = 0), and 1 if one pass is
+// enough (one_pass allowed and hn^2 > 0.1 ||w||^2), else 0. Needs 2m + 5 doubles.
+// prev: the record of the first pass, or NULL; where it says that one pass is enough nothing is done.
+constexpr int gs_record(int m) { return 2 * m + 6; }
+template <typename T>
+cudaError_t gs_dots(const T *base, long stride, int m, const T *w, long n, const RowList &rows, double *out,
+                    long ostride, bool one_pass, const double *prev, double *partials, unsigned *counters,
+                    cudaStream_t st);
+// Subtracts sum_i h_i v_i, h from the record of this pass. First pass (prev NULL): the result goes to
+// next, scaled by 1 / hn, where one pass is enough, and back to w otherwise; second pass: to next,
+// scaled, except where one pass was enough.
+template <typename T>
+cudaError_t gs_subtract(const T *base, long stride, int m, const double *h, long ostride, const double *prev, T *w,
+                        T *next, long n, const RowList &rows, cudaStream_t st);
+// x (+)= sum_i c_i v_i, complex coefficients of row k at c + 2 * m * k (device); add = false: assigned
+template <typename T>
+cudaError_t gs_combine(const T *base, long stride, int m, const double *c, T *x, bool add, long n, const RowList &rows,
+                       cudaStream_t st);
 cudaError_t dev_multiaxpy_f(const float *base, long stride, int m, const double *c, float *w, long n,
                             cudaStream_t st);
 // x[k] = seeded pseudo-random values in [-1, 1) (a counter hash of k and the seed)

@@ -385,16 +385,11 @@ __device__ __forceinline__ void sap_glob_dir(const Geom &g, const Sap32<S> &m, c
 // neighbouring blocks (the block's own x is zero and is assigned), or v - D_W x.
 enum SapStart { kSapFresh, kSapOwnZero, kSapFull };
 
-// The right-hand sides of a batch that take part: grid row y is vector row[y].
-struct SapRows {
-    int n, row[kMaxBatch];
-};
-
 // One CTA per block of the colour and right-hand side; ADD: x += e instead of x = e.
 template <int S, int START, bool ADD>
 __global__ void __launch_bounds__(2 * S, 1)
     k_sap_block32(Geom g, SapGeom sg, const float4 *__restrict__ U, const float4 *__restrict__ v, float4 *x, long stride,
-                  SapRows rows, float m4, int colour, int mr_iters, bool colour_grid) {
+                  RowList rows, float m4, int colour, int mr_iters, bool colour_grid) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ float4 red[2 * kBlock / 32];
     int B[4], rem = blockIdx.x;
@@ -580,7 +575,7 @@ static SapGrid sap_grid(const SapGeom &sg) {
 
 template <int S, int START, bool ADD>
 static cudaError_t launch_sap32_s(const Geom &g, const SapGeom &sg, const SapGrid &sp, const float4 *U, const float4 *v,
-                                  float4 *x, long stride, const SapRows &rows, float m4, int colour, int mr_iters,
+                                  float4 *x, long stride, const RowList &rows, float m4, int colour, int mr_iters,
                                   cudaStream_t st) {
     static size_t granted = 0;
     constexpr size_t smem = sizeof(Sap32<S>);
@@ -594,7 +589,7 @@ static cudaError_t launch_sap32_s(const Geom &g, const SapGeom &sg, const SapGri
 }
 template <int START, bool ADD>
 static cudaError_t launch_sap32(const Geom &g, const SapGeom &sg, const SapGrid &sp, const float4 *U, const float4 *v,
-                                float4 *x, long stride, const SapRows &rows, float m4, int colour, int mr_iters,
+                                float4 *x, long stride, const RowList &rows, float m4, int colour, int mr_iters,
                                 cudaStream_t st) {
     // blocks of up to 64 sites take 25 KB instead of 98, so that more of them fit on an SM
     return sg.nb <= 64 ? launch_sap32_s<64, START, ADD>(g, sg, sp, U, v, x, stride, rows, m4, colour, mr_iters, st)
@@ -606,7 +601,7 @@ cudaError_t sap_f32_rows(const Geom &g, const SapGeom &sg, const float4 *U, cons
     const SapGrid sp = sap_grid(sg);
     const float m4 = m0 + 4.f;
     const size_t bytes = (size_t)g.V * 6 * sizeof(float4);
-    SapRows rows{};
+    RowList rows{};
     cudaError_t e;
     for (int y = 0; y < n; y++) {
         if (!act || act[y]) rows.row[rows.n++] = y;
@@ -633,7 +628,7 @@ cudaError_t sap_f32_rows(const Geom &g, const SapGeom &sg, const float4 *U, cons
                 continue;
             }
             for (int k = 0; k < rows.n; k++) {   // r = v - D_W x on the whole lattice, then the block solves from r
-                SapRows one{};
+                RowList one{};
                 one.n = 1;
                 const long off = rows.row[k] * stride;
                 if ((e = wilson_f32(g, U, x + off, r, m0, 0, -1.f, v + off, 1.f, st)) != cudaSuccess) return e;

@@ -32,13 +32,6 @@ template <> struct Ops<double> {
     static cudaError_t axpby(Ctx *c, double a, const double *x, double b, double *y) {
         return dev_axpby(a, x, b, y, c->n64, c->stream);
     }
-    // basis vectors k = 0..m-1 at base + k * stride (stride 0: consecutive vectors)
-    static cudaError_t multidot(Ctx *c, const double *base, int m, const double *w, double *out, long stride = 0) {
-        return dev_multidot(base, stride ? stride : c->n64, m, w, c->n64, out, c->d_md_part, c->stream);
-    }
-    static cudaError_t multiaxpy(Ctx *c, const double *base, int m, const double *coef, double *w, long stride = 0) {
-        return dev_multiaxpy(base, stride ? stride : c->n64, m, coef, w, c->n64, c->stream);
-    }
     static cudaError_t wilson(Ctx *c, const double *in, double *out, double m0) {
         return wilson_f64(c->g, c->U64, (const double2 *)in, (double2 *)out, m0, 0, 1.0, nullptr, 0.0, c->stream);
     }
@@ -54,12 +47,6 @@ template <> struct Ops<float> {
     static cudaError_t axpby(Ctx *c, double a, const float *x, double b, float *y) {
         return dev_axpby_f((float)a, x, (float)b, y, c->n64, c->stream);
     }
-    static cudaError_t multidot(Ctx *c, const float *base, int m, const float *w, double *out, long stride = 0) {
-        return dev_multidot_f(base, stride ? stride : c->n64, m, w, c->n64, out, c->d_md_part, c->stream);
-    }
-    static cudaError_t multiaxpy(Ctx *c, const float *base, int m, const double *coef, float *w, long stride = 0) {
-        return dev_multiaxpy_f(base, stride ? stride : c->n64, m, coef, w, c->n64, c->stream);
-    }
     static cudaError_t wilson(Ctx *c, const float *in, float *out, double m0) {
         return wilson_f32(c->g, c->U32, (const float4 *)in, (float4 *)out, (float)m0, 0, 1.f, nullptr, 0.f,
                           c->stream);
@@ -67,15 +54,6 @@ template <> struct Ops<float> {
     static cudaError_t sap(Ctx *c, const SapGeom &sg, const float *v, float *x, float *r, double m0) {
         return sap_f32(c->g, sg, c->U32, (const float4 *)v, (float4 *)x, (float4 *)r, (float)m0, c->p.sap_cycles,
                        c->p.sap_mr_iters, c->stream);
-    }
-    // [0, 2m) = <base_j, w>, [2m] = ||w||^2 in one pass over the basis
-    static cudaError_t multidot_norm(Ctx *c, const float *base, int m, const float *w, double *out) {
-        return dev_multidot_norm_f(base, c->n64, m, w, c->n64, out, c->d_md_part, c->stream);
-    }
-    // out = scale (w - sum_j h_j base_j), h on the device
-    static cudaError_t orth_scale(Ctx *c, const float *base, int m, const double *h, double scale, const float *w,
-                                  float *out) {
-        return dev_orth_scale_f(base, c->n64, m, h, scale, w, out, c->n64, c->stream);
     }
     static constexpr bool kCgs2 = false;   // low-accuracy solves: one Gram-Schmidt pass unless it cancels
 };
@@ -116,162 +94,204 @@ ovl_status upload_coef(Ctx *c, const std::vector<cd> &v) {
     return OVL_OK;
 }
 
+// Records of the device's Gram-Schmidt kernels in c->d_gs: norms of start vectors first (gs_record(0)
+// doubles per right-hand side), then the two passes of an Arnoldi step, row by row.
+constexpr int kGsStart = 128;
+static_assert(kMaxBatch * gs_record(0) <= kGsStart && kMaxBatch <= 12, "");
+
+// V_0 = w / ||w|| for the rows (w: vector y at w + y n), ||w||^2 in the start records; no host wait.
+template <typename T>
+static ovl_status gs_start(Ctx *c, const T *w, T *v0, const RowList &rows) {
+    CK(gs_dots<T>(w, 0, 0, w, c->n64, rows, c->d_gs, gs_record(0), false, nullptr, c->d_md_part, c->gs_counters,
+                  c->stream));
+    // with one pass not enough and nothing to subtract, the second pass normalises
+    CK(gs_subtract<T>(w, 0, 0, c->d_gs, gs_record(0), c->d_gs, const_cast<T *>(w), v0, c->n64, rows, c->stream));
+    return OVL_OK;
+}
+
+// One Arnoldi step of the rows: w against m basis vectors (entry i of row y at V + i stride + y n), V_m =
+// the normalised rest, by classical Gram-Schmidt, in FP64 always with a second pass (CGS2), in FP32
+// when the first one cancels most of w (the decision is made on the device). One wait for the host,
+// which gets h (m values per row) and hn; start (nullable): also the rows' ||w||^2 of gs_start.
+template <typename T>
+static ovl_status gs_arnoldi(Ctx *c, T *V, long stride, int m, T *w, const RowList &rows, std::vector<std::vector<cd>> &h,
+                             std::vector<double> &hn, std::vector<double> *start = nullptr) {
+    const long n = c->n64, rec = gs_record(m), os = 2 * rec;
+    double *first = c->d_gs + kGsStart, *second = first + rec;
+    T *next = V + (long)m * stride;
+    if (kGsStart + rows.n * os > kScal / 2) {
+        c->err = "Krylov solver: scalar staging too small";
+        return OVL_EINVAL;
+    }
+    CK(gs_dots<T>(V, stride, m, w, n, rows, first, os, !Ops<T>::kCgs2, nullptr, c->d_md_part, c->gs_counters, c->stream));
+    CK(gs_subtract<T>(V, stride, m, first, os, nullptr, w, next, n, rows, c->stream));
+    CK(gs_dots<T>(V, stride, m, w, n, rows, second, os, false, first, c->d_md_part, c->gs_counters, c->stream));
+    CK(gs_subtract<T>(V, stride, m, second, os, first, w, next, n, rows, c->stream));
+    std::vector<double> t(kGsStart + rows.n * os);
+    ST(c->fetch(c->d_gs, (int)t.size(), t.data()));
+    h.assign(rows.n, std::vector<cd>(m));
+    hn.assign(rows.n, 0.0);
+    if (start) start->assign(rows.n, 0.0);
+    for (int r = 0; r < rows.n; r++) {
+        const double *a = t.data() + kGsStart + r * os, *b = a + rec;
+        const bool one = a[2 * m + 4] != 0.0;
+        for (int i = 0; i < m; i++) h[r][i] = cd(a[2 * i], a[2 * i + 1]) + (one ? cd(0) : cd(b[2 * i], b[2 * i + 1]));
+        hn[r] = one ? a[2 * m + 2] : b[2 * m + 2];
+        if (start) (*start)[r] = t[r * gs_record(0)];
+    }
+    return OVL_OK;
+}
+
+// x (+)= sum_i y_i Z_i for the rows (coefficients y[r], padded with zeros to the longest). The pinned
+// staging is free: a fetch has waited for the stream since the last call.
+template <typename T>
+static ovl_status gs_solution(Ctx *c, const T *Z, long stride, const std::vector<std::vector<cd>> &y, T *x, bool add,
+                              const RowList &rows) {
+    size_t m = 0;
+    for (auto &v : y) m = std::max(m, v.size());
+    for (int r = 0; r < rows.n; r++)
+        for (size_t i = 0; i < m; i++) {
+            const cd v = i < y[r].size() ? y[r][i] : cd(0);
+            c->h_gs_coef[2 * (m * r + i)] = v.real();
+            c->h_gs_coef[2 * (m * r + i) + 1] = v.imag();
+        }
+    CK(cudaMemcpyAsync(c->d_gs_coef, c->h_gs_coef, 2 * m * rows.n * sizeof(double), cudaMemcpyHostToDevice, c->stream));
+    CK(gs_combine<T>(Z, stride, (int)m, c->d_gs_coef, x, add, c->n64, rows, c->stream));
+    return OVL_OK;
+}
+
+// Givens rotations of column j of the Hessenberg matrix H (leading dimension m) and of the
+// right-hand side gv.
+static void givens_column(std::vector<cd> &H, int m, int j, std::vector<cd> &cs, std::vector<cd> &sn, std::vector<cd> &gv) {
+    for (int i = 0; i < j; i++) {
+        const cd a = H[(size_t)i * m + j], b = H[(size_t)(i + 1) * m + j];
+        H[(size_t)i * m + j] = std::conj(cs[i]) * a + std::conj(sn[i]) * b;
+        H[(size_t)(i + 1) * m + j] = -sn[i] * a + cs[i] * b;
+    }
+    const cd a = H[(size_t)j * m + j], b = H[(size_t)(j + 1) * m + j];
+    const double den = sqrt(std::norm(a) + std::norm(b));
+    cs[j] = den > 0 ? a / den : cd(1.0);
+    sn[j] = den > 0 ? b / den : cd(0.0);
+    H[(size_t)j * m + j] = den;
+    H[(size_t)(j + 1) * m + j] = 0.0;
+    gv[j + 1] = -sn[j] * gv[j];
+    gv[j] = std::conj(cs[j]) * gv[j];
+}
+// y = H^{-1} g for the leading k x k block
+static std::vector<cd> back_substitute(const std::vector<cd> &H, int m, const std::vector<cd> &gv, int k) {
+    std::vector<cd> y(k);
+    for (int i = k - 1; i >= 0; i--) {
+        cd s = gv[i];
+        for (int q = i + 1; q < k; q++) s -= H[(size_t)i * m + q] * y[q];
+        y[i] = s / H[(size_t)i * m + i];
+    }
+    return y;
+}
+
 // FGMRES(m). matvec(in, out, rel_res_now) computes out = A in; precond(in, out) gives
 // out ~ A^{-1} in (nullptr: plain GMRES). x holds the initial guess (x_zero: it is 0).
 // Stops when ||b - A x|| <= tol ||b|| (checked on the recomputed residual) or after
 // maxit iterations.
 // verify = false (preconditioner solves): return after the cycle whose Arnoldi residual
-// estimate meets tol, without recomputing the true residual.
+// estimate meets tol, without recomputing the true residual. Started from x = 0 such a solve waits
+// for the host once per Arnoldi step and not before: ||b|| comes with the first step's scalars.
 template <typename T, typename MV, typename PC>
 static ovl_status fgmres(Ctx *c, Krylov<T> &k, T *x, const T *b, double tol, int maxit, bool x_zero, MV matvec,
                          PC *precond, KrylovResult *res, bool verify = true) {
     using O = Ops<T>;
     const long n = c->n64;
     const int m = k.m;
-    double bb;
-    CK(O::norm2(c, b, c->d_scal));
-    ST(c->fetch(c->d_scal, 1, &bb));
-    const double bnorm = sqrt(bb);
+    const RowList one{1, {0}};
     res->iters = 0;
     res->converged = false;
-    if (bnorm == 0.0) {
-        CK(cudaMemsetAsync(x, 0, n * sizeof(T), c->stream));
-        res->rel_res = 0.0;
-        res->converged = true;
-        return OVL_OK;
-    }
     bool xz = x_zero;
-    if (xz) CK(cudaMemsetAsync(x, 0, n * sizeof(T), c->stream));   // x_zero: start from x = 0
-    std::vector<cd> H((size_t)(m + 1) * m), cs(m), sn(m), gv(m + 1), y(m), h1(m + 1), h2(m + 1);
-    while (true) {
-        // r = b - A x
-        if (xz) {
-            CK(cudaMemcpyAsync(k.r, b, n * sizeof(T), cudaMemcpyDeviceToDevice, c->stream));
-        } else {
-            ST(matvec(x, k.w, -1.0));
-            CK(cudaMemcpyAsync(k.r, b, n * sizeof(T), cudaMemcpyDeviceToDevice, c->stream));
-            CK(O::axpby(c, -1.0, k.w, 1.0, k.r));
-        }
-        double rr;
-        CK(O::norm2(c, k.r, c->d_scal));
-        ST(c->fetch(c->d_scal, 1, &rr));
-        const double beta = sqrt(rr);
-        res->rel_res = beta / bnorm;
-        if (!std::isfinite(beta)) {
-            c->err = "Krylov solver: non-finite residual";
-            return OVL_EBREAKDOWN;
-        }
-        if (beta <= tol * bnorm) {
+    bool late = xz && !verify && maxit > 0;   // ||b|| not yet on the host
+    double bnorm = 0.0;
+    if (!late) {
+        double bb;
+        CK(O::norm2(c, b, c->d_scal));
+        ST(c->fetch(c->d_scal, 1, &bb));
+        bnorm = sqrt(bb);
+        if (xz || bnorm == 0.0) CK(cudaMemsetAsync(x, 0, n * sizeof(T), c->stream));
+        if (bnorm == 0.0) {
+            res->rel_res = 0.0;
             res->converged = true;
             return OVL_OK;
         }
-        if (res->iters >= maxit) return OVL_OK;
-        CK(O::axpby(c, 1.0 / beta, k.r, 0.0, k.V));
+    }
+    std::vector<cd> H((size_t)(m + 1) * m), cs(m), sn(m), gv(m + 1);
+    std::vector<std::vector<cd>> hc;
+    std::vector<double> hnv, bb0;
+    while (true) {
         std::fill(gv.begin(), gv.end(), cd(0));
-        gv[0] = beta;
+        if (late) {
+            ST(gs_start(c, b, k.V, one));
+        } else {
+            // r = b - A x
+            const T *r = b;
+            if (!xz) {
+                ST(matvec(x, k.w, -1.0));
+                CK(cudaMemcpyAsync(k.r, b, n * sizeof(T), cudaMemcpyDeviceToDevice, c->stream));
+                CK(O::axpby(c, -1.0, k.w, 1.0, k.r));
+                r = k.r;
+            }
+            double rr;
+            ST(gs_start(c, r, k.V, one));
+            ST(c->fetch(c->d_gs, 1, &rr));
+            const double beta = sqrt(rr);
+            res->rel_res = beta / bnorm;
+            if (!std::isfinite(beta)) {
+                c->err = "Krylov solver: non-finite residual";
+                return OVL_EBREAKDOWN;
+            }
+            if (beta <= tol * bnorm) {
+                res->converged = true;
+                return OVL_OK;
+            }
+            if (res->iters >= maxit) return OVL_OK;
+            gv[0] = beta;
+        }
         int j = 0;
         bool stop = false;
         for (; j < m && !stop; j++) {
             T *vj = k.V + (long)j * n;
             T *zj = vj;
+            const double rel_now = late ? 1.0 : std::abs(gv[j]) / bnorm;
             if (precond) {
                 zj = k.Z + (long)j * n;
-                c->fgmres_rel = std::abs(gv[j]) / bnorm;   // read by an adaptive preconditioner
+                c->fgmres_rel = rel_now;   // read by an adaptive preconditioner
                 ST((*precond)(vj, zj));
             }
-            const double rel_now = std::abs(gv[j]) / bnorm;
             ST(matvec(zj, k.w, rel_now));
-            // Gram-Schmidt: h = V^H w and ||w||^2 in one round trip; a second pass (CGS2)
-            // always in FP64, and in FP32 only when the first pass cancels most of w.
-            double hn = 0.0;
-            bool next_done = false;   // V_{j+1} already written
-            if constexpr (!O::kCgs2) {
-                // one pass: the dots and ||w||^2 in one kernel; unless the pass cancels most of w,
-                // V_{j+1} = (w - V h) / hn in one more, with h read from device memory
-                CK(O::multidot_norm(c, k.V, j + 1, k.w, c->d_scal));
-                double tmp[2 * 128 + 2];
-                ST(c->fetch(c->d_scal, 2 * (j + 1) + 1, tmp));
-                double hsq = 0.0;
-                for (int i = 0; i <= j; i++) {
-                    h1[i] = cd(tmp[2 * i], tmp[2 * i + 1]);
-                    hsq += std::norm(h1[i]);
+            ST(gs_arnoldi<T>(c, k.V, n, j + 1, k.w, one, hc, hnv, late ? &bb0 : nullptr));
+            if (late) {
+                late = false;
+                bnorm = sqrt(bb0[0]);
+                if (!std::isfinite(bnorm)) {
+                    c->err = "Krylov solver: non-finite residual";
+                    return OVL_EBREAKDOWN;
                 }
-                const double ww = tmp[2 * (j + 1)];
-                const double left = ww - hsq;
-                if (left > 0.1 * ww) {
-                    std::fill(h2.begin(), h2.end(), cd(0));
-                    hn = sqrt(left);
-                    if (hn > 0) CK(O::orth_scale(c, k.V, j + 1, c->d_scal, 1.0 / hn, k.w, k.V + (long)(j + 1) * n));
-                    next_done = true;
-                } else {   // cancellation: subtract this pass, then a second full pass below
-                    std::vector<cd> neg(j + 1);
-                    for (int i = 0; i <= j; i++) neg[i] = -h1[i];
-                    ST(upload_coef(c, neg));
-                    CK(O::multiaxpy(c, k.V, j + 1, c->d_coef, k.w));
+                if (bnorm == 0.0) {
+                    CK(cudaMemsetAsync(x, 0, n * sizeof(T), c->stream));
+                    res->rel_res = 0.0;
+                    res->converged = true;
+                    return OVL_OK;
                 }
+                gv[0] = bnorm;
             }
-            for (int pass = next_done ? 2 : (O::kCgs2 ? 0 : 1); pass < 2; pass++) {
-                std::vector<cd> &hh = pass == 0 ? h1 : h2;
-                CK(O::multidot(c, k.V, j + 1, k.w, c->d_scal));
-                CK(O::norm2(c, k.w, c->d_scal + 2 * (j + 1)));
-                double tmp[2 * 128 + 2];
-                ST(c->fetch(c->d_scal, 2 * (j + 1) + 1, tmp));   // 2 (j + 1) + 1 <= 243 doubles
-                std::vector<cd> neg(j + 1);
-                double hsq = 0.0;
-                for (int i = 0; i <= j; i++) {
-                    hh[i] = cd(tmp[2 * i], tmp[2 * i + 1]);
-                    neg[i] = -hh[i];
-                    hsq += std::norm(hh[i]);
-                }
-                ST(upload_coef(c, neg));
-                CK(O::multiaxpy(c, k.V, j + 1, c->d_coef, k.w));
-                const double ww = tmp[2 * (j + 1)];
-                const double left = ww - hsq;   // ||w - V h||^2 for orthonormal V
-                if (pass == 0 && !O::kCgs2 && left > 0.1 * ww) {
-                    std::fill(h2.begin(), h2.end(), cd(0));
-                    hn = sqrt(left);
-                    break;
-                }
-                if (pass == 1) {
-                    double w2;
-                    CK(O::norm2(c, k.w, c->d_scal));
-                    ST(c->fetch(c->d_scal, 1, &w2));
-                    hn = sqrt(w2);
-                }
-            }
-            for (int i = 0; i <= j; i++) H[(size_t)i * m + j] = h1[i] + h2[i];
+            const double hn = hnv[0];
+            for (int i = 0; i <= j; i++) H[(size_t)i * m + j] = hc[0][i];
             H[(size_t)(j + 1) * m + j] = hn;
             if (!std::isfinite(hn)) {
                 c->err = "Krylov solver: non-finite Arnoldi coefficient";
                 return OVL_EBREAKDOWN;
             }
-            if (hn > 0 && !next_done) CK(O::axpby(c, 1.0 / hn, k.w, 0.0, k.V + (long)(j + 1) * n));
-            // rotations
-            for (int i = 0; i < j; i++) {
-                const cd a = H[(size_t)i * m + j], bq = H[(size_t)(i + 1) * m + j];
-                H[(size_t)i * m + j] = std::conj(cs[i]) * a + std::conj(sn[i]) * bq;
-                H[(size_t)(i + 1) * m + j] = -sn[i] * a + cs[i] * bq;
-            }
-            const cd a = H[(size_t)j * m + j], bq = H[(size_t)(j + 1) * m + j];
-            const double den = sqrt(std::norm(a) + std::norm(bq));
-            cs[j] = den > 0 ? a / den : cd(1.0);
-            sn[j] = den > 0 ? bq / den : cd(0.0);
-            H[(size_t)j * m + j] = den;
-            H[(size_t)(j + 1) * m + j] = 0.0;
-            gv[j + 1] = -sn[j] * gv[j];
-            gv[j] = std::conj(cs[j]) * gv[j];
+            givens_column(H, m, j, cs, sn, gv);
             res->iters++;
             if (std::abs(gv[j + 1]) <= tol * bnorm || hn == 0.0 || res->iters >= maxit) stop = true;
         }
-        // y = H^{-1} g, x += Z y
-        for (int i = j - 1; i >= 0; i--) {
-            cd s = gv[i];
-            for (int q = i + 1; q < j; q++) s -= H[(size_t)i * m + q] * y[q];
-            y[i] = s / H[(size_t)i * m + i];
-        }
-        std::vector<cd> yy(y.begin(), y.begin() + j);
-        ST(upload_coef(c, yy));
-        CK(O::multiaxpy(c, precond ? k.Z : k.V, j, c->d_coef, x));
+        // y = H^{-1} g, x += Z y (x = Z y in a first cycle from zero)
+        ST(gs_solution<T>(c, precond ? k.Z : k.V, n, {back_substitute(H, m, gv, j)}, x, !xz, one));
         xz = false;
         if (!verify && (std::abs(gv[j]) <= tol * bnorm || res->iters >= maxit)) {
             res->rel_res = std::abs(gv[j]) / bnorm;
@@ -637,20 +657,25 @@ ovl_status fgmres_batch(Ctx *c, Krylov<T> &k, int nb, T *x, const T *b, double t
             conv[y] = 1;
         }
     }
-    std::vector<double> relv(nb);
+    std::vector<double> relv(nb), hnv;
+    std::vector<std::vector<cd>> hc;
     while (true) {
         // R = B - A X for the active systems
-        if (xz) {
-            CK(cudaMemcpyAsync(k.r, b, (size_t)nb * n * sizeof(T), cudaMemcpyDeviceToDevice, c->stream));
-        } else {
+        if (!xz) {
             for (int y = 0; y < nb; y++) relv[y] = active[y] ? -1.0 : 2.0;
             ST(matvec(x, k.w, relv.data()));
             CK(cudaMemcpyAsync(k.r, b, (size_t)nb * n * sizeof(T), cudaMemcpyDeviceToDevice, c->stream));
             for (int y = 0; y < nb; y++)
                 if (active[y]) CK(O::axpby(c, -1.0, k.w + (long)y * n, 1.0, k.r + (long)y * n));
         }
-        for (int y = 0; y < nb; y++) CK(O::norm2(c, k.r + (long)y * n, c->d_scal + y));
-        ST(c->fetch(c->d_scal, nb, tmp));
+        // V_0 = r / ||r|| (0 for r = 0; rows that stop here do not use theirs)
+        const T *r0 = xz ? b : k.r;
+        RowList all{nb, {}};
+        for (int y = 0; y < nb; y++) all.row[y] = y;
+        ST(gs_start(c, r0, k.V, all));
+        std::vector<double> nr((size_t)nb * gs_record(0));
+        ST(c->fetch(c->d_gs, (int)nr.size(), nr.data()));
+        for (int y = 0; y < nb; y++) tmp[y] = nr[(size_t)y * gs_record(0)];
         bool any = false;
         for (int y = 0; y < nb; y++) {
             if (!active[y]) continue;
@@ -671,8 +696,7 @@ ovl_status fgmres_batch(Ctx *c, Krylov<T> &k, int nb, T *x, const T *b, double t
         for (int y = 0; y < nb; y++) {
             std::fill(gv[y].begin(), gv[y].end(), cd(0));
             gv[y][0] = beta[y];
-            if (active[y]) CK(O::axpby(c, 1.0 / beta[y], k.r + (long)y * n, 0.0, vec(k.V, 0, y)));
-            else CK(cudaMemsetAsync(vec(k.V, 0, y), 0, n * sizeof(T), c->stream));
+            if (!active[y]) CK(cudaMemsetAsync(vec(k.V, 0, y), 0, n * sizeof(T), c->stream));
         }
         std::vector<char> live = active;   // systems iterating in this cycle
         int j = 0;
@@ -683,77 +707,22 @@ ovl_status fgmres_batch(Ctx *c, Krylov<T> &k, int nb, T *x, const T *b, double t
             ST(precond(vec(k.V, j, 0), vec(k.Z, j, 0), live.data()));
             for (int y = 0; y < nb; y++) relv[y] = live[y] ? std::abs(gv[y][j]) / bnorm[y] : 2.0;
             ST(matvec(vec(k.Z, j, 0), k.w, relv.data()));
-            // Gram-Schmidt per system: one pass, a second when it cancels (always in FP64)
-            std::vector<std::vector<cd>> h1(nb, std::vector<cd>(j + 1)), h2(nb, std::vector<cd>(j + 1));
-            std::vector<double> hn(nb, 0.0);
-            std::vector<char> need2(nb, 0);
-            for (int pass = 0; pass < 2; pass++) {
-                int cnt = 0;
-                for (int y = 0; y < nb; y++) {
-                    if (!live[y] || (pass == 1 && !need2[y])) continue;
-                    CK(O::multidot(c, vec(k.V, 0, y), j + 1, k.w + (long)y * n, c->d_scal + cnt * (2 * (j + 1) + 1),
-                                   (long)nb * n));
-                    CK(O::norm2(c, k.w + (long)y * n, c->d_scal + cnt * (2 * (j + 1) + 1) + 2 * (j + 1)));
-                    cnt++;
-                }
-                if (!cnt) break;
-                std::vector<double> all((size_t)cnt * (2 * (j + 1) + 1));
-                if (all.size() > (size_t)kScal / 2) {
-                    c->err = "batched Krylov solver: scalar staging too small";
-                    return OVL_EINVAL;
-                }
-                ST(c->fetch(c->d_scal, (int)all.size(), all.data()));
-                cnt = 0;
-                for (int y = 0; y < nb; y++) {
-                    if (!live[y] || (pass == 1 && !need2[y])) continue;
-                    const double *t = all.data() + (size_t)cnt * (2 * (j + 1) + 1);
-                    std::vector<cd> &hh = pass == 0 ? h1[y] : h2[y];
-                    std::vector<cd> neg(j + 1);
-                    double hsq = 0.0;
-                    for (int i = 0; i <= j; i++) {
-                        hh[i] = cd(t[2 * i], t[2 * i + 1]);
-                        neg[i] = -hh[i];
-                        hsq += std::norm(hh[i]);
-                    }
-                    ST(upload_coef(c, neg));
-                    CK(O::multiaxpy(c, vec(k.V, 0, y), j + 1, c->d_coef, k.w + (long)y * n, (long)nb * n));
-                    ST(c->sync());   // the coefficient staging is reused by the next system
-                    const double ww = t[2 * (j + 1)];
-                    const double left = ww - hsq;
-                    if (pass == 0) {
-                        if (!O::kCgs2 && left > 0.1 * ww) hn[y] = sqrt(left);
-                        else need2[y] = 1;
-                    } else {
-                        hn[y] = sqrt(std::max(0.0, left));
-                    }
-                    cnt++;
-                }
-            }
-            for (int y = 0; y < nb; y++) {
-                if (!live[y]) continue;
+            // Gram-Schmidt of the live systems in the same kernels
+            RowList rows{0, {}};
+            for (int y = 0; y < nb; y++)
+                if (live[y]) rows.row[rows.n++] = y;
+            ST(gs_arnoldi<T>(c, k.V, (long)nb * n, j + 1, k.w, rows, hc, hnv));
+            for (int r = 0; r < rows.n; r++) {
+                const int y = rows.row[r];
                 std::vector<cd> &Hy = H[y];
-                for (int i = 0; i <= j; i++) Hy[(size_t)i * m + j] = h1[y][i] + (need2[y] ? h2[y][i] : cd(0));
-                Hy[(size_t)(j + 1) * m + j] = hn[y];
-                if (!std::isfinite(hn[y])) {
+                for (int i = 0; i <= j; i++) Hy[(size_t)i * m + j] = hc[r][i];
+                Hy[(size_t)(j + 1) * m + j] = hnv[r];
+                if (!std::isfinite(hnv[r])) {
                     c->err = "batched Krylov solver: non-finite Arnoldi coefficient";
                     return OVL_EBREAKDOWN;
                 }
-                if (hn[y] > 0) CK(O::axpby(c, 1.0 / hn[y], k.w + (long)y * n, 0.0, vec(k.V, j + 1, y)));
-                else CK(cudaMemsetAsync(vec(k.V, j + 1, y), 0, n * sizeof(T), c->stream));
-                for (int i = 0; i < j; i++) {
-                    const cd a = Hy[(size_t)i * m + j], bq = Hy[(size_t)(i + 1) * m + j];
-                    Hy[(size_t)i * m + j] = std::conj(cs[y][i]) * a + std::conj(sn[y][i]) * bq;
-                    Hy[(size_t)(i + 1) * m + j] = -sn[y][i] * a + cs[y][i] * bq;
-                }
-                const cd a = Hy[(size_t)j * m + j], bq = Hy[(size_t)(j + 1) * m + j];
-                const double den = sqrt(std::norm(a) + std::norm(bq));
-                cs[y][j] = den > 0 ? a / den : cd(1.0);
-                sn[y][j] = den > 0 ? bq / den : cd(0.0);
-                Hy[(size_t)j * m + j] = den;
-                Hy[(size_t)(j + 1) * m + j] = 0.0;
-                gv[y][j + 1] = -sn[y][j] * gv[y][j];
-                gv[y][j] = std::conj(cs[y][j]) * gv[y][j];
-                if (std::abs(gv[y][j + 1]) <= tol * bnorm[y] || hn[y] == 0.0) live[y] = 0;
+                givens_column(Hy, m, j, cs[y], sn[y], gv[y]);
+                if (std::abs(gv[y][j + 1]) <= tol * bnorm[y] || hnv[r] == 0.0) live[y] = 0;
             }
             its++;
             if (its >= maxit) {
@@ -762,24 +731,20 @@ ovl_status fgmres_batch(Ctx *c, Krylov<T> &k, int nb, T *x, const T *b, double t
             }
         }
         // x_y += Z_y (H_y^{-1} g_y) over the columns this system took
+        RowList rows{0, {}};
+        std::vector<std::vector<cd>> yy;
         for (int y = 0; y < nb; y++) {
             if (!active[y]) continue;
             int jy = 0;   // columns used by y: those with nonzero diagonal
             while (jy < j && std::abs(H[y][(size_t)jy * m + jy]) > 0) jy++;
             if (!jy) continue;
-            std::vector<cd> yy(jy);
-            for (int i = jy - 1; i >= 0; i--) {
-                cd sacc = gv[y][i];
-                for (int q = i + 1; q < jy; q++) sacc -= H[y][(size_t)i * m + q] * yy[q];
-                yy[i] = sacc / H[y][(size_t)i * m + i];
-            }
-            ST(upload_coef(c, yy));
-            CK(O::multiaxpy(c, vec(k.Z, 0, y), jy, c->d_coef, x + (long)y * n, (long)nb * n));
-            ST(c->sync());
+            rows.row[rows.n++] = y;
+            yy.push_back(back_substitute(H[y], m, gv[y], jy));
             rel[y] = std::abs(gv[y][jy]) / bnorm[y];
             // reset this system's Hessenberg for the next cycle
             std::fill(H[y].begin(), H[y].end(), cd(0));
         }
+        if (rows.n) ST(gs_solution<T>(c, k.Z, (long)nb * n, yy, x, true, rows));
         xz = false;
         if (!verify) {
             bool any_left = false;
