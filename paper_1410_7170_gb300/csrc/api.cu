@@ -1210,8 +1210,12 @@ static ovl_status create_impl(Ctx *c, const double *gauge, const int dims[4], do
     c->rs.counter = (unsigned *)((char *)buf + sizeof(double) * kMaxRedValues * kMaxRedBlocks);
     c->d_flag = (int *)((char *)buf + sizeof(double) * kMaxRedValues * kMaxRedBlocks + 256);
     CK(cudaMemsetAsync(buf, 0, sizeof(double) * kMaxRedValues * kMaxRedBlocks + 4096, c->stream));
-    ST(c->alloc(&buf, (size_t)kScal * sizeof(double)));
+    ST(c->alloc(&buf, (size_t)(2 * kScal + 12 * 256 + 32) * sizeof(double)));
     c->d_scal = (double *)buf;
+    c->d_gs = c->d_scal + kScal;
+    c->d_gs_coef = c->d_gs + kScal;
+    c->gs_counters = (unsigned *)(c->d_gs_coef + 12 * 256);
+    CK(cudaMemsetAsync(c->gs_counters, 0, 32 * sizeof(double), c->stream));
     ST(c->alloc(&buf, sizeof(MsState)));
     c->ms64_state = (MsState *)buf;
     ST(c->alloc(&buf, sizeof(MsState)));
@@ -1220,11 +1224,6 @@ static ovl_status create_impl(Ctx *c, const double *gauge, const int dims[4], do
     c->d_md_part = (double *)buf;
     ST(c->alloc(&buf, (size_t)2 * 128 * sizeof(double)));
     c->d_coef = (double *)buf;
-    ST(c->alloc(&buf, (size_t)(kScal + 12 * 256) * sizeof(double) + 256));
-    c->d_gs = (double *)buf;
-    c->d_gs_coef = c->d_gs + kScal;
-    c->gs_counters = (unsigned *)(c->d_gs_coef + 12 * 256);
-    CK(cudaMemsetAsync(c->gs_counters, 0, 256, c->stream));
     // gauge field
     ST(c->alloc((void **)&c->U64, (size_t)V * 4 * kLink64Words * sizeof(double2)));
     ST(c->alloc((void **)&c->U32, (size_t)V * 4 * 3 * sizeof(float4)));
@@ -1350,8 +1349,12 @@ extern "C" ovl_status wilson_apply(ovl_ctx *ctx, double *out, const double *in, 
     }
     const bool late = on_device(in, out);
     ST(c->import_vec(in, c->io_a, 1, !late));
+    if (late) {
+        CK(wilson_f64_lex(c->g, c->U64, c->io_a, out, m0, 1, c->d_flag, c->stream));
+        return c->check_finite();
+    }
     CK(wilson_f64(c->g, c->U64, c->io_a, c->io_b, m0, 0, 1.0, nullptr, 0.0, c->stream));
-    return c->export_vec(c->io_b, out, 1, late);
+    return c->export_vec(c->io_b, out);
 }
 
 static ovl_status check_tol(Ctx *c, double tol) {
@@ -1607,6 +1610,10 @@ extern "C" ovl_status wilson_apply_arith(ovl_ctx *ctx, double *out, const double
     fb = (float4 *)c->f_b;
     if (arith == OVL_ARITH_FP32) {
         ST(c->import_vec(in, fa, 1, !late));
+        if (late && c->g.tps32 == 1) {
+            CK(wilson_f32_lex(c->g, c->U32, fa, out, (float)m0, 1, c->d_flag, c->stream));
+            return c->check_finite();
+        }
         CK(wilson_f32(c->g, c->U32, fa, fb, (float)m0, 0, 1.f, nullptr, 0.f, c->stream));
     } else {
         // 16-bit links and spinors, FP32 arithmetic: FP32 -> 16 bits, stencil, and back
@@ -1638,10 +1645,20 @@ extern "C" ovl_status wilson_apply_n_arith(ovl_ctx *ctx, double *out, const doub
     }
     const long wf = (long)c->g.V * 6;
     const bool late = on_device(in, out);
+    // Where one thread per site is the faster stencil (not on small lattices), the links that a
+    // multi-RHS kernel shares do not pay for a kernel of its own on the way out (whole call, us per
+    // right-hand side, multi-RHS kernel and way out -> one stencil per right-hand side that writes the
+    // answer: 16^4 13.9 -> 12.1 at 12 and 20.4 -> 16.3 at 3, 24^4 65.6 -> 54.4, 32^4 203 -> 182).
+    const bool direct = late && c->g.tps32 == 1 && !c->p.mrhs_kernel;
     float4 *fa = (float4 *)c->fbat, *fb = fa + (size_t)blk * wf;
     for (int r0 = 0; r0 < n_rhs; r0 += blk) {
         const int nb = std::min(blk, n_rhs - r0);
         ST(c->import_vec(in + (size_t)r0 * c->n64, fa, nb, !late));
+        if (direct) {
+            CK(wilson_f32_lex(c->g, c->U32, fa, out + (size_t)r0 * c->n64, (float)m0, nb, c->d_flag, c->stream));
+            ST(c->check_finite());
+            continue;
+        }
         CK(wilson_batch_f32(c->g, c->U32, fa, fb, wf, nb, (float)m0, 0, 1.f, nullptr, 0.f, c->stream));
         ST(c->export_vec(fb, out + (size_t)r0 * c->n64, nb, late));
     }
@@ -1775,8 +1792,13 @@ extern "C" ovl_status wilson_apply_n(ovl_ctx *ctx, double *out, const double *in
     for (int r0 = 0; r0 < n_rhs; r0 += blk) {
         const int nb = std::min(blk, n_rhs - r0);
         ST(c->import_vec(in + (size_t)r0 * c->n64, c->bbat, nb, !late));
+        if (late) {
+            CK(wilson_f64_lex(c->g, c->U64, c->bbat, out + (size_t)r0 * c->n64, m0, nb, c->d_flag, c->stream));
+            ST(c->check_finite());
+            continue;
+        }
         CK(wilson_batch_f64(c->g, c->U64, c->bbat, c->xbat, w, nb, m0, 0, 1.0, nullptr, 0.0, c->stream));
-        ST(c->export_vec(c->xbat, out + (size_t)r0 * c->n64, nb, late));
+        ST(c->export_vec(c->xbat, out + (size_t)r0 * c->n64, nb));
     }
     return OVL_OK;
 }

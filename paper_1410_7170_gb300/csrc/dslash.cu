@@ -289,31 +289,80 @@ cudaError_t spinor_f2d(const Geom &g, const float4 *a, double2 *b, cudaStream_t 
 }
 
 // ------------------------------------------------------------------ stencil
-// out = a [g5] D_W(m0) in + b z, one thread per site of the full lattice
-// (threads [0, Vh) even sites, [Vh, V) odd sites).
-template <typename R, typename LT, typename ST>
-__global__ void __launch_bounds__(kBlock, MinBlocks<R>::value) k_wilson(Geom g, const LT *__restrict__ U, const ST *__restrict__ in,
-                                                   ST *__restrict__ out, R m4, int g5, R a,
-                                                   const ST *z, R b, int spb) {
-    const int t = blockIdx.x * spb + threadIdx.x;
-    if (threadIdx.x >= spb || t >= g.V) return;
-    int p, i;
-    site_of_thread(t, p, i);
-    cpx<R> hop[12], own[12], res[12];
-    wilson_hop<R>(g, U, in, p, i, hop);
-    load_spinor<R>(in, g.Vh, p, i, own);
-    wilson_combine<R>(m4, own, hop, res);
-    if (g5) apply_g5(res);
-    if (z) {
-        cpx<R> zz[12];
-        load_spinor<R>(z, g.Vh, p, i, zz);
+// out = a [g5] D_W(m0) in + b z in FP32, one thread per site. Bound: the L1 data pipe, 80% busy with the
+// neighbour gathers and with filling them from L2. One wave of blocks that stride over the lattice
+// keeps the blocks of an SM and their neighbours on other SMs close together in time: 32^4 107 -> 90
+// us, 24^4 40 -> 35, 64 x 32^3 182 -> 170 (0.70 of the copy bandwidth), 16^4 10.2 -> 9.2, against a
+// block per 256 sites.
+__global__ void __launch_bounds__(kBlock, MinBlocks<float>::value)
+    k_wilson(Geom g, const float4 *__restrict__ U, const float4 *__restrict__ in, float4 *__restrict__ out, float m4,
+             int g5, float a, const float4 *z, float b, int spb) {
+    if (threadIdx.x >= spb) return;
+    for (int t = blockIdx.x * spb + threadIdx.x; t < g.V; t += gridDim.x * spb) {
+        int p, i;
+        site_of_thread(t, p, i);
+        cpx<float> hop[12], own[12], res[12];
+        wilson_hop<float>(g, U, in, p, i, hop);
+        load_spinor<float>(in, g.Vh, p, i, own);
+        wilson_combine<float>(m4, own, hop, res);
+        if (g5) apply_g5(res);
+        if (z) {
+            cpx<float> zz[12];
+            load_spinor<float>(z, g.Vh, p, i, zz);
 #pragma unroll
-        for (int c = 0; c < 12; c++) res[c] = a * res[c] + b * zz[c];
-    } else {
+            for (int c = 0; c < 12; c++) res[c] = a * res[c] + b * zz[c];
+        } else {
 #pragma unroll
-        for (int c = 0; c < 12; c++) res[c] = a * res[c];
+            for (int c = 0; c < 12; c++) res[c] = a * res[c];
+        }
+        store_spinor<float>(out, g.Vh, p, i, res);
     }
-    store_spinor<R>(out, g.Vh, p, i, res);
+}
+
+// D_W(m0) in FP32 straight into n boundary vectors (complex doubles). The 256 sites of a block's turn
+// are consecutive in both orders, so their results go through shared memory (28 words of 4 bytes
+// per site: the 16-byte stores of a quarter warp fall on different banks) and leave in whole rows,
+// instead of going to memory in the internal format and back through a kernel of their own
+// (k_spinor_out): per site 96 B written and 96 B read less. 64 x 32^3: 170 + 114 us -> 239 us.
+constexpr int kLexRow = 28;
+__global__ void __launch_bounds__(kBlock, MinBlocks<float>::value)
+    k_wilson_lex(Geom g, const float4 *__restrict__ U, const float4 *__restrict__ in, double2 *__restrict__ lex,
+                 long stride, float m4, const int *skip) {
+    extern __shared__ float lex_rows[];   // [kBlock][kLexRow]
+    if (skip && *(const volatile int *)skip) return;
+    in += blockIdx.y * stride;
+    lex += blockIdx.y * stride * 2;
+    for (int base = blockIdx.x * kBlock; base < g.V; base += gridDim.x * kBlock) {
+        const int t = base + threadIdx.x;
+        if (t < g.V) {
+            int p, i;
+            site_of_thread(t, p, i);
+            cpx<float> hop[12], own[12], res[12];
+            wilson_hop<float>(g, U, in, p, i, hop);
+            load_spinor<float>(in, g.Vh, p, i, own);
+            wilson_combine<float>(m4, own, hop, res);
+            const int s = 2 * i + ((p + io_row_parity(g, i)) & 1) - base;
+            float4 *row = reinterpret_cast<float4 *>(lex_rows + s * kLexRow);
+#pragma unroll
+            for (int c = 0; c < 6; c++)
+                row[c] = make_float4(res[2 * c].re, res[2 * c].im, res[2 * c + 1].re, res[2 * c + 1].im);
+        }
+        __syncthreads();
+        const int n = min(kBlock, g.V - base) * 12;
+        for (int e = threadIdx.x; e < n; e += kBlock) {
+            const float2 w = *reinterpret_cast<const float2 *>(lex_rows + (e / 12) * kLexRow + 2 * (e % 12));
+            __stcs(lex + (size_t)base * 12 + e, make_double2(f2d(w.x), f2d(w.y)));
+        }
+        __syncthreads();   // the next turn overwrites the rows
+    }
+}
+cudaError_t wilson_f32_lex(const Geom &g, const float4 *U, const float4 *in, double *lex, float m0, int n,
+                           const int *skip, cudaStream_t st) {
+    constexpr int smem = kBlock * kLexRow * sizeof(float);   // 28 KB
+    const int slots = std::max(1, g.nsm * MinBlocks<float>::value / n), need = (g.V + kBlock - 1) / kBlock;
+    k_wilson_lex<<<dim3(std::min(slots, need), n), kBlock, smem, st>>>(g, U, in, (double2 *)lex, 6L * g.V, m0 + 4.f, skip);
+    count_launches(1);
+    return cudaGetLastError();
 }
 
 // out = a [g5] D_W(m0) in + b z in FP64 or float-float, one warp per hop (hops.cuh); blockIdx.y =
@@ -328,7 +377,7 @@ __global__ void __launch_bounds__(kHopBlock, HopBlocks<R>::value)
     out += blockIdx.y * stride;
     if (z) z += blockIdx.y * stride;
     const auto fm = H::factor(m4), fa = H::factor(a), fb = H::factor(b);
-    hop_tiles<R>(g, blockIdx.x, gridDim.x, U, in, [&](int p, int i, int it, int e, typename H::Elem hop) {
+    hop_tiles<R>(g, blockIdx.x, gridDim.x, U, in, [&](int p, int i, int it, int e, typename H::Elem hop, int) {
         typename H::Elem r = H::fma(fm, H::load(in, g.Vh, p, i, it, e), hop);
         r = H::mul(fa, H::neg_if(r, g5 && H::upper(it)));
         if (z) r = H::fma(fb, H::load(z, g.Vh, p, i, it, e), r);
@@ -340,6 +389,27 @@ static cudaError_t wilson_hops(const Geom &g, const LT *U, const ST *in, ST *out
                                double a, const ST *z, double b, cudaStream_t st) {
     k_wilson_hops<R><<<dim3(hop_grid<R>(g, n, false), n), kHopBlock, 0, st>>>(g, U, in, out, stride, R(m0 + 4.0), g5,
                                                                                R(a), z, R(b));
+    count_launches(1);
+    return cudaGetLastError();
+}
+// D_W(m0) in FP64 straight into n boundary vectors. The FP64 units bound the stencil at all sizes, so
+// that 8-byte stores 192 bytes apart cost nothing beside them; a kernel for the way out and its
+// launch cost 5 us of a call (35 at 4^4).
+__global__ void __launch_bounds__(kHopBlock, HopBlocks<double>::value)
+    k_wilson_hops_lex(Geom g, const double2 *__restrict__ U, const double2 *__restrict__ in, double *__restrict__ lex,
+                      long stride, double m4, const int *skip) {
+    using H = HopTiles<double>;
+    if (skip && *(const volatile int *)skip) return;
+    in += blockIdx.y * stride;
+    lex += blockIdx.y * stride * 2;
+    hop_tiles<double>(g, blockIdx.x, gridDim.x, U, in, [&](int p, int i, int it, int e, double hop, int s) {
+        H::store_lex(lex, s, it, e, H::fma(m4, H::load(in, g.Vh, p, i, it, e), hop));
+    });
+}
+cudaError_t wilson_f64_lex(const Geom &g, const double2 *U, const double2 *in, double *lex, double m0, int n,
+                           const int *skip, cudaStream_t st) {
+    k_wilson_hops_lex<<<dim3(hop_grid<double>(g, n, false), n), kHopBlock, 0, st>>>(g, U, in, lex, 12L * g.V, m0 + 4.0,
+                                                                                    skip);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -362,8 +432,8 @@ cudaError_t wilson_ff(const Geom &g, const ffl *U, const ffw *in, ffw *out, doub
 cudaError_t wilson_f32(const Geom &g, const float4 *U, const float4 *in, float4 *out, float m0, int g5,
                        float a, const float4 *z, float b, cudaStream_t st) {
     if (g.tps32 == 4) return wilson_hops<float>(g, U, in, out, 0, 1, m0, g5, a, z, b, st);
-    const LaunchShape ls = balanced_shape(g.V, g.nsm, MinBlocks<float>::value, 1 << 30);
-    k_wilson<float, float4, float4><<<ls.grid, ls.block, 0, st>>>(g, U, in, out, m0 + 4.0f, g5, a, z, b, ls.spb);
+    const LaunchShape ls = balanced_shape(g.V, g.nsm, MinBlocks<float>::value, g.nsm * MinBlocks<float>::value);
+    k_wilson<<<ls.grid, ls.block, 0, st>>>(g, U, in, out, m0 + 4.0f, g5, a, z, b, ls.spb);
     count_launches(1);
     return cudaGetLastError();
 }

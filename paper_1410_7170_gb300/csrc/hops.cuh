@@ -268,6 +268,8 @@ template <> struct HopTiles<double> {
     __device__ static void store(Store *f, int Vh, int p, int i, int it, int im, Elem v) {
         reinterpret_cast<double *>(f)[at(Vh, p, i, it, im)] = v;
     }
+    // component `it` of site s of a boundary vector ([s][12] complex doubles)
+    __device__ static void store_lex(double *f, int s, int it, int im, Elem v) { f[24 * (size_t)s + 2 * it + im] = v; }
     __device__ static Factor factor(double a) { return a; }
     __device__ static Factor minus_alpha(const MsState &s) { return -s.alpha; }
     __device__ static Factor sigma0(const MsState &s) { return s.sigma[0]; }
@@ -511,8 +513,9 @@ template <> struct HopBlocks<double> { static constexpr int value = 3; };
 template <> struct HopBlocks<ff> { static constexpr int value = 3; };
 template <> struct HopBlocks<float> { static constexpr int value = 4; };
 
-// Tiles first, first + step, ... : epi(p, i, item, sub, hop) is called for each of the warp's items in
-// every lane that holds a site, with the hopping sum (times -1/2, the stored links' factor).
+// Tiles first, first + step, ... : epi(p, i, item, sub, hop, s) is called for each of the warp's items in
+// every lane that holds a site, with the hopping sum (times -1/2, the stored links' factor) and the
+// site's lexicographic index.
 template <typename R, typename Epi>
 __device__ __forceinline__ void hop_tiles(const Geom &g, int first, int step,
                                           const typename HopTiles<R>::Link *__restrict__ U,
@@ -532,7 +535,7 @@ __device__ __forceinline__ void hop_tiles(const Geom &g, int first, int step,
 #pragma unroll
         for (int it = w; it < H::items; it += 8) {
             const typename H::Elem hop = H::sum(part + lane, it, sub);
-            if (live) epi(p, i, it, sub, hop);
+            if (live) epi(p, i, it, sub, hop, 2 * i + (x[3] & 1));
         }
         if (tile + step < tiles) __syncthreads();   // the next tile overwrites part
     }

@@ -95,6 +95,12 @@ cudaError_t wilson_f64(const Geom &g, const double2 *U, const double2 *in, doubl
                        double a, const double2 *z, double b, cudaStream_t st);
 cudaError_t wilson_f32(const Geom &g, const float4 *U, const float4 *in, float4 *out, float m0, int g5,
                        float a, const float4 *z, float b, cudaStream_t st);
+// D_W(m0) of n even-odd spinors back to back into n boundary vectors; nothing is written if *skip
+// (device memory, nullable) is set
+cudaError_t wilson_f64_lex(const Geom &g, const double2 *U, const double2 *in, double *lex, double m0, int n,
+                           const int *skip, cudaStream_t st);
+cudaError_t wilson_f32_lex(const Geom &g, const float4 *U, const float4 *in, double *lex, float m0, int n,
+                           const int *skip, cudaStream_t st);
 // float-float stencil; fields in the layouts of ff.cuh
 cudaError_t wilson_ff(const Geom &g, const ffl *U, const ffw *in, ffw *out, double m0, int g5, double a,
                       const ffw *z, double b, cudaStream_t st);

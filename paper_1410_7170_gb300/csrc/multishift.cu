@@ -389,7 +389,7 @@ __global__ void __launch_bounds__(kHopBlock, HopBlocks<R>::value)
     typename H::Store *__restrict__ t = v.t + blockIdx.y * v.stride;
     typename H::Sum sum = H::zero();
     const auto fm = H::factor(m4);
-    hop_tiles<R>(g, blockIdx.x, gridDim.x, U, p0, [&](int p, int i, int it, int e, typename H::Elem hop) {
+    hop_tiles<R>(g, blockIdx.x, gridDim.x, U, p0, [&](int p, int i, int it, int e, typename H::Elem hop, int) {
         typename H::Elem w = H::fma(fm, H::load(p0, g.Vh, p, i, it, e), hop);
         w = H::neg_if(w, H::upper(it));
         H::store(t, g.Vh, p, i, it, e, w);
@@ -415,7 +415,7 @@ __global__ void __launch_bounds__(kHopBlock, HopBlocks<R>::value)
     if (blockIdx.x == 0 && threadIdx.x < 32) ShiftScalars{s}(threadIdx.x);
     const int first = blockIdx.x ? blockIdx.x - 1 : g.V;   // block 0: past the last tile
     const auto fm = H::factor(m4), fa = H::minus_alpha(*s), fs = H::sigma0(*s);
-    hop_tiles<R>(g, first, gridDim.x - 1, U, t, [&](int p, int i, int it, int e, typename H::Elem hop) {
+    hop_tiles<R>(g, first, gridDim.x - 1, U, t, [&](int p, int i, int it, int e, typename H::Elem hop, int) {
         typename H::Elem w = H::fma(fm, H::load(t, g.Vh, p, i, it, e), hop);
         w = H::fma(fs, H::load(p0, g.Vh, p, i, it, e), H::neg_if(w, H::upper(it)));
         w = H::fma(fa, w, H::load_rw(rin, g.Vh, p, i, it, e));
@@ -593,8 +593,10 @@ cudaError_t ms_stencils_hops(const Geom &g, const LT *U, double m0, int nrhs, Ms
 cudaError_t ms_stencils_site(const Geom &g, const float4 *U, float m0, int nrhs, MsState *s, const MsBatch<float4> &v,
                              const RedScratch &rows, cudaStream_t st, const MsEvents &ev) {
     const int slots = std::max(1, g.nsm * MinBlocks<float>::value / nrhs);   // resident blocks of a row
-    const LaunchShape q = balanced_shape(g.V, slots, 1, kMaxRedBlocks);
-    const LaunchShape r = balanced_shape(g.V, std::max(1, slots - 1), 1, kMaxRedBlocks - 1);
+    // one wave of blocks that stride over the sites (at 32^4 thirteen waves, each block ending with a
+    // fence and an atomic, cost 20 us of 125)
+    const LaunchShape q = balanced_shape(g.V, slots, 1, slots);
+    const LaunchShape r = balanced_shape(g.V, std::max(1, slots - 1), 1, std::max(1, slots - 1));
     cudaError_t e;
     if ((e = ev.record(0, st)) != cudaSuccess) return e;
     k_ms_q_site<<<dim3(q.grid, nrhs), q.block, 0, st>>>(g, U, m0 + 4.f, s, v, rows, q.spb);

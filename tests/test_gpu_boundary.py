@@ -31,15 +31,16 @@ def dev(a):
     return torch.from_numpy(np.ascontiguousarray(a)).cuda()
 
 
-def _op(dims):
+def _op(dims, tps=0):
     U = synth.gauge_field(dims, 0.5, 300 + sum(dims))
-    return U, ovl.Overlap(U, dims, 1.0, 0.05, ovl.params_default(lambda_min=0.05, lambda_max=8.0))
+    return U, ovl.Overlap(U, dims, 1.0, 0.05, ovl.params_default(lambda_min=0.05, lambda_max=8.0, stencil_tps=tps))
 
 
-@pytest.mark.parametrize("dims", [(2, 2, 2, 2), (2, 2, 4, 6), (2, 6, 6, 10), (4, 4, 4, 4)])
+@pytest.mark.parametrize("tps", [1, 4])
+@pytest.mark.parametrize("dims", [(2, 2, 2, 2), (2, 2, 4, 6), (2, 6, 6, 10), (4, 4, 4, 4), (4, 4, 6, 8), (12, 10, 8, 6)])
 @pytest.mark.parametrize("arith", list(TOL))
-def test_formats_on_partial_tiles(dims, arith):
-    U, op = _op(dims)
+def test_formats_on_partial_tiles(dims, arith, tps):
+    U, op = _op(dims, tps)
     for n in (1,) if arith == ovl.OVL_ARITH_FF else (1, 3, 13):
         b = synth.rhs_gaussian(dims, 400 + n, n_rhs=n)
         ref = np.stack([sparse.wilson(b[k], U, dims, -0.7) for k in range(n)])
@@ -56,8 +57,9 @@ def test_formats_on_partial_tiles(dims, arith):
 
 @pytest.mark.parametrize("dims", [(2, 2, 2, 2), (2, 6, 6, 10), (4, 4, 4, 4)])
 @pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf])
-def test_nonfinite_device_input_leaves_output_and_context_alone(dims, bad):
-    U, op = _op(dims)
+@pytest.mark.parametrize("tps", [1, 4])
+def test_nonfinite_device_input_leaves_output_and_context_alone(dims, bad, tps):
+    U, op = _op(dims, tps)
     b = synth.rhs_gaussian(dims, 77, n_rhs=2)
     ref = sparse.wilson(b[0], U, dims, -0.7)
     at = dev(b)
