@@ -377,8 +377,10 @@ __global__ void __launch_bounds__(kHopBlock, HopBlocks<R>::value)
     out += blockIdx.y * stride;
     if (z) z += blockIdx.y * stride;
     const auto fm = H::factor(m4), fa = H::factor(a), fb = H::factor(b);
-    hop_tiles<R>(g, blockIdx.x, gridDim.x, U, in, [&](int p, int i, int it, int e, typename H::Elem hop, int) {
-        typename H::Elem r = H::fma(fm, H::load(in, g.Vh, p, i, it, e), hop);
+    const auto own = [&](int p, int i, int it, int e) { return H::load(in, g.Vh, p, i, it, e); };
+    hop_tiles<R>(g, blockIdx.x, gridDim.x, U, in, own, [&](int p, int i, int it, int e, typename H::Elem hop, int,
+                                                            typename H::Elem o) {
+        typename H::Elem r = H::fma(fm, o, hop);
         r = H::mul(fa, H::neg_if(r, g5 && H::upper(it)));
         if (z) r = H::fma(fb, H::load(z, g.Vh, p, i, it, e), r);
         H::store(out, g.Vh, p, i, it, e, r);
@@ -402,8 +404,9 @@ __global__ void __launch_bounds__(kHopBlock, HopBlocks<double>::value)
     if (skip && *(const volatile int *)skip) return;
     in += blockIdx.y * stride;
     lex += blockIdx.y * stride * 2;
-    hop_tiles<double>(g, blockIdx.x, gridDim.x, U, in, [&](int p, int i, int it, int e, double hop, int s) {
-        H::store_lex(lex, s, it, e, H::fma(m4, H::load(in, g.Vh, p, i, it, e), hop));
+    const auto own = [&](int p, int i, int it, int e) { return H::load(in, g.Vh, p, i, it, e); };
+    hop_tiles<double>(g, blockIdx.x, gridDim.x, U, in, own, [&](int p, int i, int it, int e, double hop, int s, double o) {
+        H::store_lex(lex, s, it, e, H::fma(m4, o, hop));
     });
 }
 cudaError_t wilson_f64_lex(const Geom &g, const double2 *U, const double2 *in, double *lex, double m0, int n,

@@ -383,14 +383,16 @@ __global__ void __launch_bounds__(kHopBlock, HopBlocks<R>::value)
     k_ms_q_hops(Geom g, const typename HopTiles<R>::Link *__restrict__ U, R m4, MsState *st,
                 MsBatch<typename HopTiles<R>::Store> v, RedScratch rs) {
     using H = HopTiles<R>;
+    using E = typename H::Elem;
     MsState *s = st + blockIdx.y;
     if (s->done) return;
     const typename H::Store *__restrict__ p0 = v.p0_at(blockIdx.y, s->iter);
     typename H::Store *__restrict__ t = v.t + blockIdx.y * v.stride;
     typename H::Sum sum = H::zero();
     const auto fm = H::factor(m4);
-    hop_tiles<R>(g, blockIdx.x, gridDim.x, U, p0, [&](int p, int i, int it, int e, typename H::Elem hop, int) {
-        typename H::Elem w = H::fma(fm, H::load(p0, g.Vh, p, i, it, e), hop);
+    const auto own = [&](int p, int i, int it, int e) { return H::load(p0, g.Vh, p, i, it, e); };
+    hop_tiles<R>(g, blockIdx.x, gridDim.x, U, p0, own, [&](int p, int i, int it, int e, E hop, int, E o) {
+        E w = H::fma(fm, o, hop);
         w = H::neg_if(w, H::upper(it));
         H::store(t, g.Vh, p, i, it, e, w);
         H::square_add(w, sum);
@@ -404,6 +406,7 @@ __global__ void __launch_bounds__(kHopBlock, HopBlocks<R>::value)
     k_ms_r_hops(Geom g, const typename HopTiles<R>::Link *__restrict__ U, R m4, MsState *st,
                 MsBatch<typename HopTiles<R>::Store> v, RedScratch rs) {
     using H = HopTiles<R>;
+    using E = typename H::Elem;
     MsState *s = st + blockIdx.y;
     if (s->done) return;
     const int it0 = s->iter;
@@ -415,10 +418,16 @@ __global__ void __launch_bounds__(kHopBlock, HopBlocks<R>::value)
     if (blockIdx.x == 0 && threadIdx.x < 32) ShiftScalars{s}(threadIdx.x);
     const int first = blockIdx.x ? blockIdx.x - 1 : g.V;   // block 0: past the last tile
     const auto fm = H::factor(m4), fa = H::minus_alpha(*s), fs = H::sigma0(*s);
-    hop_tiles<R>(g, first, gridDim.x - 1, U, t, [&](int p, int i, int it, int e, typename H::Elem hop, int) {
-        typename H::Elem w = H::fma(fm, H::load(t, g.Vh, p, i, it, e), hop);
-        w = H::fma(fs, H::load(p0, g.Vh, p, i, it, e), H::neg_if(w, H::upper(it)));
-        w = H::fma(fa, w, H::load_rw(rin, g.Vh, p, i, it, e));
+    struct Own {
+        E t, p0, r;
+    };
+    const auto own = [&](int p, int i, int it, int e) {
+        return Own{H::load(t, g.Vh, p, i, it, e), H::load(p0, g.Vh, p, i, it, e), H::load_rw(rin, g.Vh, p, i, it, e)};
+    };
+    hop_tiles<R>(g, first, gridDim.x - 1, U, t, own, [&](int p, int i, int it, int e, E hop, int, const Own &o) {
+        E w = H::fma(fm, o.t, hop);
+        w = H::fma(fs, o.p0, H::neg_if(w, H::upper(it)));
+        w = H::fma(fa, w, o.r);
         H::store(rout, g.Vh, p, i, it, e, w);
         H::square_add(w, sum);
     });
