@@ -10,13 +10,16 @@ namespace ovl {
 
 namespace {
 
+struct Nothing {};
 struct StoreFin1 {
     double *res;
-    __device__ void operator()(const double *s) const { res[0] = s[0]; }
+    __device__ Nothing before() const { return {}; }
+    __device__ void operator()(const double *s, Nothing) const { res[0] = s[0]; }
 };
 struct StoreFin2 {
     double *res;
-    __device__ void operator()(const double *s) const { res[0] = s[0]; res[1] = s[1]; }
+    __device__ Nothing before() const { return {}; }
+    __device__ void operator()(const double *s, Nothing) const { res[0] = s[0]; res[1] = s[1]; }
 };
 
 // Per-thread partial sums are kept in the vector's own precision T (a grid-stride
@@ -185,12 +188,10 @@ __global__ void __launch_bounds__(kBlock) k_gs_dots(const T *__restrict__ base, 
     if (threadIdx.x == 0) {
         part[((long)i * gx + blockIdx.x) * 2] = s[0];
         part[((long)i * gx + blockIdx.x) * 2 + 1] = s[1];
-        __threadfence();
-        is_last = atomicAdd(counters + z, 1u) == (unsigned)(gridDim.y * gx - 1);
+        is_last = arrive(counters + z) == (unsigned)(gridDim.y * gx - 1);
     }
     __syncthreads();
     if (!is_last) return;
-    __threadfence();
     double *o = out + z * ostride;
     const int lane = threadIdx.x & 31;
     for (int q = threadIdx.x >> 5; q <= m; q += kBlock / 32) {

@@ -65,9 +65,13 @@ __device__ __forceinline__ void store_ff(float *to, double x) {
 // holds because r_k is orthogonal to p_{k-1} in CG; this spares ms_q a second reduction.
 struct AlphaFin {
     MsState *s;
-    __device__ void operator()(const double *v) const {
-        const double pAp = v[0] + s->sigma[0] * s->pp;
-        const double a = s->rr / pAp;
+    struct In {
+        double sigma0, pp, rr;
+    };
+    __device__ In before() const { return {s->sigma[0], s->pp, s->rr}; }
+    __device__ void operator()(const double *v, const In &in) const {
+        const double pAp = v[0] + in.sigma0 * in.pp;
+        const double a = in.rr / pAp;
         if (!(pAp > 0.0) || !isfinite(a)) {
             s->status = 1;
             s->done = 1;
@@ -118,9 +122,26 @@ struct ShiftScalars {
 };
 struct ShiftFin {
     MsState *s;
-    __device__ void operator()(const double *v, int lane) const {
-        const double rr_new = v[0], rs = rr_new * s->scale;
-        const double beta = rs * s->inv_rr;
+    static constexpr int kSets = kMaxPoles / 32;
+    struct In {
+        double scale, inv_rr, inv_bb, tol, pp, alpha, ratio[kSets], critz2[kSets];
+        int n, slot, iter, hist_cap, active[kSets];
+        int *hist;
+    };
+    __device__ In before(int lane) const {
+        In in{s->scale, s->inv_rr, s->inv_bb, s->tol, s->pp, s->alpha, {}, {}, s->n, s->npend, s->iter, s->hist_cap, {},
+              s->hist};
+#pragma unroll
+        for (int j = 0; j < kSets; j++) {
+            in.ratio[j] = s->ratio[32 * j + lane];
+            in.critz2[j] = s->critz2[32 * j + lane];
+            in.active[j] = s->active[32 * j + lane];
+        }
+        return in;
+    }
+    __device__ void operator()(const double *v, int lane, const In &in) const {
+        const double rr_new = v[0], rs = rr_new * in.scale;
+        const double beta = rs * in.inv_rr;
         if (!isfinite(beta)) {
             if (lane == 0) {
                 s->status = 1;
@@ -128,34 +149,34 @@ struct ShiftFin {
             }
             return;
         }
-        const double rel = rs * s->inv_bb, tol2 = s->tol * s->tol;
-        const int slot = s->npend;
+        const double rel = rs * in.inv_bb, tol2 = in.tol * in.tol;
         int any = 0, nupd = 0;
-        for (int l0 = 0; l0 < kMaxPoles; l0 += 32) {
-            const int l = l0 + lane;
-            const bool on = l < s->n && s->active[l];
+#pragma unroll
+        for (int j = 0; j < kSets; j++) {
+            const int l = 32 * j + lane;
+            const bool on = l < in.n && in.active[j];
             const unsigned m = __ballot_sync(0xffffffffu, on);
-            if (lane == 0) s->on[slot][l0 / 32] = m;
+            if (lane == 0) s->on[in.slot][j] = m;
             nupd += __popc(m);
             if (!on) continue;
-            const double bl = beta * s->ratio[l];
-            s->bl[slot][l] = bl;
-            store_ff(s->bl_f[slot][l], bl);
+            const double bl = beta * in.ratio[j];
+            s->bl[in.slot][l] = bl;
+            store_ff(s->bl_f[in.slot][l], bl);
             // residual bound after this iteration's update: this was the shift's last one, except
             // for the base shift, whose direction drives the Krylov space
-            if (s->critz2[l] * rel > tol2) any = 1;
+            if (in.critz2[j] * rel > tol2) any = 1;
             else if (l > 0) s->active[l] = 0;
         }
         any = __any_sync(0xffffffffu, any);
         if (lane == 0) {
-            if (s->hist && s->iter < s->hist_cap) s->hist[s->iter] = nupd;
-            s->alpha_prev = s->alpha;
+            if (in.hist && in.iter < in.hist_cap) in.hist[in.iter] = nupd;
+            s->alpha_prev = in.alpha;
             s->beta_prev = beta;
             store_ff(s->beta_f, beta);
-            s->pp = rr_new + beta * beta * s->pp;
+            s->pp = rr_new + beta * beta * in.pp;
             s->rr = rr_new;
-            s->iter += 1;
-            s->npend = slot + 1;
+            s->iter = in.iter + 1;
+            s->npend = in.slot + 1;
             if (!any) s->done = 2;   // ms_shifts brings y up to date, then the solve is done
         }
     }
@@ -364,16 +385,17 @@ __global__ void __launch_bounds__(kBlock, kShiftBlocks) k_ms_shifts(MsState *st,
     __syncthreads();
     const bool go_on = !s->done;
     const typename W::C b0 = W::coef(s->beta_prev, s->beta_f);
+    // the block that arrives last, when all have read the state, clears the pending iterations and ends
+    // a finished solve
+    if (grid_last_block(counters + row) && threadIdx.x == 0) {
+        s->npend = 0;
+        if (!go_on && s->done == 2) s->done = 1;
+    }
     switch (np) {
         case 1: shift_updates<1>(sl, v, row, it, b0, go_on); break;
         case 2: shift_updates<2>(sl, v, row, it, b0, go_on); break;
         case 3: shift_updates<3>(sl, v, row, it, b0, go_on); break;
         default: shift_updates<4>(sl, v, row, it, b0, go_on); break;
-    }
-    // the last block clears the pending iterations and ends a finished solve
-    if (grid_last_block(counters + row) && threadIdx.x == 0) {
-        s->npend = 0;
-        if (s->done == 2) s->done = 1;
     }
 }
 
@@ -450,7 +472,8 @@ __global__ void __launch_bounds__(kBlock) k_ms_p0(const MsState *st, MsBatch<ST>
 
 struct InitFin {
     MsState *s;
-    __device__ void operator()(const double *v) const {
+    __device__ int before() const { return 0; }
+    __device__ void operator()(const double *v, int) const {
         s->bb = v[0];
         s->rr = v[0];
         s->pp = v[0];   // p_0 = b
