@@ -1647,8 +1647,8 @@ extern "C" ovl_status wilson_apply_n_arith(ovl_ctx *ctx, double *out, const doub
     const bool late = on_device(in, out);
     // Where one thread per site is the faster stencil (not on small lattices), the links that a
     // multi-RHS kernel shares do not pay for a kernel of its own on the way out (whole call, us per
-    // right-hand side, multi-RHS kernel and way out -> one stencil per right-hand side that writes the
-    // answer: 16^4 13.9 -> 12.1 at 12 and 20.4 -> 16.3 at 3, 24^4 65.6 -> 54.4, 32^4 203 -> 182).
+    // right-hand side, the best multi-RHS kernel and way out -> one stencil per right-hand side that
+    // writes the answer: 16^4 14.0 -> 11.7 at 12 and 20.8 -> 17.4 at 3, 24^4 60.2 -> 52.0, 32^4 201 -> 173).
     const bool direct = late && c->g.tps32 == 1 && !c->p.mrhs_kernel;
     float4 *fa = (float4 *)c->fbat, *fb = fa + (size_t)blk * wf;
     for (int r0 = 0; r0 < n_rhs; r0 += blk) {

@@ -94,13 +94,16 @@ __device__ __forceinline__ int div_mod(int n, int d, unsigned inv, int &rem) {
     return q;
 }
 
-// Site visited by thread t of a full-lattice kernel: parities interleave (t even: even
-// site, t odd: odd site, same checkerboard index), so the two sites that read a link
-// (x and x + mu) and the neighbours of a site are touched close together in time and
-// their data is still in L2.
+// Site visited by thread t of a full-lattice kernel: eight even sites, then the odd sites of the same
+// checkerboard indices, so that the two sites that read a link (x and x + mu) and the neighbours of a
+// site are touched close together in time, and so that the 16-byte words that a quarter of a warp reads
+// are one 128-byte line: a warp-wide load goes through L1 a quarter at a time, and with the parities
+// alternating from thread to thread each quarter took half a line of either parity's plane, which fall
+// on the same banks. One FP32 stencil 16^4 9.4 -> 8.3 us, 24^4 35.0 -> 31.3, 32^4 90 -> 81, 22 x 26 x 34 x 18
+// 40.8 -> 34.8. V is a multiple of 16 (even extents).
 __device__ __forceinline__ void site_of_thread(int t, int &p, int &i) {
-    p = t & 1;
-    i = t >> 1;
+    p = t >> 3 & 1;
+    i = (t >> 4 << 3) | (t & 7);
 }
 
 // Coordinates of checkerboard site (p, i).

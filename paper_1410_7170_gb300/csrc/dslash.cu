@@ -289,11 +289,12 @@ cudaError_t spinor_f2d(const Geom &g, const float4 *a, double2 *b, cudaStream_t 
 }
 
 // ------------------------------------------------------------------ stencil
-// out = a [g5] D_W(m0) in + b z in FP32, one thread per site. Bound: the L1 data pipe, 80% busy with the
-// neighbour gathers and with filling them from L2. One wave of blocks that stride over the lattice
-// keeps the blocks of an SM and their neighbours on other SMs close together in time: 32^4 107 -> 90
-// us, 24^4 40 -> 35, 64 x 32^3 182 -> 170 (0.70 of the copy bandwidth), 16^4 10.2 -> 9.2, against a
-// block per 256 sites.
+// out = a [g5] D_W(m0) in + b z in FP32, one thread per site. Bound: the L1 data pipe (neighbour gathers
+// and their fills from L2) until the vectors and links no longer fit in L2, then memory (64 x 32^3, 168
+// us: 0.70 of the copy bandwidth). One wave of blocks that stride over the lattice keeps the blocks
+// of an SM and their neighbours on other SMs close together in time: 32^4 107 -> 90 us, 24^4 40 -> 35,
+// 64 x 32^3 182 -> 170, 16^4 10.2 -> 9.2, against a block per 256 sites; with the order of
+// site_of_thread 81, 31.3, 168 and 8.3.
 __global__ void __launch_bounds__(kBlock, MinBlocks<float>::value)
     k_wilson(Geom g, const float4 *__restrict__ U, const float4 *__restrict__ in, float4 *__restrict__ out, float m4,
              int g5, float a, const float4 *z, float b, int spb) {
@@ -320,11 +321,11 @@ __global__ void __launch_bounds__(kBlock, MinBlocks<float>::value)
 }
 
 // D_W(m0) in FP32 straight into n boundary vectors (complex doubles). The 256 sites of a block's turn
-// are consecutive in both orders, so their results go through shared memory (28 words of 4 bytes
-// per site: the 16-byte stores of a quarter warp fall on different banks) and leave in whole rows,
+// are consecutive in both orders, so their results go through shared memory (26 words of 4 bytes
+// per site: the 8-byte stores of half a warp fall on different banks) and leave in whole rows,
 // instead of going to memory in the internal format and back through a kernel of their own
-// (k_spinor_out): per site 96 B written and 96 B read less. 64 x 32^3: 170 + 114 us -> 239 us.
-constexpr int kLexRow = 28;
+// (k_spinor_out): per site 96 B written and 96 B read less. 64 x 32^3: 170 + 114 us -> 226 us.
+constexpr int kLexRow = 26;
 __global__ void __launch_bounds__(kBlock, MinBlocks<float>::value)
     k_wilson_lex(Geom g, const float4 *__restrict__ U, const float4 *__restrict__ in, double2 *__restrict__ lex,
                  long stride, float m4, const int *skip) {
@@ -342,10 +343,9 @@ __global__ void __launch_bounds__(kBlock, MinBlocks<float>::value)
             load_spinor<float>(in, g.Vh, p, i, own);
             wilson_combine<float>(m4, own, hop, res);
             const int s = 2 * i + ((p + io_row_parity(g, i)) & 1) - base;
-            float4 *row = reinterpret_cast<float4 *>(lex_rows + s * kLexRow);
+            float2 *row = reinterpret_cast<float2 *>(lex_rows + s * kLexRow);
 #pragma unroll
-            for (int c = 0; c < 6; c++)
-                row[c] = make_float4(res[2 * c].re, res[2 * c].im, res[2 * c + 1].re, res[2 * c + 1].im);
+            for (int c = 0; c < 12; c++) row[c] = make_float2(res[c].re, res[c].im);
         }
         __syncthreads();
         const int n = min(kBlock, g.V - base) * 12;
@@ -358,7 +358,7 @@ __global__ void __launch_bounds__(kBlock, MinBlocks<float>::value)
 }
 cudaError_t wilson_f32_lex(const Geom &g, const float4 *U, const float4 *in, double *lex, float m0, int n,
                            const int *skip, cudaStream_t st) {
-    constexpr int smem = kBlock * kLexRow * sizeof(float);   // 28 KB
+    constexpr int smem = kBlock * kLexRow * sizeof(float);   // 26 KB
     const int slots = std::max(1, g.nsm * MinBlocks<float>::value / n), need = (g.V + kBlock - 1) / kBlock;
     k_wilson_lex<<<dim3(std::min(slots, need), n), kBlock, smem, st>>>(g, U, in, (double2 *)lex, 6L * g.V, m0 + 4.f, skip);
     count_launches(1);

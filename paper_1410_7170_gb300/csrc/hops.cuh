@@ -19,7 +19,7 @@
 // The sum of the FP64 instructions per site is that of the one-thread form. One stencil, one thread
 // per site -> one warp per hop (us): FP64 4^4 33 -> 8, 8^4 33 -> 12, 12^4 51 -> 39, 16^4 111 -> 109,
 // 32^4 1688 -> 1681 (the FP64 units' measured rate allows 1730 with the epilogue: 888 FP64
-// instructions per site); float-float 8^4 25 -> 6, 16^4 38 -> 29, 24^4 194 -> 154, 32^4 535 -> 466.
+// instructions per site); float-float 8^4 25 -> 6, 16^4 38 -> 29, 24^4 194 -> 138, 32^4 535 -> 418.
 #pragma once
 #include "reduce.cuh"
 #include "wilson_site.cuh"

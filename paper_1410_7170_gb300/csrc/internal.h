@@ -59,6 +59,7 @@ inline LaunchShape balanced_shape(long n, int nsm, int per_sm, int max_blocks) {
     if (nblk > max_blocks) nblk = (max_blocks / slots) * slots;
     if (nblk < 1) nblk = 1;
     long spb = (n + nblk - 1) / nblk;
+    spb = (spb + 7) / 8 * 8;         // quarter warps on whole lines (site_of_thread)
     if (spb > kBlock) spb = kBlock;   // more sites than threads: the kernel strides
     const int T = (int)((spb + 31) / 32 * 32);
     return LaunchShape{(int)nblk, T, (int)spb};

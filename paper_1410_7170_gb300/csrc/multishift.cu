@@ -626,7 +626,8 @@ cudaError_t ms_stencils_site(const Geom &g, const float4 *U, float m0, int nrhs,
                              const RedScratch &rows, cudaStream_t st, const MsEvents &ev) {
     const int slots = std::max(1, g.nsm * MinBlocks<float>::value / nrhs);   // resident blocks of a row
     // one wave of blocks that stride over the sites (at 32^4 thirteen waves, each block ending with a
-    // fence and an atomic, cost 20 us of 125)
+    // fence and an atomic, cost 20 us of 125; the whole FP32 sign at 32^4 14.67 ms, with the order of
+    // site_of_thread 14.17)
     const LaunchShape q = balanced_shape(g.V, slots, 1, slots);
     const LaunchShape r = balanced_shape(g.V, std::max(1, slots - 1), 1, std::max(1, slots - 1));
     cudaError_t e;
