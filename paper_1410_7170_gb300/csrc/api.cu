@@ -1601,8 +1601,12 @@ extern "C" ovl_status wilson_apply_arith(ovl_ctx *ctx, double *out, const double
     if (arith == OVL_ARITH_FF) {
         ST(c->ensure_msff());
         ST(c->import_vec(in, c->msff.t, 1, !late));
+        if (late) {
+            CK(wilson_ff_lex(c->g, c->Uff, c->msff.t, out, m0, c->d_flag, c->stream));
+            return c->check_finite();
+        }
         CK(wilson_ff(c->g, c->Uff, c->msff.t, c->msff.y, m0, 0, 1.0, nullptr, 0.0, c->stream));
-        return c->export_vec(c->msff.y, out, 1, late);
+        return c->export_vec(c->msff.y, out);
     }
     float4 *fa, *fb;
     ST(ensure_f32_buffers(c));

@@ -416,6 +416,37 @@ cudaError_t wilson_f64_lex(const Geom &g, const double2 *U, const double2 *in, d
     count_launches(1);
     return cudaGetLastError();
 }
+// The same in float-float. The tile's 32 sites are consecutive in both orders; a lane holds one real of
+// two spins, so the results go through shared memory (26 doubles per site) and leave in whole rows:
+// per site 192 B written and 192 B read less. The whole call at 24^4 209 -> 198 us.
+constexpr int kFfLexRow = 26;
+__global__ void __launch_bounds__(kHopBlock, HopBlocks<ff>::value)
+    k_wilson_ff_lex(Geom g, const ffl *__restrict__ U, const ffw *__restrict__ in, double2 *__restrict__ lex, ff m4,
+                    const int *skip) {
+    using H = HopTiles<ff>;
+    __shared__ __align__(16) double rows[H::tile * kFfLexRow];
+    if (skip && *(const volatile int *)skip) return;
+    const auto fm = H::factor(m4);
+    const int s0 = blockIdx.x * H::tile;
+    const auto own = [&](int p, int i, int it, int e) { return H::load(in, g.Vh, p, i, it, e); };
+    hop_tiles<ff>(g, blockIdx.x, gridDim.x, U, in, own, [&](int p, int i, int it, int, ff2 hop, int s, ff2 o) {
+        const float4 w = ff2_word(H::fma(fm, o, hop));
+        double *row = rows + (s - s0) * kFfLexRow + 2 * IoWord<ffw>::first(it) + (it & 1);
+        row[0] = ff2d(w.x, w.z);
+        row[6] = ff2d(w.y, w.w);
+    });
+    __syncthreads();
+    const int n = min(H::tile, g.V - s0) * 12;
+    for (int e = threadIdx.x; e < n; e += kHopBlock)
+        __stcs(lex + (size_t)s0 * 12 + e,
+               *reinterpret_cast<const double2 *>(rows + (e / 12) * kFfLexRow + 2 * (e % 12)));
+}
+cudaError_t wilson_ff_lex(const Geom &g, const ffl *U, const ffw *in, double *lex, double m0, const int *skip,
+                          cudaStream_t st) {
+    k_wilson_ff_lex<<<hop_grid<ff>(g, 1, false), kHopBlock, 0, st>>>(g, U, in, (double2 *)lex, ff(m0 + 4.0), skip);
+    count_launches(1);
+    return cudaGetLastError();
+}
 cudaError_t wilson_f64(const Geom &g, const double2 *U, const double2 *in, double2 *out, double m0, int g5,
                        double a, const double2 *z, double b, cudaStream_t st) {
     return wilson_hops<double>(g, U, in, out, 0, 1, m0, g5, a, z, b, st);

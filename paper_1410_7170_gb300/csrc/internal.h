@@ -102,6 +102,8 @@ cudaError_t wilson_f64_lex(const Geom &g, const double2 *U, const double2 *in, d
                            const int *skip, cudaStream_t st);
 cudaError_t wilson_f32_lex(const Geom &g, const float4 *U, const float4 *in, double *lex, float m0, int n,
                            const int *skip, cudaStream_t st);
+cudaError_t wilson_ff_lex(const Geom &g, const ffl *U, const ffw *in, double *lex, double m0, const int *skip,
+                          cudaStream_t st);
 // float-float stencil; fields in the layouts of ff.cuh
 cudaError_t wilson_ff(const Geom &g, const ffl *U, const ffw *in, ffw *out, double m0, int g5, double a,
                       const ffw *z, double b, cudaStream_t st);
