@@ -268,8 +268,8 @@ ovl_status ovl_krylov_sign_info(const ovl_ctx *ctx, long *cycles, long *matvecs)
 ovl_status ovl_hermitian_eig(int n, const double *A, double *w, double *Z);
 
 /* FP32 Schwarz block solves of the Wilson preconditioner (Sec. 5.1 smoother; an implementation
- * choice, the paper has no counterpart): they have one form, two threads per block site. *tps is
- * params.sap_tps if that is set and 2 otherwise; ms[0..2] the measured time of one Schwarz cycle
+ * choice, the paper has no counterpart): they have one form, one thread per block site. *tps is
+ * params.sap_tps if that is set and 1 otherwise; ms[0..2] the measured time of one Schwarz cycle
  * (zeros when sap_tps is set or precond is OVL_PREC_NONE). tps, ms nullable. */
 ovl_status ovl_tuning_sap(const ovl_ctx *ctx, int *tps, float *ms);
 

@@ -420,7 +420,7 @@ def ovl_tuning_mrhs(ctx):
 
 
 def ovl_tuning_sap(ctx):
-    """params.sap_tps or 2 (one FP32 Schwarz block kernel) and its time per cycle, three times (ms)."""
+    """params.sap_tps or 1 (one FP32 Schwarz block kernel) and its time per cycle, three times (ms)."""
     import numpy as np
     a = ctypes.c_int()
     ms = np.zeros(3, dtype=np.float32)

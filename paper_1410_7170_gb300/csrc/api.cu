@@ -1089,7 +1089,7 @@ ovl_status Ctx::autotune_mrhs() {
 }
 
 // Time of one FP32 Schwarz cycle on a constant non-zero input, for ovl_tuning_sap (the block kernel
-// has one form, two threads per block site).
+// has one form, one thread per block site).
 ovl_status Ctx::time_sap() {
     Ctx *c = this;
     void *buf;
@@ -1515,7 +1515,7 @@ extern "C" ovl_status ovl_m0_adapt_info(const ovl_ctx *ctx, double *cand, double
 extern "C" ovl_status ovl_tuning_sap(const ovl_ctx *ctx, int *tps, float *ms) {
     const Ctx *c = reinterpret_cast<const Ctx *>(ctx);
     if (!c) return OVL_EINVAL;
-    if (tps) *tps = c->p.sap_tps ? c->p.sap_tps : 2;
+    if (tps) *tps = c->p.sap_tps ? c->p.sap_tps : 1;
     if (ms)
         for (int k = 0; k < 3; k++) ms[k] = c->sap_ms[k];
     return OVL_OK;
