@@ -33,8 +33,8 @@ TOL = 1e-8
 METRIC = "overlap solves/s at 1e-8 (mixed vs FP64 GPU); Dslash GB/s % HBM; p50/p99 latency"
 UNIT = "solves/s"
 KERNEL_SOURCES = ["paper_1410_7170_gb300/csrc/multishift.cu", "paper_1410_7170_gb300/csrc/wilson_site.cuh",
-                  "paper_1410_7170_gb300/csrc/common.cuh", "paper_1410_7170_gb300/csrc/reduce.cuh",
-                  "paper_1410_7170_gb300/csrc/ff.cuh"]
+                  "paper_1410_7170_gb300/csrc/hops.cuh", "paper_1410_7170_gb300/csrc/common.cuh",
+                  "paper_1410_7170_gb300/csrc/reduce.cuh", "paper_1410_7170_gb300/csrc/ff.cuh"]
 PROF_CLASSES = ("ms_stencil_f64", "ms_shifts_f64", "ms_stencil_f32", "ms_shifts_f32", "ms_stencil_ff", "ms_shifts_ff")
 # Unpreconditioned FP64 GMRES(100) on the 16^4 workload with fixed sign accuracy 1e-10 (no
 # relaxation), the oracle's own algorithm: D_N applications per solve, measured with the
@@ -169,10 +169,10 @@ RELAX = 0.3
 # (python -m paper_1410_7170_gb300.scan --m0=-0.45:0.0:0.05 --relax 0.3) is flat from -0.25 to 0
 # (118 to 110 ms per solve) and lowest at 0 (m0^def = -0.265 gives 118 ms).
 M0_PREC = 0.0
-# Algorithmic FP32 operations per site of the float-float multishift stencils (the float-float
-# formulas of ff.cuh as written: the hopping term 9024, the (m0+4) combination 360, the norm
-# 443, and in the residual update 864 more): k_ms_q 9827, k_ms_r 10691.
-FF_OPS_PER_SITE = (9827 + 10691) / 2.0
+# Algorithmic FP32 operations per site of the float-float multishift stencils (the packed float-float
+# formulas of hops.cuh as written, two operations each: the hopping term 8832, the (m0+4) combination
+# 360, the norm 360, and in the residual update 720 more): k_ms_q_hops 9552, k_ms_r_hops 10272.
+FF_OPS_PER_SITE = (9552 + 10272) / 2.0
 
 
 def solver_params(ovl, mixed):

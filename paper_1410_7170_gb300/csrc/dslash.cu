@@ -289,9 +289,10 @@ cudaError_t spinor_f2d(const Geom &g, const float4 *a, double2 *b, cudaStream_t 
 }
 
 // ------------------------------------------------------------------ stencil
-// out = a [g5] D_W(m0) in + b z in FP32, one thread per site. Bound: the L1 data pipe (neighbour gathers
-// and their fills from L2) until the vectors and links no longer fit in L2, then memory (64 x 32^3, 168
-// us: 0.70 of the copy bandwidth). One wave of blocks that stride over the lattice keeps the blocks
+// out = a [g5] D_W(m0) in + b z in FP32, one thread per site. Bound: the latency of the neighbour gathers,
+// which go to L2 three times in four, at 16 warps per SM (128 registers); at 64 x 32^3 with memory 60%
+// and the L1 data pipe 48% busy (168 us: 0.70 of the copy bandwidth). One wave of blocks that stride
+// over the lattice keeps the blocks
 // of an SM and their neighbours on other SMs close together in time: 32^4 107 -> 90 us, 24^4 40 -> 35,
 // 64 x 32^3 182 -> 170, 16^4 10.2 -> 9.2, against a block per 256 sites; with the order of
 // site_of_thread 81, 31.3, 168 and 8.3.
