@@ -1599,14 +1599,17 @@ extern "C" ovl_status wilson_apply_arith(ovl_ctx *ctx, double *out, const double
     if (arith == OVL_ARITH_FP64) return wilson_apply(ctx, out, in, m0);
     const bool late = on_device(in, out);
     if (arith == OVL_ARITH_FF) {
-        ST(c->ensure_msff());
-        ST(c->import_vec(in, c->msff.t, 1, !late));
+        // the FP64 boundary buffers hold float-float spinors too (16 B per complex number): the stencil
+        // needs no multishift vectors
+        ST(c->ensure_ff_links());
+        ffw *a = (ffw *)c->io_a, *b = (ffw *)c->io_b;
+        ST(c->import_vec(in, a, 1, !late));
         if (late) {
-            CK(wilson_ff_lex(c->g, c->Uff, c->msff.t, out, m0, c->d_flag, c->stream));
+            CK(wilson_ff_lex(c->g, c->Uff, a, out, m0, c->d_flag, c->stream));
             return c->check_finite();
         }
-        CK(wilson_ff(c->g, c->Uff, c->msff.t, c->msff.y, m0, 0, 1.0, nullptr, 0.0, c->stream));
-        return c->export_vec(c->msff.y, out);
+        CK(wilson_ff(c->g, c->Uff, a, b, m0, 0, 1.0, nullptr, 0.0, c->stream));
+        return c->export_vec(b, out);
     }
     float4 *fa, *fb;
     ST(ensure_f32_buffers(c));
