@@ -485,11 +485,14 @@ struct InitFin {
     }
 };
 
-// r = y = p_l = b ; ||b||^2 of right-hand side blockIdx.y (b: vectors v.stride words apart)
+// r = y = p_l = b ; ||b||^2 of right-hand side blockIdx.y (b: vectors v.stride words apart). One that
+// needs no work (done already set) is left out: its b is a vector that its solver never wrote, and a NaN
+// in it would count as a breakdown of the whole batch.
 template <typename ST>
 __global__ void k_ms_init(MsState *st, const ST *__restrict__ b, MsBatch<ST> v, RedScratch rs) {
     using W = Word<ST>;
     MsState *s = st + blockIdx.y;
+    if (s->done) return;   // uniform over the blocks of this right-hand side: only the last to arrive sets it
     b += blockIdx.y * v.stride;
     ST *r = v.r_at(blockIdx.y, 0), *p0 = v.p0_at(blockIdx.y, 0), *y = v.y + blockIdx.y * v.stride;
     ST *P = v.p + blockIdx.y * v.prow;
