@@ -253,12 +253,12 @@ __global__ void __launch_bounds__(kBlock) k_gs_subtract(const T *__restrict__ ba
 template <typename T>
 __global__ void __launch_bounds__(kBlock) k_gs_combine(const T *__restrict__ base, long stride, int m,
                                                        const double *__restrict__ c, T *x, bool add, long n,
-                                                       RowList rows) {
+                                                       RowList rows, RowColumns cols) {
     using G = GsWord<T>;
     using W = typename G::W;
     __shared__ T cs[2 * kGsMax];
-    const int z = blockIdx.y;
-    for (int k = threadIdx.x; k < 2 * m; k += blockDim.x) cs[k] = (T)c[2 * m * z + k];
+    const int z = blockIdx.y, mz = cols.n[z];
+    for (int k = threadIdx.x; k < 2 * mz; k += blockDim.x) cs[k] = (T)c[2 * m * z + k];
     __syncthreads();
     const long off = (long)rows.row[z] * n, nw = n * (long)sizeof(T) / (long)sizeof(W);
     const W *v = reinterpret_cast<const W *>(base + off);
@@ -267,7 +267,7 @@ __global__ void __launch_bounds__(kBlock) k_gs_combine(const T *__restrict__ bas
     for (long k = (long)blockIdx.x * blockDim.x + threadIdx.x; k < nw; k += (long)gridDim.x * blockDim.x) {
         W a = add ? o[k] : G::zero();
 #pragma unroll 4
-        for (int j = 0; j < m; j++) G::axpy(cs[2 * j], cs[2 * j + 1], v[j * sw + k], a);
+        for (int j = 0; j < mz; j++) G::axpy(cs[2 * j], cs[2 * j + 1], v[j * sw + k], a);
         o[k] = a;
     }
 }
@@ -403,9 +403,9 @@ cudaError_t gs_subtract(const T *base, long stride, int m, const double *h, long
 }
 template <typename T>
 cudaError_t gs_combine(const T *base, long stride, int m, const double *c, T *x, bool add, long n, const RowList &rows,
-                       cudaStream_t st) {
+                       const RowColumns &cols, cudaStream_t st) {
     k_gs_combine<T><<<dim3(gs_grid(n * (long)sizeof(T) / 16, rows.n, 8), rows.n), kBlock, 0, st>>>(base, stride, m, c, x, add,
-                                                                                             n, rows);
+                                                                                             n, rows, cols);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -415,7 +415,7 @@ cudaError_t gs_combine(const T *base, long stride, int m, const double *c, T *x,
     template cudaError_t gs_subtract<T>(const T *, long, int, const double *, long, const double *, T *, T *, long,    \
                                         const RowList &, cudaStream_t);                                               \
     template cudaError_t gs_combine<T>(const T *, long, int, const double *, T *, bool, long, const RowList &,         \
-                                       cudaStream_t);
+                                       const RowColumns &, cudaStream_t);
 OVL_GS(float)
 OVL_GS(double)
 #undef OVL_GS

@@ -166,10 +166,15 @@ cudaError_t gs_dots(const T *base, long stride, int m, const T *w, long n, const
 template <typename T>
 cudaError_t gs_subtract(const T *base, long stride, int m, const double *h, long ostride, const double *prev, T *w,
                         T *next, long n, const RowList &rows, cudaStream_t st);
-// x (+)= sum_i c_i v_i, complex coefficients of row k at c + 2 * m * k (device); add = false: assigned
+// x (+)= sum_i c_i v_i, i < cols.n[k] <= m for row k, its complex coefficients at c + 2 * m * k (device);
+// add = false: assigned. Entries past a row's own columns are not read: its solver may never have
+// written them, and a zero coefficient would turn a NaN there into a NaN in x.
+struct RowColumns {
+    int n[12];
+};
 template <typename T>
 cudaError_t gs_combine(const T *base, long stride, int m, const double *c, T *x, bool add, long n, const RowList &rows,
-                       cudaStream_t st);
+                       const RowColumns &cols, cudaStream_t st);
 cudaError_t dev_multiaxpy_f(const float *base, long stride, int m, const double *c, float *w, long n,
                             cudaStream_t st);
 // x[k] = seeded pseudo-random values in [-1, 1) (a counter hash of k and the seed)

@@ -142,21 +142,23 @@ static ovl_status gs_arnoldi(Ctx *c, T *V, long stride, int m, T *w, const RowLi
     return OVL_OK;
 }
 
-// x (+)= sum_i y_i Z_i for the rows (coefficients y[r], padded with zeros to the longest). The pinned
+// x (+)= sum_i y_i Z_i for the rows (row r: coefficients y[r], i < y[r].size()). The pinned
 // staging is free: a fetch has waited for the stream since the last call.
 template <typename T>
 static ovl_status gs_solution(Ctx *c, const T *Z, long stride, const std::vector<std::vector<cd>> &y, T *x, bool add,
                               const RowList &rows) {
     size_t m = 0;
+    RowColumns cols{};
     for (auto &v : y) m = std::max(m, v.size());
-    for (int r = 0; r < rows.n; r++)
-        for (size_t i = 0; i < m; i++) {
-            const cd v = i < y[r].size() ? y[r][i] : cd(0);
-            c->h_gs_coef[2 * (m * r + i)] = v.real();
-            c->h_gs_coef[2 * (m * r + i) + 1] = v.imag();
+    for (int r = 0; r < rows.n; r++) {
+        cols.n[r] = (int)y[r].size();
+        for (size_t i = 0; i < y[r].size(); i++) {
+            c->h_gs_coef[2 * (m * r + i)] = y[r][i].real();
+            c->h_gs_coef[2 * (m * r + i) + 1] = y[r][i].imag();
         }
+    }
     CK(cudaMemcpyAsync(c->d_gs_coef, c->h_gs_coef, 2 * m * rows.n * sizeof(double), cudaMemcpyHostToDevice, c->stream));
-    CK(gs_combine<T>(Z, stride, (int)m, c->d_gs_coef, x, add, c->n64, rows, c->stream));
+    CK(gs_combine<T>(Z, stride, (int)m, c->d_gs_coef, x, add, c->n64, rows, cols, c->stream));
     return OVL_OK;
 }
 

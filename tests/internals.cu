@@ -42,3 +42,15 @@ extern "C" int t_ms_init(int nrhs, long words, const void *b, const int *skip, i
     delete[] h;
     return st;
 }
+
+// x (+)= sum_i c_i v_i of n_rows right-hand sides with cols[y] of m columns each (FP64, gs_combine)
+extern "C" int t_gs_combine_f64(const double *base, long stride, int m, const double *c, const int *cols, double *x, int add,
+                                long n, int n_rows) {
+    RowList rows{n_rows, {}};
+    RowColumns rc{};
+    for (int y = 0; y < n_rows; y++) {
+        rows.row[y] = y;
+        rc.n[y] = cols[y];
+    }
+    return done(gs_combine<double>(base, stride, m, c, x, add != 0, n, rows, rc, 0));
+}
