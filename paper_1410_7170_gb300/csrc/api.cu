@@ -216,11 +216,25 @@ template <> long spinor_words<float4>(const Geom &g) { return 6L * g.V; }
 ovl_status Ctx::check_finite() {
     Ctx *c = this;
     ST(sync());
-    if (!*(volatile int *)h_flag) return OVL_OK;
-    *h_flag = 0;
-    CK(cudaMemsetAsync(d_flag, 0, sizeof(int), stream));
-    err = "input vector holds NaN or Inf";
-    return OVL_EINVAL;
+    if (*(volatile int *)h_flag) {
+        *h_flag = 0;
+        CK(cudaMemsetAsync(d_flag, 0, sizeof(int), stream));
+        unchecked = false;
+        err = "input vector holds NaN or Inf";
+        return OVL_EINVAL;
+    }
+    unchecked = false;
+    return OVL_OK;
+}
+void Ctx::open_call() {
+    if (unchecked) check_finite();
+}
+ovl_status Ctx::close_failed(ovl_status st) {
+    if (st == OVL_OK || !unchecked) return st;
+    const std::string why = err;
+    if (check_finite() == OVL_EINVAL) return OVL_EINVAL;
+    err = why;
+    return st;
 }
 
 // Boundary vectors (host or device, lexicographic, back to back) into internal even-odd spinors.
@@ -229,6 +243,7 @@ ovl_status Ctx::import_vec(const double *src, ST *dst, int n, bool check) {
     Ctx *c = this;
     const long w = spinor_words<ST>(g);
     const InputFlags bad{d_flag, h_flag};
+    unchecked = true;
     if (is_device_ptr(src)) {
         CK(spinor_in(g, dst, w, src, n, bad, stream));
     } else {
@@ -1333,6 +1348,7 @@ static ovl_status check_ctx_ptrs(Ctx *c, const void *a, const void *b) {
         c->err = "NULL vector argument";
         return OVL_EINVAL;
     }
+    c->open_call();
     return OVL_OK;
 }
 
@@ -1574,12 +1590,12 @@ extern "C" ovl_status wilson_sap_apply(ovl_ctx *ctx, double *out, const double *
     const bool late = on_device(in, out);
     if (c->p.precision == OVL_FP64) {
         ST(c->import_vec(in, c->io_a, 1, !late));
-        ST(sap_apply_eo(c, c->io_a, c->io_b, m0));
+        ST(c->close_failed(sap_apply_eo(c, c->io_a, c->io_b, m0)));
         return c->export_vec(c->io_b, out, 1, late);
     }
     ST(ensure_f32_buffers(c));
     ST(c->import_vec(in, (float4 *)c->f_a, 1, !late));
-    ST(sap_apply_eo(c, (const float4 *)c->f_a, (float4 *)c->f_b, m0));
+    ST(c->close_failed(sap_apply_eo(c, (const float4 *)c->f_a, (float4 *)c->f_b, m0)));
     return c->export_vec((const float4 *)c->f_b, out, 1, late);
 }
 

@@ -299,6 +299,7 @@ extern "C" ovl_status ovl_mg_setup(ovl_ctx *ctx, double m0, const double *start,
         c->err = "ovl_mg_setup: need finite m0 and n_start >= 1 with start vectors";
         return OVL_EINVAL;
     }
+    c->open_call();
     return mg_setup(c, m0, start, n_start);
 }
 
@@ -309,6 +310,7 @@ extern "C" ovl_status wilson_mg_apply(ovl_ctx *ctx, double *out, const double *i
         c->err = "wilson_mg_apply: NULL vector or non-finite m0";
         return OVL_EINVAL;
     }
+    c->open_call();
     ST(mg_check(c, c->mg.ready ? c->mg.nv : c->p.mg_nv));
     ST(ensure_f32_buffers(c));
     ST(c->import_vec(in, (float4 *)c->f_a));

@@ -209,6 +209,13 @@ struct Ctx {
     template <typename ST>
     ovl_status export_vec(const ST *src, double *dst, int n = 1, bool gate = false);
     ovl_status check_finite();
+    // The flags that an import leaves belong to its call: one that ends before its check (no memory, a
+    // failed launch) must not make the next call refuse its input. open_call, first in every call that
+    // imports, drops what an earlier one left; close_failed(st) makes the check that a call failing with
+    // st has not come to, so that bad input is reported before anything else.
+    bool unchecked = false;
+    void open_call();
+    ovl_status close_failed(ovl_status st);
     int pick_poles(double tol) const;
     void fill_poles(MsState &s, int n, double tol) const;
     ovl_status ms_setup(MsState *d_state, double tol, int *n_out);
