@@ -4,6 +4,7 @@
 // finalisation functor on thread 0. The summation order depends only on the launch
 // shape, so repeated runs give bit-identical results.
 #pragma once
+#include "ff.cuh"
 #include "internal.h"
 
 namespace ovl {
@@ -111,6 +112,20 @@ __device__ __forceinline__ void block_sum(const ff vf[NV], double v[NV]) {
         warp_sum<NV, kBlockWarps>(v);
     }
 }
+// A thread's sum of many FP32 terms without the growth of its rounding error: a running sum and the
+// exact errors of its additions (TwoSum), rounded once at the end or handed on as float-float. Six FP32
+// additions for each of add's, in kernels that wait for memory.
+struct fsum {
+    float s, e;
+    __device__ __forceinline__ fsum() : s(0.f), e(0.f) {}
+    __device__ __forceinline__ void add(float x) {
+        const ff t = ff_two_sum(s, x);
+        s = t.hi;
+        e = __fadd_rn(e, t.lo);
+    }
+    __device__ __forceinline__ ff value() const { return ff_fast_two_sum(s, e); }
+};
+
 // Reduce v[NV] (per-thread FP64 or FP32 partial sums) over the grid; the last block calls
 // fin(total, fin.before()) on thread 0 and resets the counter. Must be reached by every thread of
 // every block.

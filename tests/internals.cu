@@ -54,3 +54,11 @@ extern "C" int t_gs_combine_f64(const double *base, long stride, int m, const do
     }
     return done(gs_combine<double>(base, stride, m, c, x, add != 0, n, rows, rc, 0));
 }
+
+// gs_dots of n_rows right-hand sides, all of them; out: n_rows records of gs_record(m) doubles
+extern "C" int t_gs_dots_f32(const float *base, long stride, int m, const float *w, long n, int n_rows, double *out,
+                             double *partials, unsigned *counters) {
+    RowList rows{n_rows, {}};
+    for (int y = 0; y < n_rows; y++) rows.row[y] = y;
+    return done(gs_dots<float>(base, stride, m, w, n, rows, out, gs_record(m), false, nullptr, partials, counters, 0));
+}
