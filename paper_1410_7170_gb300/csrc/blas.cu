@@ -143,12 +143,12 @@ template <> struct GsWord<double> {
 };
 template <> struct GsWord<float> {
     using W = float4;
-    using Part = ff;
+    using Part = fsum;
     struct Sum {
         fsum s;
         __device__ float open() const { return 0.f; }
         __device__ void close(float x) { s.add(x); }
-        __device__ Part value() const { return s.value(); }
+        __device__ Part value() const { return s; }
     };
     __device__ static void dot(W v, W w, float &a, float &b) {
         a += v.x * w.x + v.y * w.y + v.z * w.z + v.w * w.w;
@@ -180,7 +180,7 @@ __global__ void __launch_bounds__(kBlock) k_gs_dots(const T *__restrict__ base, 
     const W *x = reinterpret_cast<const W *>(w + off);
     const W *v = i < m ? reinterpret_cast<const W *>(base + (long)i * stride + off) : x;
     // Four words of each vector in flight per thread: the grid is small (gs_grid). In FP32 a plain sum
-    // never runs over more than four words (16 products); the groups are added without rounding error
+    // never runs over more than four words (16 products); the groups are added with their errors (fsum),
     // and so are the threads. The kernel has 2 blocks per SM over all vectors, so that with one FP32 sum
     // per thread the relative error of ||w||^2 at 32^4 was 1e-8 at 32 vectors and 4e-8 at 75 (chains of
     // 5800 products and more): 1e-10 now, at the same time (DRAM and latency bound).

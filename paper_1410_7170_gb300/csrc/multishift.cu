@@ -189,7 +189,7 @@ __global__ void __launch_bounds__(kBlock, MinBlocks<float>::value)
     if (s->done) return;
     const float4 *__restrict__ p0 = v.p0_at(blockIdx.y, s->iter);
     float4 *__restrict__ t = v.t + blockIdx.y * v.stride;
-    float sum[1] = {0.f};   // per-thread sums in FP32, FP64 from the warp sums on (grid_reduce)
+    fsum sum;   // a site's sum in FP32, a thread's and a warp's with their errors, then FP64 (grid_reduce)
     const bool lane_has_sites = threadIdx.x < spb;
     for (int k = blockIdx.x * spb + threadIdx.x; lane_has_sites && k < g.V; k += gridDim.x * spb) {
         int p, i;
@@ -203,9 +203,10 @@ __global__ void __launch_bounds__(kBlock, MinBlocks<float>::value)
         float a0 = 0.f;
 #pragma unroll
         for (int c = 0; c < 12; c++) a0 += norm2(res[c]);
-        sum[0] += a0;
+        sum.add(a0);
     }
-    grid_reduce<1>(sum, rs.row(blockIdx.y), AlphaFin{s});
+    const fsum w[1] = {sum};
+    grid_reduce<1>(w, rs.row(blockIdx.y), AlphaFin{s});
 }
 
 // r_{k+1} = r_k - alpha (gamma5 D_W(m) t + sigma0 p0) ; ||r_{k+1}||^2 -> shift scalars. Block 0 takes no
@@ -214,7 +215,7 @@ __global__ void __launch_bounds__(kBlock, MinBlocks<float>::value)
     k_ms_r_site(Geom g, const float4 *__restrict__ U, float m4, MsState *st, MsBatch<float4> v, RedScratch rs, int spb) {
     MsState *s = st + blockIdx.y;
     if (s->done) return;
-    float sum[1] = {0.f};
+    fsum sum;
     if (blockIdx.x == 0) {
         if (threadIdx.x < 32) ShiftScalars{s}(threadIdx.x);
     } else {
@@ -241,11 +242,12 @@ __global__ void __launch_bounds__(kBlock, MinBlocks<float>::value)
                 rv[c] = rv[c] + ma * (res[c] + sig0 * pp[c]);
                 a0 += norm2(rv[c]);
             }
-            sum[0] += a0;
+            sum.add(a0);
             store_spinor<float>(rout, g.Vh, p, i, rv);
         }
     }
-    grid_reduce_warp<1>(sum, rs.row(blockIdx.y), ShiftFin{s});
+    const fsum w[1] = {sum};
+    grid_reduce_warp<1>(w, rs.row(blockIdx.y), ShiftFin{s});
 }
 
 // Elementwise arithmetic on storage words: V is a word in registers, C a real coefficient in the
@@ -255,30 +257,33 @@ template <> struct Word<double2> {
     using V = double2;
     using C = double;
     using Sum = double;
+    __device__ static void add(Sum &s, double x) { s += x; }
     __device__ static V get(const double2 &w) { return w; }
     __device__ static double2 put(const V &v) { return v; }
     __device__ static C coef(double a, const float *) { return a; }
     __device__ static V fma(C a, const V &b, const V &c) {
         return make_double2(fma_r(a, b.x, c.x), fma_r(a, b.y, c.y));
     }
-    __device__ static Sum norm2(const V &v) { return v.x * v.x + v.y * v.y; }
+    __device__ static double norm2(const V &v) { return v.x * v.x + v.y * v.y; }
 };
 template <> struct Word<float4> {
     using V = float4;
     using C = float;
-    using Sum = float;
+    using Sum = fsum;
+    __device__ static void add(Sum &s, float x) { s.add(x); }
     __device__ static V get(const float4 &w) { return w; }
     __device__ static float4 put(const V &v) { return v; }
     __device__ static C coef(double, const float *f) { return f[0]; }
     __device__ static V fma(C a, const V &b, const V &c) {
         return make_float4(fma_r(a, b.x, c.x), fma_r(a, b.y, c.y), fma_r(a, b.z, c.z), fma_r(a, b.w, c.w));
     }
-    __device__ static Sum norm2(const V &v) { return v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w; }
+    __device__ static float norm2(const V &v) { return v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w; }
 };
 template <> struct Word<ffw> {
     using V = ff2;
     using C = ff2_factor;
     using Sum = ff;
+    __device__ static void add(Sum &s, ff x) { s += x; }
     __device__ static V get(const ffw &w) { return ff2_load(reinterpret_cast<const float4 &>(w)); }
     __device__ static ffw put(const V &v) {
         const float4 w = ff2_word(v);
@@ -286,7 +291,7 @@ template <> struct Word<ffw> {
     }
     __device__ static C coef(double, const float *f) { return ff2_scale(f[0], f[1]); }
     __device__ static V fma(const C &a, const V &b, const V &c) { return ff2_fma(a, b, c); }
-    __device__ static Sum norm2(const V &v) {
+    __device__ static ff norm2(const V &v) {
         return HopTiles<ff>::total(ff2_square_add(v, HopTiles<ff>::zero()));
     }
 };
@@ -419,7 +424,7 @@ __global__ void __launch_bounds__(kHopBlock, HopBlocks<R>::value)
         H::store(t, g.Vh, p, i, it, e, w);
         H::square_add(w, sum);
     });
-    const R w[1] = {H::total(sum)};
+    const decltype(H::total(sum)) w[1] = {H::total(sum)};
     grid_reduce<1>(w, rs.row(blockIdx.y), AlphaFin{s});
 }
 
@@ -453,7 +458,7 @@ __global__ void __launch_bounds__(kHopBlock, HopBlocks<R>::value)
         H::store(rout, g.Vh, p, i, it, e, w);
         H::square_add(w, sum);
     });
-    const R w[1] = {H::total(sum)};
+    const decltype(H::total(sum)) w[1] = {H::total(sum)};
     grid_reduce_warp<1>(w, rs.row(blockIdx.y), ShiftFin{s});
 }
 
@@ -497,16 +502,17 @@ __global__ void k_ms_init(MsState *st, const ST *__restrict__ b, MsBatch<ST> v, 
     ST *r = v.r_at(blockIdx.y, 0), *p0 = v.p0_at(blockIdx.y, 0), *y = v.y + blockIdx.y * v.stride;
     ST *P = v.p + blockIdx.y * v.prow;
     const int n = s->n;
-    typename W::Sum sum[1] = {typename W::Sum(0)};
+    typename W::Sum sum{};
     for (long k = (long)blockIdx.x * blockDim.x + threadIdx.x; k < v.stride; k += (long)gridDim.x * blockDim.x) {
         const ST w = b[k];
         r[k] = w;
         y[k] = w;
         p0[k] = w;
         for (int l = 1; l < n; l++) P[(l - 1) * v.stride + k] = w;
-        sum[0] += W::norm2(W::get(w));
+        W::add(sum, W::norm2(W::get(w)));
     }
-    grid_reduce<1>(sum, rs.row(blockIdx.y), InitFin{s});
+    const typename W::Sum total[1] = {sum};
+    grid_reduce<1>(total, rs.row(blockIdx.y), InitFin{s});
 }
 
 inline int stream_grid(long n) {

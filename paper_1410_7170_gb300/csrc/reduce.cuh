@@ -86,6 +86,55 @@ __device__ __forceinline__ void block_sum(const float vf[NV], double v[NV]) {
         warp_sum<NV, kBlockWarps>(v);
     }
 }
+// A sum of many FP32 terms without the growth of its rounding error: the running sum and the errors of
+// its additions (TwoSum), which are exact. Where one wave of blocks takes the whole lattice a thread
+// adds thousands of terms and a row of the grid has few warps; with plain FP32 sums in threads and
+// warps the relative error of a squared norm at 32^4 had grown tenfold against one site per thread, with
+// these it is that of the terms. Six FP32 additions for one, in kernels that wait for memory, and about
+// 100 clocks more for the shuffles at their ends.
+struct fsum {
+    float s = 0.f, e = 0.f;
+    __device__ __forceinline__ void add(float x) {
+        const ff t = ff_two_sum(s, x);
+        s = t.hi;
+        e = __fadd_rn(e, t.lo);
+    }
+    __device__ __forceinline__ void add(const fsum &x) {
+        const ff t = ff_two_sum(s, x.s);
+        s = t.hi;
+        e = __fadd_rn(__fadd_rn(e, x.e), t.lo);
+    }
+};
+// Block-wide sum of per-thread sums of this kind, blockDim.x <= kBlock: the warp stage in FP32 with its
+// errors, the sum over warps in FP64 by the first warp.
+template <int NV>
+__device__ __forceinline__ void block_sum(const fsum vf[NV], double v[NV]) {
+    __shared__ double sm[NV][kBlockWarps];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int nw = (blockDim.x + 31) >> 5;
+    fsum t[NV];
+#pragma unroll
+    for (int k = 0; k < NV; k++) {
+        t[k] = vf[k];
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+            fsum o;
+            o.s = __shfl_down_sync(0xffffffffu, t[k].s, off);
+            o.e = __shfl_down_sync(0xffffffffu, t[k].e, off);
+            t[k].add(o);
+        }
+    }
+    __syncthreads();   // protect sm from a previous use in the same kernel
+    if (lane == 0)
+#pragma unroll
+        for (int k = 0; k < NV; k++) sm[k][warp] = (double)t[k].s + (double)t[k].e;
+    __syncthreads();
+    if (warp == 0) {
+#pragma unroll
+        for (int k = 0; k < NV; k++) v[k] = lane < nw ? sm[k][lane & (kBlockWarps - 1)] : 0.0;
+        warp_sum<NV, kBlockWarps>(v);
+    }
+}
 // Block-wide sum of per-thread float-float values, blockDim.x <= kBlock: the warp stage in float-float (both
 // words shuffled), the sum over warps in FP64 by the first warp.
 template <int NV>
@@ -112,21 +161,7 @@ __device__ __forceinline__ void block_sum(const ff vf[NV], double v[NV]) {
         warp_sum<NV, kBlockWarps>(v);
     }
 }
-// A thread's sum of many FP32 terms without the growth of its rounding error: a running sum and the
-// exact errors of its additions (TwoSum), rounded once at the end or handed on as float-float. Six FP32
-// additions for each of add's, in kernels that wait for memory.
-struct fsum {
-    float s, e;
-    __device__ __forceinline__ fsum() : s(0.f), e(0.f) {}
-    __device__ __forceinline__ void add(float x) {
-        const ff t = ff_two_sum(s, x);
-        s = t.hi;
-        e = __fadd_rn(e, t.lo);
-    }
-    __device__ __forceinline__ ff value() const { return ff_fast_two_sum(s, e); }
-};
-
-// Reduce v[NV] (per-thread FP64 or FP32 partial sums) over the grid; the last block calls
+// Reduce v[NV] (per-thread FP64, FP32, fsum or float-float partial sums) over the grid; the last block calls
 // fin(total, fin.before()) on thread 0 and resets the counter. Must be reached by every thread of
 // every block.
 template <int NV, typename T, typename Fin>

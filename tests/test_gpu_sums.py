@@ -59,3 +59,39 @@ def test_gram_schmidt_dots_f32(lib, sites, m, rows):
             h = torch.vdot(torch.view_as_complex(vd.view(-1, 2)), wc)
             err = abs(complex(out[y, 2 * i].item(), out[y, 2 * i + 1].item()) - h.item())
             assert err < tol * (ww.sqrt() * vd.norm()).item()
+
+
+def multishift(lib, dims, dtype, tps, rows, ring, iters, seed):
+    """ms_probe on random links: (scalars [rows][5], t, r, p_0 as [rows][24 V])."""
+    V = dims[0] * dims[1] * dims[2] * dims[3]
+    gen = torch.Generator("cuda")
+    gen.manual_seed(seed)
+    u = torch.linalg.qr(torch.complex(*torch.randn((2, 4096, 4, 3, 3), dtype=torch.float64, device="cuda", generator=gen)))[0]
+    u = u / torch.linalg.det(u).pow(1 / 3)[..., None, None]
+    u = u[torch.randint(0, 4096, (V,), device="cuda", generator=gen)].contiguous()
+    b = torch.randn((rows, 24 * V), dtype=dtype, device="cuda", generator=gen)
+    t, r, p = torch.zeros_like(b), torch.zeros_like(b), torch.zeros_like(b)
+    scal = (ctypes.c_double * (5 * rows))()
+    torch.cuda.synchronize()
+    assert lib.t_ms_probe((ctypes.c_int * 4)(*dims), P(u), int(dtype == torch.float64), tps, rows, ring, P(b), iters, scal,
+                          P(t), P(r), P(p)) == 0
+    return torch.tensor(list(scal), dtype=torch.float64).view(rows, 5), b, t, r, p
+
+
+def squares(x):
+    return torch.stack([v.double().square().sum() for v in x]).cpu()
+
+
+@pytest.mark.parametrize("dims,tps,rows", [((32, 32, 32, 32), 1, 1), ((32, 32, 32, 32), 1, 12), ((32, 32, 32, 32), 4, 3),
+                                           ((16, 16, 16, 16), 1, 12), ((6, 4, 10, 8), 1, 5), ((6, 4, 10, 8), 4, 5)])
+def test_multishift_sums_f32(lib, dims, tps, rows):
+    """||b||^2, ||Q p_0||^2 (from alpha) and ||r_1||^2 of one iteration. One plain FP32 sum runs over a site's
+    24 products (four in ||b||^2)."""
+    scal, b, t, r, _ = multishift(lib, dims, torch.float32, tps, rows, 2, 1, 31)
+    n = b.shape[1]
+    assert bool((scal[:, 4] == 0).all())
+    bb = squares(b)
+    assert (scal[:, 0] / bb - 1).abs().max() < bar(4, n)
+    assert (scal[:, 1] / squares(r) - 1).abs().max() < bar(24, n)
+    tt = scal[:, 0] / scal[:, 3] - 0.01 * scal[:, 0]
+    assert (tt / squares(t) - 1).abs().max() < bar(24, n) + 0.01 * bar(4, n)
