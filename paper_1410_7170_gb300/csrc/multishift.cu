@@ -41,6 +41,7 @@
 #include <math.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "hops.cuh"
 #include "internal.h"
@@ -60,9 +61,12 @@ __device__ __forceinline__ void store_ff(float *to, double x) {
     to[1] = f.lo;
 }
 
-// alpha = (r, r) / (p, (Q^2 + sigma_0) p) with (p, Q^2 p) = ||Q p||^2 (v[0], reduced by ms_q)
-// and ||p||^2 from the scalar recurrence ||p_k||^2 = ||r_k||^2 + beta^2 ||p_{k-1}||^2, which
-// holds because r_k is orthogonal to p_{k-1} in CG; this spares ms_q a second reduction.
+// alpha = (r, r) / (p, (Q^2 + sigma_0) p) with (p, Q^2 p) = ||Q p||^2 (v[0], reduced by ms_q). ||p||^2 of one
+// right-hand side comes from the scalar recurrence ||p_k||^2 = ||r_k||^2 + beta^2 ||p_{k-1}||^2, which
+// holds because r_k is orthogonal to p_{k-1} in CG; this spares ms_q a second reduction. Batches (OWN)
+// reduce it too, v[1]: in FP32 the recurrence drifts to 5e-7 in 40 iterations (16^4), the sum is good to
+// 1e-9. Float-float batches use the recurrence, as one right-hand side does.
+template <bool OWN>
 struct AlphaFin {
     MsState *s;
     struct In {
@@ -70,7 +74,8 @@ struct AlphaFin {
     };
     __device__ In before() const { return {s->sigma[0], s->pp, s->rr}; }
     __device__ void operator()(const double *v, const In &in) const {
-        const double pAp = v[0] + in.sigma0 * in.pp;
+        const double pp = OWN ? v[OWN] : in.pp;
+        const double pAp = v[0] + in.sigma0 * pp;
         const double a = in.rr / pAp;
         if (!(pAp > 0.0) || !isfinite(a)) {
             s->status = 1;
@@ -79,6 +84,7 @@ struct AlphaFin {
         }
         s->alpha = a;
         store_ff(s->alpha_f, a);
+        if (OWN) s->pp = pp;
     }
 };
 
@@ -182,14 +188,16 @@ struct ShiftFin {
     }
 };
 
-// One thread per site (FP32), right-hand side blockIdx.y: t = gamma5 D_W(m) p_0 ; ||t||^2 -> alpha.
+// One thread per site (FP32), right-hand side blockIdx.y: t = gamma5 D_W(m) p_0 ; ||t||^2 (OWN: and
+// ||p_0||^2) -> alpha.
+template <bool OWN>
 __global__ void __launch_bounds__(kBlock, MinBlocks<float>::value)
     k_ms_q_site(Geom g, const float4 *__restrict__ U, float m4, MsState *st, MsBatch<float4> v, RedScratch rs, int spb) {
     MsState *s = st + blockIdx.y;
     if (s->done) return;
     const float4 *__restrict__ p0 = v.p0_at(blockIdx.y, s->iter);
     float4 *__restrict__ t = v.t + blockIdx.y * v.stride;
-    fsum sum;   // a site's sum in FP32, a thread's and a warp's with their errors, then FP64 (grid_reduce)
+    fsum sum[1 + OWN];   // a site's sum in FP32, a thread's and a warp's with their errors, then FP64 (grid_reduce)
     const bool lane_has_sites = threadIdx.x < spb;
     for (int k = blockIdx.x * spb + threadIdx.x; lane_has_sites && k < g.V; k += gridDim.x * spb) {
         int p, i;
@@ -203,10 +211,15 @@ __global__ void __launch_bounds__(kBlock, MinBlocks<float>::value)
         float a0 = 0.f;
 #pragma unroll
         for (int c = 0; c < 12; c++) a0 += norm2(res[c]);
-        sum.add(a0);
+        sum[0].add(a0);
+        if (OWN) {
+            a0 = 0.f;
+#pragma unroll
+            for (int c = 0; c < 12; c++) a0 += norm2(own[c]);
+            sum[OWN].add(a0);
+        }
     }
-    const fsum w[1] = {sum};
-    grid_reduce<1>(w, rs.row(blockIdx.y), AlphaFin{s});
+    grid_reduce<1 + OWN>(sum, rs.row(blockIdx.y), AlphaFin<OWN>{s});
 }
 
 // r_{k+1} = r_k - alpha (gamma5 D_W(m) t + sigma0 p0) ; ||r_{k+1}||^2 -> shift scalars. Block 0 takes no
@@ -405,7 +418,7 @@ __global__ void __launch_bounds__(kBlock, kShiftBlocks) k_ms_shifts(MsState *st,
 }
 
 // The same with one warp per hop (hops.cuh).
-template <typename R>
+template <typename R, bool OWN>
 __global__ void __launch_bounds__(kHopBlock, HopBlocks<R>::value)
     k_ms_q_hops(Geom g, const typename HopTiles<R>::Link *__restrict__ U, R m4, MsState *st,
                 MsBatch<typename HopTiles<R>::Store> v, RedScratch rs) {
@@ -415,7 +428,7 @@ __global__ void __launch_bounds__(kHopBlock, HopBlocks<R>::value)
     if (s->done) return;
     const typename H::Store *__restrict__ p0 = v.p0_at(blockIdx.y, s->iter);
     typename H::Store *__restrict__ t = v.t + blockIdx.y * v.stride;
-    typename H::Sum sum = H::zero();
+    typename H::Sum sum = H::zero(), psum = H::zero();
     const auto fm = H::factor(m4);
     const auto own = [&](int p, int i, int it, int e) { return H::load(p0, g.Vh, p, i, it, e); };
     hop_tiles<R>(g, blockIdx.x, gridDim.x, U, p0, own, [&](int p, int i, int it, int e, E hop, int, E o) {
@@ -423,9 +436,11 @@ __global__ void __launch_bounds__(kHopBlock, HopBlocks<R>::value)
         w = H::neg_if(w, H::upper(it));
         H::store(t, g.Vh, p, i, it, e, w);
         H::square_add(w, sum);
+        if (OWN) H::square_add(o, psum);
     });
-    const decltype(H::total(sum)) w[1] = {H::total(sum)};
-    grid_reduce<1>(w, rs.row(blockIdx.y), AlphaFin{s});
+    decltype(H::total(sum)) w[1 + OWN] = {H::total(sum)};
+    if (OWN) w[OWN] = H::total(psum);
+    grid_reduce<1 + OWN>(w, rs.row(blockIdx.y), AlphaFin<OWN>{s});
 }
 
 template <typename R>
@@ -623,7 +638,9 @@ cudaError_t ms_stencils_hops(const Geom &g, const LT *U, double m0, int nrhs, Ms
     const int gx = hop_grid<R>(g, nrhs, true);
     cudaError_t e;
     if ((e = ev.record(0, st)) != cudaSuccess) return e;
-    k_ms_q_hops<R><<<dim3(gx, nrhs), kHopBlock, 0, st>>>(g, U, R(m0 + 4.0), s, v, rows);
+    if (nrhs > 1 && !std::is_same<R, ff>::value)
+        k_ms_q_hops<R, !std::is_same<R, ff>::value><<<dim3(gx, nrhs), kHopBlock, 0, st>>>(g, U, R(m0 + 4.0), s, v, rows);
+    else k_ms_q_hops<R, false><<<dim3(gx, nrhs), kHopBlock, 0, st>>>(g, U, R(m0 + 4.0), s, v, rows);
     if ((e = ev.record(1, st)) != cudaSuccess) return e;
     // one block more for the shift scalars, within the wave
     const int gr = (long)gx * nrhs + nrhs > (long)g.nsm * HopBlocks<R>::value && gx > 1 ? gx : gx + 1;
@@ -641,7 +658,8 @@ cudaError_t ms_stencils_site(const Geom &g, const float4 *U, float m0, int nrhs,
     const LaunchShape r = balanced_shape(g.V, std::max(1, slots - 1), 1, std::max(1, slots - 1));
     cudaError_t e;
     if ((e = ev.record(0, st)) != cudaSuccess) return e;
-    k_ms_q_site<<<dim3(q.grid, nrhs), q.block, 0, st>>>(g, U, m0 + 4.f, s, v, rows, q.spb);
+    if (nrhs > 1) k_ms_q_site<true><<<dim3(q.grid, nrhs), q.block, 0, st>>>(g, U, m0 + 4.f, s, v, rows, q.spb);
+    else k_ms_q_site<false><<<dim3(q.grid, nrhs), q.block, 0, st>>>(g, U, m0 + 4.f, s, v, rows, q.spb);
     if ((e = ev.record(1, st)) != cudaSuccess) return e;
     k_ms_r_site<<<dim3(r.grid + 1, nrhs), r.block, 0, st>>>(g, U, m0 + 4.f, s, v, rows, r.spb);
     return ev.record(2, st);

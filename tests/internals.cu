@@ -72,12 +72,12 @@ extern "C" int t_gs_dots_f32(const float *base, long stride, int m, const float 
     return done(gs_dots<float>(base, stride, m, w, n, rows, out, gs_record(m), false, nullptr, partials, counters, 0));
 }
 
-// nrhs multishift solves with shifts 0.01 and 1, stopped after `iters` iterations: scal = 5 doubles per
+// nrhs multishift solves with shifts sigma0 and sigma0 + 1, stopped after `iters` iterations: scal = 5 doubles per
 // right-hand side (||b||^2, ||r||^2, ||p_0||^2 as the solver has it, alpha of the last iteration, status);
 // t, r, p0: the vectors' last values.
 template <typename ST, typename LT>
-static int ms_probe(const Geom &g, const LT *U, int nrhs, int ring, long words, const ST *b, int iters, double *scal, ST *t,
-                    ST *r, ST *p0) {
+static int ms_probe(const Geom &g, const LT *U, int nrhs, int ring, long words, const ST *b, int iters,
+                    double sigma0, double *scal, ST *t, ST *r, ST *p0) {
     const int n = 2;
     ST *d = nullptr;
     MsState *s = nullptr;
@@ -87,18 +87,18 @@ static int ms_probe(const Geom &g, const LT *U, int nrhs, int ring, long words, 
         h[y].n = n;
         h[y].tol = 1e-14;
         h[y].alpha_prev = 1.0;
-        h[y].sigma[0] = 0.01;
-        h[y].sigma[1] = 1.0;
-        h[y].sigma0_f[0] = (float)0.01;
-        h[y].sigma0_f[1] = (float)(0.01 - (double)(float)0.01);
+        h[y].sigma[0] = sigma0;
+        h[y].sigma[1] = sigma0 + 1.0;
+        h[y].sigma0_f[0] = (float)sigma0;
+        h[y].sigma0_f[1] = (float)(sigma0 - (double)(float)sigma0);
         for (int l = 0; l < n; l++) h[y].w[l] = h[y].crit[l] = h[y].zeta[l] = h[y].zeta_prev[l] = 1.0, h[y].active[l] = 1;
     }
     const long v = words * nrhs;
     cudaError_t e = cudaMalloc(&d, (size_t)v * ms_vectors(n, ring) * sizeof(ST));
     if (e == cudaSuccess) e = cudaMalloc(&s, sizeof(MsState) * nrhs);
-    if (e == cudaSuccess) e = cudaMalloc(&part, sizeof(double) * kMaxRedBlocks * nrhs + 256);
+    if (e == cudaSuccess) e = cudaMalloc(&part, sizeof(double) * kRowRedValues * kMaxRedBlocks * nrhs + 256);
     if (e == cudaSuccess) {
-        unsigned *cnt = (unsigned *)(part + (size_t)kMaxRedBlocks * nrhs);
+        unsigned *cnt = (unsigned *)(part + (size_t)kRowRedValues * kMaxRedBlocks * nrhs);
         const MsBatch<ST> w{d, d + v * ring, d + 2 * v * ring, d + (2 * ring + 1) * v, d + (2 * ring + 2) * v, words,
                             words * (n - 1), ring};
         cudaMemset(cnt, 0, 256);
@@ -124,7 +124,7 @@ static int ms_probe(const Geom &g, const LT *U, int nrhs, int ring, long words, 
     return st;
 }
 extern "C" int t_ms_probe(const int *dims, const double *gauge, int fp64, int tps32, int nrhs, int ring, const void *b, int iters,
-                          double *scal, void *t, void *r, void *p0) {
+                          double sigma0, double *scal, void *t, void *r, void *p0) {
     Geom g = geom(dims);
     g.tps32 = tps32;
     double2 *u64 = nullptr;
@@ -136,10 +136,10 @@ extern "C" int t_ms_probe(const int *dims, const double *gauge, int fp64, int tp
     if (e == cudaSuccess) e = pack_gauge(g, gauge, u64, u32, bad, 1e-10, 0);
     int st = done(e);
     if (!st && fp64)
-        st = ms_probe<double2>(g, u64, nrhs, ring, 12L * g.V, (const double2 *)b, iters, scal, (double2 *)t, (double2 *)r,
+        st = ms_probe<double2>(g, u64, nrhs, ring, 12L * g.V, (const double2 *)b, iters, sigma0, scal, (double2 *)t, (double2 *)r,
                                (double2 *)p0);
     else if (!st)
-        st = ms_probe<float4>(g, u32, nrhs, ring, 6L * g.V, (const float4 *)b, iters, scal, (float4 *)t, (float4 *)r,
+        st = ms_probe<float4>(g, u32, nrhs, ring, 6L * g.V, (const float4 *)b, iters, sigma0, scal, (float4 *)t, (float4 *)r,
                               (float4 *)p0);
     cudaFree(u64);
     cudaFree(u32);

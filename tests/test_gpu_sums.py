@@ -61,7 +61,7 @@ def test_gram_schmidt_dots_f32(lib, sites, m, rows):
             assert err < tol * (ww.sqrt() * vd.norm()).item()
 
 
-def multishift(lib, dims, dtype, tps, rows, ring, iters, seed):
+def multishift(lib, dims, dtype, tps, rows, ring, iters, seed, sigma0=0.01):
     """ms_probe on random links: (scalars [rows][5], t, r, p_0 as [rows][24 V])."""
     V = dims[0] * dims[1] * dims[2] * dims[3]
     gen = torch.Generator("cuda")
@@ -73,8 +73,8 @@ def multishift(lib, dims, dtype, tps, rows, ring, iters, seed):
     t, r, p = torch.zeros_like(b), torch.zeros_like(b), torch.zeros_like(b)
     scal = (ctypes.c_double * (5 * rows))()
     torch.cuda.synchronize()
-    assert lib.t_ms_probe((ctypes.c_int * 4)(*dims), P(u), int(dtype == torch.float64), tps, rows, ring, P(b), iters, scal,
-                          P(t), P(r), P(p)) == 0
+    assert lib.t_ms_probe((ctypes.c_int * 4)(*dims), P(u), int(dtype == torch.float64), tps, rows, ring, P(b), iters,
+                          ctypes.c_double(sigma0), scal, P(t), P(r), P(p)) == 0
     return torch.tensor(list(scal), dtype=torch.float64).view(rows, 5), b, t, r, p
 
 
@@ -95,3 +95,17 @@ def test_multishift_sums_f32(lib, dims, tps, rows):
     assert (scal[:, 1] / squares(r) - 1).abs().max() < bar(24, n)
     tt = scal[:, 0] / scal[:, 3] - 0.01 * scal[:, 0]
     assert (tt / squares(t) - 1).abs().max() < bar(24, n) + 0.01 * bar(4, n)
+
+
+@pytest.mark.parametrize("dtype,tps", [(torch.float32, 1), (torch.float32, 4), (torch.float64, 1)])
+@pytest.mark.parametrize("dims,rows", [((16, 16, 16, 16), 3), ((6, 4, 10, 8), 12)])
+def test_direction_norm_of_a_batch(lib, dtype, tps, dims, rows):
+    """||p_0||^2 in alpha of a later iteration of several right-hand sides, with a shift as large as Q^2: it is
+    summed from the vector, not carried from iteration to iteration."""
+    k, sigma0 = 6, 16.0
+    before, b, _, _, p = multishift(lib, dims, dtype, tps, rows, 2, k, 41, sigma0)
+    after, _, t, _, _ = multishift(lib, dims, dtype, tps, rows, 2, k + 1, 41, sigma0)
+    tt, pp = squares(t), squares(p)
+    got = (before[:, 1] / after[:, 3] - tt) / sigma0
+    eps = bar(24, b.shape[1]) if dtype == torch.float32 else 1e-14
+    assert ((got / pp - 1).abs() < eps * (1 + tt / (sigma0 * pp))).all()
