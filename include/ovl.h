@@ -489,7 +489,10 @@ typedef struct {
 ovl_status ovl_server_create(ovl_server **srv, int slots, size_t hbm_budget);
 /* Host only (no device call): the device memory the server reserves for req at admission,
  * an upper estimate of what ovl_create and ovl_solve allocate for its lattice, precision,
- * preconditioner, sign method, deflation and right-hand sides (params NULL = defaults).
+ * preconditioner, sign method, deflation and right-hand sides (params NULL = defaults), with
+ * all the multishift vectors that it would like to use. A request that does not fit the budget
+ * with these is admitted with fewer, down to n_poles + 3 per arithmetic and right-hand side
+ * (slower), before it is refused.
  * OVL_EINVAL for NULL pointers, n_rhs < 1 or a non-positive extent. */
 ovl_status ovl_request_bytes(const ovl_request *req, size_t *bytes);
 /* Queues a request and returns its ticket. The buffers it points to (gauge, b, x) must stay

@@ -554,7 +554,7 @@ ovl_status Ctx::ensure_msff() {
         ST(alloc(&buf, sizeof(MsState)));
         msff_state = (MsState *)buf;
     }
-    return alloc_ms(msff, 1, kMaxRing);
+    return alloc_ms(msff, 1, ring_one);
 }
 
 ovl_status Ctx::sign_outer(const double2 *b, double2 *out, double tol, int mode) {
@@ -612,7 +612,7 @@ ovl_status Ctx::sign32(const float4 *b, float4 *out, double tol, int mode, int s
     return ms;
 }
 
-ovl_status Ctx::ensure_ms64() { return ms64.r ? OVL_OK : alloc_ms(ms64, 1, kMaxRing); }
+ovl_status Ctx::ensure_ms64() { return ms64.r ? OVL_OK : alloc_ms(ms64, 1, ring_one); }
 // ---- several right-hand sides
 ovl_status Ctx::ensure_batch() {
     Ctx *c = this;
@@ -636,18 +636,21 @@ ovl_status Ctx::ensure_batch() {
 // Multishift vectors for nrhs right-hand sides, one allocation that starts at v.r.
 template <typename W>
 ovl_status Ctx::alloc_ms(MsBatch<W> &v, int nrhs, int ring) {
-    const long words = spinor_words<W>(g);
+    const long words = spinor_words<W>(g), n = words * nrhs;
     void *buf;
-    ST(alloc(&buf, (size_t)words * sizeof(W) * nrhs * ms_vectors(npole, ring)));
+    ovl_status st;
+    while ((st = alloc(&buf, (size_t)n * sizeof(W) * ms_vectors(npole, ring))) == OVL_ENOMEM && ring > 1 && !fixed_rings) {
+        ring /= 2;
+        rings_reduced = true;
+    }
+    if (st != OVL_OK) return st;
     W *d = (W *)buf;
-    const long n = words * nrhs;
     v = MsBatch<W>{d, d + n * ring, d + 2 * n * ring, d + (2 * ring + 1) * n, d + (2 * ring + 2) * n, words,
                    words * (npole - 1), ring};
     return OVL_OK;
 }
 
 // Batched multishift vectors (grown when a larger batch comes).
-constexpr int kBatchRing = 2;
 template <typename W>
 ovl_status Ctx::ensure_msb(MsBatch<W> &v, int &cap, int nrhs) {
     if (v.r && cap >= nrhs) return OVL_OK;
@@ -661,7 +664,7 @@ ovl_status Ctx::ensure_msb(MsBatch<W> &v, int &cap, int nrhs) {
                 graphs[k].exec = nullptr;
             }
     }
-    ST(alloc_ms(v, nrhs, kBatchRing));
+    ST(alloc_ms(v, nrhs, ring_batch));
     cap = nrhs;
     return OVL_OK;
 }
@@ -669,7 +672,8 @@ ovl_status Ctx::ensure_msb(MsBatch<W> &v, int &cap, int nrhs) {
 // Lock-step multishift solves of nrhs right-hand sides (tolerance tol[y] each); the
 // host polls the first four words (n, iter, done, status) of every state per chunk.
 template <typename ST, typename Init, typename Iter>
-ovl_status Ctx::msb_run(int nrhs, const double *tol, int n, int slot, Init init_fn, Iter iter_fn, long *iters_out) {
+ovl_status Ctx::msb_run(int nrhs, const double *tol, int n, int slot, int ring, Init init_fn, Iter iter_fn,
+                        long *iters_out) {
     Ctx *c = this;
     for (int y = 0; y < nrhs; y++) {
         MsState &s = h_msb[y];
@@ -692,7 +696,7 @@ ovl_status Ctx::msb_run(int nrhs, const double *tol, int n, int slot, Init init_
                 set_launch_counting(false);
                 CK(cudaStreamBeginCapture(stream, cudaStreamCaptureModeThreadLocal));
                 cudaError_t ce = cudaSuccess;
-                for (int k = 0; k < chunk && ce == cudaSuccess; k++) ce = iter_fn(ms_flush(k, chunk, kBatchRing));
+                for (int k = 0; k < chunk && ce == cudaSuccess; k++) ce = iter_fn(ms_flush(k, chunk, ring));
                 cudaError_t ee = cudaStreamEndCapture(stream, &graph);
                 set_launch_counting(true);
                 CK(ce);
@@ -706,7 +710,7 @@ ovl_status Ctx::msb_run(int nrhs, const double *tol, int n, int slot, Init init_
             CK(cudaGraphLaunch(gs.exec, stream));
             count_launches(3L * chunk);
         } else {
-            for (int k = 0; k < chunk; k++) CK(iter_fn(ms_flush(k, chunk, kBatchRing)));
+            for (int k = 0; k < chunk; k++) CK(iter_fn(ms_flush(k, chunk, ring)));
         }
         done_iters += chunk;
         CK(cudaMemcpy2DAsync(h_msb_small, 4 * sizeof(int), msb_state, sizeof(MsState), 4 * sizeof(int), nrhs,
@@ -761,7 +765,7 @@ ovl_status Ctx::sign64_batch(const double2 *b, double2 *out, int nrhs, const dou
         return ms_iter(g, U64, m0_ker, nrhs, msb_state, msb64, rsb, bcounters, flush, stream, MsEvents{});
     };
     const int n = pick_poles(min_positive(tol, nrhs));
-    ST((msb_run<double2>(nrhs, tol, n, 3, init, it, &iters)));
+    ST((msb_run<double2>(nrhs, tol, n, 3, msb64.ring, init, it, &iters)));
     stat_ms64 += iters * nrhs;
     const double sc = zs_d0[n - 1] / lam_min;
     CK(wilson_batch_f64(g, U64, msb64.y, out, msb64.stride, nrhs, m0_ker, mode == 0, sc, mode == 1 ? b : nullptr,
@@ -794,7 +798,7 @@ ovl_status Ctx::sign_ff_batch(const double2 *b, double2 *out, int nrhs, const do
         return ms_iter(g, Uff, m0_ker, nrhs, msb_state, vf, rsb, bcounters, flush, stream, MsEvents{});
     };
     const int n = pick_poles(min_positive(tol, nrhs));
-    ST((msb_run<ffw>(nrhs, tol, n, 7, init, it, &iters)));
+    ST((msb_run<ffw>(nrhs, tol, n, 7, vf.ring, init, it, &iters)));
     stat_msff += iters * nrhs;
     const double sc = zs_d0[n - 1] / lam_min;
     CK(wilson_batch_ff(g, Uff, vf.y, vf.t, words, nrhs, m0_ker, mode == 0, sc, nullptr, 0.0, stream));
@@ -819,7 +823,7 @@ ovl_status Ctx::sign32_batch(const float4 *b, float4 *out, int nrhs, const doubl
         return ms_iter(g, U32, m0_ker, nrhs, msb_state, msb32, rsb, bcounters, flush, stream, MsEvents{});
     };
     const int n = pick_poles(min_positive(tol, nrhs));
-    ST((msb_run<float4>(nrhs, tol, n, 4, init, it, &iters)));
+    ST((msb_run<float4>(nrhs, tol, n, 4, msb32.ring, init, it, &iters)));
     stat_ms32 += iters * nrhs;
     const float sc = (float)(zs_d0[n - 1] / lam_min);
     CK(wilson_batch_f32(g, U32, msb32.y, out, msb32.stride, nrhs, (float)m0_ker, mode == 0, sc,
@@ -851,7 +855,7 @@ ovl_status Ctx::ensure_msh() {
     return OVL_OK;
 }
 
-ovl_status Ctx::ensure_ms32() { return ms32.r ? OVL_OK : alloc_ms(ms32, 1, kMaxRing); }
+ovl_status Ctx::ensure_ms32() { return ms32.r ? OVL_OK : alloc_ms(ms32, 1, ring_one); }
 
 // ------------------------------------------------------------------ spectral estimates
 // Tridiagonal eigenvalue bounds by Sturm-sequence bisection.

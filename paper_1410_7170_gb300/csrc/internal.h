@@ -185,6 +185,7 @@ cudaError_t fill_random_f32(float *x, long n, unsigned seed, cudaStream_t st);
 
 // ---------------------------------------------------------------- multishift CG
 constexpr int kMaxRing = 4;   // iterations whose shift updates are done together, at most
+constexpr int kBatchRing = 2;   // the same in batches, where the rings' vectors count as often as there are right-hand sides
 
 // Device-side state of one multishift solve (Q^2 + sigma_l) x_l = b, l < n, with the
 // Zolotarev accumulation y = b + sum_l w_l x_l. sigma[0] is the base (smallest) shift.

@@ -44,6 +44,7 @@ struct Job {
     ovl_params params;
     bool has_params;
     size_t est_bytes;
+    int ring = ovl::kMaxRing;   // multishift rings that the estimate holds (ovl::Ctx::ring_one)
     Clock::time_point t_submit, t_start, t_end;
     ovl_result res;
     bool done = false;
@@ -58,6 +59,7 @@ struct CachedCtx {
     double rho, mu;
     ovl_params params;
     size_t bytes;
+    int ring;
     long last_use;
 };
 
@@ -90,16 +92,17 @@ namespace {
 
 // Device memory of one request: the context's fields and workspaces for its lattice,
 // precision, preconditioner and right-hand sides (an upper estimate of what ovl_create
-// and ovl_solve allocate).
-size_t estimate_bytes(const ovl_request &r, const ovl_params &p) {
+// and ovl_solve allocate), with rings of `ring` multishift vectors (ovl::Ctx::ring_one).
+size_t estimate_bytes(const ovl_request &r, const ovl_params &p, int ring) {
+    const int batch_ring = std::min(ring, ovl::kBatchRing);
     const double V = (double)r.dims[0] * r.dims[1] * r.dims[2] * r.dims[3];
     const double v64 = 24.0 * V * 8.0, v32 = 24.0 * V * 4.0;
     double b = V * 4 * (9 * 16 + 3 * 16);                 // links: FP64 18 reals + FP32 12 reals
     b += 3 * v64 + 6 * v32;                               // staging, Lanczos / tuning vectors
     b += 24 * v32;                                        // multi-RHS stencil tuning (12 RHS in and out)
-    b += ovl::ms_vectors(p.n_poles, ovl::kMaxRing) * v64;   // FP64 (or float-float) multishift
+    b += ovl::ms_vectors(p.n_poles, ring) * v64;            // FP64 (or float-float) multishift
     const bool mixed = p.precision != OVL_FP64 || p.precond == OVL_PREC_RECURSIVE;
-    if (mixed) b += ovl::ms_vectors(p.n_poles, ovl::kMaxRing) * v32;   // FP32 multishift
+    if (mixed) b += ovl::ms_vectors(p.n_poles, ring) * v32;   // FP32 multishift
     if (mixed && p.ff_outer) b += V * 4 * 9 * 16;          // float-float links
     if (p.sign_method == OVL_SIGN_KRYLOV) b += (p.krylov_m + p.krylov_keep + 3) * v64;   // Krylov sign basis
     if (p.n_deflate > 0) {
@@ -113,8 +116,8 @@ size_t estimate_bytes(const ovl_request &r, const ovl_params &p) {
     if (nrhs > 1 && p.rhs_block > 1) {
         const int nb = std::min(std::min(p.rhs_block, nrhs), 12);
         const int mo = std::min(p.restart, 32), mi = std::min(p.restart_inner, 32), mw = std::min(p.prec_restart, 16);
-        b += nb * ((2 * mo + 5) * v64 + ovl::ms_vectors(p.n_poles, 2) * v64);
-        if (mixed) b += nb * ((2 * mi + 3) * v32 + (2 * mw + 3) * v32 + ovl::ms_vectors(p.n_poles, 2) * v32 + 2 * v32);
+        b += nb * ((2 * mo + 5) * v64 + ovl::ms_vectors(p.n_poles, batch_ring) * v64);
+        if (mixed) b += nb * ((2 * mi + 3) * v32 + (2 * mw + 3) * v32 + ovl::ms_vectors(p.n_poles, batch_ring) * v32 + 2 * v32);
     } else {
         b += (2 * p.restart + 5) * v64;                   // outer FGMRES basis (V and Z)
         if (p.precond == OVL_PREC_RECURSIVE) b += (2 * p.restart_inner + 3) * v32;
@@ -132,14 +135,23 @@ void evict_idle(ovl_server *s) {
     s->idle.clear();
 }
 
+// The admission estimate reserved the batch workspaces and the multishift rings: the context batches by
+// rhs_block alone and takes the rings of the estimate.
+void reserve_as_admitted(ovl_ctx *ctx, const Job *j, bool fixed_rings) {
+    ovl::Ctx *c = reinterpret_cast<ovl::Ctx *>(ctx);
+    c->fixed_batch = true;
+    c->ring_one = j->ring;
+    c->ring_batch = std::min(j->ring, ovl::kBatchRing);
+    c->fixed_rings = fixed_rings;
+}
+
 void run_job(ovl_server *s, Job *j) {
     // context: the cached one claimed at admission, or a new one
     ovl_ctx *ctx = j->claimed;
     const size_t cbytes = j->claimed_bytes;
     ovl_status st = OVL_OK;
     if (!ctx) st = ovl_create(&ctx, j->req.gauge, j->req.dims, j->req.rho, j->req.mu, &j->params, nullptr);
-    // the admission estimate reserved the batch workspaces: batch by rhs_block alone
-    if (ctx) reinterpret_cast<ovl::Ctx *>(ctx)->fixed_batch = true;
+    if (ctx) reserve_as_admitted(ctx, j, true);
     ovl_stats stats;
     memset(&stats, 0, sizeof(stats));
     if (st == OVL_OK) st = ovl_solve(ctx, j->req.x, j->req.b, j->req.n_rhs, j->req.tol, &stats);
@@ -156,7 +168,7 @@ void run_job(ovl_server *s, Job *j) {
             evict_idle(s);
         }
         st = ovl_create(&ctx, j->req.gauge, j->req.dims, j->req.rho, j->req.mu, &j->params, nullptr);
-        if (ctx) reinterpret_cast<ovl::Ctx *>(ctx)->fixed_batch = true;
+        if (ctx) reserve_as_admitted(ctx, j, false);   // smaller rings rather than no answer
         if (st == OVL_OK) st = ovl_solve(ctx, j->req.x, j->req.b, j->req.n_rhs, j->req.tol, &stats);
     }
     if (st != OVL_OK && ctx) {
@@ -170,7 +182,8 @@ void run_job(ovl_server *s, Job *j) {
     std::lock_guard<std::mutex> lk(s->mu);
     s->reserved -= cbytes ? cbytes : j->est_bytes;
     if (ctx) {
-        if (j->req.gauge_key && st == OVL_OK) {
+        // one whose rings had to shrink would give its next request other roundings
+        if (j->req.gauge_key && st == OVL_OK && !reinterpret_cast<ovl::Ctx *>(ctx)->rings_reduced) {
             CachedCtx cc;
             cc.ctx = ctx;
             cc.key = j->req.gauge_key;
@@ -179,6 +192,7 @@ void run_job(ovl_server *s, Job *j) {
             cc.mu = j->req.mu;
             cc.params = j->params;
             cc.bytes = std::max(held, j->est_bytes);
+            cc.ring = j->ring;
             cc.last_use = ++s->use_clock;
             s->idle.push_back(cc);
             s->cached += cc.bytes;
@@ -234,7 +248,8 @@ void worker(ovl_server *s) {
                     if (c->req.gauge_key)
                         for (auto ci = s->idle.begin(); ci != s->idle.end(); ++ci)
                             if (ci->key == c->req.gauge_key && !memcmp(ci->dims, c->req.dims, sizeof(ci->dims)) &&
-                                ci->rho == c->req.rho && ci->mu == c->req.mu && same_params(ci->params, c->params)) {
+                                ci->rho == c->req.rho && ci->mu == c->req.mu && ci->ring == c->ring &&
+                                same_params(ci->params, c->params)) {
                                 hit = ci;
                                 break;
                             }
@@ -296,7 +311,7 @@ extern "C" ovl_status ovl_request_bytes(const ovl_request *req, size_t *bytes) {
     ovl_params p;
     if (req->params) p = *req->params;
     else ovl_params_default(&p);
-    *bytes = estimate_bytes(*req, p);
+    *bytes = estimate_bytes(*req, p, ovl::kMaxRing);
     return OVL_OK;
 }
 
@@ -307,7 +322,9 @@ extern "C" ovl_status ovl_server_submit(ovl_server *s, const ovl_request *req, l
     if (req->params) j->params = *req->params;
     else ovl_params_default(&j->params);
     j->req.params = nullptr;
-    j->est_bytes = estimate_bytes(j->req, j->params);
+    // with the full rings if they fit the budget, with smaller ones rather than not at all
+    j->ring = ovl::kMaxRing;
+    while ((j->est_bytes = estimate_bytes(j->req, j->params, j->ring)) > s->budget && j->ring > 1) j->ring /= 2;
     memset(&j->res, 0, sizeof(j->res));
     std::lock_guard<std::mutex> lk(s->mu);
     if (j->est_bytes > s->budget) {

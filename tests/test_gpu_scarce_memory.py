@@ -1,9 +1,15 @@
-"""Calls that find little device memory left: what fails reports it and leaves the context as it was.
-The lattice is 48^4 (a vector of FP64 is 1.0 GB), so that hundreds of MB stay free for the CUDA runtime
-while an allocation of the library does not fit. Links are the identity; nothing here tests numbers."""
+"""Calls that find little device memory left: what fails reports it and leaves the context as it was, and
+what is there for speed alone is left out before a call fails. The lattice is 48^4 (a vector of FP64 is 1.0 GB), so that hundreds of MB stay free for the CUDA runtime
+while an allocation of the library does not fit. Links are the identity.
+
+Bars: two evaluations with another order of the shift updates differ by rounding, 1e-11 in FP64 and
+float-float, 2e-5 in FP32 (as for the other tests of the update order)."""
 import contextlib
 
+import numpy as np
 import pytest
+
+import synth
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -63,4 +69,66 @@ def test_refused_call_leaves_no_trace_in_the_next_one(precision):
         assert status(f, op, out, good, -0.3) == ovl.OVL_ENOMEM
     assert bool((out == 7.0).all())
     assert status(f, op, out, good, -0.3) == ovl.OVL_OK
+    op.close()
+
+
+# vectors of a multishift solve with n poles and rings of one (n + 3), in units of an FP64 vector
+POLES = 4
+SIGNS = {ovl.OVL_ARITH_FP64: (1.0, 1e-11), ovl.OVL_ARITH_FF: (1.0, 1e-11), ovl.OVL_ARITH_FP32: (0.5, 2e-5)}
+
+
+@pytest.mark.parametrize("arith", list(SIGNS))
+def test_sign_with_room_for_the_smallest_rings(arith):
+    size, tol = SIGNS[arith]
+    gen = torch.Generator("cuda")
+    gen.manual_seed(51)
+    b = torch.view_as_complex(torch.randn((V, 4, 3, 2), dtype=torch.float64, device="cuda", generator=gen))
+    ref, out = torch.empty_like(b), torch.empty_like(b)
+    op = _op(n_poles=POLES)
+    op.sign_apply_arith(ref, b, 1e-5, arith)
+    op.close()
+    op = _op(n_poles=POLES)
+    op.wilson_apply_arith(out, b, -1.0, arith)   # what the call needs besides
+    f = ovl.lib().sign_apply_arith
+    with scarce(int((POLES + 3 + 0.8) * size * VEC)):
+        assert status(f, op, out, b, 1e-5, arith) == ovl.OVL_OK
+    out -= ref
+    assert (out.norm() / ref.norm()).item() < tol
+    op.close()
+
+
+def test_batch_with_room_for_the_smallest_rings():
+    b = torch.randn((2, V, 4, 3), dtype=torch.complex128, device="cuda")
+    ref, out = torch.empty_like(b), torch.empty_like(b)
+    op = _op(n_poles=POLES)
+    op.ovl_apply_n(ref, b, 2, 1e-5)
+    op.close()
+    op = _op(n_poles=POLES)
+    op.wilson_apply_n(out, b, 2, -1.0)
+    with scarce(int((2 * (POLES + 3) + 0.8) * VEC)):
+        assert status(ovl.lib().ovl_apply_n, op, out, b, 2, 1e-5) == ovl.OVL_OK
+    out -= ref
+    assert (out.norm() / ref.norm()).item() < 1e-11
+    op.close()
+
+
+@pytest.mark.parametrize("n", [1, 3])
+def test_budget_of_the_smallest_rings_admits(n):
+    """A budget that holds a request with rings of one serves it."""
+    dims = (8, 8, 8, 8)
+    U = synth.gauge_field(dims, 0.5, 52, stout_steps=3)
+    p = ovl.params_default(precond=ovl.OVL_PREC_RECURSIVE, precision=ovl.OVL_MIXED_FP32, rhs_block=4)
+    one, batch = 6 * 1.5, 2 * 1.5 * (n if n > 1 else 0)   # vectors of the larger rings, FP64 and half as much in FP32
+    budget = ovl.request_bytes(dims, n, p) - int(1.1 * (one + batch) * 8 ** 4 * 192) + (1 << 20)
+    b = synth.rhs_gaussian(dims, 53, n_rhs=n)
+    x = np.zeros_like(b)
+    srv = ovl.Server(slots=1, hbm_budget=budget)
+    res = srv.wait(srv.submit(U, dims, 1.0, 0.05, b, x, n, 1e-8, p))
+    srv.close()
+    assert res["status"] == ovl.OVL_OK, res["message"]
+    op = ovl.Overlap(U, dims, 1.0, 0.05, p)
+    for k in range(n):
+        ax = np.empty_like(x[k])
+        op.ovl_apply(ax, x[k], 1e-12)
+        assert np.linalg.norm(b[k] - ax) / np.linalg.norm(b[k]) < 1.5e-8
     op.close()
