@@ -650,9 +650,9 @@ ovl_status Ctx::alloc_ms(MsBatch<W> &v, int nrhs, int ring) {
     return OVL_OK;
 }
 
-// Batched multishift vectors (grown when a larger batch comes).
+// Batched multishift vectors (grown when a larger batch comes). whole: OVL_ENOMEM rather than smaller rings.
 template <typename W>
-ovl_status Ctx::ensure_msb(MsBatch<W> &v, int &cap, int nrhs) {
+ovl_status Ctx::ensure_msb(MsBatch<W> &v, int &cap, int nrhs, bool whole) {
     if (v.r && cap >= nrhs) return OVL_OK;
     if (v.r) {
         cudaFree(v.r);
@@ -664,17 +664,21 @@ ovl_status Ctx::ensure_msb(MsBatch<W> &v, int &cap, int nrhs) {
                 graphs[k].exec = nullptr;
             }
     }
-    ST(alloc_ms(v, nrhs, ring_batch));
-    cap = nrhs;
-    return OVL_OK;
+    const bool fixed = fixed_rings;
+    fixed_rings = fixed || whole;
+    const ovl_status st = alloc_ms(v, nrhs, ring_batch);
+    fixed_rings = fixed;
+    if (st == OVL_OK) cap = nrhs;
+    return st;
 }
 
 // Lock-step multishift solves of nrhs right-hand sides (tolerance tol[y] each); the
 // host polls the first four words (n, iter, done, status) of every state per chunk.
 template <typename ST, typename Init, typename Iter>
-ovl_status Ctx::msb_run(int nrhs, const double *tol, int n, int slot, int ring, Init init_fn, Iter iter_fn,
+ovl_status Ctx::msb_run(MsRows rows, const double *tol, int n, int slot, int ring, Init init_fn, Iter iter_fn,
                         long *iters_out) {
     Ctx *c = this;
+    const int nrhs = rows.n;
     for (int y = 0; y < nrhs; y++) {
         MsState &s = h_msb[y];
         fill_poles(s, n, tol[y] > 0 ? tol[y] : 1.0);
@@ -684,7 +688,7 @@ ovl_status Ctx::msb_run(int nrhs, const double *tol, int n, int slot, int ring, 
     CK(init_fn());
     const int chunk = std::min(p.check_every, kMaxChunk);
     GraphSlot &gs = graphs[slot];
-    if (gs.exec && (gs.nrhs != nrhs || gs.chunk != chunk)) {
+    if (gs.exec && (gs.nrhs != nrhs || gs.of != rows.of || gs.chunk != chunk)) {
         cudaGraphExecDestroy(gs.exec);
         gs.exec = nullptr;
     }
@@ -705,6 +709,7 @@ ovl_status Ctx::msb_run(int nrhs, const double *tol, int n, int slot, int ring, 
                 cudaGraphDestroy(graph);
                 CK(ie);
                 gs.nrhs = nrhs;
+                gs.of = rows.of;
                 gs.chunk = chunk;
             }
             CK(cudaGraphLaunch(gs.exec, stream));
@@ -773,14 +778,14 @@ ovl_status Ctx::sign64_batch(const double2 *b, double2 *out, int nrhs, const dou
     return OVL_OK;
 }
 
-// The same in float-float arithmetic (sign_ff).
+// The same in float-float arithmetic (sign_ff). The FP64 batch's vectors serve both arithmetics (words
+// of the same size, one call at a time). Where they don't fit for all right-hand sides these are done
+// in parts, with the degree and the launch shapes of the whole batch: the same results, bit for bit.
 ovl_status Ctx::sign_ff_batch(const double2 *b, double2 *out, int nrhs, const double *tol, int mode) {
     Ctx *c = this;
     const long words = (long)g.V * 12;
-    // the FP64 batch's vectors serve both arithmetics (words of the same size, one call at a time);
-    // a batch that does not fit runs one vector at a time in the single vector's memory
     static_assert(sizeof(ffw) == sizeof(double2), "");
-    if (nrhs == 1 || ndefl || p.sign_method == OVL_SIGN_KRYLOV || ensure_msb(msb64, msb64_cap, nrhs) != OVL_OK) {
+    if (nrhs == 1 || ndefl || p.sign_method == OVL_SIGN_KRYLOV) {
         for (int y = 0; y < nrhs; y++)
             if (tol[y] > 0) ST(sign_ff(b + y * words, out + y * words, tol[y], mode));
         return OVL_OK;
@@ -788,22 +793,31 @@ ovl_status Ctx::sign_ff_batch(const double2 *b, double2 *out, int nrhs, const do
     PhaseClock pclk(this, &t_sign64);
     ST(ensure_batch());
     ST(ensure_ff_links());
+    int part = std::min(nrhs, ff_part);
+    ovl_status st;
+    while ((st = ensure_msb(msb64, msb64_cap, part, part > 1)) == OVL_ENOMEM && part > 1) ff_part = part = (part + 1) / 2;
+    if (st != OVL_OK) return st;
     const MsBatch<ffw> vf{(ffw *)msb64.r, (ffw *)msb64.p0, (ffw *)msb64.t, (ffw *)msb64.y, (ffw *)msb64.p, msb64.stride,
                           msb64.prow, msb64.ring};
-    // b in float-float into t (t is overwritten by the first iteration's Q p)
-    CK(spinor_d2ff(g, b, vf.t, stream, nrhs));
-    long iters = 0;
-    auto init = [&]() { return ms_init(g, nrhs, msb_state, vf, vf.t, rsb, bcounters, stream); };
-    auto it = [&](bool flush) {
-        return ms_iter(g, Uff, m0_ker, nrhs, msb_state, vf, rsb, bcounters, flush, stream, MsEvents{});
-    };
     const int n = pick_poles(min_positive(tol, nrhs));
-    ST((msb_run<ffw>(nrhs, tol, n, 7, vf.ring, init, it, &iters)));
-    stat_msff += iters * nrhs;
     const double sc = zs_d0[n - 1] / lam_min;
-    CK(wilson_batch_ff(g, Uff, vf.y, vf.t, words, nrhs, m0_ker, mode == 0, sc, nullptr, 0.0, stream));
-    CK(spinor_ff2d(g, vf.t, out, stream, nrhs));
-    if (mode == 1) CK(dev_axpby(rho, (const double *)b, 1.0, (double *)out, n64 * nrhs, stream));
+    for (int r0 = 0; r0 < nrhs; r0 += part) {
+        const MsRows rows(std::min(part, nrhs - r0), nrhs);
+        const double2 *br = b + r0 * words;
+        double2 *o = out + r0 * words;
+        // b in float-float into t (t is overwritten by the first iteration's Q p)
+        CK(spinor_d2ff(g, br, vf.t, stream, rows.n));
+        long iters = 0;
+        auto init = [&]() { return ms_init(g, rows, msb_state, vf, vf.t, rsb, bcounters, stream); };
+        auto it = [&](bool flush) {
+            return ms_iter(g, Uff, m0_ker, rows, msb_state, vf, rsb, bcounters, flush, stream, MsEvents{});
+        };
+        ST((msb_run<ffw>(rows, tol + r0, n, 7, vf.ring, init, it, &iters)));
+        stat_msff += iters * rows.n;
+        CK(wilson_batch_ff(g, Uff, vf.y, vf.t, words, rows.n, m0_ker, mode == 0, sc, nullptr, 0.0, stream));
+        CK(spinor_ff2d(g, vf.t, o, stream, rows.n));
+        if (mode == 1) CK(dev_axpby(rho, (const double *)br, 1.0, (double *)o, n64 * rows.n, stream));
+    }
     return OVL_OK;
 }
 

@@ -256,21 +256,29 @@ struct MsVectorsH {
     long words_h;       // uint4 words per FP16 vector (3 V)
 };
 
+// Right-hand sides of a launch, and of the batch that they belong to: a batch that does not fit the
+// memory is done in parts, with the launch shapes of the whole (they decide the order of the
+// reductions), so that its results don't depend on the memory that was free.
+struct MsRows {
+    int n, of;
+    MsRows(int n_) : n(n_), of(n_) {}
+    MsRows(int n_, int of_) : n(n_), of(of_) {}
+};
 // One multishift iteration of nrhs right-hand sides (state st[y]; grid row y) = three launches: Q p,
 // residual update, and p_0 or, where flush is set, the pending shift updates with it. A caller sets
 // flush at least in every ring-th iteration, and in the last one before it reads y or the state.
 // rs.partials: nrhs * kRowRedValues * kMaxRedBlocks doubles; counters: nrhs words, zero between launches.
-cudaError_t ms_init(const Geom &g, int nrhs, MsState *s, MsBatch<double2> v, const double2 *b, RedScratch rs,
+cudaError_t ms_init(const Geom &g, MsRows nrhs, MsState *s, MsBatch<double2> v, const double2 *b, RedScratch rs,
                     unsigned *counters, cudaStream_t st);
-cudaError_t ms_init(const Geom &g, int nrhs, MsState *s, MsBatch<float4> v, const float4 *b, RedScratch rs,
+cudaError_t ms_init(const Geom &g, MsRows nrhs, MsState *s, MsBatch<float4> v, const float4 *b, RedScratch rs,
                     unsigned *counters, cudaStream_t st);
-cudaError_t ms_init(const Geom &g, int nrhs, MsState *s, MsBatch<ffw> v, const ffw *b, RedScratch rs,
+cudaError_t ms_init(const Geom &g, MsRows nrhs, MsState *s, MsBatch<ffw> v, const ffw *b, RedScratch rs,
                     unsigned *counters, cudaStream_t st);
-cudaError_t ms_iter(const Geom &g, const double2 *U, double m0, int nrhs, MsState *s, MsBatch<double2> v, RedScratch rs,
+cudaError_t ms_iter(const Geom &g, const double2 *U, double m0, MsRows nrhs, MsState *s, MsBatch<double2> v, RedScratch rs,
                     unsigned *counters, bool flush, cudaStream_t st, const MsEvents &ev);
-cudaError_t ms_iter(const Geom &g, const float4 *U, double m0, int nrhs, MsState *s, MsBatch<float4> v, RedScratch rs,
+cudaError_t ms_iter(const Geom &g, const float4 *U, double m0, MsRows nrhs, MsState *s, MsBatch<float4> v, RedScratch rs,
                     unsigned *counters, bool flush, cudaStream_t st, const MsEvents &ev);
-cudaError_t ms_iter(const Geom &g, const ffl *U, double m0, int nrhs, MsState *s, MsBatch<ffw> v, RedScratch rs,
+cudaError_t ms_iter(const Geom &g, const ffl *U, double m0, MsRows nrhs, MsState *s, MsBatch<ffw> v, RedScratch rs,
                     unsigned *counters, bool flush, cudaStream_t st, const MsEvents &ev);
 // one right-hand side with 16-bit shifted directions, updated in every iteration
 cudaError_t ms_init_half(const Geom &g, int n, MsState *s, MsVectorsH v, const float4 *b, RedScratch rs, bool bf16,

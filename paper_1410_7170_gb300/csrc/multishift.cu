@@ -621,36 +621,36 @@ __global__ void k_ms_init_half(Geom g, MsState *s, MsVectorsH v, const float4 *_
 
 // The third kernel of an iteration: the shift updates where `flush`, else p_0 alone.
 template <typename ST>
-cudaError_t ms_third(const Geom &g, int nrhs, MsState *s, const MsBatch<ST> &v, unsigned *counters, bool flush,
+cudaError_t ms_third(const Geom &g, MsRows nrhs, MsState *s, const MsBatch<ST> &v, unsigned *counters, bool flush,
                      cudaStream_t st) {
     const int want = stream_grid(v.stride);
     if (flush)
-        k_ms_shifts<ST><<<dim3(std::max(1, std::min(want, kShiftBlocks * g.nsm / nrhs)), nrhs), kBlock, 0, st>>>(s, v,
+        k_ms_shifts<ST><<<dim3(std::max(1, std::min(want, kShiftBlocks * g.nsm / nrhs.of)), nrhs.n), kBlock, 0, st>>>(s, v,
                                                                                                       counters);
-    else k_ms_p0<ST><<<dim3(std::max(1, std::min(want, 16 * g.nsm / nrhs)), nrhs), kBlock, 0, st>>>(s, v);
+    else k_ms_p0<ST><<<dim3(std::max(1, std::min(want, 16 * g.nsm / nrhs.of)), nrhs.n), kBlock, 0, st>>>(s, v);
     return cudaGetLastError();
 }
 
 // One iteration of nrhs right-hand sides, one warp per hop.
 template <typename R, typename LT, typename ST>
-cudaError_t ms_stencils_hops(const Geom &g, const LT *U, double m0, int nrhs, MsState *s, const MsBatch<ST> &v,
+cudaError_t ms_stencils_hops(const Geom &g, const LT *U, double m0, MsRows nrhs, MsState *s, const MsBatch<ST> &v,
                              const RedScratch &rows, cudaStream_t st, const MsEvents &ev) {
-    const int gx = hop_grid<R>(g, nrhs, true);
+    const int gx = hop_grid<R>(g, nrhs.of, true);
     cudaError_t e;
     if ((e = ev.record(0, st)) != cudaSuccess) return e;
-    if (nrhs > 1 && !std::is_same<R, ff>::value)
-        k_ms_q_hops<R, !std::is_same<R, ff>::value><<<dim3(gx, nrhs), kHopBlock, 0, st>>>(g, U, R(m0 + 4.0), s, v, rows);
-    else k_ms_q_hops<R, false><<<dim3(gx, nrhs), kHopBlock, 0, st>>>(g, U, R(m0 + 4.0), s, v, rows);
+    if (nrhs.of > 1 && !std::is_same<R, ff>::value)
+        k_ms_q_hops<R, !std::is_same<R, ff>::value><<<dim3(gx, nrhs.n), kHopBlock, 0, st>>>(g, U, R(m0 + 4.0), s, v, rows);
+    else k_ms_q_hops<R, false><<<dim3(gx, nrhs.n), kHopBlock, 0, st>>>(g, U, R(m0 + 4.0), s, v, rows);
     if ((e = ev.record(1, st)) != cudaSuccess) return e;
     // one block more for the shift scalars, within the wave
-    const int gr = (long)gx * nrhs + nrhs > (long)g.nsm * HopBlocks<R>::value && gx > 1 ? gx : gx + 1;
-    k_ms_r_hops<R><<<dim3(gr, nrhs), kHopBlock, 0, st>>>(g, U, R(m0 + 4.0), s, v, rows);
+    const int gr = (long)gx * nrhs.of + nrhs.of > (long)g.nsm * HopBlocks<R>::value && gx > 1 ? gx : gx + 1;
+    k_ms_r_hops<R><<<dim3(gr, nrhs.n), kHopBlock, 0, st>>>(g, U, R(m0 + 4.0), s, v, rows);
     return ev.record(2, st);
 }
 // FP32, one thread per site
-cudaError_t ms_stencils_site(const Geom &g, const float4 *U, float m0, int nrhs, MsState *s, const MsBatch<float4> &v,
+cudaError_t ms_stencils_site(const Geom &g, const float4 *U, float m0, MsRows nrhs, MsState *s, const MsBatch<float4> &v,
                              const RedScratch &rows, cudaStream_t st, const MsEvents &ev) {
-    const int slots = std::max(1, g.nsm * MinBlocks<float>::value / nrhs);   // resident blocks of a row
+    const int slots = std::max(1, g.nsm * MinBlocks<float>::value / nrhs.of);   // resident blocks of a row
     // one wave of blocks that stride over the sites (at 32^4 thirteen waves, each block ending with a
     // fence and an atomic, cost 20 us of 125; the whole FP32 sign at 32^4 14.67 ms, with the order of
     // site_of_thread 14.17)
@@ -658,15 +658,15 @@ cudaError_t ms_stencils_site(const Geom &g, const float4 *U, float m0, int nrhs,
     const LaunchShape r = balanced_shape(g.V, std::max(1, slots - 1), 1, std::max(1, slots - 1));
     cudaError_t e;
     if ((e = ev.record(0, st)) != cudaSuccess) return e;
-    if (nrhs > 1) k_ms_q_site<true><<<dim3(q.grid, nrhs), q.block, 0, st>>>(g, U, m0 + 4.f, s, v, rows, q.spb);
-    else k_ms_q_site<false><<<dim3(q.grid, nrhs), q.block, 0, st>>>(g, U, m0 + 4.f, s, v, rows, q.spb);
+    if (nrhs.of > 1) k_ms_q_site<true><<<dim3(q.grid, nrhs.n), q.block, 0, st>>>(g, U, m0 + 4.f, s, v, rows, q.spb);
+    else k_ms_q_site<false><<<dim3(q.grid, nrhs.n), q.block, 0, st>>>(g, U, m0 + 4.f, s, v, rows, q.spb);
     if ((e = ev.record(1, st)) != cudaSuccess) return e;
-    k_ms_r_site<<<dim3(r.grid + 1, nrhs), r.block, 0, st>>>(g, U, m0 + 4.f, s, v, rows, r.spb);
+    k_ms_r_site<<<dim3(r.grid + 1, nrhs.n), r.block, 0, st>>>(g, U, m0 + 4.f, s, v, rows, r.spb);
     return ev.record(2, st);
 }
 
 template <typename R, typename LT, typename ST>
-cudaError_t ms_iter_t(const Geom &g, const LT *U, double m0, int nrhs, MsState *s, MsBatch<ST> v, RedScratch rs,
+cudaError_t ms_iter_t(const Geom &g, const LT *U, double m0, MsRows nrhs, MsState *s, MsBatch<ST> v, RedScratch rs,
                       unsigned *counters, bool flush, cudaStream_t st, const MsEvents &ev) {
     const RedScratch rows{rs.partials, counters};
     cudaError_t e;
@@ -683,38 +683,38 @@ cudaError_t ms_iter_t(const Geom &g, const LT *U, double m0, int nrhs, MsState *
     return cudaGetLastError();
 }
 template <typename ST>
-cudaError_t ms_init_t(int nrhs, MsState *s, const MsBatch<ST> &v, const ST *b, RedScratch rs, unsigned *counters,
+cudaError_t ms_init_t(MsRows nrhs, MsState *s, const MsBatch<ST> &v, const ST *b, RedScratch rs, unsigned *counters,
                       cudaStream_t st) {
-    const int gx = std::max(1, red_grid(v.stride) / nrhs);
-    k_ms_init<ST><<<dim3(gx, nrhs), kBlock, 0, st>>>(s, b, v, RedScratch{rs.partials, counters});
+    const int gx = std::max(1, red_grid(v.stride) / nrhs.of);
+    k_ms_init<ST><<<dim3(gx, nrhs.n), kBlock, 0, st>>>(s, b, v, RedScratch{rs.partials, counters});
     count_launches(1);
     return cudaGetLastError();
 }
 
 }  // namespace
 
-cudaError_t ms_init(const Geom &g, int nrhs, MsState *s, MsBatch<double2> v, const double2 *b, RedScratch rs,
+cudaError_t ms_init(const Geom &g, MsRows nrhs, MsState *s, MsBatch<double2> v, const double2 *b, RedScratch rs,
                     unsigned *counters, cudaStream_t st) {
     return ms_init_t(nrhs, s, v, b, rs, counters, st);
 }
-cudaError_t ms_init(const Geom &g, int nrhs, MsState *s, MsBatch<float4> v, const float4 *b, RedScratch rs,
+cudaError_t ms_init(const Geom &g, MsRows nrhs, MsState *s, MsBatch<float4> v, const float4 *b, RedScratch rs,
                     unsigned *counters, cudaStream_t st) {
     return ms_init_t(nrhs, s, v, b, rs, counters, st);
 }
-cudaError_t ms_init(const Geom &g, int nrhs, MsState *s, MsBatch<ffw> v, const ffw *b, RedScratch rs,
+cudaError_t ms_init(const Geom &g, MsRows nrhs, MsState *s, MsBatch<ffw> v, const ffw *b, RedScratch rs,
                     unsigned *counters, cudaStream_t st) {
     return ms_init_t(nrhs, s, v, b, rs, counters, st);
 }
-cudaError_t ms_iter(const Geom &g, const double2 *U, double m0, int nrhs, MsState *s, MsBatch<double2> v, RedScratch rs,
+cudaError_t ms_iter(const Geom &g, const double2 *U, double m0, MsRows nrhs, MsState *s, MsBatch<double2> v, RedScratch rs,
                     unsigned *counters, bool flush, cudaStream_t st, const MsEvents &ev) {
     return ms_iter_t<double>(g, U, m0, nrhs, s, v, rs, counters, flush, st, ev);
 }
-cudaError_t ms_iter(const Geom &g, const float4 *U, double m0, int nrhs, MsState *s, MsBatch<float4> v, RedScratch rs,
+cudaError_t ms_iter(const Geom &g, const float4 *U, double m0, MsRows nrhs, MsState *s, MsBatch<float4> v, RedScratch rs,
                     unsigned *counters, bool flush, cudaStream_t st, const MsEvents &ev) {
     return ms_iter_t<float>(g, U, m0, nrhs, s, v, rs, counters, flush, st, ev);
 }
 // float-float: the scalar recurrences stay FP64 on the device
-cudaError_t ms_iter(const Geom &g, const ffl *U, double m0, int nrhs, MsState *s, MsBatch<ffw> v, RedScratch rs,
+cudaError_t ms_iter(const Geom &g, const ffl *U, double m0, MsRows nrhs, MsState *s, MsBatch<ffw> v, RedScratch rs,
                     unsigned *counters, bool flush, cudaStream_t st, const MsEvents &ev) {
     return ms_iter_t<ff>(g, U, m0, nrhs, s, v, rs, counters, flush, st, ev);
 }

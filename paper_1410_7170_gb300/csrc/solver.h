@@ -34,7 +34,7 @@ struct GraphSlot {
     cudaGraphExec_t exec = nullptr;
     int chunk = 0;
     bool prof = false;
-    int nrhs = 0;
+    int nrhs = 0, of = 0;
 };
 
 constexpr int kMaxChunk = 64;
@@ -246,19 +246,20 @@ struct Ctx {
     template <typename W>
     ovl_status alloc_ms(MsBatch<W> &v, int nrhs, int ring);
     template <typename W>
-    ovl_status ensure_msb(MsBatch<W> &v, int &cap, int nrhs);
+    ovl_status ensure_msb(MsBatch<W> &v, int &cap, int nrhs, bool whole = false);
     // Rings of one right-hand side's and of a batch's multishift vectors. They are for speed: where the
     // memory for them is not there they halve, down to one (n + 3 vectors for n poles), unless
     // fixed_rings is set (the serving loop, which reserved the memory for them and wants the same
     // results whatever else runs: the ring decides the order of additions in y).
     int ring_one = kMaxRing, ring_batch = kBatchRing;
+    int ff_part = kMaxBatch;   // right-hand sides of a float-float batch that are done together, as far as memory goes
     bool fixed_rings = false, rings_reduced = false;
     ovl_status sign64_batch(const double2 *b, double2 *out, int nrhs, const double *tol, int mode);
     ovl_status sign_ff_batch(const double2 *b, double2 *out, int nrhs, const double *tol, int mode);
     ovl_status sign_outer_batch(const double2 *b, double2 *out, int nrhs, const double *tol, int mode);
     ovl_status sign32_batch(const float4 *b, float4 *out, int nrhs, const double *tol, int mode);
     template <typename ST, typename Init, typename Iter>
-    ovl_status msb_run(int nrhs, const double *tol, int n, int slot, int ring, Init init_fn, Iter iter_fn,
+    ovl_status msb_run(MsRows rows, const double *tol, int n, int slot, int ring, Init init_fn, Iter iter_fn,
                        long *iters_out);
     ovl_status lanczos_bounds(double *lmin, double *lmax, double m0 = NAN);   // |eigenvalues| of Q(m0), default m0_ker
     ovl_status sigma_min_estimate(double *smin);

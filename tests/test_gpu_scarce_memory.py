@@ -132,3 +132,31 @@ def test_budget_of_the_smallest_rings_admits(n):
         op.ovl_apply(ax, x[k], 1e-12)
         assert np.linalg.norm(b[k] - ax) / np.linalg.norm(b[k]) < 1.5e-8
     op.close()
+
+
+def test_served_batch_in_parts_gives_the_same_bits():
+    """The float-float batch of a served request whose vectors don't fit all at once."""
+    dims, n = (16, 16, 16, 16), 4
+    U = torch.from_numpy(synth.gauge_field(dims, 0.5, 54, stout_steps=2, device="cuda")).cuda()
+    b = torch.from_numpy(synth.rhs_gaussian(dims, 55, n_rhs=n)).cuda()
+    p = ovl.params_default(precond=ovl.OVL_PREC_RECURSIVE, precision=ovl.OVL_MIXED_FP32, rhs_block=n, restart=8,
+                           restart_inner=16, prec_restart=8, lambda_min=0.15, lambda_max=8.0, m0_prec=0.0, relax_factor=0.3)
+    vec = 16 ** 4 * 192
+
+    def served(left):
+        x = torch.zeros_like(b)
+        srv = ovl.Server(slots=1)
+        with scarce(left) if left else contextlib.nullcontext():
+            free = torch.cuda.mem_get_info()[0]
+            res = srv.wait(srv.submit(U, dims, 1.0, 0.05, b, x, n, 1e-9, p, gauge_key=7))
+            used = free - torch.cuda.mem_get_info()[0]   # the resident context still holds its memory
+        srv.close()
+        assert res["status"] == ovl.OVL_OK, res["message"]
+        return x, used
+
+    ref, used = served(0)
+    batch = n * (2 * 2 + 2 + 19) * vec   # the float-float batch's vectors: 20 poles, rings of two
+    assert used > batch
+    x, less = served(used - batch // 4)
+    assert less < used - batch // 4
+    assert torch.equal(x, ref)
