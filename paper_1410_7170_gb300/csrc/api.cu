@@ -1122,9 +1122,22 @@ ovl_status Ctx::autotune_mrhs() {
 }
 
 // Time of one FP32 Schwarz cycle on a constant non-zero input, for ovl_tuning_sap (the block kernel
-// has one form, one thread per block site).
+// has one form, one thread per block site). Measured once per process, lattice shape and block shape:
+// contexts after the first (the serving loop makes one per gauge field) don't pay for it.
+static std::map<std::tuple<int, int, int, int, int, int, int, int, int>, float> g_sap_cache;
+
 ovl_status Ctx::time_sap() {
     Ctx *c = this;
+    const auto key = std::make_tuple(g.L[0], g.L[1], g.L[2], g.L[3], p.sap_block[0], p.sap_block[1], p.sap_block[2],
+                                     p.sap_block[3], p.sap_mr_iters);
+    {
+        std::lock_guard<std::mutex> lk(g_tune_mu);
+        auto it = g_sap_cache.find(key);
+        if (it != g_sap_cache.end()) {
+            sap_ms[0] = sap_ms[1] = sap_ms[2] = it->second;
+            return OVL_OK;
+        }
+    }
     void *buf;
     const size_t bytes = (size_t)n64 * sizeof(float);
     ST(alloc(&buf, bytes * 3));
@@ -1144,6 +1157,10 @@ ovl_status Ctx::time_sap() {
     float ms;
     CK(cudaEventElapsedTime(&ms, e0, e1));
     sap_ms[0] = sap_ms[1] = sap_ms[2] = ms / reps;
+    {
+        std::lock_guard<std::mutex> lk(g_tune_mu);
+        g_sap_cache[key] = ms / reps;
+    }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     cudaFree(buf);
