@@ -95,27 +95,36 @@ ovl_status upload_coef(Ctx *c, const std::vector<cd> &v) {
 }
 
 // Records of the device's Gram-Schmidt kernels in c->d_gs: norms of start vectors first (gs_record(0)
-// doubles per right-hand side), then the two passes of an Arnoldi step, row by row.
-constexpr int kGsStart = 128;
-static_assert(kMaxBatch * gs_record(0) <= kGsStart && kMaxBatch <= 12, "");
+// doubles per right-hand side), then the two passes of an Arnoldi step, row by row. A solver that reads
+// its start record only after its first step (fgmres) has one of its own per nesting level, because its
+// preconditioner may be such a solver too.
+constexpr int kGsStart = 128, kGsLevels = 8;
+static_assert((kMaxBatch + kGsLevels) * gs_record(0) <= kGsStart && kMaxBatch <= 12, "");
+struct GsLevel {
+    Ctx *c;
+    int at;   // of the start record in d_gs
+    explicit GsLevel(Ctx *c_) : c(c_), at((kMaxBatch + c_->gs_level++) * gs_record(0)) {}
+    ~GsLevel() { c->gs_level--; }
+    bool ok() const { return c->gs_level <= kGsLevels; }
+};
 
-// V_0 = w / ||w|| for the rows (w: vector y at w + y n), ||w||^2 in the start records; no host wait.
+// V_0 = w / ||w|| for the rows (w: vector y at w + y n), ||w||^2 in the start records from `at`; no host wait.
 template <typename T>
-static ovl_status gs_start(Ctx *c, const T *w, T *v0, const RowList &rows) {
-    CK(gs_dots<T>(w, 0, 0, w, c->n64, rows, c->d_gs, gs_record(0), false, nullptr, c->d_md_part, c->gs_counters,
-                  c->stream));
+static ovl_status gs_start(Ctx *c, const T *w, T *v0, const RowList &rows, int at = 0) {
+    double *rec = c->d_gs + at;
+    CK(gs_dots<T>(w, 0, 0, w, c->n64, rows, rec, gs_record(0), false, nullptr, c->d_md_part, c->gs_counters, c->stream));
     // with one pass not enough and nothing to subtract, the second pass normalises
-    CK(gs_subtract<T>(w, 0, 0, c->d_gs, gs_record(0), c->d_gs, const_cast<T *>(w), v0, c->n64, rows, c->stream));
+    CK(gs_subtract<T>(w, 0, 0, rec, gs_record(0), rec, const_cast<T *>(w), v0, c->n64, rows, c->stream));
     return OVL_OK;
 }
 
 // One Arnoldi step of the rows: w against m basis vectors (entry i of row y at V + i stride + y n), V_m =
 // the normalised rest, by classical Gram-Schmidt, in FP64 always with a second pass (CGS2), in FP32
 // when the first one cancels most of w (the decision is made on the device). One wait for the host,
-// which gets h (m values per row) and hn; start (nullable): also the rows' ||w||^2 of gs_start.
+// which gets h (m values per row) and hn; start (nullable): also the rows' ||w||^2 of gs_start(.., at).
 template <typename T>
 static ovl_status gs_arnoldi(Ctx *c, T *V, long stride, int m, T *w, const RowList &rows, std::vector<std::vector<cd>> &h,
-                             std::vector<double> &hn, std::vector<double> *start = nullptr) {
+                             std::vector<double> &hn, std::vector<double> *start = nullptr, int at = 0) {
     const long n = c->n64, rec = gs_record(m), os = 2 * rec;
     double *first = c->d_gs + kGsStart, *second = first + rec;
     T *next = V + (long)m * stride;
@@ -137,7 +146,7 @@ static ovl_status gs_arnoldi(Ctx *c, T *V, long stride, int m, T *w, const RowLi
         const bool one = a[2 * m + 4] != 0.0;
         for (int i = 0; i < m; i++) h[r][i] = cd(a[2 * i], a[2 * i + 1]) + (one ? cd(0) : cd(b[2 * i], b[2 * i + 1]));
         hn[r] = one ? a[2 * m + 2] : b[2 * m + 2];
-        if (start) (*start)[r] = t[r * gs_record(0)];
+        if (start) (*start)[r] = t[at + r * gs_record(0)];
     }
     return OVL_OK;
 }
@@ -204,6 +213,11 @@ static ovl_status fgmres(Ctx *c, Krylov<T> &k, T *x, const T *b, double tol, int
     const long n = c->n64;
     const int m = k.m;
     const RowList one{1, {0}};
+    const GsLevel level(c);
+    if (!level.ok()) {
+        c->err = "Krylov solver: nested too deep";
+        return OVL_EINVAL;
+    }
     res->iters = 0;
     res->converged = false;
     bool xz = x_zero;
@@ -227,7 +241,7 @@ static ovl_status fgmres(Ctx *c, Krylov<T> &k, T *x, const T *b, double tol, int
     while (true) {
         std::fill(gv.begin(), gv.end(), cd(0));
         if (late) {
-            ST(gs_start(c, b, k.V, one));
+            ST(gs_start(c, b, k.V, one, level.at));
         } else {
             // r = b - A x
             const T *r = b;
@@ -238,8 +252,8 @@ static ovl_status fgmres(Ctx *c, Krylov<T> &k, T *x, const T *b, double tol, int
                 r = k.r;
             }
             double rr;
-            ST(gs_start(c, r, k.V, one));
-            ST(c->fetch(c->d_gs, 1, &rr));
+            ST(gs_start(c, r, k.V, one, level.at));
+            ST(c->fetch(c->d_gs + level.at, 1, &rr));
             const double beta = sqrt(rr);
             res->rel_res = beta / bnorm;
             if (!std::isfinite(beta)) {
@@ -265,7 +279,7 @@ static ovl_status fgmres(Ctx *c, Krylov<T> &k, T *x, const T *b, double tol, int
                 ST((*precond)(vj, zj));
             }
             ST(matvec(zj, k.w, rel_now));
-            ST(gs_arnoldi<T>(c, k.V, n, j + 1, k.w, one, hc, hnv, late ? &bb0 : nullptr));
+            ST(gs_arnoldi<T>(c, k.V, n, j + 1, k.w, one, hc, hnv, late ? &bb0 : nullptr, level.at));
             if (late) {
                 late = false;
                 bnorm = sqrt(bb0[0]);

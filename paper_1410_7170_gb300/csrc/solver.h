@@ -82,6 +82,7 @@ struct Ctx {
     double *d_coef = nullptr;     // multi-axpy coefficients
     double *d_gs = nullptr;       // Gram-Schmidt records (kScal doubles)
     double *d_gs_coef = nullptr, *h_gs_coef = nullptr;   // coefficients of x += Z y (12 x 256; pinned copy)
+    int gs_level = 0;             // solvers that are running inside one another (GsLevel)
     unsigned *gs_counters = nullptr;                     // per right-hand side, zero between launches
     // gauge field (12-real links)
     double2 *U64 = nullptr;
