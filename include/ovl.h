@@ -234,7 +234,8 @@ ovl_status wilson_sap_apply(ovl_ctx *ctx, double *out, const double *in, double 
 
 /* FP32 stencil variant chosen by the autotuner (threads per site, 1 or 4) and the measured ms
  * per full-lattice stencil application of each variant (ms[2], ms[3] = FP32 x1, x4). The FP64
- * stencil is one kernel (a warp per hop) at every size: *tps64 is 1, ms[0] = ms[1] its time. All
+ * stencil's form (a warp per hop, or a thread per site on some large lattices) follows from the
+ * lattice: *tps64 is 1, ms[0] = ms[1] its time. All
  * ms are zero when the variant is forced. Nullable outputs. */
 ovl_status ovl_tuning(const ovl_ctx *ctx, int *tps64, int *tps32, float *ms);
 

@@ -289,35 +289,36 @@ cudaError_t spinor_f2d(const Geom &g, const float4 *a, double2 *b, cudaStream_t 
 }
 
 // ------------------------------------------------------------------ stencil
-// out = a [g5] D_W(m0) in + b z in FP32, one thread per site. Bound: the latency of the neighbour gathers,
+// out = a [g5] D_W(m0) in + b z, one thread per site, in FP32 and (wilson_f64) on some lattices in FP64. Bound in FP32: the latency of the neighbour gathers,
 // which go to L2 three times in four, at 16 warps per SM (128 registers); at 64 x 32^3 with memory 60%
 // and the L1 data pipe 48% busy (168 us: 0.70 of the copy bandwidth). One wave of blocks that stride
 // over the lattice keeps the blocks
 // of an SM and their neighbours on other SMs close together in time: 32^4 107 -> 90 us, 24^4 40 -> 35,
 // 64 x 32^3 182 -> 170, 16^4 10.2 -> 9.2, against a block per 256 sites; with the order of
 // site_of_thread 81, 31.3, 168 and 8.3.
-__global__ void __launch_bounds__(kBlock, MinBlocks<float>::value)
-    k_wilson(Geom g, const float4 *__restrict__ U, const float4 *__restrict__ in, float4 *__restrict__ out, float m4,
-             int g5, float a, const float4 *z, float b, int spb) {
+template <typename R, typename ST>
+__global__ void __launch_bounds__(kBlock, MinBlocks<R>::value)
+    k_wilson(Geom g, const ST *__restrict__ U, const ST *__restrict__ in, ST *__restrict__ out, R m4, int g5, R a, const ST *z,
+             R b, int spb) {
     if (threadIdx.x >= spb) return;
     for (int t = blockIdx.x * spb + threadIdx.x; t < g.V; t += gridDim.x * spb) {
         int p, i;
         site_of_thread(t, p, i);
-        cpx<float> hop[12], own[12], res[12];
-        wilson_hop<float>(g, U, in, p, i, hop);
-        load_spinor<float>(in, g.Vh, p, i, own);
-        wilson_combine<float>(m4, own, hop, res);
+        cpx<R> hop[12], own[12], res[12];
+        wilson_hop<R>(g, U, in, p, i, hop);
+        load_spinor<R>(in, g.Vh, p, i, own);
+        wilson_combine<R>(m4, own, hop, res);
         if (g5) apply_g5(res);
         if (z) {
-            cpx<float> zz[12];
-            load_spinor<float>(z, g.Vh, p, i, zz);
+            cpx<R> zz[12];
+            load_spinor<R>(z, g.Vh, p, i, zz);
 #pragma unroll
             for (int c = 0; c < 12; c++) res[c] = a * res[c] + b * zz[c];
         } else {
 #pragma unroll
             for (int c = 0; c < 12; c++) res[c] = a * res[c];
         }
-        store_spinor<float>(out, g.Vh, p, i, res);
+        store_spinor<R>(out, g.Vh, p, i, res);
     }
 }
 
@@ -448,8 +449,18 @@ cudaError_t wilson_ff_lex(const Geom &g, const ffl *U, const ffw *in, double *le
     count_launches(1);
     return cudaGetLastError();
 }
+// FP64: one warp per hop, 1.60 ns a site at all sizes (2^19 sites and more); one thread per site takes 1.55 ns
+// over the part of its threads that have a site, and is taken where that is at least 97.5% of
+// them (whole waves of 304 blocks of 256): 28^4 0.987 -> 0.967 ms, 40 x 32^3 2.10 -> 2.05, 64 x 32^3
+// 3.35 -> 3.25, but 32^4 (96%) 1.680 against 1.687 and 30^4 (95%) 1.299 against 1.326.
 cudaError_t wilson_f64(const Geom &g, const double2 *U, const double2 *in, double2 *out, double m0, int g5,
                        double a, const double2 *z, double b, cudaStream_t st) {
+    const LaunchShape ls = balanced_shape(g.V, g.nsm, MinBlocks<double>::value, 1 << 30);
+    if (g.V >= 1 << 19 && g.V >= 0.975 * ls.grid * ls.block) {
+        k_wilson<double><<<ls.grid, ls.block, 0, st>>>(g, U, in, out, m0 + 4.0, g5, a, z, b, ls.spb);
+        count_launches(1);
+        return cudaGetLastError();
+    }
     return wilson_hops<double>(g, U, in, out, 0, 1, m0, g5, a, z, b, st);
 }
 cudaError_t wilson_batch_f64(const Geom &g, const double2 *U, const double2 *in, double2 *out, long stride, int nrhs,
@@ -468,7 +479,7 @@ cudaError_t wilson_f32(const Geom &g, const float4 *U, const float4 *in, float4 
                        float a, const float4 *z, float b, cudaStream_t st) {
     if (g.tps32 == 4) return wilson_hops<float>(g, U, in, out, 0, 1, m0, g5, a, z, b, st);
     const LaunchShape ls = balanced_shape(g.V, g.nsm, MinBlocks<float>::value, g.nsm * MinBlocks<float>::value);
-    k_wilson<<<ls.grid, ls.block, 0, st>>>(g, U, in, out, m0 + 4.0f, g5, a, z, b, ls.spb);
+    k_wilson<float><<<ls.grid, ls.block, 0, st>>>(g, U, in, out, m0 + 4.0f, g5, a, z, b, ls.spb);
     count_launches(1);
     return cudaGetLastError();
 }

@@ -31,6 +31,7 @@ struct RedScratch {
 // Minimum resident blocks per SM requested from the compiler for the one-thread-per-site stencils:
 // at 128 registers two 256-thread blocks fit on an SM (one wave of 256 blocks at 16^4 on 152 SMs).
 template <typename R> struct MinBlocks { static constexpr int value = 1; };
+template <> struct MinBlocks<double> { static constexpr int value = 2; };
 template <> struct MinBlocks<float> { static constexpr int value = 2; };
 
 // SMs of the current device (queried once per device and cached).

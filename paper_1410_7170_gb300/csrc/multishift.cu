@@ -188,35 +188,42 @@ struct ShiftFin {
     }
 };
 
+// A thread's sum over its sites
+template <typename R> struct SiteSum;
+template <> struct SiteSum<float> { using type = fsum; };
+template <> struct SiteSum<double> { using type = double; };
+__device__ __forceinline__ void sum_add(fsum &s, float x) { s.add(x); }
+__device__ __forceinline__ void sum_add(double &s, double x) { s += x; }
+
 // One thread per site (FP32), right-hand side blockIdx.y: t = gamma5 D_W(m) p_0 ; ||t||^2 (OWN: and
 // ||p_0||^2) -> alpha.
-template <bool OWN>
-__global__ void __launch_bounds__(kBlock, MinBlocks<float>::value)
-    k_ms_q_site(Geom g, const float4 *__restrict__ U, float m4, MsState *st, MsBatch<float4> v, RedScratch rs, int spb) {
+template <typename R, bool OWN, typename ST>
+__global__ void __launch_bounds__(kBlock, MinBlocks<R>::value)
+    k_ms_q_site(Geom g, const ST *__restrict__ U, R m4, MsState *st, MsBatch<ST> v, RedScratch rs, int spb) {
     MsState *s = st + blockIdx.y;
     if (s->done) return;
-    const float4 *__restrict__ p0 = v.p0_at(blockIdx.y, s->iter);
-    float4 *__restrict__ t = v.t + blockIdx.y * v.stride;
-    fsum sum[1 + OWN];   // a site's sum in FP32, a thread's and a warp's with their errors, then FP64 (grid_reduce)
+    const ST *__restrict__ p0 = v.p0_at(blockIdx.y, s->iter);
+    ST *__restrict__ t = v.t + blockIdx.y * v.stride;
+    typename SiteSum<R>::type sum[1 + OWN] = {};   // a site's sum in FP32, a thread's and a warp's with their errors, then FP64 (grid_reduce)
     const bool lane_has_sites = threadIdx.x < spb;
     for (int k = blockIdx.x * spb + threadIdx.x; lane_has_sites && k < g.V; k += gridDim.x * spb) {
         int p, i;
         site_of_thread(k, p, i);
-        cpx<float> hop[12], own[12], res[12];
-        wilson_hop<float>(g, U, p0, p, i, hop);
-        load_spinor<float>(p0, g.Vh, p, i, own);
-        wilson_combine<float>(m4, own, hop, res);
+        cpx<R> hop[12], own[12], res[12];
+        wilson_hop<R>(g, U, p0, p, i, hop);
+        load_spinor<R>(p0, g.Vh, p, i, own);
+        wilson_combine<R>(m4, own, hop, res);
         apply_g5(res);
-        store_spinor<float>(t, g.Vh, p, i, res);
-        float a0 = 0.f;
+        store_spinor<R>(t, g.Vh, p, i, res);
+        R a0 = 0;
 #pragma unroll
         for (int c = 0; c < 12; c++) a0 += norm2(res[c]);
-        sum[0].add(a0);
+        sum_add(sum[0], a0);
         if (OWN) {
-            a0 = 0.f;
+            a0 = 0;
 #pragma unroll
             for (int c = 0; c < 12; c++) a0 += norm2(own[c]);
-            sum[OWN].add(a0);
+            sum_add(sum[OWN], a0);
         }
     }
     grid_reduce<1 + OWN>(sum, rs.row(blockIdx.y), AlphaFin<OWN>{s});
@@ -224,43 +231,43 @@ __global__ void __launch_bounds__(kBlock, MinBlocks<float>::value)
 
 // r_{k+1} = r_k - alpha (gamma5 D_W(m) t + sigma0 p0) ; ||r_{k+1}||^2 -> shift scalars. Block 0 takes no
 // sites: it forms the shift scalars that need only alpha_k while the others compute (ShiftScalars).
-__global__ void __launch_bounds__(kBlock, MinBlocks<float>::value)
-    k_ms_r_site(Geom g, const float4 *__restrict__ U, float m4, MsState *st, MsBatch<float4> v, RedScratch rs, int spb) {
+template <typename R, typename ST>
+__global__ void __launch_bounds__(kBlock, MinBlocks<R>::value)
+    k_ms_r_site(Geom g, const ST *__restrict__ U, R m4, MsState *st, MsBatch<ST> v, RedScratch rs, int spb) {
     MsState *s = st + blockIdx.y;
     if (s->done) return;
-    fsum sum;
+    typename SiteSum<R>::type sum[1] = {};
     if (blockIdx.x == 0) {
         if (threadIdx.x < 32) ShiftScalars{s}(threadIdx.x);
     } else {
         const int it = s->iter;
-        const float4 *__restrict__ p0 = v.p0_at(blockIdx.y, it);
-        const float4 *__restrict__ t = v.t + blockIdx.y * v.stride;
-        const float4 *rin = v.r_at(blockIdx.y, it);
-        float4 *rout = v.r_at(blockIdx.y, it + 1);
-        const float ma = -s->alpha_f[0], sig0 = s->sigma0_f[0];
+        const ST *__restrict__ p0 = v.p0_at(blockIdx.y, it);
+        const ST *__restrict__ t = v.t + blockIdx.y * v.stride;
+        const ST *rin = v.r_at(blockIdx.y, it);
+        ST *rout = v.r_at(blockIdx.y, it + 1);
+        const R ma = HopTiles<R>::minus_alpha(*s), sig0 = HopTiles<R>::sigma0(*s);
         const bool lane_has_sites = threadIdx.x < spb;
         for (int k = (blockIdx.x - 1) * spb + threadIdx.x; lane_has_sites && k < g.V; k += (gridDim.x - 1) * spb) {
             int p, i;
             site_of_thread(k, p, i);
-            cpx<float> hop[12], own[12], res[12], pp[12], rv[12];
-            wilson_hop<float>(g, U, t, p, i, hop);
-            load_spinor<float>(t, g.Vh, p, i, own);
-            wilson_combine<float>(m4, own, hop, res);
+            cpx<R> hop[12], own[12], res[12], pp[12], rv[12];
+            wilson_hop<R>(g, U, t, p, i, hop);
+            load_spinor<R>(t, g.Vh, p, i, own);
+            wilson_combine<R>(m4, own, hop, res);
             apply_g5(res);
-            load_spinor<float>(p0, g.Vh, p, i, pp);
-            load_spinor<float>(rin, g.Vh, p, i, rv);
-            float a0 = 0.f;
+            load_spinor<R>(p0, g.Vh, p, i, pp);
+            load_spinor<R>(rin, g.Vh, p, i, rv);
+            R a0 = 0;
 #pragma unroll
             for (int c = 0; c < 12; c++) {
                 rv[c] = rv[c] + ma * (res[c] + sig0 * pp[c]);
                 a0 += norm2(rv[c]);
             }
-            sum.add(a0);
-            store_spinor<float>(rout, g.Vh, p, i, rv);
+            sum_add(sum[0], a0);
+            store_spinor<R>(rout, g.Vh, p, i, rv);
         }
     }
-    const fsum w[1] = {sum};
-    grid_reduce_warp<1>(w, rs.row(blockIdx.y), ShiftFin{s});
+    grid_reduce_warp<1>(sum, rs.row(blockIdx.y), ShiftFin{s});
 }
 
 // Elementwise arithmetic on storage words: V is a word in registers, C a real coefficient in the
@@ -647,35 +654,44 @@ cudaError_t ms_stencils_hops(const Geom &g, const LT *U, double m0, MsRows nrhs,
     k_ms_r_hops<R><<<dim3(gr, nrhs.n), kHopBlock, 0, st>>>(g, U, R(m0 + 4.0), s, v, rows);
     return ev.record(2, st);
 }
-// FP32, one thread per site
-cudaError_t ms_stencils_site(const Geom &g, const float4 *U, float m0, MsRows nrhs, MsState *s, const MsBatch<float4> &v,
+// One thread per site, in FP32 and for one right-hand side in FP64 (ms_fp64_per_site). FP32: one wave of
+// blocks that stride over the sites (at 32^4 thirteen waves, each block ending with a fence and an atomic,
+// cost 20 us of 125; the whole FP32 sign at 32^4 14.67 ms, with the order of site_of_thread 14.17).
+// FP64, ten times as long a site: as many blocks as the reduction's scratch holds, which even out what
+// a last wave leaves.
+template <typename R, typename ST>
+cudaError_t ms_stencils_site(const Geom &g, const ST *U, R m0, MsRows nrhs, MsState *s, const MsBatch<ST> &v,
                              const RedScratch &rows, cudaStream_t st, const MsEvents &ev) {
-    const int slots = std::max(1, g.nsm * MinBlocks<float>::value / nrhs.of);   // resident blocks of a row
-    // one wave of blocks that stride over the sites (at 32^4 thirteen waves, each block ending with a
-    // fence and an atomic, cost 20 us of 125; the whole FP32 sign at 32^4 14.67 ms, with the order of
-    // site_of_thread 14.17)
-    const LaunchShape q = balanced_shape(g.V, slots, 1, slots);
-    const LaunchShape r = balanced_shape(g.V, std::max(1, slots - 1), 1, std::max(1, slots - 1));
+    constexpr bool fp64 = std::is_same<R, double>::value;
+    const int slots = std::max(1, g.nsm * MinBlocks<R>::value / nrhs.of);   // resident blocks of a row
+    const LaunchShape q = fp64 ? balanced_shape(g.V, slots, 1, kMaxRedBlocks - 1) : balanced_shape(g.V, slots, 1, slots);
+    const LaunchShape r = fp64 ? q : balanced_shape(g.V, std::max(1, slots - 1), 1, std::max(1, slots - 1));
     cudaError_t e;
     if ((e = ev.record(0, st)) != cudaSuccess) return e;
-    if (nrhs.of > 1) k_ms_q_site<true><<<dim3(q.grid, nrhs.n), q.block, 0, st>>>(g, U, m0 + 4.f, s, v, rows, q.spb);
-    else k_ms_q_site<false><<<dim3(q.grid, nrhs.n), q.block, 0, st>>>(g, U, m0 + 4.f, s, v, rows, q.spb);
+    if (!fp64 && nrhs.of > 1)
+        k_ms_q_site<R, !fp64><<<dim3(q.grid, nrhs.n), q.block, 0, st>>>(g, U, m0 + (R)4, s, v, rows, q.spb);
+    else k_ms_q_site<R, false><<<dim3(q.grid, nrhs.n), q.block, 0, st>>>(g, U, m0 + (R)4, s, v, rows, q.spb);
     if ((e = ev.record(1, st)) != cudaSuccess) return e;
-    k_ms_r_site<<<dim3(r.grid + 1, nrhs.n), r.block, 0, st>>>(g, U, m0 + 4.f, s, v, rows, r.spb);
+    k_ms_r_site<R><<<dim3(r.grid + 1, nrhs.n), r.block, 0, st>>>(g, U, m0 + (R)4, s, v, rows, r.spb);
     return ev.record(2, st);
 }
+// FP64: one warp per hop, or on large lattices one thread per site. The whole sign (ms) with the one and
+// the other: 24^4 126.4 / 127.9, 30^4 304.9 / 313.7, 32^4 394.8 / 382.3, 48 x 32^3 590.9 / 582.9, 64 x 32^3
+// 894.9 / 872.3, 40^4 1063 / 1039; in batches, which have fewer blocks a row, 2 at 24^4 253.8 / 265.0, 8
+// at 24^4 1018 / 1059, 2 at 32^4 787 / 778.
+inline bool ms_fp64_per_site(const Geom &g, MsRows nrhs) { return nrhs.of == 1 && g.V >= 1 << 20; }
 
 template <typename R, typename LT, typename ST>
 cudaError_t ms_iter_t(const Geom &g, const LT *U, double m0, MsRows nrhs, MsState *s, MsBatch<ST> v, RedScratch rs,
                       unsigned *counters, bool flush, cudaStream_t st, const MsEvents &ev) {
     const RedScratch rows{rs.partials, counters};
     cudaError_t e;
-    if constexpr (sizeof(R) == 4) {
-        e = g.tps32 == 4 ? ms_stencils_hops<R>(g, U, m0, nrhs, s, v, rows, st, ev)
-                         : ms_stencils_site(g, U, (float)m0, nrhs, s, v, rows, st, ev);
-    } else {
-        e = ms_stencils_hops<R>(g, U, m0, nrhs, s, v, rows, st, ev);
+    bool per_site = false;
+    if constexpr (!std::is_same<R, ff>::value) {
+        per_site = sizeof(R) == 4 ? g.tps32 != 4 : ms_fp64_per_site(g, nrhs);
+        if (per_site) e = ms_stencils_site<R>(g, U, (R)m0, nrhs, s, v, rows, st, ev);
     }
+    if (!per_site) e = ms_stencils_hops<R>(g, U, m0, nrhs, s, v, rows, st, ev);
     if (e != cudaSuccess || (e = ms_third(g, nrhs, s, v, counters, flush, st)) != cudaSuccess ||
         (e = ev.record(3, st)) != cudaSuccess)
         return e;
@@ -732,7 +748,7 @@ cudaError_t ms_init_half(const Geom &g, int n, MsState *s, MsVectorsH v, const f
 cudaError_t ms_iter_half(const Geom &g, const float4 *U, double m0, MsState *s, MsVectorsH v, RedScratch rs, bool bf16,
                          cudaStream_t st, const MsEvents &ev) {
     const MsBatch<float4> w{v.r, v.p0, v.t, v.y, nullptr, v.words, 0, 1};
-    cudaError_t e = ms_stencils_site(g, U, (float)m0, 1, s, w, RedScratch{rs.partials, rs.counter}, st, ev);
+    cudaError_t e = ms_stencils_site<float>(g, U, (float)m0, 1, s, w, RedScratch{rs.partials, rs.counter}, st, ev);
     if (e != cudaSuccess) return e;
     const int gsh = balanced_shape(g.V, g.nsm, 2, 1 << 30).grid;
     if (bf16) k_ms_shifts_half<true><<<gsh, kBlock, 0, st>>>(g, s, v, rs.counter);
