@@ -620,9 +620,9 @@ ovl_status Ctx::ensure_batch() {
     void *buf;
     ST(alloc(&buf, sizeof(MsState) * kMaxBatch));
     msb_state = (MsState *)buf;
-    ST(alloc(&buf, sizeof(double) * (size_t)kMaxBatch * kRowRedValues * kMaxRedBlocks + 256));
+    ST(alloc(&buf, sizeof(double) * (size_t)kMaxBatch * kMaxRedBlocks + 256));
     rsb.partials = (double *)buf;
-    rsb.counter = (unsigned *)((char *)buf + sizeof(double) * (size_t)kMaxBatch * kRowRedValues * kMaxRedBlocks);
+    rsb.counter = (unsigned *)((char *)buf + sizeof(double) * (size_t)kMaxBatch * kMaxRedBlocks);
     ST(alloc(&buf, sizeof(unsigned) * kMaxBatch));
     bcounters = (unsigned *)buf;
     CK(cudaMemsetAsync(rsb.counter, 0, sizeof(unsigned), stream));

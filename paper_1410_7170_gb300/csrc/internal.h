@@ -15,17 +15,14 @@ constexpr int kMaxPoles = 64;
 constexpr int kBlock = 256;             // threads per block of site-parallel kernels
 constexpr int kMaxRedBlocks = 4096;     // cap on blocks of a reducing kernel (grid-stride beyond)
 constexpr int kMaxRedValues = 4;        // doubles reduced by one kernel
-constexpr int kRowRedValues = 2;        // and by each grid row of a kernel for several right-hand sides
 
 // Scratch of the deterministic two-level reductions: per-block partial sums, and
 // a counter the last finishing block uses to find that it is last.
 struct RedScratch {
     double *partials;      // [kMaxRedValues][kMaxRedBlocks]
     unsigned *counter;     // one word, zero between launches
-    // of grid row y, where each has up to kRowRedValues reduced values and a counter of its own
-    __device__ RedScratch row(int y) const {
-        return RedScratch{partials + (size_t)y * kRowRedValues * kMaxRedBlocks, counter + y};
-    }
+    // of grid row y, where each has one reduced value and a counter of its own
+    __device__ RedScratch row(int y) const { return RedScratch{partials + (size_t)y * kMaxRedBlocks, counter + y}; }
 };
 
 // Minimum resident blocks per SM requested from the compiler for the one-thread-per-site stencils:
@@ -268,7 +265,7 @@ struct MsRows {
 // One multishift iteration of nrhs right-hand sides (state st[y]; grid row y) = three launches: Q p,
 // residual update, and p_0 or, where flush is set, the pending shift updates with it. A caller sets
 // flush at least in every ring-th iteration, and in the last one before it reads y or the state.
-// rs.partials: nrhs * kRowRedValues * kMaxRedBlocks doubles; counters: nrhs words, zero between launches.
+// rs.partials: nrhs * kMaxRedBlocks doubles; counters: nrhs words, zero between launches.
 cudaError_t ms_init(const Geom &g, MsRows nrhs, MsState *s, MsBatch<double2> v, const double2 *b, RedScratch rs,
                     unsigned *counters, cudaStream_t st);
 cudaError_t ms_init(const Geom &g, MsRows nrhs, MsState *s, MsBatch<float4> v, const float4 *b, RedScratch rs,

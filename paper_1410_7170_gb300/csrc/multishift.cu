@@ -61,11 +61,11 @@ __device__ __forceinline__ void store_ff(float *to, double x) {
     to[1] = f.lo;
 }
 
-// alpha = (r, r) / (p, (Q^2 + sigma_0) p) with (p, Q^2 p) = ||Q p||^2 (v[0], reduced by ms_q). ||p||^2 of one
+// alpha = (r, r) / (p, (Q^2 + sigma_0) p) with (p, Q^2 p) = ||Q p||^2, reduced by ms_q. ||p||^2 of one
 // right-hand side comes from the scalar recurrence ||p_k||^2 = ||r_k||^2 + beta^2 ||p_{k-1}||^2, which
-// holds because r_k is orthogonal to p_{k-1} in CG; this spares ms_q a second reduction. Batches (OWN)
-// reduce it too, v[1]: in FP32 the recurrence drifts to 5e-7 in 40 iterations (16^4), the sum is good to
-// 1e-9. Float-float batches use the recurrence, as one right-hand side does.
+// holds because r_k is orthogonal to p_{k-1} in CG; this spares ms_q the sum. Batches (OWN) sum it, into the
+// same number, ||Q p||^2 + sigma_0 ||p||^2: in FP32 the recurrence drifts to 5e-7 in 40 iterations (16^4),
+// the sum is good to 1e-9. Float-float batches use the recurrence, as one right-hand side does.
 template <bool OWN>
 struct AlphaFin {
     MsState *s;
@@ -74,8 +74,7 @@ struct AlphaFin {
     };
     __device__ In before() const { return {s->sigma[0], s->pp, s->rr}; }
     __device__ void operator()(const double *v, const In &in) const {
-        const double pp = OWN ? v[OWN] : in.pp;
-        const double pAp = v[0] + in.sigma0 * pp;
+        const double pAp = OWN ? v[0] : v[0] + in.sigma0 * in.pp;
         const double a = in.rr / pAp;
         if (!(pAp > 0.0) || !isfinite(a)) {
             s->status = 1;
@@ -84,9 +83,15 @@ struct AlphaFin {
         }
         s->alpha = a;
         store_ff(s->alpha_f, a);
-        if (OWN) s->pp = pp;
     }
 };
+// sum + sigma_0 b for a thread's sums of ||Q p||^2 and ||p||^2; in FP32 with both words of sigma_0, whose
+// rounding all threads would share
+__device__ __forceinline__ void add_shifted(const MsState &s, double b, double &sum) { sum = fma_r(s.sigma[0], b, sum); }
+__device__ __forceinline__ void add_shifted(const MsState &s, const fsum &b, fsum &sum) {
+    sum.add(__fmul_rn(s.sigma0_f[0], b.s));
+    sum.add(fma_r(s.sigma0_f[1], b.s, __fmul_rn(s.sigma0_f[0], b.e)));
+}
 
 // Shift scalars of an iteration, in two parts, one lane per shift (lane j: shifts j, j + 32). A
 // dependent FP64 instruction takes 64 clocks or more on GB300 (half a lane per clock and scheduler),
@@ -195,8 +200,8 @@ template <> struct SiteSum<double> { using type = double; };
 __device__ __forceinline__ void sum_add(fsum &s, float x) { s.add(x); }
 __device__ __forceinline__ void sum_add(double &s, double x) { s += x; }
 
-// One thread per site (FP32), right-hand side blockIdx.y: t = gamma5 D_W(m) p_0 ; ||t||^2 (OWN: and
-// ||p_0||^2) -> alpha.
+// One thread per site (FP32; FP64 on large lattices), right-hand side blockIdx.y:
+// t = gamma5 D_W(m) p_0 ; ||t||^2 (OWN: + sigma_0 ||p_0||^2) -> alpha.
 template <typename R, bool OWN, typename ST>
 __global__ void __launch_bounds__(kBlock, MinBlocks<R>::value)
     k_ms_q_site(Geom g, const ST *__restrict__ U, R m4, MsState *st, MsBatch<ST> v, RedScratch rs, int spb) {
@@ -204,7 +209,8 @@ __global__ void __launch_bounds__(kBlock, MinBlocks<R>::value)
     if (s->done) return;
     const ST *__restrict__ p0 = v.p0_at(blockIdx.y, s->iter);
     ST *__restrict__ t = v.t + blockIdx.y * v.stride;
-    typename SiteSum<R>::type sum[1 + OWN] = {};   // a site's sum in FP32, a thread's and a warp's with their errors, then FP64 (grid_reduce)
+    // FP32: a site's sum plain, a thread's and a warp's with their errors, then FP64 (grid_reduce)
+    typename SiteSum<R>::type sum[1] = {}, psum = {};
     const bool lane_has_sites = threadIdx.x < spb;
     for (int k = blockIdx.x * spb + threadIdx.x; lane_has_sites && k < g.V; k += gridDim.x * spb) {
         int p, i;
@@ -223,10 +229,11 @@ __global__ void __launch_bounds__(kBlock, MinBlocks<R>::value)
             a0 = 0;
 #pragma unroll
             for (int c = 0; c < 12; c++) a0 += norm2(own[c]);
-            sum_add(sum[OWN], a0);
+            sum_add(psum, a0);
         }
     }
-    grid_reduce<1 + OWN>(sum, rs.row(blockIdx.y), AlphaFin<OWN>{s});
+    if (OWN) add_shifted(*s, psum, sum[0]);
+    grid_reduce<1>(sum, rs.row(blockIdx.y), AlphaFin<OWN>{s});
 }
 
 // r_{k+1} = r_k - alpha (gamma5 D_W(m) t + sigma0 p0) ; ||r_{k+1}||^2 -> shift scalars. Block 0 takes no
@@ -445,9 +452,9 @@ __global__ void __launch_bounds__(kHopBlock, HopBlocks<R>::value)
         H::square_add(w, sum);
         if (OWN) H::square_add(o, psum);
     });
-    decltype(H::total(sum)) w[1 + OWN] = {H::total(sum)};
-    if (OWN) w[OWN] = H::total(psum);
-    grid_reduce<1 + OWN>(w, rs.row(blockIdx.y), AlphaFin<OWN>{s});
+    if constexpr (OWN) add_shifted(*s, psum, sum);
+    const decltype(H::total(sum)) w[1] = {H::total(sum)};
+    grid_reduce<1>(w, rs.row(blockIdx.y), AlphaFin<OWN>{s});
 }
 
 template <typename R>

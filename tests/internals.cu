@@ -96,9 +96,9 @@ static int ms_probe(const Geom &g, const LT *U, int nrhs, int ring, long words, 
     const long v = words * nrhs;
     cudaError_t e = cudaMalloc(&d, (size_t)v * ms_vectors(n, ring) * sizeof(ST));
     if (e == cudaSuccess) e = cudaMalloc(&s, sizeof(MsState) * nrhs);
-    if (e == cudaSuccess) e = cudaMalloc(&part, sizeof(double) * kRowRedValues * kMaxRedBlocks * nrhs + 256);
+    if (e == cudaSuccess) e = cudaMalloc(&part, sizeof(double) * kMaxRedBlocks * nrhs + 256);
     if (e == cudaSuccess) {
-        unsigned *cnt = (unsigned *)(part + (size_t)kRowRedValues * kMaxRedBlocks * nrhs);
+        unsigned *cnt = (unsigned *)(part + (size_t)kMaxRedBlocks * nrhs);
         const MsBatch<ST> w{d, d + v * ring, d + 2 * v * ring, d + (2 * ring + 1) * v, d + (2 * ring + 2) * v, words,
                             words * (n - 1), ring};
         cudaMemset(cnt, 0, 256);
