@@ -236,17 +236,16 @@ __global__ void __launch_bounds__(kBlock, MinBlocks<R>::value)
     grid_reduce<1>(sum, rs.row(blockIdx.y), AlphaFin<OWN>{s});
 }
 
-// r_{k+1} = r_k - alpha (gamma5 D_W(m) t + sigma0 p0) ; ||r_{k+1}||^2 -> shift scalars. Block 0 takes no
-// sites: it forms the shift scalars that need only alpha_k while the others compute (ShiftScalars).
+// r_{k+1} = r_k - alpha (gamma5 D_W(m) t + sigma0 p0) ; ||r_{k+1}||^2 -> shift scalars. Block 0 forms the shift
+// scalars that need only alpha_k (ShiftScalars); it takes no sites, unless `share` is set (ms_share).
 template <typename R, typename ST>
 __global__ void __launch_bounds__(kBlock, MinBlocks<R>::value)
-    k_ms_r_site(Geom g, const ST *__restrict__ U, R m4, MsState *st, MsBatch<ST> v, RedScratch rs, int spb) {
+    k_ms_r_site(Geom g, const ST *__restrict__ U, R m4, MsState *st, MsBatch<ST> v, RedScratch rs, int spb, bool share) {
     MsState *s = st + blockIdx.y;
     if (s->done) return;
     typename SiteSum<R>::type sum[1] = {};
-    if (blockIdx.x == 0) {
-        if (threadIdx.x < 32) ShiftScalars{s}(threadIdx.x);
-    } else {
+    if (blockIdx.x == 0 && threadIdx.x < 32) ShiftScalars{s}(threadIdx.x);
+    if (share || blockIdx.x) {
         const int it = s->iter;
         const ST *__restrict__ p0 = v.p0_at(blockIdx.y, it);
         const ST *__restrict__ t = v.t + blockIdx.y * v.stride;
@@ -254,7 +253,8 @@ __global__ void __launch_bounds__(kBlock, MinBlocks<R>::value)
         ST *rout = v.r_at(blockIdx.y, it + 1);
         const R ma = HopTiles<R>::minus_alpha(*s), sig0 = HopTiles<R>::sigma0(*s);
         const bool lane_has_sites = threadIdx.x < spb;
-        for (int k = (blockIdx.x - 1) * spb + threadIdx.x; lane_has_sites && k < g.V; k += (gridDim.x - 1) * spb) {
+        const int first = blockIdx.x - !share, blocks = gridDim.x - !share;
+        for (int k = first * spb + threadIdx.x; lane_has_sites && k < g.V; k += blocks * spb) {
             int p, i;
             site_of_thread(k, p, i);
             cpx<R> hop[12], own[12], res[12], pp[12], rv[12];
@@ -460,7 +460,7 @@ __global__ void __launch_bounds__(kHopBlock, HopBlocks<R>::value)
 template <typename R>
 __global__ void __launch_bounds__(kHopBlock, HopBlocks<R>::value)
     k_ms_r_hops(Geom g, const typename HopTiles<R>::Link *__restrict__ U, R m4, MsState *st,
-                MsBatch<typename HopTiles<R>::Store> v, RedScratch rs) {
+                MsBatch<typename HopTiles<R>::Store> v, RedScratch rs, bool share) {
     using H = HopTiles<R>;
     using E = typename H::Elem;
     MsState *s = st + blockIdx.y;
@@ -472,7 +472,7 @@ __global__ void __launch_bounds__(kHopBlock, HopBlocks<R>::value)
     typename H::Store *rout = v.r_at(blockIdx.y, it0 + 1);
     typename H::Sum sum = H::zero();
     if (blockIdx.x == 0 && threadIdx.x < 32) ShiftScalars{s}(threadIdx.x);
-    const int first = blockIdx.x ? blockIdx.x - 1 : g.V;   // block 0: past the last tile
+    const int first = share ? blockIdx.x : blockIdx.x ? blockIdx.x - 1 : g.V;   // block 0: past the last tile
     const auto fm = H::factor(m4), fa = H::minus_alpha(*s), fs = H::sigma0(*s);
     struct Own {
         E t, p0, r;
@@ -480,7 +480,7 @@ __global__ void __launch_bounds__(kHopBlock, HopBlocks<R>::value)
     const auto own = [&](int p, int i, int it, int e) {
         return Own{H::load(t, g.Vh, p, i, it, e), H::load(p0, g.Vh, p, i, it, e), H::load_rw(rin, g.Vh, p, i, it, e)};
     };
-    hop_tiles<R>(g, first, gridDim.x - 1, U, t, own, [&](int p, int i, int it, int e, E hop, int, const Own &o) {
+    hop_tiles<R>(g, first, gridDim.x - !share, U, t, own, [&](int p, int i, int it, int e, E hop, int, const Own &o) {
         E w = H::fma(fm, o.t, hop);
         w = H::fma(fs, o.p0, H::neg_if(w, H::upper(it)));
         w = H::fma(fa, w, o.r);
@@ -645,6 +645,12 @@ cudaError_t ms_third(const Geom &g, MsRows nrhs, MsState *s, const MsBatch<ST> &
     return cudaGetLastError();
 }
 
+// Whether block 0 of a residual kernel takes its share of a row's `turns` per block after the shift
+// scalars (3 us) instead of none: a batch has few blocks a row (38 of 456 for 12 right-hand sides in FP64, 25 of
+// 304 in FP32), and one without work costs as much as the row's 1/blocks. A turn takes 4 to 12 us, so the
+// line is safely where a block has as many turns as there are blocks.
+inline bool ms_share(long turns, int blocks) { return turns >= blocks; }
+
 // One iteration of nrhs right-hand sides, one warp per hop.
 template <typename R, typename LT, typename ST>
 cudaError_t ms_stencils_hops(const Geom &g, const LT *U, double m0, MsRows nrhs, MsState *s, const MsBatch<ST> &v,
@@ -657,8 +663,9 @@ cudaError_t ms_stencils_hops(const Geom &g, const LT *U, double m0, MsRows nrhs,
     else k_ms_q_hops<R, false><<<dim3(gx, nrhs.n), kHopBlock, 0, st>>>(g, U, R(m0 + 4.0), s, v, rows);
     if ((e = ev.record(1, st)) != cudaSuccess) return e;
     // one block more for the shift scalars, within the wave
-    const int gr = (long)gx * nrhs.of + nrhs.of > (long)g.nsm * HopBlocks<R>::value && gx > 1 ? gx : gx + 1;
-    k_ms_r_hops<R><<<dim3(gr, nrhs.n), kHopBlock, 0, st>>>(g, U, R(m0 + 4.0), s, v, rows);
+    const bool full = (long)gx * nrhs.of + nrhs.of > (long)g.nsm * HopBlocks<R>::value && gx > 1;
+    const bool share = full && ms_share(hop_grid<R>(g, 1, false) / gx, gx);
+    k_ms_r_hops<R><<<dim3(full ? gx : gx + 1, nrhs.n), kHopBlock, 0, st>>>(g, U, R(m0 + 4.0), s, v, rows, share);
     return ev.record(2, st);
 }
 // One thread per site, in FP32 and for one right-hand side in FP64 (ms_fp64_per_site). FP32: one wave of
@@ -672,14 +679,15 @@ cudaError_t ms_stencils_site(const Geom &g, const ST *U, R m0, MsRows nrhs, MsSt
     constexpr bool fp64 = std::is_same<R, double>::value;
     const int slots = std::max(1, g.nsm * MinBlocks<R>::value / nrhs.of);   // resident blocks of a row
     const LaunchShape q = fp64 ? balanced_shape(g.V, slots, 1, kMaxRedBlocks - 1) : balanced_shape(g.V, slots, 1, slots);
-    const LaunchShape r = fp64 ? q : balanced_shape(g.V, std::max(1, slots - 1), 1, std::max(1, slots - 1));
+    const bool share = !fp64 && ms_share(g.V / (slots * kBlock), slots);
+    const LaunchShape r = fp64 || share ? q : balanced_shape(g.V, std::max(1, slots - 1), 1, std::max(1, slots - 1));
     cudaError_t e;
     if ((e = ev.record(0, st)) != cudaSuccess) return e;
     if (!fp64 && nrhs.of > 1)
         k_ms_q_site<R, !fp64><<<dim3(q.grid, nrhs.n), q.block, 0, st>>>(g, U, m0 + (R)4, s, v, rows, q.spb);
     else k_ms_q_site<R, false><<<dim3(q.grid, nrhs.n), q.block, 0, st>>>(g, U, m0 + (R)4, s, v, rows, q.spb);
     if ((e = ev.record(1, st)) != cudaSuccess) return e;
-    k_ms_r_site<R><<<dim3(r.grid + 1, nrhs.n), r.block, 0, st>>>(g, U, m0 + (R)4, s, v, rows, r.spb);
+    k_ms_r_site<R><<<dim3(r.grid + !share, nrhs.n), r.block, 0, st>>>(g, U, m0 + (R)4, s, v, rows, r.spb, share);
     return ev.record(2, st);
 }
 // FP64: one warp per hop, or on large lattices one thread per site. The whole sign (ms) with the one and

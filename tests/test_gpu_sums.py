@@ -61,15 +61,16 @@ def test_gram_schmidt_dots_f32(lib, sites, m, rows):
             assert err < tol * (ww.sqrt() * vd.norm()).item()
 
 
-def multishift(lib, dims, dtype, tps, rows, ring, iters, seed, sigma0=0.01):
-    """ms_probe on random links: (scalars [rows][5], t, r, p_0 as [rows][24 V])."""
+def multishift(lib, dims, dtype, tps, rows, ring, iters, seed, sigma0=0.01, b=None):
+    """ms_probe on random links (and vectors unless given): (scalars [rows][5], t, r, p_0 as [rows][24 V])."""
     V = dims[0] * dims[1] * dims[2] * dims[3]
     gen = torch.Generator("cuda")
     gen.manual_seed(seed)
     u = torch.linalg.qr(torch.complex(*torch.randn((2, 4096, 4, 3, 3), dtype=torch.float64, device="cuda", generator=gen)))[0]
     u = u / torch.linalg.det(u).pow(1 / 3)[..., None, None]
     u = u[torch.randint(0, 4096, (V,), device="cuda", generator=gen)].contiguous()
-    b = torch.randn((rows, 24 * V), dtype=dtype, device="cuda", generator=gen)
+    if b is None:
+        b = torch.randn((rows, 24 * V), dtype=dtype, device="cuda", generator=gen)
     t, r, p = torch.zeros_like(b), torch.zeros_like(b), torch.zeros_like(b)
     scal = (ctypes.c_double * (5 * rows))()
     torch.cuda.synchronize()
@@ -109,3 +110,16 @@ def test_direction_norm_of_a_batch(lib, dtype, tps, dims, rows):
     got = (before[:, 1] / after[:, 3] - tt) / sigma0
     eps = bar(24, b.shape[1]) if dtype == torch.float32 else 1e-14
     assert ((got / pp - 1).abs() < eps * (1 + tt / (sigma0 * pp))).all()
+
+
+@pytest.mark.parametrize("dtype,tps,dims", [(torch.float64, 1, (14, 12, 12, 12)), (torch.float64, 1, (12, 10, 10, 10)),
+                                            (torch.float32, 1, (20, 20, 20, 20)), (torch.float32, 1, (16, 16, 16, 16)),
+                                            (torch.float32, 4, (20, 20, 20, 20))])
+def test_rows_of_a_batch_cover_the_lattice(lib, dtype, tps, dims):
+    """r, t and p_0 of twelve right-hand sides after three iterations against one alone, on either side of the
+    size from which block 0 takes sites too. The scalars differ by rounding: 100 units of the arithmetic."""
+    _, b, t, r, p = multishift(lib, dims, dtype, tps, 12, 2, 3, 61)
+    for y in (0, 11):
+        _, _, t1, r1, p1 = multishift(lib, dims, dtype, tps, 1, 2, 3, 61, b=b[y:y + 1].contiguous())
+        for x, x1 in ((t[y], t1[0]), (r[y], r1[0]), (p[y], p1[0])):
+            assert (x - x1).abs().max() < 100 * torch.finfo(dtype).eps * x1.abs().max()
