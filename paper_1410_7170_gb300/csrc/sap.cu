@@ -78,8 +78,46 @@ __device__ __forceinline__ void sm_load_link(const float4 *u, int nb, int mu, in
     }
     reconstruct_row2(m);
 }
-// q = D_BB s at local site t (local coords l, extents bx), links of the block in smem.
-template <typename R, typename LT, typename ST>
+// The one hop of a site of a 2^4 block in direction mu, to site n, forward or backward: with sg = -1 forward and +1
+// backward, h = up + sg c low and the lower spins sg c^* a; the link is the site's, or the neighbour's
+// adjoint. The same sums in the same order as the two branches of block_apply.
+__device__ __forceinline__ void sap_one_hop(const float4 *s, const float4 *u, int nb, int mu, int t, int n, bool fwd,
+                                            cpx<float> acc[12]) {
+    const float sg = fwd ? -1.f : 1.f;
+    cpx<float> v[12], h0[3], h1[3], a0[3], a1[3], m[3][3];
+    sm_load_sp(s, nb, n, v);
+    sm_load_link(u, nb, mu, fwd ? t : n, m);
+    const bool cross = mu == 1 || mu == 2, turn = mu == 1 || mu == 3;
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+        const cpx<float> low0 = v[(cross ? 9 : 6) + c], low1 = v[(cross ? 6 : 9) + c];
+        const float s0 = mu == 0 ? sg : -sg, s1 = mu == 1 ? -sg : sg;
+        h0[c] = v[c] + s0 * (turn ? mul_i(low0) : low0);
+        h1[c] = v[3 + c] + s1 * (turn ? mul_i(low1) : low1);
+    }
+#pragma unroll
+    for (int a = 0; a < 3; a++)
+#pragma unroll
+        for (int b = a; b < 3; b++) {
+            const cpx<float> x = m[a][b], y = m[b][a];
+            m[a][b] = cpx<float>{fwd ? x.re : y.re, fwd ? x.im : -y.im};
+            m[b][a] = cpx<float>{fwd ? y.re : x.re, fwd ? y.im : -x.im};
+        }
+    su3_mul(m, h0, a0);
+    su3_mul(m, h1, a1);
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+        const cpx<float> l2 = cross ? a1[c] : a0[c], l3 = cross ? a0[c] : a1[c];
+        acc[c] = acc[c] + a0[c];
+        acc[3 + c] = acc[3 + c] + a1[c];
+        acc[6 + c] = acc[6 + c] + sg * (turn ? mul_i(l2) : l2);
+        acc[9 + c] = acc[9 + c] + (mu >= 2 ? -sg : sg) * (turn ? mul_i(l3) : l3);
+    }
+}
+
+// q = D_BB s at local site t (local coords l, extents bx), links of the block in smem. TWO (FP32): all
+// extents are 2, where a site has one hop per direction and its warp would run through both branches.
+template <typename R, typename LT, typename ST, bool TWO = false>
 __device__ __forceinline__ void block_apply(const ST *s, const LT *u, int nb, int t, const int l[4], const int bx[4],
                                             const int stride[4], R m4, cpx<R> q[12]) {
     cpx<R> acc[12];
@@ -87,6 +125,10 @@ __device__ __forceinline__ void block_apply(const ST *s, const LT *u, int nb, in
     for (int c = 0; c < 12; c++) acc[c] = cpx<R>{0, 0};
 #pragma unroll
     for (int mu = 0; mu < 4; mu++) {
+        if constexpr (TWO) {
+            sap_one_hop(s, u, nb, mu, t, t ^ (8 >> mu), l[mu] == 0, acc);
+            continue;
+        }
         if (l[mu] + 1 < bx[mu]) {
             cpx<R> v[12], h0[3], h1[3], a0[3], a1[3], m[3][3];
             sm_load_sp(s, nb, t + stride[mu], v);
@@ -289,12 +331,12 @@ __device__ __forceinline__ void sap_out_dir(const Geom &g, const SapGeom &sg, co
 // second colour's blocks. Right-hand sides of a batch are grid rows. One Schwarz application (two
 // cycles, 6 MR steps), one thread per site without these savings -> two threads per site with them ->
 // this form: 16^4 183 -> 142 -> 139 us, 24^4 621 -> 586 -> 492, 32^4 1593 -> 1632 -> 1254.
-template <int START, bool ADD>
+template <int START, bool ADD, bool TWO>
 __global__ void __launch_bounds__(kBlock, 2)
     k_sap_site32(Geom g, SapGeom sg, const float4 *__restrict__ U, const float4 *__restrict__ v, float4 *x, long stride,
                  RowList rows, float m4, int colour, int mr_iters, bool colour_grid) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int nb = sg.nb;
+    const int nb = TWO ? 16 : sg.nb;
     int B[4];
     if (!sap_block_of(sg, blockIdx.x, colour, colour_grid, B)) return;   // uniform over the CTA
     v += rows.row[blockIdx.y] * stride;
@@ -346,7 +388,7 @@ __global__ void __launch_bounds__(kBlock, 2)
             for (int c = 0; c < 6; c++)
                 s[c * nb + t] = make_float4(res[2 * c].re, res[2 * c].im, res[2 * c + 1].re, res[2 * c + 1].im);
         __syncthreads();
-        if (act) block_apply<float, float4, float4>(s, u, nb, t, l, sg.b, sg.stride, m4, q);
+        if (act) block_apply<float, float4, float4, TWO>(s, u, nb, t, l, sg.b, sg.stride, m4, q);
         float a0 = 0.f, a1 = 0.f, a2 = 0.f;
 #pragma unroll
         for (int c = 0; c < 12; c++) {
@@ -401,18 +443,29 @@ static SapGrid sap_grid(const SapGeom &sg) {
     return SapGrid{even, even ? n / 2 : n};
 }
 
-template <int START, bool ADD>
-static cudaError_t launch_sap32(const Geom &g, const SapGeom &sg, const SapGrid &sp, const float4 *U, const float4 *v,
+template <int START, bool ADD, bool TWO>
+static cudaError_t launch_sap32_form(const Geom &g, const SapGeom &sg, const SapGrid &sp, const float4 *U, const float4 *v,
                                 float4 *x, long stride, const RowList &rows, float m4, int colour, int mr_iters,
                                 cudaStream_t st) {
     static size_t granted = 0;
     const size_t smem = (size_t)sg.nb * (kSapSpinor32 + 4 * kSapLink32) * sizeof(float4);
-    cudaError_t e = grant_smem(k_sap_site32<START, ADD>, smem, granted);
+    cudaError_t e = grant_smem(k_sap_site32<START, ADD, TWO>, smem, granted);
     if (e != cudaSuccess) return e;
-    k_sap_site32<START, ADD><<<dim3(sp.blocks, rows.n), (sg.nb + 31) / 32 * 32, smem, st>>>(
+    k_sap_site32<START, ADD, TWO><<<dim3(sp.blocks, rows.n), (sg.nb + 31) / 32 * 32, smem, st>>>(
         g, sg, U, v, x, stride, rows, m4, colour, mr_iters, sp.even);
     count_launches(1);
     return cudaGetLastError();
+}
+
+template <int START, bool ADD>
+static cudaError_t launch_sap32(const Geom &g, const SapGeom &sg, const SapGrid &sp, const float4 *U, const float4 *v,
+                                float4 *x, long stride, const RowList &rows, float m4, int colour, int mr_iters,
+                                cudaStream_t st) {
+    // blocks of 16 sites are 2^4. One cycle (us) with the best of one, two and four threads per site, with
+    // the general form, and with the one for 2^4: 4^4 30 / 37 / 25, 8^4 35 / 37 / 28, 12^4 47 / 47 / 35, 16^4
+    // 82 / 76 / 54, 24^4 332 / 316 / 223. A CTA is one warp there, bound by fetching its instructions.
+    return sg.nb == 16 ? launch_sap32_form<START, ADD, true>(g, sg, sp, U, v, x, stride, rows, m4, colour, mr_iters, st)
+               : launch_sap32_form<START, ADD, false>(g, sg, sp, U, v, x, stride, rows, m4, colour, mr_iters, st);
 }
 
 cudaError_t sap_f32_rows(const Geom &g, const SapGeom &sg, const float4 *U, const float4 *v, float4 *x, float4 *r,

@@ -1,5 +1,6 @@
 // Host functions of the library that no entry point reaches alone, with C linkage for the tests.
 #include "../paper_1410_7170_gb300/csrc/internal.h"
+#include "../paper_1410_7170_gb300/csrc/sap.h"
 
 using namespace ovl;
 
@@ -143,6 +144,33 @@ extern "C" int t_ms_probe(const int *dims, const double *gauge, int fp64, int tp
                               (float4 *)p0);
     cudaFree(u64);
     cudaFree(u32);
+    cudaFree(bad);
+    return st;
+}
+
+// One Schwarz application to n boundary vectors (device memory, back to back) as the batched solvers make
+// it: rows with act[y] = 0 are left out
+extern "C" int t_sap_rows_f32(const int *dims, const double *gauge, const int *block, const double *in, double *out,
+                              const char *act, int n, double m0, int cycles, int mr_iters) {
+    const Geom g = geom(dims);
+    const long words = 6L * g.V;
+    double2 *u64 = nullptr;
+    float4 *u32 = nullptr, *v = nullptr;
+    int *bad = nullptr;
+    cudaError_t e = cudaMalloc(&u64, (size_t)g.V * 4 * kLink64Words * sizeof(double2));
+    if (e == cudaSuccess) e = cudaMalloc(&u32, (size_t)g.V * 4 * 3 * sizeof(float4));
+    if (e == cudaSuccess) e = cudaMalloc(&v, (size_t)words * (2 * n + 1) * sizeof(float4));
+    if (e == cudaSuccess) e = cudaMalloc(&bad, sizeof(int));
+    if (e == cudaSuccess) e = cudaMemset(v, 0xff, (size_t)words * (2 * n + 1) * sizeof(float4));   // NaN
+    if (e == cudaSuccess) e = pack_gauge(g, gauge, u64, u32, bad, 1e-10, 0);
+    if (e == cudaSuccess) e = spinor_in(g, v, words, in, n, InputFlags{nullptr, nullptr}, 0);
+    float4 *x = v + words * n, *r = x + words * n;
+    if (e == cudaSuccess) e = sap_f32_rows(g, make_sap_geom(g, block), u32, v, x, r, words, n, act, (float)m0, cycles, mr_iters, 0);
+    if (e == cudaSuccess) e = spinor_out(g, out, x, words, n, nullptr, 0);
+    const int st = done(e);
+    cudaFree(u64);
+    cudaFree(u32);
+    cudaFree(v);
     cudaFree(bad);
     return st;
 }
