@@ -318,10 +318,12 @@ ovl_status ovl_zolotarev(double k, int n, double *d0, double *a, double *c, doub
 /* Instrumentation of the running library (used by the benchmark; not part of the
  * paper's method). With profiling enabled, the multishift CG records CUDA events around
  * the three kernels of one iteration of every queued chunk of check_every iterations
- * (the middle one; event nodes inside the captured graphs), a sample that keeps the
+ * (the first that updates the shifts, and the p_0 kernel of the one before it; event nodes
+ * inside the captured graphs), a sample that keeps the
  * event nodes from slowing the other iterations, and logs the shifts each iteration
- * updated, so that algorithmic bytes (reals per site: Q p 96, residual update 144, shift
- * update 72 + 48 per updated shift) are known for every launch. The achieved rate of a
+ * updated, so that algorithmic bytes are known for every launch (reals per site: Q p 96, residual
+ * update 144; p_0 and the shift updates of k iterations together 120 k + 48 per updated
+ * shift, an iteration counting its share). The achieved rate of a
  * class is timed_bytes / ms (or timed flops / ms); its total time is estimated as
  * ms / timed * launches. */
 typedef struct {

@@ -982,8 +982,9 @@ ovl_status Ctx::sigma_min_estimate(double *smin) {
 
 // ------------------------------------------------------------------ autotuner
 // Threads per site of the FP32 stencil (1 or 4) for this lattice shape: both variants are timed
-// with CUDA events on the context's stream and the faster is kept; the FP64 stencil (one kernel
-// for all sizes) is timed beside them. Results are cached per process and shape.
+// with CUDA events on the context's stream and the faster is kept (for the stencils inside the solvers: one
+// FP32 sign at 8^4 1.50 -> 1.19 ms); the FP64 stencil (its form follows from the lattice) is timed
+// beside them. Results are cached per process and shape.
 static std::mutex g_tune_mu;
 struct TuneEntry {
     int tps32;
@@ -1707,6 +1708,7 @@ extern "C" ovl_status wilson_apply_n_arith(ovl_ctx *ctx, double *out, const doub
     // multi-RHS kernel shares do not pay for a kernel of its own on the way out (whole call, us per
     // right-hand side, the best multi-RHS kernel and way out -> one stencil per right-hand side that
     // writes the answer: 16^4 14.0 -> 11.7 at 12 and 20.8 -> 17.4 at 3, 24^4 60.2 -> 52.0, 32^4 201 -> 173).
+    // On the small ones the two ways differ by less than 1 us a call (one vector at 8^4 27.0 against 27.4).
     const bool direct = late && c->g.tps32 == 1 && !c->p.mrhs_kernel;
     float4 *fa = (float4 *)c->fbat, *fb = fa + (size_t)blk * wf;
     for (int r0 = 0; r0 < n_rhs; r0 += blk) {

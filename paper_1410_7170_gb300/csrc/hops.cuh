@@ -6,20 +6,21 @@
 // and run the caller's epilogue.
 //
 // Used for small lattices in FP32 (the autotuner's choice: 8^4 5.8 -> 4.2 us a stencil, 16^4 8.3 -> 12.4,
-// where the shared memory traffic costs more than the extra warps give) and at all sizes for the
-// arithmetics that are bound by their own instructions, FP64 (2 lanes per clock and
-// SM on GB300, so a warp's FP64 instruction holds the SM's unit for 16 clocks) and float-float
-// (about 10k FP32 operations per site):
+// where the shared memory traffic costs more than the extra warps give), at all sizes in float-float (about
+// 10k FP32 operations per site), and in FP64 (2 lanes per clock and SM on GB300, so a warp's FP64
+// instruction holds the SM's unit for 16 clocks) but for some large lattices, where one thread per
+// site is up to 3% faster (wilson_f64, ms_fp64_per_site):
 //   * the work of a tile is spread evenly over the four schedulers. One thread per site fills
 //     them only from about 150 x 2 x 256 sites on; at 8^4 its 304 blocks of 14 sites used two
 //     schedulers of each SM with 14 of 32 lanes live;
 //   * no thread holds the 24 accumulators of a site while it computes a hop, so three blocks
 //     fit on an SM at 80 registers instead of two of one-thread-per-site blocks at 128;
 //   * the direction is uniform in a warp: no divergence and no multiplications by spin units.
-// The sum of the FP64 instructions per site is that of the one-thread form. One stencil, one thread
-// per site -> one warp per hop (us): FP64 4^4 33 -> 8, 8^4 33 -> 12, 12^4 51 -> 39, 16^4 111 -> 109,
-// 32^4 1688 -> 1681 (the FP64 units' measured rate allows 1730 with the epilogue: 888 FP64
-// instructions per site); float-float 8^4 25 -> 6, 16^4 38 -> 29, 24^4 194 -> 138, 32^4 535 -> 418.
+// The sum of the FP64 instructions per site is that of the one-thread form, 888 with the epilogue. One
+// stencil, one thread per site -> one warp per hop (us): FP64 4^4 33 -> 8, 8^4 33 -> 12, 12^4 51 -> 39,
+// 16^4 111 -> 109, 32^4 1687 -> 1680; float-float 8^4 25 -> 6, 16^4 38 -> 29, 24^4 194 -> 138, 32^4 535 ->
+// 418. 32^4 in FP64 is 0.88 of the units' 2 lanes a clock (1479 us at the 2070 MHz of the run), 1.76 lanes;
+// ovl_fma_peak's chains of fused multiply-adds reach 1.68 and are no bound for it.
 #pragma once
 #include "reduce.cuh"
 #include "wilson_site.cuh"

@@ -53,8 +53,9 @@ __global__ void __launch_bounds__(384) k_wilson_mrhs(Geom g, const LT *__restric
 // and loops over the right-hand sides two at a time, applying every link it loads to both
 // (wilson_hop2). A block of 32 sites x nr right-hand sides (k_wilson_mrhs) shares the links
 // across right-hand sides too, but its blocks span one x3 row, so the x2 neighbours miss L1 and
-// the spinor gathers that bound this stencil grow; measured per right-hand side at 12 of them it
-// ran 1.16x the single-RHS time at 64x32^3, this loop 0.95x (32^4: 0.88x, 16^4: 0.52x).
+// the spinor gathers that bound this stencil grow. Per right-hand side at 12 of them, against one stencil of
+// one right-hand side (k_wilson, strided over the lattice in one wave): 64x32^3 171 against 168 us, 32^4 89
+// against 81, 24^4 25.5 against 31.3, 16^4 5.0 against 8.3.
 __global__ void __launch_bounds__(kBlock, 2) k_wilson_mrhs_pairs(Geom g, const float4 *__restrict__ U,
                                                                const float4 *__restrict__ in, float4 *__restrict__ out,
                                                                long stride, int nrhs, float m4, int g5, float a,
