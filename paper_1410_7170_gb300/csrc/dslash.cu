@@ -289,17 +289,16 @@ cudaError_t spinor_f2d(const Geom &g, const float4 *a, double2 *b, cudaStream_t 
 }
 
 // ------------------------------------------------------------------ stencil
-// out = a [g5] D_W(m0) in + b z, one thread per site, in FP32 and (wilson_f64) on some lattices in FP64. Bound in FP32: the latency of the neighbour gathers,
-// which go to L2 three times in four, at 16 warps per SM (128 registers); at 64 x 32^3 with memory 60%
-// and the L1 data pipe 48% busy (168 us: 0.70 of the copy bandwidth). One wave of blocks that stride
-// over the lattice keeps the blocks
-// of an SM and their neighbours on other SMs close together in time: 32^4 107 -> 90 us, 24^4 40 -> 35,
-// 64 x 32^3 182 -> 170, 16^4 10.2 -> 9.2, against a block per 256 sites; with the order of
-// site_of_thread 81, 31.3, 168 and 8.3.
+// out = a [g5] D_W(m0) in + b z, one thread per site, in FP32 and on some lattices in FP64 (wilson_f64).
+// Bound in FP32: the latency of the neighbour gathers, which go to L2 three times in four, at 16 warps
+// per SM (128 registers); at 64 x 32^3 with memory 60% and the L1 data pipe 48% busy (167 us: 0.71 of the
+// copy bandwidth). One wave of blocks that stride over the lattice keeps the blocks of an SM and their
+// neighbours on other SMs close together in time: 32^4 107 -> 90 us, 24^4 40 -> 35, 64 x 32^3 182 -> 170,
+// 16^4 10.2 -> 9.2, against a block per 256 sites; with the order of site_of_thread 81, 31.3, 168 and 8.3.
 template <typename R, typename ST>
 __global__ void __launch_bounds__(kBlock, MinBlocks<R>::value)
-    k_wilson(Geom g, const ST *__restrict__ U, const ST *__restrict__ in, ST *__restrict__ out, R m4, int g5, R a, const ST *z,
-             R b, int spb) {
+    k_wilson(Geom g, const ST *__restrict__ U, const ST *__restrict__ in, ST *__restrict__ out, R m4, int g5, R a,
+             const ST *z, R b, int spb) {
     if (threadIdx.x >= spb) return;
     for (int t = blockIdx.x * spb + threadIdx.x; t < g.V; t += gridDim.x * spb) {
         int p, i;

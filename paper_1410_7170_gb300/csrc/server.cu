@@ -117,7 +117,8 @@ size_t estimate_bytes(const ovl_request &r, const ovl_params &p, int ring) {
         const int nb = std::min(std::min(p.rhs_block, nrhs), 12);
         const int mo = std::min(p.restart, 32), mi = std::min(p.restart_inner, 32), mw = std::min(p.prec_restart, 16);
         b += nb * ((2 * mo + 5) * v64 + ovl::ms_vectors(p.n_poles, batch_ring) * v64);
-        if (mixed) b += nb * ((2 * mi + 3) * v32 + (2 * mw + 3) * v32 + ovl::ms_vectors(p.n_poles, batch_ring) * v32 + 2 * v32);
+        if (mixed)
+            b += nb * ((2 * mi + 3) * v32 + (2 * mw + 3) * v32 + ovl::ms_vectors(p.n_poles, batch_ring) * v32 + 2 * v32);
     } else {
         b += (2 * p.restart + 5) * v64;                   // outer FGMRES basis (V and Z)
         if (p.precond == OVL_PREC_RECURSIVE) b += (2 * p.restart_inner + 3) * v32;

@@ -82,8 +82,8 @@ struct Ctx {
     double *d_coef = nullptr;     // multi-axpy coefficients
     double *d_gs = nullptr;       // Gram-Schmidt records (kScal doubles)
     double *d_gs_coef = nullptr, *h_gs_coef = nullptr;   // coefficients of x += Z y (12 x 256; pinned copy)
-    int gs_level = 0;             // solvers that are running inside one another (GsLevel)
     unsigned *gs_counters = nullptr;                     // per right-hand side, zero between launches
+    int gs_level = 0;             // solvers that are running inside one another (GsLevel)
     // gauge field (12-real links)
     double2 *U64 = nullptr;
     float4 *U32 = nullptr;
@@ -253,8 +253,8 @@ struct Ctx {
     // fixed_rings is set (the serving loop, which reserved the memory for them and wants the same
     // results whatever else runs: the ring decides the order of additions in y).
     int ring_one = kMaxRing, ring_batch = kBatchRing;
-    int ff_part = kMaxBatch;   // right-hand sides of a float-float batch that are done together, as far as memory goes
     bool fixed_rings = false, rings_reduced = false;
+    int ff_part = kMaxBatch;   // right-hand sides of a float-float batch that the memory holds together
     ovl_status sign64_batch(const double2 *b, double2 *out, int nrhs, const double *tol, int mode);
     ovl_status sign_ff_batch(const double2 *b, double2 *out, int nrhs, const double *tol, int mode);
     ovl_status sign_outer_batch(const double2 *b, double2 *out, int nrhs, const double *tol, int mode);
